@@ -63,8 +63,10 @@ __device__ __forceinline__ void slab_gate(const float* __restrict__ qpart, int q
   }
   __syncthreads();
   float u = 0.f;   // (then a fixed-order butterfly)
+  if (gate_w != nullptr) {   // without weights the logits are the bias alone, whatever q-bar is (0 * inf)
 #pragma unroll
-  for (int j = 0; j < 4; ++j) u += gw[j] * qs[seg * 4 + j];
+    for (int j = 0; j < 4; ++j) u += gw[j] * qs[seg * 4 + j];
+  }
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
   if (i < L1 && seg == 0) {
@@ -335,7 +337,7 @@ __global__ void __launch_bounds__(256) k_gate_backward(
             const float du = dus[q + 4 * r][i];
             gw_acc[i] += qb[r] * du;
             gb_acc[i] += du;
-            dq += gw[i] * du;
+            if (gate_w != nullptr) dq += gw[i] * du;   // (none without weights, whatever du is)
           }
         dqbar[((size_t)b * H + h) * kD + c] = dq;
       }
