@@ -714,7 +714,7 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
         const float* zr = zs + 32 * wq;
         // ---- R, D'
         uint32_t rp[NH][16];
-        float den = 0.f, den2 = 0.f;   // (twice their share of D')
+        float den = 0.f, den2 = 0.f;
         f32x2 num = pk2(0.f, 0.f);
         if (__any_sync(0xffffffffu, *abort_flag != 0)) ok = false;
         wait_all(&bars->a_full, par);
@@ -739,11 +739,10 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
               if constexpr (!kGroup) {
                 if ((j & 3) == 0) asm volatile("" ::: "memory");   // (z' is read as it is used, not kept in registers)
                 const float4 z = *reinterpret_cast<const float4*>(zr + h * 128 + 2 * j);
-                // 2 ReLU(a) = a + |a|: an add at full rate where a maximum would take two cycles
-                den = fmaf(a[0] + fabsf(a[0]), z.x, den);
-                den2 = fmaf(a[1] + fabsf(a[1]), z.y, den2);
-                den = fmaf(a[2] + fabsf(a[2]), z.z, den);
-                den2 = fmaf(a[3] + fabsf(a[3]), z.w, den2);
+                den = fmaf(fmaxf(a[0], 0.f), z.x, den);
+                den2 = fmaf(fmaxf(a[1], 0.f), z.y, den2);
+                den = fmaf(fmaxf(a[2], 0.f), z.z, den);
+                den2 = fmaf(fmaxf(a[3], 0.f), z.w, den2);
               }
             }
           }
@@ -769,7 +768,7 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
 #pragma unroll
               for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(rp[h][8 + j]), pk2u(b[2 * j], b[2 * j + 1]), num);
             }
-            const uint32_t st[2] = {__float_as_uint(0.5f * (den + den2)), __float_as_uint(sum2(num))};
+            const uint32_t st[2] = {__float_as_uint(den + den2), __float_as_uint(sum2(num))};
             tmem_st2(trow + kStat + 2 * wq, st);
             tmem_st_wait();
             tc_fence_before_sync();
