@@ -336,9 +336,8 @@ k_tc_bwd_kside(const __grid_constant__ CUtensorMap map_kf, const __grid_constant
     const uint32_t trow = tmem + ((32u * (warp & 3)) << 16) + 32 * wq;   // this warp's lane quarter and columns
     uint32_t b = 0, par = 0;   // accumulator and phase of the next unit
     bool ok = true;
-    auto wait_unit = [&]() {   // one warp of a lane quarter polls, the others sleep (see k_tc_bwd_qside)
-      if (wq == 0 && ok) ok = __all_sync(0xffffffffu, mbar_wait(&bars->d_full[b], par, abort_flag, status, kErrBwdMma));
-      named_bar_sync(2 + (warp & 3), 128);
+    auto wait_unit = [&]() {   // one warp of a lane quarter polls
+      ok = group_wait(&bars->d_full[b], par, wq == 0, ok, 2 + (warp & 3), 128, abort_flag, status, kErrBwdMma);
       if (ok) tc_fence_after_sync();
     };
     auto done_unit = [&]() {
@@ -352,7 +351,6 @@ k_tc_bwd_kside(const __grid_constant__ CUtensorMap map_kf, const __grid_constant
     };
     for (int it = 0; it < nt; ++it) {
       const int slab = (g0 + it) / tps;
-      if (__any_sync(0xffffffffu, *abort_flag != 0)) ok = false;
       uint32_t rp[NH][16];
 #pragma unroll
       for (int h = 0; h < NH; ++h) {
@@ -692,15 +690,13 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
     const int dz_ch = et % kChunks, dz_t0 = (et / kChunks) * kDzTok;
     bool ok = true;
     float sum_dd = 0.f;   // wq = 0: sum of dD' over this thread's tokens
-    // One of the four warps of a lane quarter polls the barrier, the others sleep at a named barrier: polls are
-    // shared-memory reads, and the tensor core needs that bandwidth for its operands.
+    // One of the four warps of a lane quarter polls the barrier; the quarter goes on as one or not at all.
     auto wait_all = [&](uint64_t* bar, uint32_t par) {
-      if (wq == 0 && ok) ok = __all_sync(0xffffffffu, mbar_wait(bar, par, abort_flag, status, kErrBwdMma));
-      named_bar_sync(2 + (warp & 3), 128);
+      ok = group_wait(bar, par, wq == 0, ok, 2 + (warp & 3), 128, abort_flag, status, kErrBwdMma);
       if (ok) tc_fence_after_sync();
     };
     int it = 0;
-    for (int gt = g0; gt < g1;) {
+    for (int gt = g0; gt < g1 && ok;) {
       const int slab = gt / tps, seg_end = min(g1, (slab + 1) * tps);
       // (every thread is past its last use of z' and of the scratch)
       if (et < m) zs[et] = zg[(size_t)slab * z_stride + et];
@@ -713,143 +709,143 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
         const int row0 = (gt - slab * tps) * kTile, row = row0 + tl;
         const float* zr = zs + 32 * wq;
         // ---- R, D'
-        uint32_t rp[NH][16];
-        float den = 0.f, den2 = 0.f;
-        f32x2 num = pk2(0.f, 0.f);
-        if (__any_sync(0xffffffffu, *abort_flag != 0)) ok = false;
+        float inv = 0.f, c = 0.f;
         wait_all(&bars->a_full, par);
-        if (ok) {
-          uint32_t r[NH][32];
+        if (ok) {   // (every wait has one answer for the lane quarter: its barriers may stand inside)
+          uint32_t rp[NH][16];
+          float den = 0.f, den2 = 0.f;
+          f32x2 num = pk2(0.f, 0.f);
+          {
+            uint32_t r[NH][32];
 #pragma unroll
-          for (int h = 0; h < NH; ++h) tmem_ld32(trow + h * 128 + 32 * wq, r[h]);
-          tmem_ld_wait();
+            for (int h = 0; h < NH; ++h) tmem_ld32(trow + h * 128 + 32 * wq, r[h]);
+            tmem_ld_wait();
 #pragma unroll
-          for (int h = 0; h < NH; ++h) reg_fence32(r[h]);
-          tc_fence_before_sync();
-          warp_arrive(&bars->a_read);   // X may become G
+            for (int h = 0; h < NH; ++h) reg_fence32(r[h]);
+            tc_fence_before_sync();
+            warp_arrive(&bars->a_read);   // X may become G
 #pragma unroll
-          for (int h = 0; h < NH; ++h) {
+            for (int h = 0; h < NH; ++h) {
 #pragma unroll
-            for (int j = 0; j < 16; j += 2) {
-              float a[4];
+              for (int j = 0; j < 16; j += 2) {
+                float a[4];
 #pragma unroll
-              for (int i = 0; i < 4; ++i) a[i] = __uint_as_float(r[h][2 * j + i]);
-              rp[h][j] = relu_pack_bf16x2(a[0], a[1]);
-              rp[h][j + 1] = relu_pack_bf16x2(a[2], a[3]);
-              if constexpr (!kGroup) {
-                if ((j & 3) == 0) asm volatile("" ::: "memory");   // (z' is read as it is used, not kept in registers)
-                const float4 z = *reinterpret_cast<const float4*>(zr + h * 128 + 2 * j);
-                den = fmaf(fmaxf(a[0], 0.f), z.x, den);
-                den2 = fmaf(fmaxf(a[1], 0.f), z.y, den2);
-                den = fmaf(fmaxf(a[2], 0.f), z.z, den);
-                den2 = fmaf(fmaxf(a[3], 0.f), z.w, den2);
+                for (int i = 0; i < 4; ++i) a[i] = __uint_as_float(r[h][2 * j + i]);
+                rp[h][j] = relu_pack_bf16x2(a[0], a[1]);
+                rp[h][j + 1] = relu_pack_bf16x2(a[2], a[3]);
+                if constexpr (!kGroup) {
+                  if ((j & 3) == 0) asm volatile("" ::: "memory");   // (z' is read as it is used, not kept in registers)
+                  const float4 z = *reinterpret_cast<const float4*>(zr + h * 128 + 2 * j);
+                  den = fmaf(fmaxf(a[0], 0.f), z.x, den);
+                  den2 = fmaf(fmaxf(a[1], 0.f), z.y, den2);
+                  den = fmaf(fmaxf(a[2], 0.f), z.z, den);
+                  den2 = fmaf(fmaxf(a[3], 0.f), z.w, den2);
+                }
               }
             }
           }
-        }
-        float inv = 0.f, c = 0.f;
-        if constexpr (!kGroup) {
           // ---- num = R . G, and the row sums over the four threads of a token
           wait_all(&bars->g_full, par);
+          if constexpr (!kGroup) {
+            if (ok) {
+              uint32_t a[16], b[16];
+              tmem_ld16(trow + 32 * wq, a);
+#pragma unroll
+              for (int h = 0; h < NH; ++h) {
+                reg_fence16(rp[h]);   // (R is unpacked again in every pass, not kept unpacked)
+                tmem_ld_wait();
+                reg_fence16(a);
+                tmem_ld16(trow + h * 128 + 32 * wq + 16, b);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(rp[h][j]), pk2u(a[2 * j], a[2 * j + 1]), num);
+                tmem_ld_wait();
+                reg_fence16(b);
+                if (h + 1 < NH) tmem_ld16(trow + (h + 1) * 128 + 32 * wq, a);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(rp[h][8 + j]), pk2u(b[2 * j], b[2 * j + 1]), num);
+              }
+              const uint32_t st[2] = {__float_as_uint(den + den2), __float_as_uint(sum2(num))};
+              tmem_st2(trow + kStat + 2 * wq, st);
+              tmem_st_wait();
+              tc_fence_before_sync();
+            }
+          }
+          if (it > 0) wait_all(&bars->p_free, par ^ 1);   // (long past, as a rule; also the barrier behind the row sums)
+          else named_bar_sync(2 + (warp & 3), 128);
           if (ok) {
-            uint32_t a[16], b[16];
-            tmem_ld16(trow + 32 * wq, a);
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-              reg_fence16(rp[h]);   // (R is unpacked again in every pass, not kept unpacked)
+            if constexpr (kGroup) {
+              if (row < n) {
+                const float D = den_ext[(size_t)slab * n + row];
+                inv = 1.f / D;
+                c = dd_ext[(size_t)slab * n + row] * D;
+              }
+            } else {
+              tc_fence_after_sync();
+              uint32_t st[8];
+              tmem_ld8(trow + kStat, st);
               tmem_ld_wait();
-              reg_fence16(a);
-              tmem_ld16(trow + h * 128 + 32 * wq + 16, b);
+              reg_fence8(st);
+              auto total = [&](int i) {
+                return (__uint_as_float(st[i]) + __uint_as_float(st[2 + i])) +
+                       (__uint_as_float(st[4 + i]) + __uint_as_float(st[6 + i]));
+              };
+              if (row < n) {   // rows past the end contribute nothing
+                inv = 1.f / (epsp + total(0));
+                c = -total(1) * inv;
+              }
+            }
+            if (wq == 0) {
+              cs[tl] = c;
+              sum_dd += c * inv;
+            }
+            // ---- dA D (hi + lo, in place) and R / D, 16 features at a time
+            // (an instruction on the ALU pipe takes a scheduler two cycles, one on the FMA pipe one: the mask 1[R > 0]
+            // is a saturating product, 1 for every normal R > 0, and multiplies dA, instead of compares and selects)
+            uint32_t a[2][16];
+            tmem_ld16(trow + 32 * wq, a[0]);
 #pragma unroll
-              for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(rp[h][j]), pk2u(a[2 * j], a[2 * j + 1]), num);
+            for (int h = 0; h < NH; ++h) reg_fence16(rp[h]);
+#pragma unroll
+            for (int s = 0; s < 2 * NH; ++s) {
+              const int h = s >> 1, q = s & 1;
+              const uint32_t col = trow + h * 128 + 32 * wq + 16 * q;
+              uint32_t(&g)[16] = a[s & 1];
               tmem_ld_wait();
-              reg_fence16(b);
-              if (h + 1 < NH) tmem_ld16(trow + (h + 1) * 128 + 32 * wq, a);
+              reg_fence16(g);
+              if (s + 1 < 2 * NH) tmem_ld16(trow + ((s + 1) >> 1) * 128 + 32 * wq + 16 * ((s + 1) & 1), a[(s + 1) & 1]);
+              const float* z = zr + h * 128 + 16 * q;
+              uint32_t ph[8], pl[8], pp[8];
 #pragma unroll
-              for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(rp[h][8 + j]), pk2u(b[2 * j], b[2 * j + 1]), num);
+              for (int j = 0; j < 8; ++j) {
+                if ((j & 1) == 0) asm volatile("" ::: "memory");
+                const float2 zz = *reinterpret_cast<const float2*>(z + 2 * j);
+                const uint32_t rw = rp[h][8 * q + j];
+                const float r0 = __uint_as_float(rw << 16), r1 = __uint_as_float(rw & 0xFFFF0000u);
+                const float v0 = fmaf(c, zz.x, __uint_as_float(g[2 * j])) * __saturatef(r0 * 0x1p127f);
+                const float v1 = fmaf(c, zz.y, __uint_as_float(g[2 * j + 1])) * __saturatef(r1 * 0x1p127f);
+                ph[j] = pack_bf16x2(v0, v1);
+                pl[j] = pack_bf16x2(v0 - __uint_as_float(ph[j] << 16), v1 - __uint_as_float(ph[j] & 0xFFFF0000u));
+                pp[j] = pack_bf16x2(r0 * inv, r1 * inv);
+              }
+              tmem_st8(col, ph);
+              tmem_st8(col + 8, pl);
+              uint8_t* blk = pt + (2 * h + (wq >> 1)) * kTileBytes;
+              const uint32_t ch = 4 * (wq & 1) + 2 * q;
+              *reinterpret_cast<uint4*>(blk + swz128(tl, ch)) = make_uint4(pp[0], pp[1], pp[2], pp[3]);
+              *reinterpret_cast<uint4*>(blk + swz128(tl, ch + 1)) = make_uint4(pp[4], pp[5], pp[6], pp[7]);
+              tmem_st_wait();
+              if (q == 1) fence_proxy_async_smem();   // R / D of the half, for the MMA of dS'
+              else asm volatile("" ::: "memory");
+              tc_fence_before_sync();
+              warp_arrive(&bars->da_ready[s]);
             }
-            const uint32_t st[2] = {__float_as_uint(den + den2), __float_as_uint(sum2(num))};
-            tmem_st2(trow + kStat + 2 * wq, st);
-            tmem_st_wait();
-            tc_fence_before_sync();
-          }
-        } else {
-          wait_all(&bars->g_full, par);
-        }
-        if (it > 0) wait_all(&bars->p_free, par ^ 1);   // (long past, as a rule; also the barrier behind the row sums)
-        else named_bar_sync(2 + (warp & 3), 128);
-        if (ok) {
-          if constexpr (kGroup) {
-            if (row < n) {
-              const float D = den_ext[(size_t)slab * n + row];
-              inv = 1.f / D;
-              c = dd_ext[(size_t)slab * n + row] * D;
-            }
-          } else {
-            tc_fence_after_sync();
-            uint32_t st[8];
-            tmem_ld8(trow + kStat, st);
-            tmem_ld_wait();
-            reg_fence8(st);
-            auto total = [&](int i) {
-              return (__uint_as_float(st[i]) + __uint_as_float(st[2 + i])) +
-                     (__uint_as_float(st[4 + i]) + __uint_as_float(st[6 + i]));
-            };
-            if (row < n) {   // rows past the end contribute nothing
-              inv = 1.f / (epsp + total(0));
-              c = -total(1) * inv;
-            }
-          }
-          if (wq == 0) {
-            cs[tl] = c;
-            sum_dd += c * inv;
-          }
-          // ---- dA D (hi + lo, in place) and R / D, 16 features at a time
-          // (an instruction on the ALU pipe takes a scheduler two cycles, one on the FMA pipe one: the mask 1[R > 0]
-          // is a saturating product, 1 for every normal R > 0, and multiplies dA, instead of compares and selects)
-          uint32_t a[2][16];
-          tmem_ld16(trow + 32 * wq, a[0]);
-#pragma unroll
-          for (int h = 0; h < NH; ++h) reg_fence16(rp[h]);
-#pragma unroll
-          for (int s = 0; s < 2 * NH; ++s) {
-            const int h = s >> 1, q = s & 1;
-            const uint32_t col = trow + h * 128 + 32 * wq + 16 * q;
-            uint32_t(&g)[16] = a[s & 1];
-            tmem_ld_wait();
-            reg_fence16(g);
-            if (s + 1 < 2 * NH) tmem_ld16(trow + ((s + 1) >> 1) * 128 + 32 * wq + 16 * ((s + 1) & 1), a[(s + 1) & 1]);
-            const float* z = zr + h * 128 + 16 * q;
-            uint32_t ph[8], pl[8], pp[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              if ((j & 1) == 0) asm volatile("" ::: "memory");
-              const float2 zz = *reinterpret_cast<const float2*>(z + 2 * j);
-              const uint32_t rw = rp[h][8 * q + j];
-              const float r0 = __uint_as_float(rw << 16), r1 = __uint_as_float(rw & 0xFFFF0000u);
-              const float v0 = fmaf(c, zz.x, __uint_as_float(g[2 * j])) * __saturatef(r0 * 0x1p127f);
-              const float v1 = fmaf(c, zz.y, __uint_as_float(g[2 * j + 1])) * __saturatef(r1 * 0x1p127f);
-              ph[j] = pack_bf16x2(v0, v1);
-              pl[j] = pack_bf16x2(v0 - __uint_as_float(ph[j] << 16), v1 - __uint_as_float(ph[j] & 0xFFFF0000u));
-              pp[j] = pack_bf16x2(r0 * inv, r1 * inv);
-            }
-            tmem_st8(col, ph);
-            tmem_st8(col + 8, pl);
-            uint8_t* blk = pt + (2 * h + (wq >> 1)) * kTileBytes;
-            const uint32_t ch = 4 * (wq & 1) + 2 * q;
-            *reinterpret_cast<uint4*>(blk + swz128(tl, ch)) = make_uint4(pp[0], pp[1], pp[2], pp[3]);
-            *reinterpret_cast<uint4*>(blk + swz128(tl, ch + 1)) = make_uint4(pp[4], pp[5], pp[6], pp[7]);
-            tmem_st_wait();
-            if (q == 1) fence_proxy_async_smem();   // R / D of the half, for the MMA of dS'
-            else asm volatile("" ::: "memory");
-            tc_fence_before_sync();
-            warp_arrive(&bars->da_ready[s]);
           }
         }
-        named_bar_sync(1, kQElem);
+        ok = named_bar_all(1, kQElem, ok);
+        if (!ok) break;   // (all quarters together)
         // ---- dz' += (R / D)^T c: thread = eight features (a 16-byte chunk) x kDzTok tokens.  (As warp-level MMAs the
         // same sums waited for the tensor pipe, which is busy here: 2.9 k cycles.)
-        if (ok) {
+        {
           const uint8_t* blk = pt + (dz_ch >> 3) * kTileBytes;
 #pragma unroll
           for (int t = 0; t < kDzTok; t += 4) {
@@ -876,8 +872,9 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
           reg_fence16(r);
           tc_fence_before_sync();
         }
-        named_bar_sync(1, kQElem);   // the dz' pass has read R / D (and dS' has: its MMAs precede dq_full)
-        if (ok) {
+        ok = named_bar_all(1, kQElem, ok);   // the dz' pass has read R / D (and dS' has: its MMAs precede dq_full)
+        if (!ok) break;
+        {
           uint8_t* box = pt + (wq >> 1) * kTileBytes;
 #pragma unroll
           for (int q = 0; q < 4; ++q)
@@ -886,10 +883,11 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
                             __uint_as_float(r[4 * q + 2]) * inv, __uint_as_float(r[4 * q + 3]) * inv);
           fence_proxy_async_smem();
         }
-        if (ok) warp_arrive(&bars->staged);
+        warp_arrive(&bars->staged);
       }
+      if (!ok) break;
       // ---- end of the segment: partial dS', dz' (every MMA of the segment has completed)
-      if (et == 0 && ok && gt < g1) mbar_arrive(&bars->s_free);
+      if (et == 0 && gt < g1) mbar_arrive(&bars->s_free);
       {
         float* dst = scratch + (et / kChunks) * m + 8 * dz_ch;
         *reinterpret_cast<float4*>(dst) = make_float4(dz[0], dz[1], dz[2], dz[3]);
@@ -897,28 +895,26 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
       }
       named_bar_sync(1, kQElem);
       const size_t pidx = (size_t)blockIdx.x + slab;
-      if (ok) {
-        tc_fence_after_sync();
-        if (et < m) {
-          float s = 0.f;
+      tc_fence_after_sync();
+      if (et < m) {
+        float s = 0.f;
 #pragma unroll
-          for (int q = 0; q < kQElem / kChunks; ++q) s += scratch[q * m + et];
-          dzpart[pidx * m + et] = s;
-        }
-#pragma unroll
-        for (int ii = 0; ii < NH; ++ii) {
-          const int i = wq * NH + ii, h = i >> 2, cc = i & 3;   // 16 columns of one half
-          uint32_t r[16];
-          tmem_ld16(trow + kAccS + h * 64 + 16 * cc, r);
-          tmem_ld_wait();
-          reg_fence16(r);
-          float* dst = dspart + (pidx * m + h * 128 + tl) * kD + 16 * cc;
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<uint4*>(dst + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
-        }
-        tc_fence_before_sync();
+        for (int q = 0; q < kQElem / kChunks; ++q) s += scratch[q * m + et];
+        dzpart[pidx * m + et] = s;
       }
+#pragma unroll
+      for (int ii = 0; ii < NH; ++ii) {
+        const int i = wq * NH + ii, h = i >> 2, cc = i & 3;   // 16 columns of one half
+        uint32_t r[16];
+        tmem_ld16(trow + kAccS + h * 64 + 16 * cc, r);
+        tmem_ld_wait();
+        reg_fence16(r);
+        float* dst = dspart + (pidx * m + h * 128 + tl) * kD + 16 * cc;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          *reinterpret_cast<uint4*>(dst + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+      }
+      tc_fence_before_sync();
       named_bar_sync(1, kQElem);   // the scratch and z' may be written again
     }
     // sum of dD' of this CTA (zero if it gave up)

@@ -104,6 +104,29 @@ __device__ __forceinline__ void named_bar_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
+// The same, and every thread learns whether all of them came with `ok`.
+__device__ __forceinline__ bool named_bar_all(int id, int threads, bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 q, %1, 0;\n\t"
+      "barrier.cta.red.and.pred p, %2, %3, q;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r)
+      : "r"(ok ? 1u : 0u), "r"(id), "r"(threads)
+      : "memory");
+  return r != 0;
+}
+// Wait of a group of warps on an mbarrier: those with `polls` poll it, the others sleep at the named barrier (polls are
+// shared-memory reads, and the tensor core needs that bandwidth for its operands).  All of the group's threads return
+// the same answer: after a wait that ran out, or one of them coming with ok = false, none of them goes on.
+__device__ __forceinline__ bool group_wait(uint64_t* bar, uint32_t parity, bool polls, bool ok, int id, int threads,
+                                           volatile int* abort_flag, int* status, int code,
+                                           unsigned long long limit_ns = kWaitLimitNs) {
+  if (polls && ok) ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, code, limit_ns));
+  return named_bar_all(id, threads, ok);
+}
+
 // ---- TMA ----------------------------------------------------------------------------------------
 // 2-D tiled load: box starting at element (x, y) -> shared memory, completion on an mbarrier.
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
