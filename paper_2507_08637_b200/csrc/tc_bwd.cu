@@ -799,8 +799,9 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
               sum_dd += c * inv;
             }
             // ---- dA D (hi + lo, in place) and R / D, 16 features at a time
-            // (an instruction on the ALU pipe takes a scheduler two cycles, one on the FMA pipe one: the mask 1[R > 0]
-            // is a saturating product, 1 for every normal R > 0, and multiplies dA, instead of compares and selects)
+            // (the mask 1[R > 0] cuts the packed pairs: a factor would have to be 1 for the smallest R too, and would let
+            // an infinity or NaN of a feature that is off through)
+            const f32x2 c2 = pk2(c, c), minus1 = pk2(-1.f, -1.f);
             uint32_t a[2][16];
             tmem_ld16(trow + 32 * wq, a[0]);
 #pragma unroll
@@ -819,12 +820,12 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
               for (int j = 0; j < 8; ++j) {
                 if ((j & 1) == 0) asm volatile("" ::: "memory");
                 const float2 zz = *reinterpret_cast<const float2*>(z + 2 * j);
-                const uint32_t rw = rp[h][8 * q + j];
+                const uint32_t rw = rp[h][8 * q + j], mk = positive_mask_bf16x2(rw);
                 const float r0 = __uint_as_float(rw << 16), r1 = __uint_as_float(rw & 0xFFFF0000u);
-                const float v0 = fmaf(c, zz.x, __uint_as_float(g[2 * j])) * __saturatef(r0 * 0x1p127f);
-                const float v1 = fmaf(c, zz.y, __uint_as_float(g[2 * j + 1])) * __saturatef(r1 * 0x1p127f);
-                ph[j] = pack_bf16x2(v0, v1);
-                pl[j] = pack_bf16x2(v0 - __uint_as_float(ph[j] << 16), v1 - __uint_as_float(ph[j] & 0xFFFF0000u));
+                const f32x2 val = fma2(c2, pk2(zz.x, zz.y), pk2u(g[2 * j], g[2 * j + 1]));
+                const uint32_t hv = pack2_bf16(val);
+                ph[j] = hv & mk;
+                pl[j] = pack2_bf16(fma2(minus1, unpack2_bf16(hv), val)) & mk;
                 pp[j] = pack_bf16x2(r0 * inv, r1 * inv);
               }
               tmem_st8(col, ph);
