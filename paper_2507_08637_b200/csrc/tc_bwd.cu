@@ -475,10 +475,10 @@ constexpr uint32_t kIdescT = make_idesc_bf16(128, 64, true, true);   // contract
 // list either index steps, so slots are distinct and those of one slab are consecutive) and takes up the next one.
 // Warp 0: TMA copies.  Warp 1: every MMA.  Warp 2: dQ_F stores.  Warps 4-19: elementwise, thread = token tl (TMEM lane) and features
 // 128 h + 32 wq .. + 31 of every half h.  Per tile, all in the accumulator X (m columns of TMEM):
-//   MMA:  X = A (three planes)             threads: R = ReLU(A) -> bf16 pairs in registers, D' = R . z'
-//   MMA:  X = G = dO S'^T (S' as hi + lo)  threads: num = R . G, sums over the four threads of a token (through
-//                                          spare TMEM columns), c = - num / D, then half by half
-//                                          R / D -> shared memory, dA D = (G + c z') 1[R > 0] -> X as hi + lo pairs
+//   MMA:  X = A (three planes)             threads: R = ReLU(A), D' = R . z', summed over the four threads of a token
+//                                          (through spare TMEM columns), R / D -> bf16 pairs in registers
+//   MMA:  X = G = dO S'^T (S' as hi + lo)  threads: num / D = (R / D) . G, summed likewise, c = - num / D, then half by
+//                                          half R / D -> shared memory, dA D = (G + c z') 1[R > 0] -> X as hi + lo pairs
 //   MMA, half by half: dS'_h += (R / D)_h^T dO,  dQ_F D += dA_h D W_h^T;  then X = A of the next tile
 //   threads meanwhile: dz' += (R / D)^T c from shared memory, then dQ_F (row scaled by 1 / D) -> staging
 // dO . O = num / D, so N' is never formed, and dO enters both contractions as it is (bf16, exact).  What bounds a tile (m = 256): 4.8 k cycles of tensor pipe (1.5 A, 1.0 G, 0.8 dS', 1.4 dQ_F) plus
@@ -708,104 +708,103 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
         const uint32_t par = it & 1;
         const int row0 = (gt - slab * tps) * kTile, row = row0 + tl;
         const float* zr = zs + 32 * wq;
-        // ---- R, D'
-        float inv = 0.f, c = 0.f;
+        // ---- D', and R / D, rounded to bf16 once from R in 32 bits
+        float inv = 0.f, c = 0.f;   // (rows past the end contribute nothing)
         wait_all(&bars->a_full, par);
         if (ok) {   // (every wait has one answer for the lane quarter: its barriers may stand inside)
-          uint32_t rp[NH][16];
-          float den = 0.f, den2 = 0.f;
-          f32x2 num = pk2(0.f, 0.f);
+          // row sums over the four threads of a token, through spare TMEM columns (four for D', four for num / D)
+          auto row_total = [&](uint32_t col, float share) {
+            tmem_st1(trow + kStat + col + wq, __float_as_uint(share));
+            tmem_st_wait();
+            tc_fence_before_sync();
+            if (it > 0 && col > 0) wait_all(&bars->p_free, par ^ 1);   // (long past, as a rule)
+            else named_bar_sync(2 + (warp & 3), 128);
+            tc_fence_after_sync();
+            uint32_t st[4];
+            tmem_ld4(trow + kStat + col, st);
+            tmem_ld_wait();
+            reg_fence4(st);
+            return (__uint_as_float(st[0]) + __uint_as_float(st[1])) + (__uint_as_float(st[2]) + __uint_as_float(st[3]));
+          };
+          uint32_t pp[NH][16];
           {
             uint32_t r[NH][32];
 #pragma unroll
             for (int h = 0; h < NH; ++h) tmem_ld32(trow + h * 128 + 32 * wq, r[h]);
-            tmem_ld_wait();
-#pragma unroll
-            for (int h = 0; h < NH; ++h) reg_fence32(r[h]);
-            tc_fence_before_sync();
-            warp_arrive(&bars->a_read);   // X may become G
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-#pragma unroll
-              for (int j = 0; j < 16; j += 2) {
-                float a[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[i] = __uint_as_float(r[h][2 * j + i]);
-                rp[h][j] = relu_pack_bf16x2(a[0], a[1]);
-                rp[h][j + 1] = relu_pack_bf16x2(a[2], a[3]);
-                if constexpr (!kGroup) {
-                  if ((j & 3) == 0) asm volatile("" ::: "memory");   // (z' is read as it is used, not kept in registers)
-                  const float4 z = *reinterpret_cast<const float4*>(zr + h * 128 + 2 * j);
-                  den = fmaf(fmaxf(a[0], 0.f), z.x, den);
-                  den2 = fmaf(fmaxf(a[1], 0.f), z.y, den2);
-                  den = fmaf(fmaxf(a[2], 0.f), z.z, den);
-                  den2 = fmaf(fmaxf(a[3], 0.f), z.w, den2);
-                }
-              }
-            }
-          }
-          // ---- num = R . G, and the row sums over the four threads of a token
-          wait_all(&bars->g_full, par);
-          if constexpr (!kGroup) {
-            if (ok) {
-              uint32_t a[16], b[16];
-              tmem_ld16(trow + 32 * wq, a);
-#pragma unroll
-              for (int h = 0; h < NH; ++h) {
-                reg_fence16(rp[h]);   // (R is unpacked again in every pass, not kept unpacked)
-                tmem_ld_wait();
-                reg_fence16(a);
-                tmem_ld16(trow + h * 128 + 32 * wq + 16, b);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(rp[h][j]), pk2u(a[2 * j], a[2 * j + 1]), num);
-                tmem_ld_wait();
-                reg_fence16(b);
-                if (h + 1 < NH) tmem_ld16(trow + (h + 1) * 128 + 32 * wq, a);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(rp[h][8 + j]), pk2u(b[2 * j], b[2 * j + 1]), num);
-              }
-              const uint32_t st[2] = {__float_as_uint(den + den2), __float_as_uint(sum2(num))};
-              tmem_st2(trow + kStat + 2 * wq, st);
-              tmem_st_wait();
-              tc_fence_before_sync();
-            }
-          }
-          if (it > 0) wait_all(&bars->p_free, par ^ 1);   // (long past, as a rule; also the barrier behind the row sums)
-          else named_bar_sync(2 + (warp & 3), 128);
-          if (ok) {
             if constexpr (kGroup) {
               if (row < n) {
                 const float D = den_ext[(size_t)slab * n + row];
                 inv = 1.f / D;
                 c = dd_ext[(size_t)slab * n + row] * D;
               }
-            } else {
-              tc_fence_after_sync();
-              uint32_t st[8];
-              tmem_ld8(trow + kStat, st);
-              tmem_ld_wait();
-              reg_fence8(st);
-              auto total = [&](int i) {
-                return (__uint_as_float(st[i]) + __uint_as_float(st[2 + i])) +
-                       (__uint_as_float(st[4 + i]) + __uint_as_float(st[6 + i]));
-              };
-              if (row < n) {   // rows past the end contribute nothing
-                inv = 1.f / (epsp + total(0));
-                c = -total(1) * inv;
-              }
             }
+            tmem_ld_wait();
+#pragma unroll
+            for (int h = 0; h < NH; ++h) reg_fence32(r[h]);
+            tc_fence_before_sync();
+            warp_arrive(&bars->a_read);   // X may become G
+            if constexpr (!kGroup) {
+              float den = 0.f, den2 = 0.f;
+#pragma unroll
+              for (int h = 0; h < NH; ++h) {
+#pragma unroll
+                for (int j = 0; j < 32; j += 4) {
+                  if ((j & 7) == 0) asm volatile("" ::: "memory");   // (z' is read as it is used, not kept in registers)
+                  const float4 z = *reinterpret_cast<const float4*>(zr + h * 128 + j);
+                  den = fmaf(fmaxf(__uint_as_float(r[h][j]), 0.f), z.x, den);
+                  den2 = fmaf(fmaxf(__uint_as_float(r[h][j + 1]), 0.f), z.y, den2);
+                  den = fmaf(fmaxf(__uint_as_float(r[h][j + 2]), 0.f), z.z, den);
+                  den2 = fmaf(fmaxf(__uint_as_float(r[h][j + 3]), 0.f), z.w, den2);
+                }
+              }
+              const float total = row_total(0, den + den2);
+              if (row < n) inv = 1.f / (epsp + total);
+            }
+#pragma unroll
+            for (int h = 0; h < NH; ++h)
+#pragma unroll
+              for (int j = 0; j < 16; ++j)
+                pp[h][j] = relu_pack_bf16x2(__uint_as_float(r[h][2 * j]) * inv, __uint_as_float(r[h][2 * j + 1]) * inv);
+          }
+          // ---- num / D = (R / D) . G
+          wait_all(&bars->g_full, par);
+          if constexpr (!kGroup) {
+            if (ok) {
+              f32x2 num = pk2(0.f, 0.f);
+              uint32_t a[16], b[16];
+              tmem_ld16(trow + 32 * wq, a);
+#pragma unroll
+              for (int h = 0; h < NH; ++h) {
+                reg_fence16(pp[h]);   // (R / D is unpacked again in every pass, not kept unpacked)
+                tmem_ld_wait();
+                reg_fence16(a);
+                tmem_ld16(trow + h * 128 + 32 * wq + 16, b);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(pp[h][j]), pk2u(a[2 * j], a[2 * j + 1]), num);
+                tmem_ld_wait();
+                reg_fence16(b);
+                if (h + 1 < NH) tmem_ld16(trow + (h + 1) * 128 + 32 * wq, a);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(pp[h][8 + j]), pk2u(b[2 * j], b[2 * j + 1]), num);
+              }
+              c = -row_total(4, sum2(num));
+            }
+          } else if (it > 0) {
+            wait_all(&bars->p_free, par ^ 1);
+          }
+          if (ok) {
             if (wq == 0) {
               cs[tl] = c;
               sum_dd += c * inv;
             }
-            // ---- dA D (hi + lo, in place) and R / D, 16 features at a time
-            // (the mask 1[R > 0] cuts the packed pairs: a factor would have to be 1 for the smallest R too, and would let
-            // an infinity or NaN of a feature that is off through)
+            // ---- dA D (hi + lo, in place) and R / D to shared memory, 16 features at a time
+            // (the mask 1[R > 0], taken from R / D, cuts the packed pairs: a factor would have to be 1 for the smallest R
+            // too, and would let an infinity or NaN of a feature that is off through)
             const f32x2 c2 = pk2(c, c), minus1 = pk2(-1.f, -1.f);
             uint32_t a[2][16];
             tmem_ld16(trow + 32 * wq, a[0]);
 #pragma unroll
-            for (int h = 0; h < NH; ++h) reg_fence16(rp[h]);
+            for (int h = 0; h < NH; ++h) reg_fence16(pp[h]);
 #pragma unroll
             for (int s = 0; s < 2 * NH; ++s) {
               const int h = s >> 1, q = s & 1;
@@ -815,25 +814,24 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
               reg_fence16(g);
               if (s + 1 < 2 * NH) tmem_ld16(trow + ((s + 1) >> 1) * 128 + 32 * wq + 16 * ((s + 1) & 1), a[(s + 1) & 1]);
               const float* z = zr + h * 128 + 16 * q;
-              uint32_t ph[8], pl[8], pp[8];
+              uint32_t ph[8], pl[8];
 #pragma unroll
               for (int j = 0; j < 8; ++j) {
                 if ((j & 1) == 0) asm volatile("" ::: "memory");
                 const float2 zz = *reinterpret_cast<const float2*>(z + 2 * j);
-                const uint32_t rw = rp[h][8 * q + j], mk = positive_mask_bf16x2(rw);
-                const float r0 = __uint_as_float(rw << 16), r1 = __uint_as_float(rw & 0xFFFF0000u);
+                const uint32_t mk = positive_mask_bf16x2(pp[h][8 * q + j]);
                 const f32x2 val = fma2(c2, pk2(zz.x, zz.y), pk2u(g[2 * j], g[2 * j + 1]));
                 const uint32_t hv = pack2_bf16(val);
                 ph[j] = hv & mk;
                 pl[j] = pack2_bf16(fma2(minus1, unpack2_bf16(hv), val)) & mk;
-                pp[j] = pack_bf16x2(r0 * inv, r1 * inv);
               }
               tmem_st8(col, ph);
               tmem_st8(col + 8, pl);
               uint8_t* blk = pt + (2 * h + (wq >> 1)) * kTileBytes;
               const uint32_t ch = 4 * (wq & 1) + 2 * q;
-              *reinterpret_cast<uint4*>(blk + swz128(tl, ch)) = make_uint4(pp[0], pp[1], pp[2], pp[3]);
-              *reinterpret_cast<uint4*>(blk + swz128(tl, ch + 1)) = make_uint4(pp[4], pp[5], pp[6], pp[7]);
+              const uint32_t* pq = pp[h] + 8 * q;
+              *reinterpret_cast<uint4*>(blk + swz128(tl, ch)) = make_uint4(pq[0], pq[1], pq[2], pq[3]);
+              *reinterpret_cast<uint4*>(blk + swz128(tl, ch + 1)) = make_uint4(pq[4], pq[5], pq[6], pq[7]);
               tmem_st_wait();
               if (q == 1) fence_proxy_async_smem();   // R / D of the half, for the MMA of dS'
               else asm volatile("" ::: "memory");
