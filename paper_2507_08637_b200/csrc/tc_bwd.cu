@@ -875,11 +875,13 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
         if (!ok) break;
         {
           uint8_t* box = pt + (wq >> 1) * kTileBytes;
+          // (with eps = 0 a token without an active feature has D = 0; its dA is zero, and so is its dQ_F)
+          const float scale = inv <= 3.402823466e38f ? inv : 0.f;
 #pragma unroll
           for (int q = 0; q < 4; ++q)
             *reinterpret_cast<float4*>(box + swz128(tl, 4 * (wq & 1) + q)) =
-                make_float4(__uint_as_float(r[4 * q]) * inv, __uint_as_float(r[4 * q + 1]) * inv,
-                            __uint_as_float(r[4 * q + 2]) * inv, __uint_as_float(r[4 * q + 3]) * inv);
+                make_float4(__uint_as_float(r[4 * q]) * scale, __uint_as_float(r[4 * q + 1]) * scale,
+                            __uint_as_float(r[4 * q + 2]) * scale, __uint_as_float(r[4 * q + 3]) * scale);
           fence_proxy_async_smem();
         }
         warp_arrive(&bars->staged);
