@@ -654,8 +654,10 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
           }
           if (ok && h == NH - 1) mma_commit(&bars->dq_full);   // (every MMA of the tile)
         }
-        if (ok && it + 1 < nt) {   // A of the next tile follows in the pipe behind the MMAs that still read X
-          ok = mbar_wait(&bars->x_full, par ^ 1, abort_flag, status, kErrBwdCopy);
+        if (ok && it + 1 < nt) {   // A of the next tile overwrites X once the MMAs that read dA there have completed
+          // (instructions with different shapes and accumulators are not ordered by being issued one after the other)
+          ok = mbar_wait(&bars->dq_full, par, abort_flag, status, kErrBwdMma) &&
+               mbar_wait(&bars->x_full, par ^ 1, abort_flag, status, kErrBwdCopy);
           if (!ok) break;
           tc_fence_after_sync();
           issue_a();
