@@ -112,7 +112,7 @@ k_tc_bwd_kside(const __grid_constant__ CUtensorMap map_kf, const __grid_constant
                const __grid_constant__ CUtensorMap map_dkf, int n, int d, int slabs, int* __restrict__ status) {
   wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = align_smem(smem_raw);
   using SL = BwdKSmem<NH>;
   BwdKBars* bars = reinterpret_cast<BwdKBars*>(smem + SL::bars);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

@@ -20,7 +20,8 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // First 1024-byte boundary of the dynamic shared memory.  The offset is added to the array itself: rounding the
 // address through an integer makes the compiler lose the address space, and every access to shared memory becomes a
 // generic load or store, slower and waited for like one to global memory (B=1 H=8 n=131072 m=256: key side 79.9 ->
-// 73.7 us, query side 79.9 -> 77.8; B=64 H=12 n=1024 m=128: query side 63.5 -> 55.3).
+// 73.7 us, query side 79.9 -> 77.8; B=64 H=12 n=1024 m=128: query side 63.5 -> 55.3; backward, key side: B=4 H=8 n=16384
+// m=256 146 -> 138 us, B=32 H=4 n=4096 d=32 m=1024 498 -> 453 us).
 __device__ __forceinline__ uint8_t* align_smem(uint8_t* raw) { return raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u); }
 __device__ __forceinline__ unsigned long long global_timer_ns() {
   unsigned long long t;
