@@ -185,6 +185,7 @@ wersa_status wersa_gate_static(const wersa_config* cfg, const void* Q, const flo
  *                       caller adds the S' and the z' of all shards (Eq. 7's sums over the tokens).
  *   wersa_shard_output  Q shard, the added S_total (batch*heads, features, 64) and z_total (batch*heads,
  *                       features), beta -> O shard.
+ * The sums that come back (qsum_total, S_total, z_total and those of the backward) may lie at any float.
  * The two additions are the only exchange between ranks (an all-reduce each; the library does not do them).
  * bf16 tensor-core contexts with features <= 256 only, else WERSA_ERR_UNSUPPORTED.
  *

@@ -816,8 +816,11 @@ static cudaError_t launch_reduce(const Plan& p, int groups, const float* spart, 
                                  float* S, float* z, __nv_bfloat16* Sbf, uint8_t* Simg, cudaStream_t st, int* launches) {
   const int m = p.cfg.features;
   const dim3 grid(m / 8, p.slabs, groups);
-  const cudaError_t err =   // (four CTAs per SM: see k_reduce_partials)
-      grid.x * grid.y * grid.z > 4u * p.sms
+  // (four CTAs per SM: see k_reduce_partials; a sequence shard's caller may hand in sums that lie at any float, such as a
+  // view into the buffer of a larger all-reduce, and those are read one by one)
+  const bool aligned = (reinterpret_cast<uintptr_t>(spart) & 15u) == 0;
+  const cudaError_t err =
+      aligned && grid.x * grid.y * grid.z > 4u * p.sms
           ? launch_after(k_reduce_partials<4>, grid, dim3(160), 0, st, spart, zpart, chunks, tps, ctas, m, S, z, Sbf, Simg)
           : launch_after(k_reduce_partials<1>, grid, dim3(544), 0, st, spart, zpart, chunks, tps, ctas, m, S, z, Sbf, Simg);
   *launches += 1;
