@@ -97,3 +97,25 @@ def test_status_strings(lib):
     lib.wersa_status_string.restype = ctypes.c_char_p
     seen = {lib.wersa_status_string(i) for i in range(7)}
     assert len(seen) == 7 and all(s for s in seen)
+
+
+def test_static_gate_makes_no_tile_plan():
+    """wersa_gate_static needs none of the choices that fp32 contexts search for: refusing a problem that does not fit its
+    array takes an fp32 call the time it takes a bf16 one (least of 20 batches of 200 calls)."""
+    import time
+    import paper_2507_08637_b200 as w
+    from paper_2507_08637_b200 import binding
+    lib, at = binding._lib(), ctypes.c_void_p(256)
+    least = {}
+    for dtype, features in (("f32", 64), ("bf16", 128)):
+        cfg = _cfg(batch=8000, heads=1, seq_len=20000, levels=3, features=features, dtype=dtype)   # 16000 counters: too many
+        args = (ctypes.byref(cfg), at, None, None, at, at, at, None)
+        assert lib.wersa_gate_static(*args) == 7
+        times = []
+        for _ in range(20):
+            t0 = time.perf_counter()
+            for _ in range(200):
+                lib.wersa_gate_static(*args)
+            times.append((time.perf_counter() - t0) / 200)
+        least[dtype] = min(times)
+    assert least["f32"] <= least["bf16"] + 1e-6, least
