@@ -143,10 +143,17 @@ def _host_ptr(t, dtype, name):
     return ctypes.c_void_p(t.data_ptr())
 
 
+# Where torch has them: the handle of a device's current stream without a Stream object (3 us of host time per call).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream_ptr(stream):
-    if stream is None:   # the current stream of the current device, without a Stream object (3 us of host time per call)
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
-    return stream.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None or _current_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
 
 
 class WersaContext:

@@ -119,3 +119,19 @@ def test_static_gate_makes_no_tile_plan():
             times.append((time.perf_counter() - t0) / 200)
         least[dtype] = min(times)
     assert least["f32"] <= least["bf16"] + 1e-6, least
+
+
+def test_current_stream_without_torch_internals(monkeypatch):
+    """The current stream's handle comes from torch's public interface where the internal calls are missing."""
+    import types
+    import torch
+    from paper_2507_08637_b200 import binding
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=4321))
+    for name in ("_raw_stream", "_current_device"):
+        with monkeypatch.context() as m:
+            m.setattr(binding, name, None)
+            assert binding._stream_ptr(None) == 4321
+    monkeypatch.setattr(binding, "_current_device", lambda: 3)
+    monkeypatch.setattr(binding, "_raw_stream", lambda device: 100 + device)
+    assert binding._stream_ptr(None) == 103
+    assert binding._stream_ptr(types.SimpleNamespace(cuda_stream=7)) == 7
