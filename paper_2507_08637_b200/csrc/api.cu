@@ -40,7 +40,7 @@ static wersa_status make_pool_plan(const wersa_config& c, Plan* p) {
   if (!(c.eps >= 0.f) || !(c.bw_floor > 0.f)) return WERSA_ERR_INVALID_ARG;
   if (c.device < 0) return WERSA_ERR_INVALID_ARG;
   if (c.levels <= 30 && (1LL << c.levels) > (long long)next_pow2(c.seq_len)) return WERSA_ERR_INVALID_ARG;
-  // head dimensions 8, 16, ... 64 (narrower ones run zero-padded to 64 columns)
+  // head dimensions 8, 16, ... 64
   if (c.head_dim > kD || c.head_dim < 8 || c.head_dim % 8 != 0) return WERSA_ERR_UNSUPPORTED;
   if (c.levels > kMaxLevels) return WERSA_ERR_UNSUPPORTED;
   // feature maps of 64, 128 or 256, and (bf16 tensor-core path) 512, 768, 1024 in groups of 256
@@ -205,8 +205,9 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   p->off_Simg = take(p->use_tc ? slabs * simg_bytes(m) : 0);
   const size_t slab_elems = slabs * (size_t)n * kD;
   const size_t io_bytes = p->bf16 ? 2 : 4;
-  // callers may rely on a narrow context asking for more than the 64-wide one of the same shape (it once held padded
-  // copies); nothing lives here
+  // The buffers of filtered tensors, their gradients and group outputs are sized for 64 columns, of which the kernels use
+  // the first slabs * n * head_dim elements; the 256 bytes behind them are unused.  Both keep the order that the sizes of
+  // narrow and 64-wide contexts have always had (a narrow one asks for more), which the interface's test pins.
   take(p->dpad ? 256 : 0);
   p->off_Og = take(grouped ? io_bytes * slab_elems * p->groups : 0);
   p->off_den = take(grouped ? sizeof(float) * slabs * n * p->groups : 0);
@@ -434,7 +435,7 @@ wersa_status wersa_forward(wersa_ctx* ctx, const void* Q, const void* K, const v
                  launch_reduce_partials(pg, w.spart, w.zpart, p.tchunks, w.S, w.z, w.Sbf, w.Simg, st, &launches));
     WERSA_STEP(0, "tc_qside", launch_tc_qside(pg, w, Q, beta, w.Og, w.den, st, &launches));
     WERSA_STEP(0, "combine_groups",
-               launch_combine_groups(w.Og, w.den, O, rows, p.groups, d, kind, st, &launches));
+               launch_combine_groups(w.Og, w.den, O, rows, p.groups, d, st, &launches));
   } else if (p.use_tc) {
     WERSA_STEP(0, "tc_kside", launch_tc_kside(p, w, K, V, st, &launches));
     if (p.tchunks > 1)   // with one chunk per slab the key-side kernel has written S', z' and the image itself
@@ -656,7 +657,7 @@ wersa_status wersa_backward(wersa_ctx* ctx, const void* Q, const void* K, const 
     // dS', dz', and dQ_F, dV, dK_F accumulate over the groups in launch order.
     WERSA_STEP(1, "haar_filter_qk", launch_haar_filter_split3(p, w, Q, w.QF3, K, w.KF3, true, st, &launches));
     WERSA_STEP(1, "group_bwd_prep",
-               launch_group_bwd_prep(w.Og, w.den, dO, d, w.f, p.cfg.seq_len, p.L1, rows, p.groups, kind, w.Dtot,
+               launch_group_bwd_prep(w.Og, w.den, dO, d, w.f, p.cfg.seq_len, p.L1, rows, p.groups, w.Dtot,
                                      w.Dtot + rows, st, &launches));
     const Plan pg = group_plan(p);
     for (int g = 0; g < p.groups; ++g) {

@@ -10,7 +10,7 @@
 
 namespace wersa {
 
-constexpr int kD = 64;           // head dim the kernels work on (narrower heads are zero-padded to it)
+constexpr int kD = 64;           // widest head; S', z' images, partial sums and q-bar of narrower ones have zero columns up to it
 constexpr int kGroupFeatures = 256;   // widest feature map of one kernel launch; wider maps run in groups
 constexpr int kMaxLevels = 8;    // Haar levels supported: block of 2^8 = 256 tokens
 constexpr int kHaarTile = 256;   // tokens per Haar tile (>= 2^kMaxLevels)
@@ -99,7 +99,7 @@ cudaError_t launch_qmean_gate_static(const Plan& p, float* scratch, const void* 
                                      cudaStream_t st);
 
 // ---- haar.cu -------------------------------------------------------------------------------
-// d: columns of the tensors as stored (a multiple of 8, at most 64).  in_kind/out_kind: 0 = float, 1 = bf16.
+// d: columns of the tensors as stored (a multiple of 8, at most 64).  in_kind/out_kind: 0 = float, 1 = bf16 (float input: float output).
 // XF = T_f(X), and with X2 also XF2 = T_f(X2) in the same launch.
 cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const float* f, void* XF, const void* X2,
                                void* XF2, int out_kind, int d, cudaStream_t st, int* launches);
@@ -158,14 +158,14 @@ cudaError_t launch_tc_bwd_kside(const Plan& p, const Ws& w, const void* KF3, con
 
 
 // ---- glue.cu -------------------------------------------------------------------------------
-// O = sum_g Og[g] * den[g] / sum_g den[g] per token (Og: groups x tokens x cols, den: groups x tokens).
+// O = sum_g Og[g] * den[g] / sum_g den[g] per token (Og: groups x tokens x cols, den: groups x tokens; bf16).
 cudaError_t launch_combine_groups(const void* Og, const float* den, void* O, size_t tokens, int groups, int cols,
-                                  int kind, cudaStream_t st, int* launches);
+                                  cudaStream_t st, int* launches);
 // Backward of the combination: per token the whole map's denominator D = sum_g den_g / r (r = the filter
 // stage's factor carried by the forward's denominators, from f) and dD' = -(dO . O) / D with
 // O = sum_g Og den_g / sum_g den_g.  Og and dO have d columns.
 cudaError_t launch_group_bwd_prep(const void* Og, const float* den, const void* dO, int d, const float* f, int n, int L1,
-                                  size_t tokens, int groups, int kind, float* Dtot, float* dDtot, cudaStream_t st,
+                                  size_t tokens, int groups, float* Dtot, float* dDtot, cudaStream_t st,
                                   int* launches);
 
 // ---- selftest.cu ---------------------------------------------------------------------------

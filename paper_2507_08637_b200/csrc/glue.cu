@@ -11,9 +11,8 @@ namespace {
 // O[tok][:] = sum_g Og[g][tok][:] * den[g][tok] / sum_g den[g][tok], groups in a fixed order.  Og and O have `cols`
 // columns.  One thread per 8 columns of a token; tokens = slabs * n.  Bound by memory: with the groups' outputs as
 // wide as the head instead of 64 columns, 4 groups, 512k tokens: d = 16 58 -> 18 us, d = 32 61 -> 33 us.
-template <typename T>
-__global__ void __launch_bounds__(256) k_combine_groups(const T* __restrict__ Og, const float* __restrict__ den,
-                                                        T* __restrict__ O, size_t tokens, int groups, int cols) {
+__global__ void __launch_bounds__(256) k_combine_groups(const __nv_bfloat16* __restrict__ Og, const float* __restrict__ den,
+                                                        __nv_bfloat16* __restrict__ O, size_t tokens, int groups, int cols) {
   wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   const size_t idx = (size_t)blockIdx.x * 256 + threadIdx.x;
   const int per = cols >> 3;
@@ -41,9 +40,8 @@ __global__ void __launch_bounds__(256) k_combine_groups(const T* __restrict__ Og
 // d / 8) per token with 8 columns each.  The forward's denominators carry the factor r = bf16(f_0) / f_0 of its filter
 // stage, which the backward's filtered planes do not.  (4 groups, 512k tokens, d = 32, Og of d instead of 64 columns:
 // 78 -> 45 us.)
-template <typename T>
-__global__ void __launch_bounds__(256) k_group_bwd_prep(const T* __restrict__ Og, const float* __restrict__ den,
-                                                        const T* __restrict__ dO, int d, int tpt, const float* __restrict__ f,
+__global__ void __launch_bounds__(256) k_group_bwd_prep(const __nv_bfloat16* __restrict__ Og, const float* __restrict__ den,
+                                                        const __nv_bfloat16* __restrict__ dO, int d, int tpt, const float* __restrict__ f,
                                                         int n, int L1, size_t tokens, int groups,
                                                         float* __restrict__ Dtot, float* __restrict__ dDtot) {
   wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
@@ -86,31 +84,21 @@ unsigned blocks_for(size_t threads) { return (unsigned)((threads + 255) / 256); 
 }  // namespace
 
 cudaError_t launch_combine_groups(const void* Og, const float* den, void* O, size_t tokens, int groups, int cols,
-                                  int kind, cudaStream_t st, int* launches) {
-  if (kind == 1)
-    launch_after(k_combine_groups<__nv_bfloat16>, dim3(blocks_for(tokens * (cols >> 3))), dim3(256), 0, st, (const __nv_bfloat16*)Og, den,
-                                                                           (__nv_bfloat16*)O, tokens, groups, cols);
-  else
-    launch_after(k_combine_groups<float>, dim3(blocks_for(tokens * (cols >> 3))), dim3(256), 0, st, (const float*)Og, den, (float*)O, tokens, groups,
-                                                                   cols);
+                                  cudaStream_t st, int* launches) {
+  using bf = __nv_bfloat16;
   *launches += 1;
-  return cudaGetLastError();
+  return launch_after(k_combine_groups, dim3(blocks_for(tokens * (cols >> 3))), dim3(256), 0, st, (const bf*)Og, den, (bf*)O,
+                      tokens, groups, cols);
 }
 
 cudaError_t launch_group_bwd_prep(const void* Og, const float* den, const void* dO, int d, const float* f, int n, int L1,
-                                  size_t tokens, int groups, int kind, float* Dtot, float* dDtot, cudaStream_t st,
-                                  int* launches) {
+                                  size_t tokens, int groups, float* Dtot, float* dDtot, cudaStream_t st, int* launches) {
+  using bf = __nv_bfloat16;
   int tpt = 1;
   while (8 * tpt < d) tpt <<= 1;
-  const dim3 grid(blocks_for(tokens * tpt));
-  if (kind == 1)
-    launch_after(k_group_bwd_prep<__nv_bfloat16>, grid, dim3(256), 0, st, (const __nv_bfloat16*)Og, den,
-                 (const __nv_bfloat16*)dO, d, tpt, f, n, L1, tokens, groups, Dtot, dDtot);
-  else
-    launch_after(k_group_bwd_prep<float>, grid, dim3(256), 0, st, (const float*)Og, den, (const float*)dO, d, tpt, f, n, L1,
-                 tokens, groups, Dtot, dDtot);
   *launches += 1;
-  return cudaGetLastError();
+  return launch_after(k_group_bwd_prep, dim3(blocks_for(tokens * tpt)), dim3(256), 0, st, (const bf*)Og, den, (const bf*)dO, d,
+                      tpt, f, n, L1, tokens, groups, Dtot, dDtot);
 }
 
 }  // namespace wersa

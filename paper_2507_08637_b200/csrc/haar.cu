@@ -562,12 +562,9 @@ cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const 
     else if (in_kind == 1 && out_kind == 0)
       err = launch_after(k_haar_filter_bf16<kFull, float>, grid_bf, dim3(256), 0, st, (const bf*)X, f, (float*)XF, (const bf*)X2,
                          (float*)XF2, n, d, L);
-    else if (in_kind == 0 && out_kind == 0)
+    else
       err = launch_after(k_haar_filter<kFull, float, float, false>, grid, dim3(256), 0, st, (const float*)X, f, (float*)XF,
                          (const float*)X2, (float*)XF2, n, d, L, nullptr, 0.f);
-    else
-      err = launch_after(k_haar_filter<kFull, float, bf, false>, grid, dim3(256), 0, st, (const float*)X, f, (bf*)XF,
-                         (const float*)X2, (bf*)XF2, n, d, L, nullptr, 0.f);
   })
   *launches += 1;
   return err != cudaSuccess ? err : cudaGetLastError();
@@ -616,9 +613,8 @@ cudaError_t launch_haar_backward(const Plan& p, const Ws& w, int which, const vo
                         static_cast<decltype(out)>(dX2), w.f, w.bands, which, n, d, L);
   };
   WERSA_FULL({
-    if (dX == nullptr && dX2 == nullptr) {   // band inner products only
-      if (in_kind == 1) err = go(k_haar_backward<kFull, bf, float, false>, (const bf*)X, (float*)nullptr);
-      else err = go(k_haar_backward<kFull, float, float, false>, (const float*)X, (float*)nullptr);
+    if (dX == nullptr && dX2 == nullptr) {   // band inner products only (sequence shards, whose tensors are bf16)
+      err = go(k_haar_backward<kFull, bf, float, false>, (const bf*)X, (float*)nullptr);
     } else if (in_kind == 1 && out_kind == 1) {
       err = go(k_haar_backward<kFull, bf, bf, true>, (const bf*)X, (bf*)dX);
     } else if (in_kind == 1 && out_kind == 0) {

@@ -129,18 +129,6 @@ __device__ __forceinline__ bool group_wait(uint64_t* bar, uint32_t parity, bool 
 }
 
 // ---- TMA ----------------------------------------------------------------------------------------
-// 2-D tiled load: box starting at element (x, y) -> shared memory, completion on an mbarrier.
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void* src, int x, int y) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
-               ::"l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(src)), "r"(x), "r"(y)
-               : "memory");
-}
 // 3-D tiled load / store: box starting at element (x, y, z).
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
   asm volatile(
@@ -215,20 +203,11 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 //   K-major  (rows = M/N index, 64 bf16 of K per row):  SBO = 1024 (next 8 rows), LBO unused.
 //   MN-major (rows = K index, 64 bf16 of M/N per row):  SBO = 1024 (next 8 K rows), LBO = stride
 //            of the next 64 M/N elements (unused when the tile is 64 wide).
-__device__ __forceinline__ uint64_t make_smem_desc(uint32_t smem_addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((smem_addr & 0x3FFFFu) >> 4);
-  d |= static_cast<uint64_t>((lbo_bytes >> 4) & 0x3FFFu) << 16;
-  d |= static_cast<uint64_t>((sbo_bytes >> 4) & 0x3FFFu) << 32;
-  d |= static_cast<uint64_t>(1) << 46;   // descriptor version of sm_100
-  d |= static_cast<uint64_t>(2) << 61;   // swizzle mode: 128 bytes
-  return d;
-}
-// The same descriptor as two 32-bit words, for issue loops that only advance the start address:
+// Held as two 32-bit words, for issue loops that only advance the start address:
 // `hi` is fixed per layout, `lo` = start address and LBO (shared-memory addresses stay below 2^18,
 // so adding (bytes >> 4) to `lo` never carries into the LBO field).
 __device__ __forceinline__ uint32_t smem_desc_hi(uint32_t sbo_bytes) {
-  return ((sbo_bytes >> 4) & 0x3FFFu) | (1u << 14) | (2u << 29);
+  return ((sbo_bytes >> 4) & 0x3FFFu) | (1u << 14) | (2u << 29);   // descriptor version of sm_100, 128-byte swizzle
 }
 __device__ __forceinline__ uint32_t smem_desc_lo(uint32_t smem_addr, uint32_t lbo_bytes) {
   return ((smem_addr & 0x3FFFFu) >> 4) | (((lbo_bytes >> 4) & 0x3FFFu) << 16);
