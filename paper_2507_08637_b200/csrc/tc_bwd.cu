@@ -102,8 +102,8 @@ static_assert(BwdKSmem<2>::total <= 232448 && BwdKSmem<1>::total <= 232448, "sha
 //              MMA dK_F += dB_h W_h^T
 // Warp 0: TMA copies; warp 1: the MMAs that fill units; warp 2: those of dV; warp 3: those of dK_F; warps 4-19
 // elementwise (thread = token tl, features 32 wq .. + 31 of the unit); warps 20-23 drain dV and dK_F to shared memory,
-// from where warp 0 stores them before it refills the stage.  The tensor pipe takes 4.2 k cycles a tile with m = 256 (1.5 B, 0.5 G, 0.7 dV, 1.4 dK_F) and
-// is the bound as long as the three accumulators hide the hand-offs.
+// from where warp 0 stores them before it refills the stage.  The tensor pipe takes 4.2 k cycles a tile with m = 256 (1.5 B, 0.5 G, 0.7 dV,
+// 1.4 dK_F), 49 % of the time: three accumulators do not hide all of the hand-offs (B=4 H=8 n=16384: 132 us).
 template <int NH, typename TG, bool kAdd = false>
 __global__ void __launch_bounds__(kKThreads, 1)
 k_tc_bwd_kside(const __grid_constant__ CUtensorMap map_kf, const __grid_constant__ CUtensorMap map_v,
@@ -481,8 +481,11 @@ constexpr uint32_t kIdescT = make_idesc_bf16(128, 64, true, true);   // contract
 //                                          half R / D -> shared memory, dA D = (G + c z') 1[R > 0] -> X as hi + lo pairs
 //   MMA, half by half: dS'_h += (R / D)_h^T dO,  dQ_F D += dA_h D W_h^T;  then X = A of the next tile
 //   threads meanwhile: dz' += (R / D)^T c from shared memory, then dQ_F (row scaled by 1 / D) -> staging
-// dO . O = num / D, so N' is never formed, and dO enters both contractions as it is (bf16, exact).  What bounds a tile (m = 256): 4.8 k cycles of tensor pipe (1.5 A, 1.0 G, 0.8 dS', 1.4 dQ_F) plus
-// num and the first half of dA, during which the pipe has nothing to do (X is the only accumulator that fits).
+// dO . O = num / D, so N' is never formed, and dO enters both contractions as it is (bf16, exact).  R / D is rounded from the
+// 32-bit R while G is formed: of the weights of dS' and dz' one rounding and no more, and nothing left to pack in the last
+// pass (B=4 H=8 n=16384 m=256 202 us; 205 with R rounded first).  What bounds a tile (m = 256): 4.8 k cycles of tensor
+// pipe (1.5 A, 1.0 G, 0.8 dS', 1.4 dQ_F; 35 % of the time) plus num and the first half of dA, during which the pipe has
+// nothing to do (X is the only accumulator that fits).
 // kGroup: the launch handles one group of 256 features of a wider feature map.  The denominator of Eq. 7 and
 // dD' then belong to the whole map and come from den_ext / dd_ext (one float per token), and with kAdd the
 // group's share of dQ_F is added to what the groups before it left.
