@@ -87,7 +87,7 @@ static_assert(4 * kRegsCtlQ + 8 * kRegsReluQ + 4 * kRegsEpiQ + 8 * kRegsAux <= (
 static_assert(4 * kRegsCtl + 8 * 96 + 8 * kRegsAux <= (kThreads / 32) * 96, "key-side register split");
 
 // Named barriers (id 0 is __syncthreads).
-enum { kBarZsum = 1, kBarCoef = 3, kBarHaar = 4, kBarOut0 = 5 };
+enum { kBarZsum = 1, kBarCoef = 3, kBarHaar = 4, kBarOut0 = 5, kBarHaarGroup0 = 8 };
 enum { kErrProducer = 11, kErrMma = 12, kErrRelu = 13, kErrEpilogue = 14, kErrHaar = 15 };
 
 struct alignas(8) KsideBars {
@@ -200,7 +200,7 @@ __device__ __forceinline__ float relu_unit(uint32_t taddr) {
 // out again where they leave results (S', z': divided by r; output: eps' scaled by r).
 //
 // Coefficient table in shared memory, written once per CTA by the Haar warps:
-//   hc[0] = bf16(f_0) in both halves (bit pattern), hc[i] = r k_i = r (f_i - f_{i-1}) / 2^i for i = 1..5
+//   hc[0] = bf16(f_0) in both halves (bit pattern), hc[i] = r k_i = r (f_i - f_{i-1}) / 2^i for i = 1..7
 //   (0 beyond L), hc[8 + 8 hw + w] = weight of warp w's 32-row sum in warp hw's levels 6-8 term
 //                                  = r (k_8 + [same 128-row group] k_7 + [same 64-row group] k_6).
 constexpr int kHaarCoefs = 8 + 64;
@@ -224,10 +224,10 @@ __device__ __forceinline__ void haar_coef_init(float* hc, const float* __restric
     scale *= 0.5f;
   }
   if (ht == 0) hc[0] = __uint_as_float(pack_bf16x2(k[0], k[0]));
-  if (ht >= 1 && ht < 6) {
+  if (ht >= 1 && ht < 8) {
     float v = k[1];
 #pragma unroll
-    for (int i = 2; i < 6; ++i) v = (ht == i) ? k[i] : v;
+    for (int i = 2; i < 8; ++i) v = (ht == i) ? k[i] : v;
     hc[ht] = v;
   }
   if (ht < 64) {
@@ -242,25 +242,34 @@ __device__ __forceinline__ uint32_t fma_bf16x2(uint32_t a, uint32_t b, uint32_t 
   return r;
 }
 
-// 256 threads (ht = 0..255) filter the block (two 128-row tiles) in place.  Thread (c = ht & 7, rg = ht >> 3) owns rows
-// 8 rg .. 8 rg + 7 of 16-byte chunk c: levels 1-3 in registers, levels 4-5 through warp shuffles
-// (a warp covers 32 consecutive rows), levels 6-8 through the 32-row sums the eight warps leave in
-// `xch` (8 x 64 floats, double-buffered by the caller) around one named barrier of the 256 threads.
-// The barrier is executed whether or not `ok` holds, so that a role that gave up on a wait keeps the
-// barrier balanced; with ok = false no memory is touched.  Rows >= valid_rows lie past the end of the
-// sequence: they arrive as zeros (the zero padding of Algorithm 2) and leave as zeros (the trim
-// before the feature map).
+// CW 16-byte chunks of columns (8: heads of more than 32 dimensions, 4: of more than 16, 2: of up to 16): 32 CW threads
+// (gt = 0 .. 32 CW - 1, CW warps, one of the 8 / CW groups of the filter role) filter the block (two 128-row tiles) in
+// place.  Thread (c = gt % CW, rg = gt / CW) owns rows 8 rg .. 8 rg + 7 of chunk c: levels 1-3 in registers, as many of
+// the following ones as a warp's 256 / CW consecutive rows cover (4-5, 4-6, 4-7) through shuffles, and the others through
+// the sums of the warps' rows, which they leave in `xch` (CW rows of 8 CW floats, double-buffered by the caller) around one
+// named barrier of the group.  The barrier is executed whether or not `ok` holds, so that a role that gave up on a wait
+// keeps the barrier balanced; with ok = false no memory is touched.  Rows >= valid_rows lie past the end of the
+// sequence: they arrive as zeros (the zero padding of Algorithm 2) and leave as zeros (the trim before the feature map).
+// Shared-memory accesses of 8 lanes cover CW chunks of 8 / CW row groups; the row groups' rows are taken in the order
+// j ^ (CW (rg mod 8 / CW)), so that the swizzle spreads them over all banks.  It only swaps halves of the blocks of 2, 4
+// and 8 rows, whose sums do not notice.
+template <int CW>
 __device__ __forceinline__ void haar_block_inplace(uint8_t* tile0, uint8_t* tile1, const float* hc, bool cross,
-                                                   float* xch, int ht, int valid_rows, bool ok) {
-  const int c = ht & 7, rg = ht >> 3, lane = ht & 31, hw = ht >> 5;
+                                                   float* xch, int gt, int bar, int valid_rows, bool ok) {
+  const int c = gt & (CW - 1), rg = gt / CW, lane = gt & 31, hw = gt >> 5;
+  const int swap = CW == 8 ? 0 : CW * (rg & (8 / CW - 1));
   uint8_t* base = (rg < 16 ? tile0 : tile1) + (rg & 15) * 1024;   // rows 0-127 / 128-255 of the block
+  auto chunk = [&](int j) {   // of the thread's j-th row; row 8 rg + jj has swizzle phase jj
+    const int jj = j ^ swap;
+    return reinterpret_cast<uint4*>(base + jj * 128 + ((c ^ jj) << 4));
+  };
   uint32_t u[8][4];   // 8 rows x 4 column pairs, as loaded
   float a[4][8];      // sums of row pairs, then the additive term c of each row pair
-  float hi[8], s5[8];
+  float hi[8], top[8];   // coarse part; sums over the warp's rows
   if (ok) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {   // row 8 rg + j has swizzle phase j
-      const uint4 raw = *reinterpret_cast<const uint4*>(base + j * 128 + ((c ^ j) << 4));
+    for (int j = 0; j < 8; ++j) {
+      const uint4 raw = *chunk(j);
       u[j][0] = raw.x; u[j][1] = raw.y; u[j][2] = raw.z; u[j][3] = raw.w;
     }
 #pragma unroll
@@ -271,43 +280,67 @@ __device__ __forceinline__ void haar_block_inplace(uint8_t* tile0, uint8_t* tile
         a[p][2 * i] = __uint_as_float(s << 16);
         a[p][2 * i + 1] = __uint_as_float(s & 0xFFFF0000u);
       }
-    const float k3 = hc[3], k4 = hc[4], k5 = hc[5];
+    const float k3 = hc[3], k4 = hc[4], k5 = hc[5], k6 = hc[6], k7 = hc[7];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const float s3 = (a[0][q] + a[1][q]) + (a[2][q] + a[3][q]);
-      const float s4 = s3 + __shfl_xor_sync(0xffffffffu, s3, 8);
-      s5[q] = s4 + __shfl_xor_sync(0xffffffffu, s4, 16);
-      hi[q] = fmaf(k3, s3, fmaf(k4, s4, k5 * s5[q]));
+      const float s4 = s3 + __shfl_xor_sync(0xffffffffu, s3, CW);
+      const float s5 = s4 + __shfl_xor_sync(0xffffffffu, s4, 2 * CW);
+      float coarse = k5 * s5;
+      top[q] = s5;
+      if constexpr (CW <= 4) {
+        const float s6 = s5 + __shfl_xor_sync(0xffffffffu, s5, 4 * CW);
+        coarse = k6 != 0.f ? fmaf(k6, s6, coarse) : coarse;   // (levels past L stay out of it: 0 * inf)
+        top[q] = s6;
+        if constexpr (CW == 2) {
+          const float s7 = s6 + __shfl_xor_sync(0xffffffffu, s6, 8 * CW);
+          coarse = k7 != 0.f ? fmaf(k7, s7, coarse) : coarse;
+          top[q] = s7;
+        }
+      }
+      hi[q] = fmaf(k3, s3, fmaf(k4, s4, coarse));
     }
   }
-  if (cross) {   // uniform over the kernel: L > 5
-    if (ok && (lane >> 3) == 0) {
-      float4* dst = reinterpret_cast<float4*>(xch + hw * kD + c * 8);
-      dst[0] = make_float4(s5[0], s5[1], s5[2], s5[3]);
-      dst[1] = make_float4(s5[4], s5[5], s5[6], s5[7]);
+  if (cross) {   // uniform over the kernel: levels that a warp's rows do not cover
+    if (ok && lane < CW) {
+      float4* dst = reinterpret_cast<float4*>(xch + hw * (8 * CW) + c * 8);
+      dst[0] = make_float4(top[0], top[1], top[2], top[3]);
+      dst[1] = make_float4(top[4], top[5], top[6], top[7]);
     }
-    named_bar_sync(kBarHaar, 256);
-    if (ok) {
-      // lane (c, q = lane >> 3) combines the eight warps' sums of columns 2 q, 2 q + 1 of chunk c (two
-      // independent chains of four), then the four lanes that share a chunk swap their pairs
-      const int qq = lane >> 3;
-      const float2* src = reinterpret_cast<const float2*>(xch + c * 8 + 2 * qq);
-      const float* cf = hc + 8 + 8 * hw;
-      float a0 = 0.f, a1 = 0.f, b0 = 0.f, b1 = 0.f;
+    named_bar_sync(bar, 32 * CW);
+    if constexpr (CW == 8) {
+      if (ok) {
+        // lane (c, q = lane >> 3) combines the eight warps' sums of columns 2 q, 2 q + 1 of chunk c (two
+        // independent chains of four), then the four lanes that share a chunk swap their pairs
+        const int qq = lane >> 3;
+        const float2* src = reinterpret_cast<const float2*>(xch + c * 8 + 2 * qq);
+        const float* cf = hc + 8 + 8 * hw;
+        float a0 = 0.f, a1 = 0.f, b0 = 0.f, b1 = 0.f;
 #pragma unroll
-      for (int w = 0; w < 8; w += 2) {
-        const float2 v0 = src[w * (kD / 2)], v1 = src[(w + 1) * (kD / 2)];
-        a0 = fmaf(cf[w], v0.x, a0);
-        a1 = fmaf(cf[w], v0.y, a1);
-        b0 = fmaf(cf[w + 1], v1.x, b0);
-        b1 = fmaf(cf[w + 1], v1.y, b1);
+        for (int w = 0; w < 8; w += 2) {
+          const float2 v0 = src[w * (kD / 2)], v1 = src[(w + 1) * (kD / 2)];
+          a0 = fmaf(cf[w], v0.x, a0);
+          a1 = fmaf(cf[w], v0.y, a1);
+          b0 = fmaf(cf[w + 1], v1.x, b0);
+          b1 = fmaf(cf[w + 1], v1.y, b1);
+        }
+        const float lo = a0 + b0, hi_ = a1 + b1;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int sl = (q << 3) | c;
+          hi[2 * q] += __shfl_sync(0xffffffffu, lo, sl);
+          hi[2 * q + 1] += __shfl_sync(0xffffffffu, hi_, sl);
+        }
       }
-      const float lo = a0 + b0, hi_ = a1 + b1;
+    } else if (ok) {
+      const float k8 = hc[8 + 7], k78 = hc[7] + k8;   // (hc[8 + 7]: weight of the last 32 rows in the first ones, k_8 alone)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int sl = (q << 3) | c;
-        hi[2 * q] += __shfl_sync(0xffffffffu, lo, sl);
-        hi[2 * q + 1] += __shfl_sync(0xffffffffu, hi_, sl);
+      for (int w = 0; w < CW; ++w) {
+        const float kw = CW == 4 && (w >> 1) == (hw >> 1) ? k78 : k8;
+        const float4* src = reinterpret_cast<const float4*>(xch + w * (8 * CW) + c * 8);
+        const float4 v0 = src[0], v1 = src[1];
+        hi[0] = fmaf(kw, v0.x, hi[0]); hi[1] = fmaf(kw, v0.y, hi[1]); hi[2] = fmaf(kw, v0.z, hi[2]); hi[3] = fmaf(kw, v0.w, hi[3]);
+        hi[4] = fmaf(kw, v1.x, hi[4]); hi[5] = fmaf(kw, v1.y, hi[5]); hi[6] = fmaf(kw, v1.z, hi[6]); hi[7] = fmaf(kw, v1.w, hi[7]);
       }
     }
   }
@@ -332,37 +365,65 @@ __device__ __forceinline__ void haar_block_inplace(uint8_t* tile0, uint8_t* tile
       }
     if (rg * 8 + 8 <= valid_rows) {   // the usual case: every row of this thread lies inside the sequence
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        *reinterpret_cast<uint4*>(base + j * 128 + ((c ^ j) << 4)) = make_uint4(u[j][0], u[j][1], u[j][2], u[j][3]);
+      for (int j = 0; j < 8; ++j) *chunk(j) = make_uint4(u[j][0], u[j][1], u[j][2], u[j][3]);
     } else {
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         uint4 out = make_uint4(u[j][0], u[j][1], u[j][2], u[j][3]);
-        if (rg * 8 + j >= valid_rows) out = make_uint4(0u, 0u, 0u, 0u);
-        *reinterpret_cast<uint4*>(base + j * 128 + ((c ^ j) << 4)) = out;
+        if (rg * 8 + (j ^ swap) >= valid_rows) out = make_uint4(0u, 0u, 0u, 0u);
+        *chunk(j) = out;
       }
     }
   }
 }
 
-// One Haar step: wait for the two raw tiles of block b (counted over all the work items of the CTA, like
+// One Haar step of a group: wait for the two raw tiles of block b (counted over all the work items of the CTA, like
 // the ring slots and barrier phases), filter them in place, hand the block to the MMA issuer.  NX = number
 // of tile slots in the ring; valid_rows = rows of the block that lie inside the sequence.
-template <int NX, typename Bars>
+template <int NX, int CW, typename Bars>
 __device__ __forceinline__ bool haar_step(uint8_t* xring, Bars* bars, float* xch, const float* hcoef, bool cross,
-                                          int b, int valid_rows, int ht, bool ok, volatile int* abort_flag,
+                                          int b, int valid_rows, int gt, int bar, bool ok, volatile int* abort_flag,
                                           int* status) {
   const int t0 = 2 * b, t1 = 2 * b + 1;
   const int s0 = t0 % NX, s1 = t1 % NX;
   if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&bars->x_full[s0], (t0 / NX) & 1, abort_flag, status, kErrHaar));
   if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&bars->x_full[s1], (t1 / NX) & 1, abort_flag, status, kErrHaar));
-  haar_block_inplace(xring + s0 * kTileBytes, xring + s1 * kTileBytes, hcoef, cross, xch + (b & 1) * 8 * kD, ht,
-                     valid_rows, ok);
+  haar_block_inplace<CW>(xring + s0 * kTileBytes, xring + s1 * kTileBytes, hcoef, cross, xch, gt, bar, valid_rows, ok);
   if (ok) {
     fence_proxy_async_smem();   // generic-proxy writes -> visible to the tensor core's reads
     warp_arrive(&bars->xf_ready[b & (kNF - 1)]);
   }
   return ok;
+}
+
+// The filter role of both kernels (256 threads): every block of the CTA's items.  Narrow heads occupy only the first
+// columns of a tile, so the warps split into 8 / CW groups that take the blocks in turn, each on the columns that are
+// there; zero columns, which no MMA reads, are left alone.  What bounds narrow heads otherwise is this stage, which works
+// on one block at a time and takes 2.0 k cycles for it whatever the columns hold.  With all warps on every block against the
+// groups: 1 x 4 x 131072, d = 16, m = 1024 key side 110 -> 98 us, query side 117 -> 99, the forward 252 -> 224 us;
+// 32 x 4 x 4096, d = 32, m = 1024 key and query side 152 + 143 -> 141 + 129 us.
+template <int NX, int CW, typename Bars>
+__device__ __forceinline__ void haar_role(uint8_t* xring, Bars* bars, float* xch, float* hcoef, const float* f, int n, int L,
+                                          int chunk_blocks, int chunks, int item0, int items, int item_step, int ht,
+                                          volatile int* abort_flag, int* status) {
+  constexpr int kGroups = 8 / CW;
+  const int grp = CW == 8 ? 0 : ht / (32 * CW), gt = CW == 8 ? ht : ht & (32 * CW - 1);
+  const bool cross = L > (CW == 8 ? 5 : CW == 4 ? 6 : 7);
+  bool ok = true;
+  int gb0 = 0;                                      // blocks of the items before
+  for (int it = item0; it < items; it += item_step) {
+    const int slab = it / chunks, blk0 = (it % chunks) * chunk_blocks;
+    const int nblk = min(chunk_blocks, (n + kBlk - 1) / kBlk - blk0);
+    named_bar_sync(kBarCoef, 256);                  // nobody reads the coefficients of the item before any more
+    haar_coef_init(hcoef, f + (size_t)slab * (L + 1), L, ht);
+    named_bar_sync(kBarCoef, 256);
+    for (int b = (grp - gb0) & (kGroups - 1); b < nblk; b += kGroups) {
+      const int gb = gb0 + b, turn = gb / kGroups;   // the group's blocks so far
+      ok = haar_step<NX, CW>(xring, bars, xch + (2 * grp + (turn & 1)) * (8 * CW * CW), hcoef, cross, gb,
+                             n - (blk0 + b) * kBlk, gt, CW == 8 ? (int)kBarHaar : kBarHaarGroup0 + grp, ok, abort_flag, status);
+    }
+    gb0 += nblk;
+  }
 }
 
 // ---- work items ---------------------------------------------------------------------------------
@@ -379,7 +440,8 @@ __device__ __forceinline__ int item_blocks(int item, int chunks, int chunk_block
 // grid (chunks * slabs, 1, feature groups) when every CTA has one item, else (min(SMs, items)); block 640.  TMEM: D1[3] at columns 0 / 128 / 256, S' half h at 384 + 64 h.
 // kMulti = false: every CTA has exactly one work item (the item loops run once and the code of the item
 // boundaries drops out).
-template <int NH, bool kMulti>
+// CW: 16-byte chunks of columns that the filter works on (see haar_block_inplace).
+template <int NH, bool kMulti, int CW>
 __global__ void __launch_bounds__(kThreads, 1)
 k_tc_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
            const __grid_constant__ CUtensorMap map_w, const float* __restrict__ f, float* __restrict__ spart,
@@ -405,7 +467,7 @@ k_tc_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CU
       mbar_init(&bars->x_full[s], 1);
       mbar_init(&bars->x_empty[s], 1);
     }
-    for (int s = 0; s < kNF; ++s) mbar_init(&bars->xf_ready[s], 8);
+    for (int s = 0; s < kNF; ++s) mbar_init(&bars->xf_ready[s], CW);
     for (int s = 0; s < kNV; ++s) {
       mbar_init(&bars->v_full[s], 1);
       mbar_init(&bars->v_empty[s], NH);
@@ -727,19 +789,8 @@ k_tc_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CU
     reg_inc<kRegsAux>();
     const int ht = threadIdx.x - 32 * kAuxWarp0;
     float* hcoef = reinterpret_cast<float*>(smem + SL::hcoef);
-    bool ok = true;
-    int gb0 = 0;                                      // blocks of the items before
-    for (int it = item0; it < items; it += item_step) {
-      const int slab = it / chunks, blk0 = (it % chunks) * chunk_blocks;
-      const int nblk = item_blocks(it, chunks, chunk_blocks, n);
-      named_bar_sync(kBarCoef, 256);                  // nobody reads the coefficients of the item before any more
-      haar_coef_init(hcoef, f + (size_t)slab * (L + 1), L, ht);
-      named_bar_sync(kBarCoef, 256);
-      for (int b = 0; b < nblk; ++b)
-        ok = haar_step<kNXK>(smem + SL::x, bars, reinterpret_cast<float*>(smem + SL::xch), hcoef, L > 5, gb0 + b,
-                             n - (blk0 + b) * kBlk, ht, ok, abort_flag, status);
-      gb0 += nblk;
-    }
+    haar_role<kNXK, CW>(smem + SL::x, bars, reinterpret_cast<float*>(smem + SL::xch), hcoef, f, n, L, chunk_blocks, chunks,
+                        item0, items, item_step, ht, abort_flag, status);
   }
   tc_fence_before_sync();
   __syncthreads();
@@ -798,7 +849,7 @@ __device__ __forceinline__ void relu_span(uint32_t in, uint32_t out) {
 // kDen: the kernel also leaves every token's denominator D' + eps' (as it divides by it, i.e. carrying the
 // filter stage's factor r) in den_out[(slab_out + slab) * n + token]: a caller that splits the features into groups
 // combines the groups' outputs with these weights.
-template <int NH, bool kMulti, bool kDen = false>
+template <int NH, bool kMulti, int CW, bool kDen = false>
 __global__ void __launch_bounds__(kThreadsQ, 1)
 k_tc_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o,
            const __grid_constant__ CUtensorMap map_w, const uint8_t* __restrict__ simg_g,
@@ -823,7 +874,7 @@ k_tc_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
       mbar_init(&bars->x_full[s], 1);
       mbar_init(&bars->x_empty[s], 1);
     }
-    for (int s = 0; s < kNF; ++s) mbar_init(&bars->xf_ready[s], 8);
+    for (int s = 0; s < kNF; ++s) mbar_init(&bars->xf_ready[s], CW);
     for (int b = 0; b < 2; ++b) {
       mbar_init(&bars->d1_full[b], 1);
       mbar_init(&bars->phi_ready[b], 8);
@@ -1064,19 +1115,8 @@ k_tc_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
     reg_inc<kRegsAux>();
     const int ht = threadIdx.x - 32 * kAuxWarp0Q;
     float* hcoef = reinterpret_cast<float*>(smem + SL::hcoef);
-    bool ok = true;
-    int gb0 = 0;                                      // blocks of the items before
-    for (int it = item0; it < items; it += item_step) {
-      const int slab = it / chunks, blk0 = (it % chunks) * chunk_blocks;
-      const int nblk = item_blocks(it, chunks, chunk_blocks, n);
-      named_bar_sync(kBarCoef, 256);                  // nobody reads the coefficients of the item before any more
-      haar_coef_init(hcoef, f + (size_t)slab * (L + 1), L, ht);
-      named_bar_sync(kBarCoef, 256);
-      for (int b = 0; b < nblk; ++b)
-        ok = haar_step<kNXQ>(smem + SL::x, bars, reinterpret_cast<float*>(smem + SL::xch), hcoef, L > 5, gb0 + b,
-                             n - (blk0 + b) * kBlk, ht, ok, abort_flag, status);
-      gb0 += nblk;
-    }
+    haar_role<kNXQ, CW>(smem + SL::x, bars, reinterpret_cast<float*>(smem + SL::xch), hcoef, f, n, L, chunk_blocks, chunks,
+                        item0, items, item_step, ht, abort_flag, status);
   }
   tc_fence_before_sync();
   __syncthreads();
@@ -1130,6 +1170,12 @@ bool tc_supported(const wersa_config& cfg) {
           (cfg.features > kGroupFeatures && cfg.features % kGroupFeatures == 0));
 }
 
+// Runs the statements with CW = the 16-byte chunks of columns that the filter stage works on as a constant.
+#define WERSA_HEAD_CHUNKS(...)                                                \
+  if (p.cfg.head_dim > 32) { constexpr int CW = 8; __VA_ARGS__ }               \
+  else if (p.cfg.head_dim > 16) { constexpr int CW = 4; __VA_ARGS__ }          \
+  else { constexpr int CW = 2; __VA_ARGS__ }
+
 // Both tensor-core kernels are launched as programmatic dependents of the kernel before them.
 template <typename... Args>
 static cudaError_t launch_pdl(void (*k)(Args...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
@@ -1173,10 +1219,12 @@ cudaError_t launch_tc_kside(const Plan& p, const Ws& w, const void* K, const voi
     return launch_pdl(kernel, grid, kThreads, smem_bytes, st, map_k, map_v, map_w, (const float*)w.f, sp, zp, sb, si,
                       p.cfg.seq_len, p.cfg.head_dim, p.cfg.levels, p.tchunk_blocks, p.tchunks, items, w.status);
   };
-  if (p.cfg.features == 256)
-    err = multi ? launch(k_tc_kside<2, true>, KsideSmem<2>::total) : launch(k_tc_kside<2, false>, KsideSmem<2>::total);
-  else
-    err = multi ? launch(k_tc_kside<1, true>, KsideSmem<1>::total) : launch(k_tc_kside<1, false>, KsideSmem<1>::total);
+  WERSA_HEAD_CHUNKS({
+    if (p.cfg.features == 256)
+      err = multi ? launch(k_tc_kside<2, true, CW>, KsideSmem<2>::total) : launch(k_tc_kside<2, false, CW>, KsideSmem<2>::total);
+    else
+      err = multi ? launch(k_tc_kside<1, true, CW>, KsideSmem<1>::total) : launch(k_tc_kside<1, false, CW>, KsideSmem<1>::total);
+  })
   *launches += 1;
   return err != cudaSuccess ? err : cudaGetLastError();
 }
@@ -1201,13 +1249,15 @@ cudaError_t launch_tc_qside(const Plan& p, const Ws& w, const void* Q, const flo
                       (const float*)w.f, beta, p.cfg.eps, p.cfg.bw_floor, p.cfg.seq_len, p.cfg.head_dim, p.cfg.levels,
                       p.tqchunk_blocks, p.tqchunks, items, w.status, den);
   };
-  if (den != nullptr) {   // groups of 256 features of a wider feature map
-    if (p.cfg.features != 256) return cudaErrorInvalidValue;
-    err = launch(k_tc_qside<2, false, true>, QsideSmem<2>::total);
-  } else if (p.cfg.features == 256)
-    err = multi ? launch(k_tc_qside<2, true>, QsideSmem<2>::total) : launch(k_tc_qside<2, false>, QsideSmem<2>::total);
-  else
-    err = multi ? launch(k_tc_qside<1, true>, QsideSmem<1>::total) : launch(k_tc_qside<1, false>, QsideSmem<1>::total);
+  if (den != nullptr && p.cfg.features != 256) return cudaErrorInvalidValue;   // (groups of 256 features of a wider map)
+  WERSA_HEAD_CHUNKS({
+    if (den != nullptr)
+      err = launch(k_tc_qside<2, false, CW, true>, QsideSmem<2>::total);
+    else if (p.cfg.features == 256)
+      err = multi ? launch(k_tc_qside<2, true, CW>, QsideSmem<2>::total) : launch(k_tc_qside<2, false, CW>, QsideSmem<2>::total);
+    else
+      err = multi ? launch(k_tc_qside<1, true, CW>, QsideSmem<1>::total) : launch(k_tc_qside<1, false, CW>, QsideSmem<1>::total);
+  })
   *launches += 1;
   return err != cudaSuccess ? err : cudaGetLastError();
 }
