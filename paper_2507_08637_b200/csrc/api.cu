@@ -443,7 +443,7 @@ wersa_status wersa_forward(wersa_ctx* ctx, const void* Q, const void* K, const v
                  launch_reduce_partials(p, w.spart, w.zpart, p.tchunks, w.S, w.z, w.Sbf, w.Simg, st, &launches));
     WERSA_STEP(0, "tc_qside", launch_tc_qside(p, w, Q, beta, O, nullptr, st, &launches));
   } else {
-    WERSA_STEP(0, "haar_filter_qk", launch_haar_filter(p, Q, kind, w.f, w.QF, K, w.KF, 0, d, st, &launches));
+    WERSA_STEP(0, "haar_filter_qk", launch_haar_filter(p, Q, kind, w.f, w.QF, K, w.KF, 0, d, true, st, &launches));
     WERSA_STEP(0, "simt_kside", launch_simt_kside(p, w, V, W, st, &launches));
     WERSA_STEP(0, "reduce_partials",
                launch_reduce_partials(p, w.spart, w.zpart, p.schunks, w.S, w.z, nullptr, nullptr, st, &launches));
@@ -711,7 +711,7 @@ wersa_status wersa_haar_filter(wersa_ctx* ctx, const void* X, const float* f, vo
   int launches = 0;
   const int kind = p.bf16 ? 1 : 0;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  WERSA_CUDA(launch_haar_filter(p, X, kind, f, XF, nullptr, nullptr, kind, p.cfg.head_dim, st, &launches));
+  WERSA_CUDA(launch_haar_filter(p, X, kind, f, XF, nullptr, nullptr, kind, p.cfg.head_dim, false, st, &launches));
   return WERSA_OK;
 }
 

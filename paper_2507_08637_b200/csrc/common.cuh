@@ -102,7 +102,7 @@ cudaError_t launch_qmean_gate_static(const Plan& p, float* scratch, const void* 
 // d: columns of the tensors as stored (a multiple of 8, at most 64).  in_kind/out_kind: 0 = float, 1 = bf16 (float input: float output).
 // XF = T_f(X), and with X2 also XF2 = T_f(X2) in the same launch.
 cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const float* f, void* XF, const void* X2,
-                               void* XF2, int out_kind, int d, cudaStream_t st, int* launches);
+                               void* XF2, int out_kind, int d, bool inputs_ready, cudaStream_t st, int* launches);
 // XF3 = T_f(X) (X bf16) as three bf16 planes hi, mid, lo (each slabs x n x head_dim) whose sum is the fp32 result;
 // with X2 also XF3_2 from X2 in the same launch, with split_S also w.Slo = bf16(w.S - w.Sbf).
 cudaError_t launch_haar_filter_split3(const Plan& p, const Ws& w, const void* X, __nv_bfloat16* XF3, const void* X2,
@@ -214,9 +214,14 @@ __device__ __forceinline__ float sum2(f32x2 v) {
   return lo + hi;
 }
 
-// Launch as a programmatic dependent of the work before it in the stream.  The kernel's first instruction
-// must be griddepcontrol.wait (nothing is read or written before that work has completed), so ordering and
-// visibility are those of a plain launch; only the placement of the CTAs overlaps the end of that work.
+// Launch as a programmatic dependent of the work before it in the stream.  Ordering and visibility are those of a plain
+// launch, since the kernel writes nothing and reads nothing of that work before wait_for_stream_predecessor(); only the
+// placement of its CTAs, and what they set up or fetch ahead of the wait, overlaps the end of that work.  What may be
+// fetched ahead: what was complete before the kernel in front of this one in its pass passed its own wait (the arguments
+// of the call and the results of earlier kernels), hence nothing in the first kernel of a pass.  Where work stands ahead of
+// the wait, results of the kernel in front are read with load_after_wait (or __ldcg where the L1 has no use for them), not
+// through a const __restrict__ pointer: such a load counts as free of order with anything, and the compiler did move the row
+// vector of dQ above the wait.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                 Args&&... args) {
@@ -233,6 +238,21 @@ inline cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block,
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 __device__ __forceinline__ void wait_for_stream_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ float load_after_wait(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 load4_after_wait(const float* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+  return v;
+}
+// The kernel behind this one may be placed once every CTA of this grid has got here (or has ended).  Not where that kernel
+// is bound by memory and several of its CTAs share an SM: placed as the SMs fall free, they gather on some and all start at
+// once, and the passes of the first ones stay in step (the mean pool behind the query side of 1 x 8 x 131072: 16 us more a
+// forward; k_haar_backward behind the key side of 4 x 8 x 16384: 160 instead of 105 us).
+__device__ __forceinline__ void let_stream_successor_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---- device helpers ------------------------------------------------------------------------
 __device__ __forceinline__ float to_f32(float x) { return x; }

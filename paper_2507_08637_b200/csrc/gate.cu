@@ -230,7 +230,10 @@ __global__ void __launch_bounds__(32) k_batch_gate(int H, int L1, const float* _
 // (four loads in flight), the 16 parts are added in a fixed order: the result repeats bit for bit.
 __global__ void __launch_bounds__(256) k_band_reduce(const float* __restrict__ bands, int slabs, int htiles,
                                                      int L, float* __restrict__ df) {
-  wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
+  // (launched as a programmatic dependent: see launch_after; the gate backward, which may be placed ahead of this kernel's
+  // wait, reads nothing of the passes over dK_F and dQ_F but what this kernel leaves it)
+  let_stream_successor_start();
+  wait_for_stream_predecessor();
   __shared__ float part[16][kBandVals];
   const int slab = blockIdx.x, j = threadIdx.x & (kBandVals - 1), pt = threadIdx.x >> 4;
   float s = 0.f;
@@ -238,11 +241,11 @@ __global__ void __launch_bounds__(256) k_band_reduce(const float* __restrict__ b
     const float* src = bands + (((size_t)which * slabs + slab) * htiles) * kBandVals + j;
     int t = pt;
     for (; t + 48 < htiles; t += 64) {
-      const float v0 = src[(size_t)t * kBandVals], v1 = src[(size_t)(t + 16) * kBandVals];
-      const float v2 = src[(size_t)(t + 32) * kBandVals], v3 = src[(size_t)(t + 48) * kBandVals];
+      const float v0 = __ldcg(src + (size_t)t * kBandVals), v1 = __ldcg(src + (size_t)(t + 16) * kBandVals);
+      const float v2 = __ldcg(src + (size_t)(t + 32) * kBandVals), v3 = __ldcg(src + (size_t)(t + 48) * kBandVals);
       s += (v0 + v1) + (v2 + v3);
     }
-    for (; t < htiles; t += 16) s += src[(size_t)t * kBandVals];
+    for (; t < htiles; t += 16) s += __ldcg(src + (size_t)t * kBandVals);
   }
   part[pt][j] = s;
   __syncthreads();
@@ -281,10 +284,10 @@ __global__ void __launch_bounds__(kD) k_sum_floats(const float* __restrict__ x, 
 // 20 us with every thread working out du itself (with the gate shared by the heads nine loads after one another:
 // 19 us at B=5 H=3), 11 now (9 at B=5 H=3).
 __device__ __forceinline__ float gate_df(const float* __restrict__ df, int b, int h, int H, int per_head, int i) {
-  if (per_head) return df[((size_t)b * H + h) * kBandVals + i];
+  if (per_head) return __ldcg(df + ((size_t)b * H + h) * kBandVals + i);
   float s = 0.f;
 #pragma unroll 4
-  for (int hh = 0; hh < H; ++hh) s += df[((size_t)b * H + hh) * kBandVals + i];
+  for (int hh = 0; hh < H; ++hh) s += __ldcg(df + ((size_t)b * H + hh) * kBandVals + i);
   return s;
 }
 constexpr int kGateRound = 28;   // batch elements of a round: a multiple of four, 28 x 9 values for the 256 threads
@@ -293,8 +296,11 @@ __global__ void __launch_bounds__(256) k_gate_backward(
     const float* __restrict__ gate_w, const float* __restrict__ omega, const float* __restrict__ sumdD,
     int n_sumdD, const float* __restrict__ beta, float eps, float bw_floor, int m, int B, int H, int dcols, int L1,
     int per_head, float* __restrict__ dbeta, float* __restrict__ dgate_w, float* __restrict__ dgate_b,
-    float* __restrict__ domega, float* __restrict__ dqbar) {
-  wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
+    float* __restrict__ domega, float* __restrict__ dqbar, bool first) {
+  // (launched as a programmatic dependent: see launch_after; the pass that writes dQ may be placed ahead of this kernel's
+  // wait, and unless it is the first one of its pass the gate weights are fetched ahead of it)
+  if (first) wait_for_stream_predecessor();
+  let_stream_successor_start();
   __shared__ float part[4][kMaxLevels + 1][kD];
   __shared__ float gbs[4][kMaxLevels + 1];
   __shared__ float dus[kGateRound][kMaxLevels + 1];
@@ -308,6 +314,7 @@ __global__ void __launch_bounds__(256) k_gate_backward(
       gw_acc[i] = gb_acc[i] = 0.f;
       gw[i] = i < L1 && gate_w != nullptr && c < dcols ? gate_w[((size_t)h * dcols + c) * L1 + i] : 0.f;
     }
+    wait_for_stream_predecessor();
     const int db = tid / (kMaxLevels + 1), di = tid - db * (kMaxLevels + 1);   // this thread's du of a round
     for (int b0 = 0; b0 < B; b0 += kGateRound) {
       float qb[kGateRound / 4];
@@ -360,13 +367,14 @@ __global__ void __launch_bounds__(256) k_gate_backward(
     // element, then the parts are added in order
     const int i = tid & 15, q = tid >> 4;
     float acc = 0.f;
+    wait_for_stream_predecessor();
     if (domega != nullptr && i < L1) {
       for (int b = q; b < B; b += 16) {
         if (per_head) {
 #pragma unroll 4
           for (int h = 0; h < H; ++h) {
             const int slab = b * H + h;
-            acc += df[(size_t)slab * kBandVals + i] * sg[(size_t)slab * L1 + i];
+            acc += __ldcg(df + (size_t)slab * kBandVals + i) * sg[(size_t)slab * L1 + i];
           }
         } else {
           acc += gate_df(df, b, 0, H, 0, i) * sg[((size_t)b * H) * L1 + i];
@@ -382,9 +390,10 @@ __global__ void __launch_bounds__(256) k_gate_backward(
       domega[tid] = s;
     }
   } else {
+    wait_for_stream_predecessor();
     float tot = 0.f;
 #pragma unroll 4
-    for (int i = tid; i < n_sumdD; i += 256) tot += sumdD[i];
+    for (int i = tid; i < n_sumdD; i += 256) tot += __ldcg(sumdD + i);
     flat[tid] = tot;
     __syncthreads();
     for (int o = 128; o > 0; o >>= 1) {
@@ -516,7 +525,7 @@ cudaError_t launch_gate_backward_from(const Plan& p, const Ws& w, const float* d
                                       float* dgate_w, float* dgate_b, float* domega, cudaStream_t st, int* launches) {
   launch_after(k_gate_backward, dim3(p.cfg.heads + 2), dim3(256), 0, st, df, w.sg, w.qbar, gate_w, omega, sumdD_total, 1,
                beta, p.cfg.eps, p.cfg.bw_floor, p.cfg.features, p.cfg.batch, p.cfg.heads, p.cfg.head_dim, p.L1, p.cfg.gate_per_head,
-               dbeta, dgate_w, dgate_b, domega, w.dqbar);
+               dbeta, dgate_w, dgate_b, domega, w.dqbar, true);
   *launches += 1;
   return cudaGetLastError();
 }
@@ -528,7 +537,8 @@ cudaError_t launch_gate_backward(const Plan& p, const Ws& w, int band_blocks, co
   launch_after(k_band_reduce, dim3(p.slabs), dim3(256), 0, st, w.bands, p.slabs, band_blocks, p.cfg.levels, df);
   launch_after(k_gate_backward, dim3(p.cfg.heads + 2), dim3(256), 0, st, df, w.sg, w.qbar, gate_w, omega, w.sumdD, n_sumdD, beta,
                                     p.cfg.eps, p.cfg.bw_floor, p.cfg.features, p.cfg.batch, p.cfg.heads,
-                                    p.cfg.head_dim, p.L1, p.cfg.gate_per_head, dbeta, dgate_w, dgate_b, domega, w.dqbar);
+                                    p.cfg.head_dim, p.L1, p.cfg.gate_per_head, dbeta, dgate_w, dgate_b, domega, w.dqbar,
+                                    false);
   *launches += 2;
   return cudaGetLastError();
 }

@@ -45,6 +45,7 @@ __global__ void __launch_bounds__(256) k_group_bwd_prep(const __nv_bfloat16* __r
                                                         int n, int L1, size_t tokens, int groups,
                                                         float* __restrict__ Dtot, float* __restrict__ dDtot) {
   wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
+  let_stream_successor_start();
   const size_t idx = (size_t)blockIdx.x * 256 + threadIdx.x;
   const size_t tok = idx / tpt;
   const int c0 = (int)(idx & (tpt - 1)) * 8;

@@ -20,13 +20,20 @@ struct LevelCoef {
   float k[kMaxLevels + 1];   // k[i] = (f_i - f_{i-1}) / 2^i for 1 <= i <= L, else 0
 };
 
-__device__ __forceinline__ LevelCoef level_coef(const float* __restrict__ f, int L) {
+// kOrdered: f is the result of the kernel in front (see launch_after).
+template <bool kOrdered = false> __device__ __forceinline__ LevelCoef level_coef(const float* __restrict__ f, int L) {
+  float v[kMaxLevels + 1];   // (no load depends on another one or on a branch)
+#pragma unroll
+  for (int i = 0; i <= kMaxLevels; ++i) {
+    const float* p = f + (i <= L ? i : L);
+    v[i] = kOrdered ? load_after_wait(p) : *p;
+  }
   LevelCoef c;
-  c.f0 = f[0];
+  c.f0 = v[0];
   float scale = 0.5f;
 #pragma unroll
   for (int i = 1; i <= kMaxLevels; ++i) {
-    c.k[i] = (i <= L) ? (f[i] - f[i - 1]) * scale : 0.f;
+    c.k[i] = (i <= L) ? (v[i] - v[i - 1]) * scale : 0.f;
     scale *= 0.5f;
   }
   c.k[0] = 0.f;
@@ -117,13 +124,17 @@ __device__ __forceinline__ void add_coarse4(const float (*ex)[W], const LevelCoe
 // the others (the pass is bound by memory bandwidth).
 // With kAddVec every output row of slab s also gets vec[s][:] * vec_scale added (the mean-pool term of dQ); that pass
 // goes through the blocks backwards, since the end of its input is what k_haar_backward has left in the L2.
+// inputs_ready: X and X2 were complete before the kernel in front of this one passed its wait (see launch_after), and are
+// fetched ahead of this one's.  That holds for dQ_F too, and the rows of the pass that writes dQ are on their way while the
+// gate backward is still at work.
 // grid (col_blocks<32>, slabs, 1 or 2 tensors: X -> XF, X2 -> XF2); block 256.
 template <bool kFull, typename Tin, typename Tout, bool kAddVec>
 __global__ void __launch_bounds__(256, 4) k_haar_filter(const Tin* __restrict__ X, const float* __restrict__ f,
                                                      Tout* __restrict__ XF, const Tin* __restrict__ X2,
                                                      Tout* __restrict__ XF2, int n, int d_arg, int L,
-                                                     const float* __restrict__ vec, float vec_scale) {
-  wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
+                                                     const float* __restrict__ vec, float vec_scale, bool inputs_ready) {
+  // (launched as a programmatic dependent: see launch_after)
+  if (!kAddVec && !inputs_ready) wait_for_stream_predecessor();
   const int d = kFull ? kD : d_arg;
   __shared__ __align__(16) float ex[8][kHalfD];   // 32-row sums of the warps
   const int bx = kAddVec ? gridDim.x - 1 - blockIdx.x : blockIdx.x, slab = kAddVec ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
@@ -132,7 +143,6 @@ __global__ void __launch_bounds__(256, 4) k_haar_filter(const Tin* __restrict__ 
   const int row0 = at.row0 + rg * 8;
   const int col0 = at.col;   // first of this thread's four columns
   const int rows = at.on ? n - row0 : 0;   // rows of this thread inside the sequence
-  const LevelCoef k = level_coef(f + (size_t)slab * (L + 1), L);
   float x[8][4];
   {
     const Tin* xp = (blockIdx.z == 0 ? X : X2) + ((size_t)slab * n + row0) * d + col0;
@@ -146,6 +156,11 @@ __global__ void __launch_bounds__(256, 4) k_haar_filter(const Tin* __restrict__ 
       }
     }
   }
+  if constexpr (!kAddVec) {   // (with the row vector it is the last kernel of its pass, and f is the forward's)
+    wait_for_stream_predecessor();
+    let_stream_successor_start();
+  }
+  const LevelCoef k = level_coef<!kAddVec>(f + (size_t)slab * (L + 1), L);
   float hi[4], s5[4];
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
@@ -153,8 +168,15 @@ __global__ void __launch_bounds__(256, 4) k_haar_filter(const Tin* __restrict__ 
     const float s4 = sum16(s3);
     s5[c] = sum32(s4);
     hi[c] = fmaf(k.k[3], s3, fmaf(k.k[4], s4, k.k[5] * s5[c]));
-    if constexpr (kAddVec) {
-      if (at.on) hi[c] = fmaf(vec[(size_t)slab * kD + col0 + c], vec_scale, hi[c]);
+  }
+  if constexpr (kAddVec) {
+    wait_for_stream_predecessor();   // the row vector is the gate backward's result
+    if (at.on) {
+      const float4 v = load4_after_wait(vec + (size_t)slab * kD + col0);
+      hi[0] = fmaf(v.x, vec_scale, hi[0]);
+      hi[1] = fmaf(v.y, vec_scale, hi[1]);
+      hi[2] = fmaf(v.z, vec_scale, hi[2]);
+      hi[3] = fmaf(v.w, vec_scale, hi[3]);
     }
   }
   if (L > 5) {
@@ -222,8 +244,9 @@ template <bool kFull, typename Tout>
 __global__ void __launch_bounds__(256, 3) k_haar_filter_bf16(const __nv_bfloat16* __restrict__ X,
                                                              const float* __restrict__ f, Tout* __restrict__ XF,
                                                              const __nv_bfloat16* __restrict__ X2,
-                                                             Tout* __restrict__ XF2, int n, int d_arg, int L) {
-  wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
+                                                             Tout* __restrict__ XF2, int n, int d_arg, int L,
+                                                             bool inputs_ready) {
+  if (!inputs_ready) wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   const int d = kFull ? kD : d_arg;
   __shared__ __align__(16) float ex[8][kD];   // 32-row sums of the warps
   const int slab = blockIdx.y;
@@ -231,7 +254,6 @@ __global__ void __launch_bounds__(256, 3) k_haar_filter_bf16(const __nv_bfloat16
   const ColMap<64> at(blockIdx.x, cg * 8, d);
   const int row0 = at.row0 + rg * 8;
   const int rows = at.on ? n - row0 : 0;   // rows of this thread inside the sequence
-  const LevelCoef k = level_coef(f + (size_t)slab * (L + 1), L);
   uint32_t u[8][4];
   {
     const __nv_bfloat16* xp = (blockIdx.z == 0 ? X : X2) + ((size_t)slab * n + row0) * d + at.col;
@@ -242,6 +264,9 @@ __global__ void __launch_bounds__(256, 3) k_haar_filter_bf16(const __nv_bfloat16
       u[j][0] = raw.x; u[j][1] = raw.y; u[j][2] = raw.z; u[j][3] = raw.w;
     }
   }
+  wait_for_stream_predecessor();   // f may be the gate kernel's result
+  let_stream_successor_start();
+  const LevelCoef k = level_coef<true>(f + (size_t)slab * (L + 1), L);
   float hi[8];
   packed_coarse(u, k, L, ex, hi);
   rows_fence(u);
@@ -321,6 +346,7 @@ __global__ void __launch_bounds__(256, 3) k_haar_filter_split3(const __nv_bfloat
                                                                const __nv_bfloat16* __restrict__ Sbf,
                                                                __nv_bfloat16* __restrict__ Slo, int features, int groups) {
   wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
+  let_stream_successor_start();
   if (S != nullptr && blockIdx.z == gridDim.z - 1) {   // the last layer of the grid: Slo = bf16(S - Sbf)
     const int per = features * kD;   // of one group (S has a slab's features together, Sbf and Slo a group's slabs)
     for (int i = (blockIdx.x * 256 + threadIdx.x) * 4; i < per * groups; i += gridDim.x * 1024) {
@@ -409,6 +435,7 @@ k_haar_backward(const Tin* __restrict__ X1, const float* __restrict__ G1, Tout* 
                 const Tin* __restrict__ X2, const float* __restrict__ G2, Tout* __restrict__ dX2,
                 const float* __restrict__ f, float* __restrict__ bands, int which, int n, int d_arg, int L) {
   wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
+  let_stream_successor_start();
   const bool second = blockIdx.z != 0;
   const Tin* __restrict__ X = second ? X2 : X1;
   const float* __restrict__ G = second ? G2 : G1;
@@ -550,7 +577,7 @@ int haar_band_blocks(const Plan& p, int d) { return col_blocks<32>(p.htiles, d);
 
 // X2 / XF2: a second tensor of the same shape in the same launch (or null).
 cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const float* f, void* XF, const void* X2,
-                               void* XF2, int out_kind, int d, cudaStream_t st, int* launches) {
+                               void* XF2, int out_kind, int d, bool inputs_ready, cudaStream_t st, int* launches) {
   const unsigned z = X2 != nullptr ? 2 : 1;
   const dim3 grid(col_blocks<32>(p.htiles, d), p.slabs, z), grid_bf(col_blocks<64>(p.htiles, d), p.slabs, z);
   const int n = p.cfg.seq_len, L = p.cfg.levels;
@@ -558,13 +585,14 @@ cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const 
   cudaError_t err;
   WERSA_FULL({
     if (in_kind == 1 && out_kind == 1)
-      err = launch_after(k_haar_filter_bf16<kFull, bf>, grid_bf, dim3(256), 0, st, (const bf*)X, f, (bf*)XF, (const bf*)X2, (bf*)XF2, n, d, L);
+      err = launch_after(k_haar_filter_bf16<kFull, bf>, grid_bf, dim3(256), 0, st, (const bf*)X, f, (bf*)XF, (const bf*)X2, (bf*)XF2, n, d, L,
+                         inputs_ready);
     else if (in_kind == 1 && out_kind == 0)
       err = launch_after(k_haar_filter_bf16<kFull, float>, grid_bf, dim3(256), 0, st, (const bf*)X, f, (float*)XF, (const bf*)X2,
-                         (float*)XF2, n, d, L);
+                         (float*)XF2, n, d, L, inputs_ready);
     else
       err = launch_after(k_haar_filter<kFull, float, float, false>, grid, dim3(256), 0, st, (const float*)X, f, (float*)XF,
-                         (const float*)X2, (float*)XF2, n, d, L, nullptr, 0.f);
+                         (const float*)X2, (float*)XF2, n, d, L, nullptr, 0.f, inputs_ready);
   })
   *launches += 1;
   return err != cudaSuccess ? err : cudaGetLastError();
@@ -578,9 +606,9 @@ cudaError_t launch_haar_filter_addvec(const Plan& p, const float* G, const float
   cudaError_t err;
   WERSA_FULL({
     if (out_kind == 0)
-      err = launch_after(k_haar_filter<kFull, float, float, true>, grid, dim3(256), 0, st, G, f, (float*)dX, nullptr, nullptr, n, d, L, vec, vec_scale);
+      err = launch_after(k_haar_filter<kFull, float, float, true>, grid, dim3(256), 0, st, G, f, (float*)dX, nullptr, nullptr, n, d, L, vec, vec_scale, true);
     else
-      err = launch_after(k_haar_filter<kFull, float, bf, true>, grid, dim3(256), 0, st, G, f, (bf*)dX, nullptr, nullptr, n, d, L, vec, vec_scale);
+      err = launch_after(k_haar_filter<kFull, float, bf, true>, grid, dim3(256), 0, st, G, f, (bf*)dX, nullptr, nullptr, n, d, L, vec, vec_scale, true);
   })
   *launches += 1;
   return err != cudaSuccess ? err : cudaGetLastError();

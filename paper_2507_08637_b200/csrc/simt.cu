@@ -361,7 +361,6 @@ template <int M, int DP, int TI, int TG>
 __global__ void __launch_bounds__(M * TG, 1)
 k_simt_kside(const float* __restrict__ KF, const void* __restrict__ V, const void* __restrict__ W, int kind,
              float* __restrict__ spart, float* __restrict__ zpart, int n, int d, int chunk_rows) {
-  wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   using C = Cfg<M, DP, TI, TG, false, true>;
   extern __shared__ __align__(16) float sm[];
   const Who<C> me;
@@ -370,9 +369,12 @@ k_simt_kside(const float* __restrict__ KF, const void* __restrict__ V, const voi
   const void* v = kind == 0 ? (const void*)(static_cast<const float*>(V) + (size_t)slab * n * d)
                             : (const void*)(static_cast<const __nv_bfloat16*>(V) + (size_t)slab * n * d);
   const int first = chunk * chunk_rows, last = min(n, first + chunk_rows);
-  load_rows<DP, C::CT, C::kThreads>(kf, 0, d, last, first, sm + C::x);
+  // (launched as a programmatic dependent, see launch_after: V and W are arguments, K_F comes from the kernel before)
   load_rows<DP, C::CT, C::kThreads>(v, kind, d, last, first, sm + C::g);
   load_wt<M, DP, C::kThreads>(W, kind, d, sm + C::wt);
+  wait_for_stream_predecessor();
+  if constexpr (TI == 2) let_stream_successor_start();   // (with full tiles: 2 x 4 x 4096, d = 32, m = 128 146 instead of 141 us)
+  load_rows<DP, C::CT, C::kThreads>(kf, 0, d, last, first, sm + C::x);
   f32x2 acc[8][DP / 16];
   float zacc[8];
 #pragma unroll
@@ -416,7 +418,6 @@ __global__ void __launch_bounds__(M * TG, 1)
 k_simt_qside(const float* __restrict__ QF, const void* __restrict__ W, int kind, const float* __restrict__ Sg,
              const float* __restrict__ zg, const float* __restrict__ beta, float eps, float bw_floor,
              void* __restrict__ O, int n, int d, int chunk_rows) {
-  wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   using C = Cfg<M, DP, TI, TG, true, false>;
   extern __shared__ __align__(16) float sm[];
   const Who<C> me;
@@ -425,10 +426,12 @@ k_simt_qside(const float* __restrict__ QF, const void* __restrict__ W, int kind,
   void* o = kind == 0 ? (void*)(static_cast<float*>(O) + (size_t)slab * n * d)
                       : (void*)(static_cast<__nv_bfloat16*>(O) + (size_t)slab * n * d);
   const int first = chunk * chunk_rows, last = min(n, first + chunk_rows);
+  // (launched as a programmatic dependent, see launch_after: Q_F is older than the reduction, which leaves S' and z')
   load_rows<DP, C::CT, C::kThreads>(qf, 0, d, last, first, sm + C::x);
-  load_b<M, DP, C::kThreads>(Sg + (size_t)slab * M * kD, sm + C::b);
   load_wt<M, DP, C::kThreads>(W, kind, d, sm + C::wt);
-  for (int i = threadIdx.x; i < M; i += C::kThreads) sm[C::zs + i] = zg[(size_t)slab * M + i];
+  wait_for_stream_predecessor();
+  load_b<M, DP, C::kThreads>(Sg + (size_t)slab * M * kD, sm + C::b);
+  for (int i = threadIdx.x; i < M; i += C::kThreads) sm[C::zs + i] = __ldcg(zg + (size_t)slab * M + i);
   const float bw = fmaxf(beta[0], bw_floor);
   const float epsp = eps * (float)M * bw * bw;
   float* R = sm + C::r + me.gid * C::TT * 64;
@@ -480,6 +483,7 @@ k_simt_bwd_qside(const float* __restrict__ QF, const void* __restrict__ W, int k
                  const void* __restrict__ dO, float* __restrict__ dQF, float* __restrict__ dspart,
                  float* __restrict__ dzpart, float* __restrict__ sumdD, int n, int d, int chunk_rows) {
   wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
+  if constexpr (TI == 2) let_stream_successor_start();   // (with full tiles: 2 x 4 x 4096, d = 32, m = 128 146 instead of 141 us)
   using C = Cfg<M, DP, TI, TG, true, true>;
   extern __shared__ __align__(16) float sm[];
   const Who<C> me;
@@ -493,7 +497,7 @@ k_simt_bwd_qside(const float* __restrict__ QF, const void* __restrict__ W, int k
   load_rows<DP, C::CT, C::kThreads>(go, kind, d, last, first, sm + C::g);
   load_b<M, DP, C::kThreads>(Sg + (size_t)slab * M * kD, sm + C::b);
   load_wt<M, DP, C::kThreads>(W, kind, d, sm + C::wt);
-  for (int i = threadIdx.x; i < M; i += C::kThreads) sm[C::zs + i] = zg[(size_t)slab * M + i];
+  for (int i = threadIdx.x; i < M; i += C::kThreads) sm[C::zs + i] = __ldcg(zg + (size_t)slab * M + i);
   const float bw = fmaxf(beta[0], bw_floor);
   const float epsp = eps * (float)M * bw * bw;
   f32x2 acc[8][DP / 16];
@@ -602,7 +606,6 @@ __global__ void __launch_bounds__(M * TG, 1)
 k_simt_bwd_kside(const float* __restrict__ KF, const void* __restrict__ V, const void* __restrict__ W, int kind,
                  const float* __restrict__ dSg, const float* __restrict__ dzg, void* __restrict__ dV, int gkind,
                  float* __restrict__ dKF, int n, int d, int chunk_rows) {
-  wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   using C = Cfg<M, DP, TI, TG, true, true>;
   extern __shared__ __align__(16) float sm[];
   const Who<C> me;
@@ -614,11 +617,13 @@ k_simt_bwd_kside(const float* __restrict__ KF, const void* __restrict__ V, const
                         : (void*)(static_cast<__nv_bfloat16*>(dV) + (size_t)slab * n * d);
   float* dkf = dKF + (size_t)slab * n * d;
   const int first = chunk * chunk_rows, last = min(n, first + chunk_rows);
+  // (launched as a programmatic dependent, see launch_after: K_F is the forward's, the reduction leaves dS' and dz')
   load_rows<DP, C::CT, C::kThreads>(kf, 0, d, last, first, sm + C::x);
   load_rows<DP, C::CT, C::kThreads>(v, kind, d, last, first, sm + C::g);
-  load_b<M, DP, C::kThreads>(dSg + (size_t)slab * M * kD, sm + C::b);
   load_wt<M, DP, C::kThreads>(W, kind, d, sm + C::wt);
-  for (int i = threadIdx.x; i < M; i += C::kThreads) sm[C::zs + i] = dzg[(size_t)slab * M + i];
+  wait_for_stream_predecessor();
+  load_b<M, DP, C::kThreads>(dSg + (size_t)slab * M * kD, sm + C::b);
+  for (int i = threadIdx.x; i < M; i += C::kThreads) sm[C::zs + i] = __ldcg(dzg + (size_t)slab * M + i);
   float* R = sm + C::r + me.gid * C::TT * 64;
   const float* zs = sm + C::zs + me.fg * 64 + me.tx;
   cp_async_wait_all();

@@ -110,7 +110,6 @@ k_tc_bwd_kside(const __grid_constant__ CUtensorMap map_kf, const __grid_constant
                const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_ds,
                const float* __restrict__ dzg, const __grid_constant__ CUtensorMap map_dv,
                const __grid_constant__ CUtensorMap map_dkf, int n, int d, int slabs, int* __restrict__ status) {
-  wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
   using SL = BwdKSmem<NH>;
@@ -163,6 +162,7 @@ k_tc_bwd_kside(const __grid_constant__ CUtensorMap map_kf, const __grid_constant
       mbar_arrive_expect_tx(&bars->w_full, NH * kTileBytes);
 #pragma unroll
       for (int h = 0; h < NH; ++h) tma_load_3d(smem + SL::wt + h * kTileBytes, &map_w, 0, h * kTile, 0, &bars->w_full);
+      griddep_wait();   // (W^T is the forward's; nothing else is read or written before: see launch_after)
       int sent = 0, seg = 0, slab_now = -1;
       bool ok = true;
       auto store_results = [&](int it) {   // of tile `it`, from its stage
@@ -332,6 +332,7 @@ k_tc_bwd_kside(const __grid_constant__ CUtensorMap map_kf, const __grid_constant
     }
   } else if (warp < kKEpiWarp0) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kKRegsElem));
+    griddep_wait();   // (and no let_stream_successor_start: see there)
     const int wq = (warp - 4) >> 2;
     const uint32_t trow = tmem + ((32u * (warp & 3)) << 16) + 32 * wq;   // this warp's lane quarter and columns
     uint32_t b = 0, par = 0;   // accumulator and phase of the next unit
@@ -385,7 +386,7 @@ k_tc_bwd_kside(const __grid_constant__ CUtensorMap map_kf, const __grid_constant
             uint32_t ph[8], pl[8];
 #pragma unroll
             for (int j = 0; j < 8; j += 2) {
-              const float4 zz = __ldg(reinterpret_cast<const float4*>(z + 16 * q + 2 * j));
+              const float4 zz = load4_after_wait(z + 16 * q + 2 * j);
               const f32x2 zp[2] = {pk2(zz.x, zz.y), pk2(zz.z, zz.w)};
 #pragma unroll
               for (int i = 0; i < 2; ++i) {
@@ -498,7 +499,6 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
                const __grid_constant__ CUtensorMap map_dqf, float* __restrict__ dspart, float* __restrict__ dzpart,
                float* __restrict__ sumdD, int n, int d, int slabs, int* __restrict__ status,
                const float* __restrict__ den_ext, const float* __restrict__ dd_ext) {
-  wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
   using SL = BwdQSmem<NH>;
@@ -539,6 +539,7 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
       mbar_arrive_expect_tx(&bars->w_full, NH * kTileBytes);
 #pragma unroll
       for (int h = 0; h < NH; ++h) tma_load_3d(smem + SL::wt + h * kTileBytes, &map_w, 0, h * kTile, 0, &bars->w_full);
+      griddep_wait();   // (W^T is the forward's; nothing else is read or written before: see launch_after)
       int it = 0, seg = -1, slab_now = -1, x_sent = 0, do_sent = 0, s_sent = 0;
       bool ok = true;
       for (int gt = g0; gt < g1; ++gt, ++it) {
@@ -684,6 +685,8 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
     const int et = threadIdx.x - 128, wq = (warp - 4) >> 2;
     const int tl = 32 * (warp & 3) + lane;                     // token = TMEM lane
     const uint32_t trow = tmem + ((32u * (warp & 3)) << 16);   // this warp's lane quarter
+    griddep_wait();
+    griddep_launch();
     float* zs = reinterpret_cast<float*>(smem + SL::zs);
     float* cs = reinterpret_cast<float*>(smem + SL::cs);
     float* scratch = reinterpret_cast<float*>(smem + SL::scratch);
@@ -738,9 +741,9 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
             for (int h = 0; h < NH; ++h) tmem_ld32(trow + h * 128 + 32 * wq, r[h]);
             if constexpr (kGroup) {
               if (row < n) {
-                const float D = den_ext[(size_t)slab * n + row];
+                const float D = __ldcg(den_ext + (size_t)slab * n + row);
                 inv = 1.f / D;
-                c = dd_ext[(size_t)slab * n + row] * D;
+                c = __ldcg(dd_ext + (size_t)slab * n + row) * D;
               }
             }
             tmem_ld_wait();
