@@ -11,6 +11,7 @@ bool tc_supported(const wersa_config& cfg);   // tc_fwd.cu
 namespace {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+constexpr long long kXUnits = 64;   // (see make_plan)
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 int next_pow2(int n) {
   int p = 1;
@@ -122,6 +123,27 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     p->schunks = ceil_div(n, rows_best);
   }
 
+  // fp32 forward on the tensor cores, from kXUnits tiles x groups of 128 features on: 2 x 4 x 1024, m = 128 (64 units) 49 -> 26
+  // us, in d = 32 37 -> 23; 1 x 4 x 1024, m = 256 (64) 40 -> 26.  One CTA per SM and group, in chunks that minimise
+  // waves x (tiles + 3), 3 tiles being about what a CTA spends before its first and after its last one.
+  p->use_x = false;
+  p->xchunks = 1;
+  p->xchunk_tiles = 1;
+  if (!p->bf16 && !(c.flags & WERSA_FLAG_SIMT_ONLY) && m >= 128) {
+    const int tiles = ceil_div(n, 128), groups = m / 128;
+    p->use_x = (long long)p->slabs * tiles * groups >= kXUnits;
+    long long best = 0;
+    for (int ch = 1; ch <= tiles && ch <= 64; ++ch) {
+      const long long cost = (long long)ceil_div(p->slabs * groups * ch, p->sms) * (ceil_div(tiles, ch) + 3);
+      if (ch == 1 || cost < best) {
+        best = cost;
+        p->xchunks = ch;
+      }
+    }
+    p->xchunk_tiles = ceil_div(tiles, p->xchunks);
+    p->xchunks = ceil_div(tiles, p->xchunk_tiles);
+  }
+
   p->tchunks = 0;
   p->tchunk_blocks = 0;
   p->tqchunks = 0;
@@ -192,6 +214,7 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   // rows of partial sums: chunks of the forward or of the fp32 kernels, or the segments of the tensor-core
   // backward (slot = CTA + slab) of one feature group; of all feature groups in the forward
   size_t part_rows = slabs * p->groups * (p->use_tc ? p->tchunks : p->schunks) * (m < kGroupFeatures ? m : kGroupFeatures);
+  if (p->use_x && p->xchunks > p->schunks) part_rows = slabs * p->xchunks * m;
   if (p->use_tc && p->with_backward) {
     const size_t seg_rows = ((size_t)p->bctas + slabs) * (m < kGroupFeatures ? m : kGroupFeatures);
     if (seg_rows > part_rows) part_rows = seg_rows;
@@ -211,9 +234,16 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   take(p->dpad ? 256 : 0);
   p->off_Og = take(grouped ? io_bytes * slab_elems * p->groups : 0);
   p->off_den = take(grouped ? sizeof(float) * slabs * n * p->groups : 0);
-  const bool need_xf = !p->use_tc;   // the tensor-core kernels filter on chip (forward) or read bf16 planes (backward)
+  const bool need_xf = !p->use_tc && (!p->use_x || p->with_backward);   // the tensor-core kernels filter on chip (forward) or read bf16 planes (backward)
   p->off_QF = take(need_xf ? sizeof(float) * slab_elems : 0);
   p->off_KF = take(need_xf ? sizeof(float) * slab_elems : 0);
+  if (p->use_x) {   // (the query side's shares follow on from KF3 into V3: see launch_tcx_qside)
+    p->off_QF3 = take(3 * sizeof(__nv_bfloat16) * slab_elems);
+    p->off_KF3 = take(3 * sizeof(__nv_bfloat16) * slab_elems);
+    p->off_V3 = take(3 * sizeof(__nv_bfloat16) * slab_elems);
+  } else {
+    p->off_QF3 = p->off_KF3 = p->off_V3 = 0;
+  }
   if (p->with_backward) {
     p->off_dS = take(sizeof(float) * slabs * m * kD);
     p->off_dz = take(sizeof(float) * slabs * m);
@@ -223,14 +253,16 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     p->off_dQF = take(sizeof(float) * slab_elems);
     p->off_dKF = take(sizeof(float) * slab_elems);
     p->off_dSbf = take(sizeof(__nv_bfloat16) * slabs * m * kD);
-    p->off_KF3 = take(p->use_tc ? 3 * sizeof(__nv_bfloat16) * slab_elems : 0);
-    p->off_QF3 = take(p->use_tc ? 3 * sizeof(__nv_bfloat16) * slab_elems : 0);
+    if (p->use_tc) {
+      p->off_KF3 = take(3 * sizeof(__nv_bfloat16) * slab_elems);
+      p->off_QF3 = take(3 * sizeof(__nv_bfloat16) * slab_elems);
+    }
     p->off_Slo = take(p->use_tc ? sizeof(__nv_bfloat16) * slabs * m * kD : 0);
     p->off_Dtot = take(grouped ? sizeof(float) * 2 * slabs * n : 0);
     p->off_shardtot = take(256);
   } else {
     p->off_Dtot = p->off_shardtot = 0;
-    p->off_dS = p->off_dz = p->off_sumdD = p->off_bands = p->off_dqbar = p->off_dQF = p->off_dKF = p->off_dSbf = p->off_KF3 = p->off_QF3 = p->off_Slo = 0;
+    p->off_dS = p->off_dz = p->off_sumdD = p->off_bands = p->off_dqbar = p->off_dQF = p->off_dKF = p->off_dSbf = p->off_Slo = 0;
   }
   p->total = off;
   return WERSA_OK;
@@ -264,6 +296,7 @@ Ws resolve(const Plan& p, void* workspace) {
   w.dSbf = reinterpret_cast<__nv_bfloat16*>(b + p.off_dSbf);
   w.KF3 = reinterpret_cast<__nv_bfloat16*>(b + p.off_KF3);
   w.QF3 = reinterpret_cast<__nv_bfloat16*>(b + p.off_QF3);
+  w.V3 = reinterpret_cast<__nv_bfloat16*>(b + p.off_V3);
   w.Slo = reinterpret_cast<__nv_bfloat16*>(b + p.off_Slo);
   w.Og = b + p.off_Og;
   w.den = reinterpret_cast<float*>(b + p.off_den);
@@ -442,6 +475,13 @@ wersa_status wersa_forward(wersa_ctx* ctx, const void* Q, const void* K, const v
       WERSA_STEP(0, "reduce_partials",
                  launch_reduce_partials(p, w.spart, w.zpart, p.tchunks, w.S, w.z, w.Sbf, w.Simg, st, &launches));
     WERSA_STEP(0, "tc_qside", launch_tc_qside(p, w, Q, beta, O, nullptr, st, &launches));
+  } else if (p.use_x) {
+    WERSA_STEP(0, "f32_planes", launch_f32_planes(p, w, static_cast<const float*>(Q), static_cast<const float*>(K),
+                                                  static_cast<const float*>(V), p.with_backward, st, &launches));
+    WERSA_STEP(0, "tcx_kside", launch_tcx_kside(p, w, W, st, &launches));
+    WERSA_STEP(0, "reduce_partials",
+               launch_reduce_partials(p, w.spart, w.zpart, p.xchunks, w.S, w.z, nullptr, nullptr, st, &launches));
+    WERSA_STEP(0, "tcx_qside", launch_tcx_qside(p, w, W, beta, O, st, &launches));
   } else {
     WERSA_STEP(0, "haar_filter_qk", launch_haar_filter(p, Q, kind, w.f, w.QF, K, w.KF, 0, d, true, st, &launches));
     WERSA_STEP(0, "simt_kside", launch_simt_kside(p, w, V, W, st, &launches));

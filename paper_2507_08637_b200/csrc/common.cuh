@@ -38,11 +38,13 @@ struct Plan {
   // tcgen05 key-side split
   int tchunks, tchunk_blocks;  // chunks per slab, 256-token blocks per chunk
   int tqchunks, tqchunk_blocks;  // the same for the query side of the forward
+  bool use_x;         // fp32 forward on the tensor cores (tc_f32.cu)
+  int xchunks, xchunk_tiles;   // its chunks per slab, 128-token tiles per chunk
   int bctas;          // tcgen05 backward: CTAs that share the list of all 128-token tiles
   // workspace offsets (bytes)
   size_t off_status, off_counters, status_bytes, off_qpart, off_qbar, off_sg, off_f, off_spart, off_zpart, off_S, off_z,
       off_Sbf, off_Wt, off_dS, off_dz, off_sumdD, off_bands, off_dqbar, off_QF, off_KF, off_dQF,
-      off_dKF, off_dSbf, off_KF3, off_QF3, off_Slo, off_Simg, off_Og, off_den, off_Dtot, off_shardtot, total;
+      off_dKF, off_dSbf, off_KF3, off_QF3, off_Slo, off_Simg, off_Og, off_den, off_Dtot, off_shardtot, off_V3, total;
 };
 
 // Fills `p` from `cfg`; returns WERSA_OK, WERSA_ERR_INVALID_ARG or WERSA_ERR_UNSUPPORTED.
@@ -52,7 +54,7 @@ struct Ws {   // resolved workspace pointers
   int* status;
   int* counters;   // arrival counters (slabs + batch + slabs ints), zero between launches
   float *qpart, *qbar, *sg, *f, *spart, *zpart, *S, *z, *dS, *dz, *sumdD, *bands, *dqbar;
-  __nv_bfloat16 *Sbf, *Wt, *dSbf, *KF3, *QF3, *Slo;   // Slo = bf16(S' - bf16(S')), built by the backward
+  __nv_bfloat16 *Sbf, *Wt, *dSbf, *KF3, *QF3, *V3, *Slo;   // Slo = bf16(S' - bf16(S')), built by the backward
   uint8_t* Simg;   // [S' | z' | 0]^T operand images of the query-side kernel, one per slab (see simg_offset)
   float *QF, *KF, *dQF, *dKF;
   // features > 256: per-group outputs and denominators
@@ -107,6 +109,9 @@ cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const 
 // with X2 also XF3_2 from X2 in the same launch, with split_S also w.Slo = bf16(w.S - w.Sbf).
 cudaError_t launch_haar_filter_split3(const Plan& p, const Ws& w, const void* X, __nv_bfloat16* XF3, const void* X2,
                                       __nv_bfloat16* XF3_2, bool split_S, cudaStream_t st, int* launches);
+// fp32 tensors: w.QF3 = T_f(Q), w.KF3 = T_f(K) and w.V3 = V as planes; with keep also w.QF and w.KF.
+cudaError_t launch_f32_planes(const Plan& p, const Ws& w, const float* Q, const float* K, const float* V, bool keep,
+                              cudaStream_t st, int* launches);
 // dX = T_f(G) + vec[slab] * vec_scale on every row (G fp32, vec = slabs x 64 floats).
 cudaError_t launch_haar_filter_addvec(const Plan& p, const float* G, const float* f, const float* vec,
                                       float vec_scale, void* dX, int out_kind, int d, cudaStream_t st, int* launches);
@@ -134,6 +139,11 @@ cudaError_t launch_simt_bwd_qside(const Plan& p, const Ws& w, const void* W, con
                                   const void* dO, cudaStream_t st, int* launches);
 cudaError_t launch_simt_bwd_kside(const Plan& p, const Ws& w, const void* V, const void* W, void* dV,
                                   cudaStream_t st, int* launches);
+
+// ---- tc_f32.cu -----------------------------------------------------------------------------
+// fp32 forward on the tensor cores: partial S', z' (p.xchunks per slab) from w.KF3 and w.V3; O from w.QF3, w.S and w.z.
+cudaError_t launch_tcx_kside(const Plan& p, const Ws& w, const void* W, cudaStream_t st, int* launches);
+cudaError_t launch_tcx_qside(const Plan& p, const Ws& w, const void* W, const float* beta, void* O, cudaStream_t st, int* launches);
 
 // ---- tc_fwd.cu -----------------------------------------------------------------------------
 // Both read the raw bf16 tensors and apply the Haar filter (coefficients from w.f) on chip.

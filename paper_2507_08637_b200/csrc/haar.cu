@@ -204,6 +204,86 @@ __global__ void __launch_bounds__(256, 4) k_haar_filter(const Tin* __restrict__ 
   }
 }
 
+// What the fp32 kernels of the tensor cores read: T_f(Q), T_f(K) and V as three bf16 planes hi, mid, lo each (their sum
+// carries the fp32 value; see k_haar_filter_split3), and for a backward that will want them T_f(Q) and T_f(K) themselves.
+// Tiles and arithmetic are those of k_haar_filter; all three tensors are arguments and fetched ahead of the wait.  Bound by
+// memory: 640 bytes a row of 64 columns and tensor, 2 x 8 x 4096 19 us, 6.6 TB/s.
+// grid (col_blocks<32>, slabs, 3), block 256.
+template <bool kFull, bool kKeep>
+__global__ void __launch_bounds__(256, 3) k_f32_planes(const float* __restrict__ Q, const float* __restrict__ K,
+                                                       const float* __restrict__ V, const float* __restrict__ f,
+                                                       __nv_bfloat16* __restrict__ Q3, __nv_bfloat16* __restrict__ K3,
+                                                       __nv_bfloat16* __restrict__ V3, float* __restrict__ QF,
+                                                       float* __restrict__ KF, size_t plane, int n, int d_arg, int L) {
+  const int d = kFull ? kD : d_arg;
+  __shared__ __align__(16) float ex[8][kHalfD];   // 32-row sums of the warps
+  const int slab = blockIdx.y, warp = threadIdx.x >> 5, cg = threadIdx.x & 7, rg = threadIdx.x >> 3;
+  const ColMap<32> at(blockIdx.x, cg * 4, d);
+  const int row0 = at.row0 + rg * 8;
+  const int rows = at.on ? n - row0 : 0;   // rows of this thread inside the sequence
+  const size_t first = ((size_t)slab * n + row0) * d + at.col;
+  const bool filtered = blockIdx.z < 2;
+  const float* __restrict__ X = blockIdx.z == 0 ? Q : blockIdx.z == 1 ? K : V;
+  float x[8][4];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    if (j < rows) {
+      load4<true>(X + first + (size_t)j * d, x[j]);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) x[j][c] = 0.f;
+    }
+  }
+  wait_for_stream_predecessor();   // (launched as a programmatic dependent, see launch_after: f is the gate kernel's)
+  let_stream_successor_start();
+  if (filtered) {
+    const LevelCoef k = level_coef<true>(f + (size_t)slab * (L + 1), L);
+    float hi[4], s5[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float s3 = ((x[0][c] + x[1][c]) + (x[2][c] + x[3][c])) + ((x[4][c] + x[5][c]) + (x[6][c] + x[7][c]));
+      const float s4 = sum16(s3);
+      s5[c] = sum32(s4);
+      hi[c] = fmaf(k.k[3], s3, fmaf(k.k[4], s4, k.k[5] * s5[c]));
+    }
+    if (L > 5) {
+      if ((threadIdx.x & 24) == 0) *reinterpret_cast<float4*>(&ex[warp][cg * 4]) = make_float4(s5[0], s5[1], s5[2], s5[3]);
+      __syncthreads();
+      add_coarse4(ex, k, warp, cg * 4, hi);
+    }
+#pragma unroll
+    for (int j = 0; j < 8; j += 4) {   // four rows (one level-2 block) at a time
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float a0 = x[j][c] + x[j + 1][c], a1 = x[j + 2][c] + x[j + 3][c];
+        const float c2 = fmaf(k.k[2], a0 + a1, hi[c]);
+        const float c10 = fmaf(k.k[1], a0, c2), c11 = fmaf(k.k[1], a1, c2);
+        x[j][c] = fmaf(k.f0, x[j][c], c10);
+        x[j + 1][c] = fmaf(k.f0, x[j + 1][c], c10);
+        x[j + 2][c] = fmaf(k.f0, x[j + 2][c], c11);
+        x[j + 3][c] = fmaf(k.f0, x[j + 3][c], c11);
+      }
+    }
+  }
+  __nv_bfloat16* dst = (blockIdx.z == 0 ? Q3 : blockIdx.z == 1 ? K3 : V3) + first;
+  float* keep = blockIdx.z == 0 ? QF : KF;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    if (j >= rows) break;
+    if (kKeep && filtered) store4(keep + first + (size_t)j * d, x[j]);
+#pragma unroll
+    for (int pl = 0; pl < 3; ++pl) {   // what a plane leaves is the next one's input
+      const __nv_bfloat162 a = __floats2bfloat162_rn(x[j][0], x[j][1]), b = __floats2bfloat162_rn(x[j][2], x[j][3]);
+      const uint2 w = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+      *reinterpret_cast<uint2*>(dst + (size_t)pl * plane + (size_t)j * d) = w;
+      x[j][0] -= __uint_as_float(w.x << 16);
+      x[j][1] -= __uint_as_float(w.x & 0xFFFF0000u);
+      x[j][2] -= __uint_as_float(w.y << 16);
+      x[j][3] -= __uint_as_float(w.y & 0xFFFF0000u);
+    }
+  }
+}
+
 // The same pass for bf16 input: a thread keeps its 8 rows x 8 columns as the 32 packed words it loaded
 // (16-byte loads; unpacked where they are used, twice), so that three CTAs of 256 rows x 64 columns share an
 // SM with 16-byte accesses in flight.  grid (htiles, slabs), block 256.
@@ -594,6 +674,20 @@ cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const 
       err = launch_after(k_haar_filter<kFull, float, float, false>, grid, dim3(256), 0, st, (const float*)X, f, (float*)XF,
                          (const float*)X2, (float*)XF2, n, d, L, nullptr, 0.f, inputs_ready);
   })
+  *launches += 1;
+  return err != cudaSuccess ? err : cudaGetLastError();
+}
+
+cudaError_t launch_f32_planes(const Plan& p, const Ws& w, const float* Q, const float* K, const float* V, bool keep,
+                              cudaStream_t st, int* launches) {
+  const int n = p.cfg.seq_len, L = p.cfg.levels, d = p.cfg.head_dim;
+  const dim3 grid(col_blocks<32>(p.htiles, d), p.slabs, 3);
+  const size_t plane = (size_t)p.slabs * n * d;
+  cudaError_t err;
+  auto go = [&](auto kernel) {
+    return launch_after(kernel, grid, dim3(256), 0, st, Q, K, V, (const float*)w.f, w.QF3, w.KF3, w.V3, w.QF, w.KF, plane, n, d, L);
+  };
+  WERSA_FULL({ err = keep ? go(k_f32_planes<kFull, true>) : go(k_f32_planes<kFull, false>); })
   *launches += 1;
   return err != cudaSuccess ? err : cudaGetLastError();
 }

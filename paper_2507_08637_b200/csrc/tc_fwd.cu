@@ -30,6 +30,7 @@
 // group barriers stay balanced) but skips all further work, and the host sees the status word.
 #include "common.cuh"
 #include "tc_common.cuh"
+#include "tc_maps.cuh"
 
 namespace wersa {
 using namespace tc;
@@ -1126,40 +1127,6 @@ k_tc_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
   }
 }
 
-// ---- host side: tensor maps ---------------------------------------------------------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (fn == nullptr) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
-  return fn;
-}
-
-// (slabs x n x 64) bf16 row-major tensor, boxes of `box_rows` rows x 64 columns of one slab, 128-byte
-// swizzle.  Rows past the end of a slab read as zeros and are not written.
-// Rows of `cols` bf16 values (a multiple of 8: row pitches are multiples of 16 bytes); the box is always 64
-// columns wide, so that a narrower tensor arrives zero-filled up to column 63 and is stored clipped.
-cudaError_t make_tile_map(const void* base, int slabs, int n, int box_rows, CUtensorMap* out, int cols = kD) {
-  EncodeTiledFn fn = encode_fn();
-  if (fn == nullptr) return cudaErrorNotSupported;
-  const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)n, (cuuint64_t)slabs};
-  const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)n * cols * 2};
-  const cuuint32_t box[3] = {kD, (cuuint32_t)box_rows, 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  const CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
 }  // namespace
 
 // (the head dimension does not enter: the tensor maps zero-fill narrower heads up to 64 columns, and feature
@@ -1198,10 +1165,10 @@ cudaError_t launch_tc_kside(const Plan& p, const Ws& w, const void* K, const voi
                             int* launches) {
   CUtensorMap map_k, map_v;
   cudaError_t err;
-  if ((err = make_tile_map(K, p.slabs, p.cfg.seq_len, kTile, &map_k, p.cfg.head_dim)) != cudaSuccess) return err;
-  if ((err = make_tile_map(V, p.slabs, p.cfg.seq_len, kTile, &map_v, p.cfg.head_dim)) != cudaSuccess) return err;
+  if ((err = make_tile_map(K, p.slabs, p.cfg.seq_len, &map_k, p.cfg.head_dim)) != cudaSuccess) return err;
+  if ((err = make_tile_map(V, p.slabs, p.cfg.seq_len, &map_v, p.cfg.head_dim)) != cudaSuccess) return err;
   CUtensorMap map_w;   // W^T (m x 64) as one slab of m rows
-  if ((err = make_tile_map(w.Wt, 1, p.cfg.features * p.groups, kTile, &map_w)) != cudaSuccess) return err;
+  if ((err = make_tile_map(w.Wt, 1, p.cfg.features * p.groups, &map_w)) != cudaSuccess) return err;
   const int items = p.tchunks * p.slabs;   // (slab, chunk) pairs; one CTA per SM walks them
   dim3 grid(items < p.sms ? items : p.sms);
   // With one chunk per slab the "partial" is the result: the kernel writes S', z' and the bf16 image
@@ -1233,13 +1200,13 @@ cudaError_t launch_tc_qside(const Plan& p, const Ws& w, const void* Q, const flo
                             cudaStream_t st, int* launches) {
   CUtensorMap map_q, map_o;
   cudaError_t err;
-  if ((err = make_tile_map(Q, p.slabs, p.cfg.seq_len, kTile, &map_q, p.cfg.head_dim)) != cudaSuccess) return err;
-  if ((err = make_tile_map(O, p.slabs * p.groups, p.cfg.seq_len, kTile, &map_o, p.cfg.head_dim)) != cudaSuccess)
+  if ((err = make_tile_map(Q, p.slabs, p.cfg.seq_len, &map_q, p.cfg.head_dim)) != cudaSuccess) return err;
+  if ((err = make_tile_map(O, p.slabs * p.groups, p.cfg.seq_len, &map_o, p.cfg.head_dim)) != cudaSuccess)
     return err;
   // (the query side may start while the reduction that produces S', z' is still running; it waits for
   // that kernel where it first needs its results)
   CUtensorMap map_w;
-  if ((err = make_tile_map(w.Wt, 1, p.cfg.features * p.groups, kTile, &map_w)) != cudaSuccess) return err;
+  if ((err = make_tile_map(w.Wt, 1, p.cfg.features * p.groups, &map_w)) != cudaSuccess) return err;
   const int items = p.tqchunks * p.slabs;
   dim3 grid(items < p.sms ? items : p.sms);
   const bool multi = p.groups == 1 && items > (int)grid.x;
