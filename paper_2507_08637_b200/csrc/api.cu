@@ -126,9 +126,14 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   // fp32 forward on the tensor cores, from kXUnits tiles x groups of 128 features on: 2 x 4 x 1024, m = 128 (64 units) 49 -> 26
   // us, in d = 32 37 -> 23; 1 x 4 x 1024, m = 256 (64) 40 -> 26.  One CTA per SM and group, in chunks that minimise
   // waves x (tiles + 3), 3 tiles being about what a CTA spends before its first and after its last one.
-  p->use_x = false;
-  p->xchunks = 1;
-  p->xchunk_tiles = 1;
+  // The backward from one tile per SM on: 2 x 3 x 4097, m = 128 150 -> 72 us, 5 x 4223, m = 256 203 -> 115, 8 x 4 x 1024,
+  // d = 32 92 -> 65, narrower heads about as fast as before (40 x 4 x 130, d = 24 106 -> 107).  It is ahead below that line
+  // too (64 tiles, m = 128 66 -> 48; 32 tiles 46 -> 46), but a feature within rounding of zero, which planes may decide
+  // otherwise than 32-bit sums, shows in a whole block of the coarsest level: in slabs of few tokens that is much of dQ.
+  p->use_x = p->use_xb = false;
+  p->xchunks = p->xbchunks = 1;
+  p->xchunk_tiles = p->xbchunk_tiles = 1;
+  p->xprep = 0;
   if (!p->bf16 && !(c.flags & WERSA_FLAG_SIMT_ONLY) && m >= 128) {
     const int tiles = ceil_div(n, 128), groups = m / 128;
     p->use_x = (long long)p->slabs * tiles * groups >= kXUnits;
@@ -142,6 +147,17 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     }
     p->xchunk_tiles = ceil_div(tiles, p->xchunks);
     p->xchunks = ceil_div(tiles, p->xchunk_tiles);
+    p->use_xb = p->use_x && p->with_backward && !p->grad_bf16 && (long long)p->slabs * tiles >= p->sms;
+    for (int ch = 1; ch <= tiles && ch <= 64; ++ch) {
+      const long long cost = (long long)ceil_div(p->slabs * ch, p->sms) * (ceil_div(tiles, ch) + 1);
+      if (ch == 1 || cost < best) {
+        best = cost;
+        p->xbchunks = ch;
+      }
+    }
+    p->xbchunk_tiles = ceil_div(tiles, p->xbchunks);
+    p->xbchunks = ceil_div(tiles, p->xbchunk_tiles);
+    p->xprep = (int)std::min<long long>(((long long)p->slabs * n * 8 + 255) / 256, 8LL * p->sms);
   }
 
   p->tchunks = 0;
@@ -234,7 +250,8 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   take(p->dpad ? 256 : 0);
   p->off_Og = take(grouped ? io_bytes * slab_elems * p->groups : 0);
   p->off_den = take(grouped ? sizeof(float) * slabs * n * p->groups : 0);
-  const bool need_xf = !p->use_tc && (!p->use_x || p->with_backward);   // the tensor-core kernels filter on chip (forward) or read bf16 planes (backward)
+  p->off_dO3 = p->off_xO = p->off_xden = p->off_xinv = p->off_xc = p->off_xshare = 0;
+  const bool need_xf = !p->use_tc && (!p->use_x || (p->with_backward && !p->use_xb));   // the tensor-core kernels filter on chip (forward) or read bf16 planes (backward)
   p->off_QF = take(need_xf ? sizeof(float) * slab_elems : 0);
   p->off_KF = take(need_xf ? sizeof(float) * slab_elems : 0);
   if (p->use_x) {   // (the query side's shares follow on from KF3 into V3: see launch_tcx_qside)
@@ -247,7 +264,16 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   if (p->with_backward) {
     p->off_dS = take(sizeof(float) * slabs * m * kD);
     p->off_dz = take(sizeof(float) * slabs * m);
-    p->off_sumdD = take(sizeof(float) * (p->use_tc ? (size_t)p->bctas : slabs * p->schunks));
+    p->off_sumdD = take(sizeof(float) * (p->use_tc ? (size_t)p->bctas : p->use_xb ? (size_t)p->xprep : slabs * p->schunks));
+    if (p->use_xb) {
+      const size_t groups = c.features / 128, padded = (size_t)ceil_div(c.seq_len, 128) * 128;
+      p->off_dO3 = take(3 * sizeof(__nv_bfloat16) * slab_elems);
+      p->off_xO = take(sizeof(float) * slab_elems);
+      p->off_xden = take(sizeof(float) * groups * slabs * c.seq_len);
+      p->off_xinv = take(sizeof(float) * slabs * padded);
+      p->off_xc = take(sizeof(float) * slabs * padded);
+      p->off_xshare = take(groups > 1 ? sizeof(float) * groups * slab_elems : 0);
+    }
     p->off_bands = take(sizeof(float) * 2 * slabs * 2 * p->htiles * kBandVals);   // Q and K; two column halves per tile
     p->off_dqbar = take(sizeof(float) * slabs * (kD + kBandVals));
     p->off_dQF = take(sizeof(float) * slab_elems);
@@ -297,6 +323,12 @@ Ws resolve(const Plan& p, void* workspace) {
   w.KF3 = reinterpret_cast<__nv_bfloat16*>(b + p.off_KF3);
   w.QF3 = reinterpret_cast<__nv_bfloat16*>(b + p.off_QF3);
   w.V3 = reinterpret_cast<__nv_bfloat16*>(b + p.off_V3);
+  w.dO3 = reinterpret_cast<__nv_bfloat16*>(b + p.off_dO3);
+  w.xO = reinterpret_cast<float*>(b + p.off_xO);
+  w.xden = reinterpret_cast<float*>(b + p.off_xden);
+  w.xinv = reinterpret_cast<float*>(b + p.off_xinv);
+  w.xc = reinterpret_cast<float*>(b + p.off_xc);
+  w.xshare = reinterpret_cast<float*>(b + p.off_xshare);
   w.Slo = reinterpret_cast<__nv_bfloat16*>(b + p.off_Slo);
   w.Og = b + p.off_Og;
   w.den = reinterpret_cast<float*>(b + p.off_den);
@@ -477,7 +509,7 @@ wersa_status wersa_forward(wersa_ctx* ctx, const void* Q, const void* K, const v
     WERSA_STEP(0, "tc_qside", launch_tc_qside(p, w, Q, beta, O, nullptr, st, &launches));
   } else if (p.use_x) {
     WERSA_STEP(0, "f32_planes", launch_f32_planes(p, w, static_cast<const float*>(Q), static_cast<const float*>(K),
-                                                  static_cast<const float*>(V), p.with_backward, st, &launches));
+                                                  static_cast<const float*>(V), p.with_backward && !p.use_xb, st, &launches));
     WERSA_STEP(0, "tcx_kside", launch_tcx_kside(p, w, W, st, &launches));
     WERSA_STEP(0, "reduce_partials",
                launch_reduce_partials(p, w.spart, w.zpart, p.xchunks, w.S, w.z, nullptr, nullptr, st, &launches));
@@ -712,17 +744,23 @@ wersa_status wersa_backward(wersa_ctx* ctx, const void* Q, const void* K, const 
     // the tensor-core forward keeps Q_F, K_F on chip: rebuild them, as three bf16 planes each
     WERSA_STEP(1, "haar_filter_qk", launch_haar_filter_split3(p, w, Q, w.QF3, K, w.KF3, true, st, &launches));
     WERSA_STEP(1, "tc_bwd_qside", launch_tc_bwd_qside(p, w, w.QF3, beta, dO, nullptr, nullptr, false, st, &launches));
+  } else if (p.use_xb) {
+    WERSA_STEP(1, "tcx_bwd_prep", launch_tcx_bwd_prep(p, w, dO, beta, st, &launches));
+    WERSA_STEP(1, "tcx_bwd_qside", launch_tcx_bwd_qside(p, w, W, st, &launches));
   } else {
     WERSA_STEP(1, "simt_bwd_qside", launch_simt_bwd_qside(p, w, W, beta, dO, st, &launches));
   }
   if (p.groups == 1)
     WERSA_STEP(1, "reduce_partials",
                p.use_tc ? launch_reduce_segments(p, w, st, &launches)
-                        : launch_reduce_partials(p, w.spart, w.zpart, p.schunks, w.dS, w.dz, nullptr, nullptr, st, &launches));
+                        : launch_reduce_partials(p, w.spart, w.zpart, p.use_xb ? p.xchunks : p.schunks, w.dS, w.dz, nullptr,
+                                                 nullptr, st, &launches));
   if (p.groups > 1) {
     // (done group by group above)
   } else if (p.use_tc) {
     WERSA_STEP(1, "tc_bwd_kside", launch_tc_bwd_kside(p, w, w.KF3, V, dV, false, st, &launches));
+  } else if (p.use_xb) {
+    WERSA_STEP(1, "tcx_bwd_kside", launch_tcx_bwd_kside(p, w, W, dV, st, &launches));
   } else {
     WERSA_STEP(1, "simt_bwd_kside", launch_simt_bwd_kside(p, w, V, W, dV, st, &launches));
   }
@@ -733,8 +771,9 @@ wersa_status wersa_backward(wersa_ctx* ctx, const void* Q, const void* K, const 
   WERSA_STEP(1, "haar_backward_kq",
              launch_haar_backward(p, w, 1, K, w.dKF, dK, Q, w.dQF, pooled_term ? nullptr : dQ, kind, gkind, d, st, &launches));
   WERSA_STEP(1, "gate_backward",
-             launch_gate_backward(p, w, haar_band_blocks(p, d), beta, gate_w, omega, p.use_tc ? p.bctas : p.slabs * p.schunks, dbeta, dgate_w, dgate_b, domega, st,
-                                  &launches));
+             launch_gate_backward(p, w, haar_band_blocks(p, d), beta, gate_w, omega,
+                                  p.use_tc ? p.bctas : p.use_xb ? p.xprep : p.slabs * p.schunks, dbeta, dgate_w, dgate_b, domega,
+                                  st, &launches));
   if (pooled_term)
     WERSA_STEP(1, "haar_filter_dq",
                launch_haar_filter_addvec(p, w.dQF, w.f, w.dqbar, 1.f / (float)p.cfg.seq_len, dQ, gkind, d, st, &launches));

@@ -40,11 +40,13 @@ struct Plan {
   int tqchunks, tqchunk_blocks;  // the same for the query side of the forward
   bool use_x;         // fp32 forward on the tensor cores (tc_f32.cu)
   int xchunks, xchunk_tiles;   // its chunks per slab, 128-token tiles per chunk
+  bool use_xb;        // fp32 backward on them too: chunks and tiles of its gradient kernels, CTAs of its first pass
+  int xbchunks, xbchunk_tiles, xprep;
   int bctas;          // tcgen05 backward: CTAs that share the list of all 128-token tiles
   // workspace offsets (bytes)
   size_t off_status, off_counters, status_bytes, off_qpart, off_qbar, off_sg, off_f, off_spart, off_zpart, off_S, off_z,
       off_Sbf, off_Wt, off_dS, off_dz, off_sumdD, off_bands, off_dqbar, off_QF, off_KF, off_dQF,
-      off_dKF, off_dSbf, off_KF3, off_QF3, off_Slo, off_Simg, off_Og, off_den, off_Dtot, off_shardtot, off_V3, total;
+      off_dKF, off_dSbf, off_KF3, off_QF3, off_Slo, off_Simg, off_Og, off_den, off_Dtot, off_shardtot, off_V3, off_dO3, off_xO, off_xden, off_xinv, off_xc, off_xshare, total;
 };
 
 // Fills `p` from `cfg`; returns WERSA_OK, WERSA_ERR_INVALID_ARG or WERSA_ERR_UNSUPPORTED.
@@ -54,7 +56,8 @@ struct Ws {   // resolved workspace pointers
   int* status;
   int* counters;   // arrival counters (slabs + batch + slabs ints), zero between launches
   float *qpart, *qbar, *sg, *f, *spart, *zpart, *S, *z, *dS, *dz, *sumdD, *bands, *dqbar;
-  __nv_bfloat16 *Sbf, *Wt, *dSbf, *KF3, *QF3, *V3, *Slo;   // Slo = bf16(S' - bf16(S')), built by the backward
+  float *xO, *xden, *xinv, *xc, *xshare;   // fp32 on the tensor cores: O and D'_g for the backward, 1 / D and -dO.O per token, shares of N'
+  __nv_bfloat16 *Sbf, *Wt, *dSbf, *KF3, *QF3, *V3, *dO3, *Slo;   // Slo = bf16(S' - bf16(S')), built by the backward
   uint8_t* Simg;   // [S' | z' | 0]^T operand images of the query-side kernel, one per slab (see simg_offset)
   float *QF, *KF, *dQF, *dKF;
   // features > 256: per-group outputs and denominators
@@ -141,9 +144,15 @@ cudaError_t launch_simt_bwd_kside(const Plan& p, const Ws& w, const void* V, con
                                   cudaStream_t st, int* launches);
 
 // ---- tc_f32.cu -----------------------------------------------------------------------------
-// fp32 forward on the tensor cores: partial S', z' (p.xchunks per slab) from w.KF3 and w.V3; O from w.QF3, w.S and w.z.
+// fp32 on the tensor cores.  Forward: partial S', z' (p.xchunks per slab) from w.KF3 and w.V3; O from w.QF3, w.S and w.z,
+// with a backward also w.xO and w.xden.  Backward: dO as planes and what the division leaves per token; dQ_F, partial dS',
+// dz'; dK_F and dV.
 cudaError_t launch_tcx_kside(const Plan& p, const Ws& w, const void* W, cudaStream_t st, int* launches);
 cudaError_t launch_tcx_qside(const Plan& p, const Ws& w, const void* W, const float* beta, void* O, cudaStream_t st, int* launches);
+
+cudaError_t launch_tcx_bwd_prep(const Plan& p, const Ws& w, const void* dO, const float* beta, cudaStream_t st, int* launches);
+cudaError_t launch_tcx_bwd_qside(const Plan& p, const Ws& w, const void* W, cudaStream_t st, int* launches);
+cudaError_t launch_tcx_bwd_kside(const Plan& p, const Ws& w, const void* W, void* dV, cudaStream_t st, int* launches);
 
 // ---- tc_fwd.cu -----------------------------------------------------------------------------
 // Both read the raw bf16 tensors and apply the Haar filter (coefficients from w.f) on chip.

@@ -14,11 +14,14 @@
 // k_tcx_kside      : S' = ReLU(K_F W)^T V, z' per sequence chunk and group of 128 features
 // k_tcx_qside      : O = ReLU(Q_F W) S' / (ReLU(Q_F W) z' + eps'); with two groups each leaves N'_g and D'_g
 // k_tcx_combine    : O = sum_g N'_g / (sum_g D'_g + eps')
+// k_tcx_bwd_prep   : dO as planes; 1 / D, -dO.O (per token) and sum dD
+// k_tcx_kside again: dS' = ReLU(Q_F W)^T (dO / D), dz' = sum of ReLU(Q_F W) dD
+// k_tcx_bwd        : dQ_F, or dK_F and dV; a launch per group of 128 features
 //
-// Both tensor-core kernels: 512 threads, 128 registers each.  Warp 0 copies, warp 1 issues the projections (MMA1), warp 2
+// The tensor-core kernels: 512 threads, 128 registers each.  Warp 0 copies, warp 1 issues the projections (MMA1), warp 2
 // the contractions (MMA2), warps 4-11 two groups that take the tiles in turn: accumulator -> ReLU -> planes back into
 // TMEM; warps 12-15 drain.  TMEM: two buffers of 192 columns (128 of D1, replaced in place by the hi and mid planes, 64 of
-// the lo plane), two accumulators of 64.  Every wait is bounded, as in tc_fwd.cu.
+// the lo plane), two accumulators of 64 (k_tcx_bwd has its own).  Every wait is bounded, as in tc_fwd.cu.
 // 2 x 8 x 4096, d = 64, m = 256: planes 19 us, key side 28, query side 29, combining 7; the forward 235 -> 95 us.  A tile and
 // group takes some 5 k cycles of tensor pipe (MMA1 reads both operands of its 24 instructions from shared memory, 105-115
 // cycles each instead of 64; the 48 of MMA2 45 each), 60 % of the time.
@@ -76,6 +79,10 @@ struct QxSmem {
 };
 static_assert(QxSmem::total <= 232448 && KxSmem::total <= 232448 && sizeof(XBars) <= 256, "shared memory of an SM");
 
+// Tokens of a slab in the per-token arrays of the backward: whole tiles, since they are read past n and in pairs (a slab has
+// to begin on an 8-byte boundary where n is odd).
+__host__ __device__ __forceinline__ int padded_tokens(int n) { return (n + kTile - 1) / kTile * kTile; }
+
 // Two floats -> one packed pair per plane.
 __device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
   hi = pack_bf16x2(a, b);
@@ -126,8 +133,10 @@ __device__ __forceinline__ void load_s_planes(const float* S, const float* zg, s
 // One D1 buffer: 128 fp32 columns -> ReLU -> planes.  32 columns hold 16 hi and 16 mid pairs of their features, the lo pairs
 // go to the columns behind them.  Returns the sum of the row's values, kWeighted: each times w[column], in chains of
 // eight, as few additions in a row as the FFMA kernels have (two chains of 64: D' 8e-8 off, more than all else together).
-template <bool kWeighted>
-__device__ __forceinline__ float relu_planes(uint32_t taddr, const float* w) {
+// kScaled: the values are multiplied by s[column] first, and the sum is of those times w[column]; both arrays in global
+// memory, on an 8-byte boundary, and may hold anything where the value is zero.
+template <bool kWeighted, bool kScaled = false>
+__device__ __forceinline__ float relu_planes(uint32_t taddr, const float* w, const float* s = nullptr) {
   uint32_t r[32];
   float total = 0.f;
 #pragma unroll 1
@@ -141,7 +150,14 @@ __device__ __forceinline__ float relu_planes(uint32_t taddr, const float* w) {
     for (int j = 0; j < 16; ++j) {
       float a = fmaxf(put_back(__uint_as_float(r[2 * j])), 0.f), b = fmaxf(put_back(__uint_as_float(r[2 * j + 1])), 0.f);
       const int k = 2 * (j & 1);
-      if constexpr (kWeighted) {
+      if constexpr (kScaled) {
+        const float2 z = __ldg(reinterpret_cast<const float2*>(w + 32 * c + 2 * j));
+        const float2 f = __ldg(reinterpret_cast<const float2*>(s + 32 * c + 2 * j));
+        a = a > 0.f ? a * f.x : 0.f;
+        b = b > 0.f ? b * f.y : 0.f;
+        e[k] += a > 0.f ? a * z.x : 0.f;
+        e[k + 1] += b > 0.f ? b * z.y : 0.f;
+      } else if constexpr (kWeighted) {
         const float2 z = *reinterpret_cast<const float2*>(w + 32 * c + 2 * j);
         e[k] = fmaf(a, z.x, e[k]);
         e[k + 1] = fmaf(b, z.y, e[k + 1]);
@@ -260,9 +276,13 @@ __device__ __forceinline__ bool drain_tile(Bars* bars, uint32_t taddr, int t, fl
 }
 
 // ---- key side.  grid (chunks, slabs, feature groups) ---------------------------------------------
+// kScaled: the query side of the backward, with Q_F and dO in the place of K_F and V.  Feature values are divided by their
+// token's D (scale, slabs of padded_tokens(n)), the sums weighted by c = -dO.O on top: dS' and dz'.
+template <bool kScaled>
 __global__ void __launch_bounds__(kXThreads, 1)
 k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const float* __restrict__ W,
-            float* __restrict__ spart, float* __restrict__ zpart, int n, int d, int m, int chunk_tiles, int* __restrict__ status) {
+            float* __restrict__ spart, float* __restrict__ zpart, int n, int d, int m, int chunk_tiles, int* __restrict__ status,
+            const float* __restrict__ scale, const float* __restrict__ weight) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
   using SL = KxSmem;
@@ -330,7 +350,12 @@ k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ C
       ok = __all_sync(0xffffffffu, mbar_wait(&bars->d1_full[g], (t >> 1) & 1, abort_flag, status, kErrXElem));
       if (!ok) break;
       tc_fence_after_sync();
-      z += relu_planes<false>(taddr, nullptr);
+      if constexpr (kScaled) {
+        const size_t tok = (size_t)slab * padded_tokens(n) + (size_t)(t0 + t) * kTile;
+        z += relu_planes<true, true>(taddr, weight + tok, scale + tok);
+      } else {
+        z += relu_planes<false>(taddr, nullptr);
+      }
       tc_fence_before_sync();
       warp_arrive(&bars->phi_ready[g]);
     }
@@ -370,11 +395,13 @@ k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ C
 }
 
 // ---- query side.  grid (chunks, slabs, feature groups) -------------------------------------------
-// One group: O, divided.  Several: N'_g into map_o (group-major slabs) and D'_g into den_out[(group * slabs + slab) * n + token].
+// One group: O, divided, and with keep (for a backward) once more into map_keep.  Several: N'_g into map_o (group-major
+// slabs).  den_out, where given: D'_g at [(group * slabs + slab) * n + token].
 __global__ void __launch_bounds__(kXThreads, 1)
 k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o, const float* __restrict__ W,
             const float* __restrict__ S, const float* __restrict__ zg, const float* __restrict__ beta, float eps, float bw_floor,
-            float* __restrict__ den_out, int n, int d, int m, int chunk_tiles, int* __restrict__ status) {
+            float* __restrict__ den_out, const __grid_constant__ CUtensorMap map_keep, int keep, int n, int d, int m, int chunk_tiles,
+            int* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
   using SL = QxSmem;
@@ -474,6 +501,10 @@ k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
       if (et == 0 && ok) {   // rows past n and columns past d are clipped
         tma_store_3d(&map_o, out, 0, row0, out_slab);
         if (d > 32) tma_store_3d(&map_o, out + kTileBytes, 32, row0, out_slab);
+        if (keep) {
+          tma_store_3d(&map_keep, out, 0, row0, out_slab);
+          if (d > 32) tma_store_3d(&map_keep, out + kTileBytes, 32, row0, out_slab);
+        }
         bulk_commit_group();
       }
     }
@@ -487,10 +518,10 @@ k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   }
 }
 
-// O = (N'_0 + N'_1) / (D'_0 + D'_1 + eps'), one thread per four columns.
+// O = (N'_0 + N'_1) / (D'_0 + D'_1 + eps'), one thread per four columns; with keep (for a backward) there too.
 __global__ void __launch_bounds__(256) k_tcx_combine(const float* __restrict__ N, const float* __restrict__ den,
                                                      const float* __restrict__ beta, float eps, float bw_floor, int m,
-                                                     float* __restrict__ O, size_t tokens, int d) {
+                                                     float* __restrict__ O, float* __restrict__ keep, size_t tokens, int d) {
   wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   const size_t idx = (size_t)blockIdx.x * 256 + threadIdx.x;
   const int per = d >> 2;
@@ -499,42 +530,381 @@ __global__ void __launch_bounds__(256) k_tcx_combine(const float* __restrict__ N
   const float bw = fmaxf(beta[0], bw_floor);
   const float inv = put_back(1.f / ((load_after_wait(den + tok) + load_after_wait(den + tokens + tok)) + eps * (float)m * bw * bw));
   const float4 a = load4_after_wait(N + idx * 4), b = load4_after_wait(N + tokens * d + idx * 4);
-  *reinterpret_cast<float4*>(O + idx * 4) =
-      make_float4((a.x + b.x) * inv, (a.y + b.y) * inv, (a.z + b.z) * inv, (a.w + b.w) * inv);
+  const float4 o = make_float4((a.x + b.x) * inv, (a.y + b.y) * inv, (a.z + b.z) * inv, (a.w + b.w) * inv);
+  *reinterpret_cast<float4*>(O + idx * 4) = o;
+  if (keep != nullptr) *reinterpret_cast<float4*>(keep + idx * 4) = o;
+}
+
+// ---- backward ------------------------------------------------------------------------------------
+// Per token: planes of dO, 1 / D (D = sum_g D'_g + eps'), c = -dO.O; sum of dD = c / D per CTA.  tpt threads (a power of
+// two >= d / 8) on a token, eight columns each.  Bound by memory (2 x 8 x 4096, d = 64: 59 MB).
+__global__ void __launch_bounds__(256)
+k_tcx_bwd_prep(const float* __restrict__ dO, const float* __restrict__ O, const float* __restrict__ den, int groups,
+               const float* __restrict__ beta, float eps, float bw_floor, int m, int d, int tpt, size_t tokens, int n,
+               __nv_bfloat16* __restrict__ dO3, float* __restrict__ inv, float* __restrict__ c, float* __restrict__ sumdD) {
+  __shared__ float sums[8];
+  wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
+  let_stream_successor_start();
+  const float bw = fmaxf(beta[0], bw_floor);
+  const float epsp = eps * (float)m * bw * bw;
+  const size_t total = tokens * tpt, plane = tokens * d;
+  const size_t warp_first = (size_t)blockIdx.x * 256 + (threadIdx.x & ~31u);
+  float dd = 0.f;
+  for (size_t w0 = warp_first; w0 < total; w0 += (size_t)gridDim.x * 256) {   // whole warps: the shuffles want all lanes
+    const size_t i = w0 + (threadIdx.x & 31), tok = i / tpt;
+    const int c0 = 8 * (int)(i % tpt);
+    float dot = 0.f;
+    if (tok < tokens && c0 < d) {
+      const float4 ga = *reinterpret_cast<const float4*>(dO + tok * d + c0), gb = *reinterpret_cast<const float4*>(dO + tok * d + c0 + 4);
+      const float4 oa = load4_after_wait(O + tok * d + c0), ob = load4_after_wait(O + tok * d + c0 + 4);
+      const float g[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w}, o[8] = {oa.x, oa.y, oa.z, oa.w, ob.x, ob.y, ob.z, ob.w};
+      uint32_t pl[3][4];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) dot = fmaf(g[j], o[j], dot);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) split3(g[2 * j], g[2 * j + 1], pl[0][j], pl[1][j], pl[2][j]);
+#pragma unroll
+      for (int s = 0; s < 3; ++s)
+        *reinterpret_cast<uint4*>(dO3 + s * plane + tok * d + c0) = make_uint4(pl[s][0], pl[s][1], pl[s][2], pl[s][3]);
+    }
+    for (int o = tpt >> 1; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+    if (tok < tokens && c0 == 0) {
+      float D = 0.f;
+      for (int g = 0; g < groups; ++g) D += load_after_wait(den + g * tokens + tok);
+      const float iv = 1.f / (D + epsp);
+      const size_t slab = tok / n, at = slab * padded_tokens(n) + (tok - slab * n);
+      inv[at] = iv;
+      c[at] = -dot;
+      dd = fmaf(-dot, iv, dd);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) dd += __shfl_xor_sync(0xffffffffu, dd, o);
+  if ((threadIdx.x & 31) == 0) sums[threadIdx.x >> 5] = dd;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s += sums[i];
+    sumdD[blockIdx.x] = s;
+  }
+}
+
+struct alignas(8) YBars {
+  uint64_t x_full, x_empty, y_full, y_empty, a_full, a_done, g_full, g_done, a_ready, g_ready, acc_full[2], acc_free[2];
+  uint32_t tmem_base;
+  int abort_flag;
+};
+struct YSmem {
+  static constexpr uint32_t wt = 0;                          // planes of W^T (128 features x 64)
+  static constexpr uint32_t s = wt + 3 * kTileBytes;         // planes of S' or dS'
+  static constexpr uint32_t x = s + 3 * kTileBytes;          // planes of Q_F or K_F
+  static constexpr uint32_t y = x + 3 * kTileBytes;          // planes of dO or V
+  static constexpr uint32_t out = y + 3 * kTileBytes;        // result tile: two boxes of 128 rows x 32 floats
+  static constexpr uint32_t zs = out + 2 * kTileBytes;       // z' or dz' of the group
+  static constexpr uint32_t bars = zs + 512;
+  static constexpr uint32_t total = bars + 256 + 1024;
+};
+static_assert(YSmem::total <= 232448 && sizeof(YBars) <= 256, "shared memory of an SM");
+
+// Chunk `chunk` (32 of 128 values) of a row -> planes, laid out as relu_planes leaves them.
+__device__ __forceinline__ void store_chunk_planes(uint32_t buf, int chunk, const float (&v)[32]) {
+  uint32_t hi[16], mid[16], lo[16];
+#pragma unroll
+  for (int j = 0; j < 16; ++j) split3(v[2 * j], v[2 * j + 1], hi[j], mid[j], lo[j]);
+  tmem_st16(buf + 32 * chunk, hi);
+  tmem_st16(buf + 32 * chunk + 16, mid);
+  tmem_st16(buf + kLoCol + 16 * chunk, lo);
+}
+
+// Per 128-token tile and group: A = X W (which features are on) and G = Y S^T, then
+// queries (X = Q_F, Y = dO, S = S'):  dQ_F = [(G + c z') / D where on] W^T
+// keys    (X = K_F, Y = V, S = dS'):  dK_F = [(G + dz') where on] W^T,  dV = ReLU(A) dS'
+// Both accumulators of a tile wait for the groups of warps 4-7 and 8-11, half the features each; dQ_F, dK_F and dV of a second
+// group of features are added by the copy engine (the launches follow one another).
+// Bound by latency: a tile is one chain copy -> MMA1 -> ReLU -> MMA2 -> drain with nothing of the next tile beside it but its
+// copies.  2 x 4 x 4096, d = 32, m = 128 (two tiles a CTA): queries 15 us, keys some 22; the backward of 8 x 4 x 1024 92 -> 65 us.
+// TMEM: keys: A and its planes 192, G and its planes 192; queries: A 128, G 192; then two accumulators of 64.
+template <bool kKeys>
+__global__ void __launch_bounds__(kXThreads, 1)
+k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y, const float* __restrict__ W,
+          const float* __restrict__ S, const float* __restrict__ zg, const float* __restrict__ tok_inv,
+          const float* __restrict__ tok_c, const __grid_constant__ CUtensorMap map_dx, const __grid_constant__ CUtensorMap map_dv,
+          int add, int n, int d, int m, int f0, int chunk_tiles, int* __restrict__ status) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = align_smem(smem_raw);
+  using SL = YSmem;
+  constexpr uint32_t kG = kKeys ? kBufCols : 128, kAcc = kG + kBufCols;
+  constexpr int kPer = kKeys ? 2 : 1;   // contractions of a tile
+  YBars* bars = reinterpret_cast<YBars*>(smem + SL::bars);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int chunk = blockIdx.x, slab = blockIdx.y, slabs = gridDim.y;
+  const int t0 = chunk * chunk_tiles, nt = min(chunk_tiles, (n + kTile - 1) / kTile - t0);
+  float* zs = reinterpret_cast<float*>(smem + SL::zs);
+  if (threadIdx.x == 0) {
+    mbar_init(&bars->x_full, 1);
+    mbar_init(&bars->x_empty, 1);
+    mbar_init(&bars->y_full, 1);
+    mbar_init(&bars->y_empty, 1);
+    mbar_init(&bars->a_full, 1);
+    mbar_init(&bars->a_done, kKeys ? 1 : 8);   // keys: MMA2 has read the planes; queries: the warps have read A
+    mbar_init(&bars->g_full, 1);
+    mbar_init(&bars->g_done, 1);
+    mbar_init(&bars->a_ready, 8);
+    mbar_init(&bars->g_ready, 8);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&bars->acc_full[i], 1);
+      mbar_init(&bars->acc_free[i], 4);
+    }
+    bars->abort_flag = 0;
+    fence_mbar_init();
+  }
+  if (warp == 1) {
+    tmem_alloc(&bars->tmem_base, 512);
+    tmem_relinquish();
+  }
+  load_w_planes(W, d, m, f0, smem + SL::wt);
+  wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
+  // (behind the key side come kernels that start with reads of what it writes and that lost time placed early)
+  if constexpr (!kKeys) let_stream_successor_start();
+  load_s_planes(S, zg, (size_t)slab * m + f0, smem + SL::s, zs);
+  fence_proxy_async_smem();
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem = bars->tmem_base;
+  volatile int* abort_flag = &bars->abort_flag;
+  const uint32_t hi = smem_desc_hi(1024);
+  if (warp == 0 && lane == 0) {
+    int xs = 0, ys = 0;
+    for (int t = 0; t < nt; ++t) {
+      if (t > 0 && !mbar_wait(&bars->x_empty, (t - 1) & 1, abort_flag, status, kErrXCopy)) break;
+      load_planes(smem + SL::x, &map_x, (t0 + t) * kTile, slab, slabs, &bars->x_full);
+      ++xs;
+      if (t > 0 && !mbar_wait(&bars->y_empty, (t - 1) & 1, abort_flag, status, kErrXCopy)) break;
+      load_planes(smem + SL::y, &map_y, (t0 + t) * kTile, slab, slabs, &bars->y_full);
+      ++ys;
+    }
+    if (*abort_flag != 0) {   // let copies in flight land before the CTA's shared memory goes away
+      if (xs > 0) mbar_wait_drain(&bars->x_full, (xs - 1) & 1);
+      if (ys > 0) mbar_wait_drain(&bars->y_full, (ys - 1) & 1);
+    }
+  } else if (warp == 1 && lane == 0) {
+    const uint32_t x_lo = smem_desc_lo(smem_u32(smem + SL::x), 16), y_lo = smem_desc_lo(smem_u32(smem + SL::y), 16);
+    const uint32_t wt_lo = smem_desc_lo(smem_u32(smem + SL::wt), 16), s_lo = smem_desc_lo(smem_u32(smem + SL::s), 16);
+    const int ksteps = (d + 15) >> 4;
+    for (int t = 0; t < nt; ++t) {
+      if (!mbar_wait(&bars->x_full, t & 1, abort_flag, status, kErrXMma)) break;
+      if (t > 0 && !mbar_wait(&bars->a_done, (t - 1) & 1, abort_flag, status, kErrXMma)) break;
+      tc_fence_after_sync();
+      issue_planes(tmem, x_lo, wt_lo, ksteps, hi);
+      mma_commit(&bars->a_full);
+      mma_commit(&bars->x_empty);
+      if (!mbar_wait(&bars->y_full, t & 1, abort_flag, status, kErrXMma)) break;
+      if (t > 0 && !mbar_wait(&bars->g_done, (t - 1) & 1, abort_flag, status, kErrXMma)) break;
+      tc_fence_after_sync();
+      issue_planes(tmem + kG, y_lo, s_lo, ksteps, hi);
+      mma_commit(&bars->g_full);
+      mma_commit(&bars->y_empty);
+    }
+  } else if (warp == 2 && lane == 0) {
+    const uint32_t s_lo = smem_desc_lo(smem_u32(smem + SL::s), 1024), wt_lo = smem_desc_lo(smem_u32(smem + SL::wt), 1024);
+    for (int t = 0; t < nt; ++t) {
+      if constexpr (kKeys) {
+        if (!mbar_wait(&bars->a_ready, t & 1, abort_flag, status, kErrXMma)) break;
+        if (!issue_mma2(bars, tmem + kAcc, tmem, 2 * t, s_lo, hi, abort_flag, status)) break;
+        mma_commit(&bars->a_done);
+      }
+      if (!mbar_wait(&bars->g_ready, t & 1, abort_flag, status, kErrXMma)) break;
+      if (!issue_mma2(bars, tmem + kAcc, tmem + kG, kPer * t + kPer - 1, wt_lo, hi, abort_flag, status)) break;
+      mma_commit(&bars->g_done);
+    }
+  } else if (warp >= 4 && warp < 12) {
+    const int g = (warp - 4) >> 2;                        // features 64 g .. 64 g + 63
+    const uint32_t row = 32u * (warp & 3) + lane;         // token of the tile = TMEM lane
+    const uint32_t lanes = tmem + ((32u * (warp & 3)) << 16);
+    bool ok = true;
+    for (int t = 0; t < nt && ok; ++t) {
+      float inv = 0.f, c = 0.f;
+      if constexpr (!kKeys) {
+        const int tok = (t0 + t) * kTile + row;
+        if (tok < n) {
+          inv = __ldcg(tok_inv + (size_t)slab * padded_tokens(n) + tok);
+          c = __ldcg(tok_c + (size_t)slab * padded_tokens(n) + tok);
+        }
+      }
+      ok = __all_sync(0xffffffffu, mbar_wait(&bars->a_full, t & 1, abort_flag, status, kErrXElem));
+      if (!ok) break;
+      tc_fence_after_sync();
+      uint32_t on[2];
+      uint32_t r[32];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        tmem_ld32(lanes + 64 * g + 32 * h, r);
+        tmem_ld_wait();
+        reg_fence32(r);
+        on[h] = 0;
+        float v[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const float x = __uint_as_float(r[j]);
+          on[h] |= (x > 0.f ? 1u : 0u) << j;
+          v[j] = fmaxf(put_back(x), 0.f);
+        }
+        if constexpr (kKeys) store_chunk_planes(lanes, 2 * g + h, v);
+      }
+      if constexpr (kKeys) tmem_st_wait();
+      tc_fence_before_sync();
+      warp_arrive(kKeys ? &bars->a_ready : &bars->a_done);
+      ok = __all_sync(0xffffffffu, mbar_wait(&bars->g_full, t & 1, abort_flag, status, kErrXElem));
+      if (!ok) break;
+      tc_fence_after_sync();
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        tmem_ld32(lanes + kG + 64 * g + 32 * h, r);
+        tmem_ld_wait();
+        reg_fence32(r);
+        float v[32];
+        const float* z = zs + 64 * g + 32 * h;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const float x = put_back(__uint_as_float(r[j]));
+          const float y = kKeys ? x + z[j] : fmaf(c, z[j], x) * inv;
+          v[j] = ((on[h] >> j) & 1u) ? y : 0.f;
+        }
+        store_chunk_planes(lanes + kG, 2 * g + h, v);
+      }
+      tmem_st_wait();
+      tc_fence_before_sync();
+      warp_arrive(&bars->g_ready);
+    }
+  } else if (warp >= 12) {
+    const int et = threadIdx.x - 384;               // token of the tile = TMEM lane
+    const uint32_t taddr = tmem + ((32u * (warp & 3)) << 16) + kAcc;
+    uint8_t* out = smem + SL::out;
+    bool ok = true;
+    for (int v = 0; v < kPer * nt; ++v) {
+      const int row0 = (t0 + v / kPer) * kTile;
+      float s[64];
+#pragma unroll
+      for (int j = 0; j < 64; ++j) s[j] = 0.f;
+      if (ok) ok = drain_tile(bars, taddr, v, s, abort_flag, status);
+      if (et == 0) bulk_wait_group_read0();   // the tile before has left the staging boxes
+      named_bar_sync(kBarDrain, 128);
+      if (ok) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          *reinterpret_cast<float4*>(out + (j >> 3) * kTileBytes + swz128(et, j & 7)) =
+              make_float4(put_back(s[4 * j]), put_back(s[4 * j + 1]), put_back(s[4 * j + 2]), put_back(s[4 * j + 3]));
+        fence_proxy_async_smem();
+      }
+      named_bar_sync(kBarDrain, 128);
+      if (et == 0 && ok) {   // rows past n and columns past d are clipped
+        const CUtensorMap* map = kKeys && (v & 1) == 0 ? &map_dv : &map_dx;
+        for (int c = 0; c < (d > 32 ? 2 : 1); ++c) {
+          if (add)
+            tma_reduce_add_3d(map, out + c * kTileBytes, 32 * c, row0, slab);
+          else
+            tma_store_3d(map, out + c * kTileBytes, 32 * c, row0, slab);
+        }
+        bulk_commit_group();
+      }
+    }
+    if (et == 0) bulk_wait_group0();
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after_sync();
+    tmem_dealloc(tmem, 512);
+  }
+}
+
+// S' and z' (or dS' and dz') per chunk from planes of X (the projected operand) and Y.
+template <bool kScaled>
+cudaError_t launch_summary(const Plan& p, const Ws& w, const __nv_bfloat16* x3, const __nv_bfloat16* y3, const void* W,
+                           const float* scale, const float* weight, cudaStream_t st, int* launches) {
+  auto kernel = k_tcx_kside<kScaled>;
+  CUtensorMap map_x, map_y;
+  cudaError_t err;
+  if ((err = make_tile_map(x3, 3 * p.slabs, p.cfg.seq_len, &map_x, p.cfg.head_dim)) != cudaSuccess) return err;
+  if ((err = make_tile_map(y3, 3 * p.slabs, p.cfg.seq_len, &map_y, p.cfg.head_dim)) != cudaSuccess) return err;
+  if ((err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, KxSmem::total)) != cudaSuccess) return err;
+  *launches += 1;
+  return launch_after(kernel, dim3(p.xchunks, p.slabs, p.cfg.features / kXFeatures), dim3(kXThreads), KxSmem::total, st, map_x, map_y,
+                      (const float*)W, w.spart, w.zpart, p.cfg.seq_len, p.cfg.head_dim, p.cfg.features, p.xchunk_tiles, w.status, scale,
+                      weight);
+}
+
+template <bool kKeys>
+cudaError_t launch_bwd(const Plan& p, const Ws& w, const __nv_bfloat16* x3, const __nv_bfloat16* y3, const void* W, const float* S,
+                       const float* z, float* dx, float* dv, cudaStream_t st, int* launches) {
+  auto kernel = k_tcx_bwd<kKeys>;
+  const int n = p.cfg.seq_len, d = p.cfg.head_dim;
+  CUtensorMap map_x, map_y, map_dx, map_dv;
+  cudaError_t err;
+  if ((err = make_tile_map(x3, 3 * p.slabs, n, &map_x, d)) != cudaSuccess) return err;
+  if ((err = make_tile_map(y3, 3 * p.slabs, n, &map_y, d)) != cudaSuccess) return err;
+  if ((err = make_out_map(dx, p.slabs, n, d, false, &map_dx)) != cudaSuccess) return err;
+  if ((err = make_out_map(dv, p.slabs, n, d, false, &map_dv)) != cudaSuccess) return err;
+  if ((err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, YSmem::total)) != cudaSuccess) return err;
+  for (int f0 = 0; f0 < p.cfg.features; f0 += kXFeatures) {
+    *launches += 1;
+    err = launch_after(kernel, dim3(p.xbchunks, p.slabs), dim3(kXThreads), YSmem::total, st, map_x, map_y, (const float*)W, S, z,
+                       (const float*)w.xinv, (const float*)w.xc, map_dx, map_dv, f0 > 0 ? 1 : 0, n, d, p.cfg.features, f0,
+                       p.xbchunk_tiles, w.status);
+    if (err != cudaSuccess) return err;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace
 
 cudaError_t launch_tcx_kside(const Plan& p, const Ws& w, const void* W, cudaStream_t st, int* launches) {
-  CUtensorMap map_k, map_v;
-  cudaError_t err;
-  if ((err = make_tile_map(w.KF3, 3 * p.slabs, p.cfg.seq_len, &map_k, p.cfg.head_dim)) != cudaSuccess) return err;
-  if ((err = make_tile_map(w.V3, 3 * p.slabs, p.cfg.seq_len, &map_v, p.cfg.head_dim)) != cudaSuccess) return err;
-  if ((err = cudaFuncSetAttribute(k_tcx_kside, cudaFuncAttributeMaxDynamicSharedMemorySize, KxSmem::total)) != cudaSuccess) return err;
-  *launches += 1;
-  return launch_after(k_tcx_kside, dim3(p.xchunks, p.slabs, p.cfg.features / kXFeatures), dim3(kXThreads), KxSmem::total, st, map_k,
-                      map_v, (const float*)W, w.spart, w.zpart, p.cfg.seq_len, p.cfg.head_dim, p.cfg.features, p.xchunk_tiles,
-                      w.status);
+  return launch_summary<false>(p, w, w.KF3, w.V3, W, nullptr, nullptr, st, launches);
 }
 
 cudaError_t launch_tcx_qside(const Plan& p, const Ws& w, const void* W, const float* beta, void* O, cudaStream_t st, int* launches) {
   const int groups = p.cfg.features / kXFeatures, n = p.cfg.seq_len, d = p.cfg.head_dim;
   const size_t tokens = (size_t)p.slabs * n;
-  // several groups leave their shares where the planes of K_F and V were (which the key side has read)
-  float* share = groups > 1 ? reinterpret_cast<float*>(w.KF3) : static_cast<float*>(O);
-  float* den = groups > 1 ? share + groups * tokens * d : nullptr;
-  CUtensorMap map_q, map_o;
+  // Several groups leave their shares where the planes of K_F and V were (which the key side has read), unless a backward
+  // reads those again.
+  float* share = groups == 1 ? static_cast<float*>(O) : p.use_xb ? w.xshare : reinterpret_cast<float*>(w.KF3);
+  float* den = p.use_xb ? w.xden : groups > 1 ? share + groups * tokens * d : nullptr;
+  float* keep = p.use_xb ? w.xO : nullptr;
+  CUtensorMap map_q, map_o, map_keep;
   cudaError_t err;
   if ((err = make_tile_map(w.QF3, 3 * p.slabs, n, &map_q, d)) != cudaSuccess) return err;
   if ((err = make_out_map(share, groups * p.slabs, n, d, false, &map_o)) != cudaSuccess) return err;
+  if ((err = make_out_map(keep != nullptr ? keep : share, p.slabs, n, d, false, &map_keep)) != cudaSuccess) return err;
   if ((err = cudaFuncSetAttribute(k_tcx_qside, cudaFuncAttributeMaxDynamicSharedMemorySize, QxSmem::total)) != cudaSuccess) return err;
   *launches += 1;
   err = launch_after(k_tcx_qside, dim3(p.xchunks, p.slabs, groups), dim3(kXThreads), QxSmem::total, st, map_q, map_o, (const float*)W,
-                     w.S, w.z, beta, p.cfg.eps, p.cfg.bw_floor, den, n, d, p.cfg.features, p.xchunk_tiles, w.status);
+                     (const float*)w.S, (const float*)w.z, beta, p.cfg.eps, p.cfg.bw_floor, den, map_keep,
+                     keep != nullptr && groups == 1 ? 1 : 0, n, d, p.cfg.features, p.xchunk_tiles, w.status);
   if (err != cudaSuccess || groups == 1) return err;
   *launches += 1;
-  return launch_after(k_tcx_combine, dim3((unsigned)((tokens * (d >> 2) + 255) / 256)), dim3(256), 0, st, share, den, beta, p.cfg.eps,
-                      p.cfg.bw_floor, p.cfg.features, (float*)O, tokens, d);
+  return launch_after(k_tcx_combine, dim3((unsigned)((tokens * (d >> 2) + 255) / 256)), dim3(256), 0, st, (const float*)share,
+                      (const float*)den, beta, p.cfg.eps, p.cfg.bw_floor, p.cfg.features, (float*)O, keep, tokens, d);
+}
+
+cudaError_t launch_tcx_bwd_prep(const Plan& p, const Ws& w, const void* dO, const float* beta, cudaStream_t st, int* launches) {
+  int tpt = 1;
+  while (tpt * 8 < p.cfg.head_dim) tpt *= 2;
+  *launches += 1;
+  return launch_after(k_tcx_bwd_prep, dim3(p.xprep), dim3(256), 0, st, (const float*)dO, (const float*)w.xO, (const float*)w.xden,
+                      p.cfg.features / kXFeatures, beta, p.cfg.eps, p.cfg.bw_floor, p.cfg.features, p.cfg.head_dim, tpt,
+                      (size_t)p.slabs * p.cfg.seq_len, p.cfg.seq_len, w.dO3, w.xinv, w.xc, w.sumdD);
+}
+
+cudaError_t launch_tcx_bwd_qside(const Plan& p, const Ws& w, const void* W, cudaStream_t st, int* launches) {
+  const cudaError_t err = launch_bwd<false>(p, w, w.QF3, w.dO3, W, w.S, w.z, w.dQF, w.dQF, st, launches);
+  if (err != cudaSuccess) return err;
+  return launch_summary<true>(p, w, w.QF3, w.dO3, W, w.xinv, w.xc, st, launches);
+}
+
+cudaError_t launch_tcx_bwd_kside(const Plan& p, const Ws& w, const void* W, void* dV, cudaStream_t st, int* launches) {
+  return launch_bwd<true>(p, w, w.KF3, w.V3, W, w.dS, w.dz, w.dKF, (float*)dV, st, launches);
 }
 
 }  // namespace wersa
