@@ -497,7 +497,7 @@ wersa_status wersa_forward(wersa_ctx* ctx, const void* Q, const void* K, const v
     WERSA_STEP(0, "tc_kside", launch_tc_kside(pg, w, K, V, st, &launches));
     if (p.tchunks > 1)
       WERSA_STEP(0, "reduce_partials",
-                 launch_reduce_partials(pg, w.spart, w.zpart, p.tchunks, w.S, w.z, w.Sbf, w.Simg, st, &launches));
+                 launch_reduce_partials(pg, w.spart, w.zpart, p.tchunks, w.S, w.z, p.with_backward ? w.Sbf : nullptr, w.Simg, st, &launches));
     WERSA_STEP(0, "tc_qside", launch_tc_qside(pg, w, Q, beta, w.Og, w.den, st, &launches));
     WERSA_STEP(0, "combine_groups",
                launch_combine_groups(w.Og, w.den, O, rows, p.groups, d, st, &launches));
@@ -505,7 +505,7 @@ wersa_status wersa_forward(wersa_ctx* ctx, const void* Q, const void* K, const v
     WERSA_STEP(0, "tc_kside", launch_tc_kside(p, w, K, V, st, &launches));
     if (p.tchunks > 1)   // with one chunk per slab the key-side kernel has written S', z' and the image itself
       WERSA_STEP(0, "reduce_partials",
-                 launch_reduce_partials(p, w.spart, w.zpart, p.tchunks, w.S, w.z, w.Sbf, w.Simg, st, &launches));
+                 launch_reduce_partials(p, w.spart, w.zpart, p.tchunks, w.S, w.z, p.with_backward ? w.Sbf : nullptr, w.Simg, st, &launches));
     WERSA_STEP(0, "tc_qside", launch_tc_qside(p, w, Q, beta, O, nullptr, st, &launches));
   } else if (p.use_x) {
     WERSA_STEP(0, "f32_planes", launch_f32_planes(p, w, static_cast<const float*>(Q), static_cast<const float*>(K),
@@ -579,7 +579,7 @@ wersa_status wersa_shard_keys(wersa_ctx* ctx, const void* K, const void* V, void
   int launches = 0;
   WERSA_CUDA(launch_tc_kside(p, w, K, V, st, &launches));
   if (p.tchunks > 1)
-    WERSA_CUDA(launch_reduce_partials(p, w.spart, w.zpart, p.tchunks, w.S, w.z, w.Sbf, w.Simg, st, &launches));
+    WERSA_CUDA(launch_reduce_partials(p, w.spart, w.zpart, p.tchunks, w.S, w.z, p.with_backward ? w.Sbf : nullptr, w.Simg, st, &launches));
   ctx->launches_fwd += launches;
   ctx->forward_done = true;   // S', z' of this shard can be read with wersa_saved
   return WERSA_OK;
@@ -598,7 +598,7 @@ wersa_status wersa_shard_output(wersa_ctx* ctx, const void* Q, const float* S_to
   if (guard.err != cudaSuccess) return WERSA_ERR_CUDA;
   int launches = 0;
   // the totals take the place of a single partial: the reduction copies them and writes the operand images
-  WERSA_CUDA(launch_reduce_partials(p, S_total, z_total, 1, w.S, w.z, w.Sbf, w.Simg, st, &launches));
+  WERSA_CUDA(launch_reduce_partials(p, S_total, z_total, 1, w.S, w.z, p.with_backward ? w.Sbf : nullptr, w.Simg, st, &launches));
   WERSA_CUDA(launch_tc_qside(p, w, Q, beta, O, nullptr, st, &launches));
   ctx->launches_fwd += launches;
   return WERSA_OK;

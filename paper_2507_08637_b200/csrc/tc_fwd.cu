@@ -75,6 +75,8 @@ constexpr int kThreads = 32 * (kAuxWarp0 + 8);      // 640 threads, 96 registers
 // Registers per thread after the roles have traded: the Haar step holds a 256 x 64 block in registers
 // and gets what the producer / MMA warpgroup gives up.
 constexpr int kRegsCtl = 40, kRegsAux = 120;
+// Key side, m = 128: units that the ReLU group without an item's summary to write takes alone (see k_tc_kside).
+constexpr int kDrainUnits = 5;
 // Query side: four more warps (12-15) form the epilogue, the Haar warps follow (16-23).  768 threads
 // start with kRegsLaunchQ registers each; the roles re-split exactly that pool (an increase waits
 // until other warps of the CTA have released enough, so the split must never exceed it).
@@ -111,9 +113,11 @@ template <int NH> struct KsideSmem {
   static constexpr uint32_t xch = v + kNV * kTileBytes;           // 2 x 8 x 64 floats
   static constexpr uint32_t hcoef = xch + 4096;                  // kHaarCoefs floats
   static constexpr uint32_t zx = hcoef + 1024;                   // 128 floats
-  static constexpr uint32_t bars = zx + 512;
+  static constexpr uint32_t stage = zx + 512;                    // 8 warps x 32 rows x 12 floats (see drain_columns)
+  static constexpr uint32_t bars = stage + 8 * 32 * 48;
   static constexpr uint32_t total = bars + 512 + 1024;           // + alignment slack
 };
+static_assert(KsideSmem<2>::total <= 232448, "shared memory of an SM");
 template <int NH> struct QsideSmem {
   static constexpr uint32_t wt = 0;
   static constexpr uint32_t simg = wt + NH * kTileBytes;          // 2 NH K blocks of [S' | z' | 0]^T
@@ -427,6 +431,45 @@ __device__ __forceinline__ void haar_role(uint8_t* xring, Bars* bars, float* xch
   }
 }
 
+// 32 columns of S' (col0 ..), 32 features in the lanes of one warp -> memory: fp32 rows at dst, with bdst also bf16 rows, with
+// img the operand image of the query side, where eight features of a column are 16 bytes.  Eight columns at a time
+// turn around in `stage` (32 rows of 12 floats: 48 bytes apart, 16-byte accesses without bank conflicts), so that every store
+// fills its 32-byte sectors.  (Written from the registers, a row per thread in 16-byte pieces and the image in 2-byte ones, an
+// item of 1024 tokens, m = 128 took 8.8 k cycles for that, in which the two ReLU groups and the tensor pipe stood still,
+// beside 9.5 k for its four blocks.)
+__device__ __forceinline__ void drain_columns(const uint32_t (&r)[32], float scale, float* stage, float* __restrict__ dst,
+                                              __nv_bfloat16* __restrict__ bdst, uint8_t* __restrict__ img, int feat0, int col0,
+                                              int lane) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    asm volatile("" : "+r"(lane));   // (the addresses of all four steps computed at once spill)
+    float v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[8 * q + j]) * scale;
+    float* mine = stage + lane * 12;
+    *reinterpret_cast<float4*>(mine) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4*>(mine + 4) = make_float4(v[4], v[5], v[6], v[7]);
+    const int c0 = col0 + 8 * q;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {   // 16 rows x 32 bytes
+      const int row = 16 * i + (lane >> 1), half = 4 * (lane & 1);
+      *reinterpret_cast<float4*>(dst + (size_t)row * kD + c0 + half) = *reinterpret_cast<const float4*>(stage + row * 12 + half);
+    }
+    if (bdst != nullptr)
+      *reinterpret_cast<uint4*>(bdst + (size_t)lane * kD + c0) =
+          make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
+    if (img != nullptr) {
+      const int j = lane >> 2, f = 8 * (lane & 3);   // column and first of eight features
+      const float* col = stage + f * 12 + j;
+      *reinterpret_cast<uint4*>(img + simg_offset(feat0 + f, c0 + j)) =
+          make_uint4(pack_bf16x2(col[0], col[12]), pack_bf16x2(col[24], col[36]), pack_bf16x2(col[48], col[60]),
+                     pack_bf16x2(col[72], col[84]));
+    }
+    __syncwarp();
+  }
+}
+
 // ---- work items ---------------------------------------------------------------------------------
 // Both kernels run one CTA per SM that walks work items: item = slab * chunks + chunk is one sequence
 // chunk of one slab, CTA c takes items c, c + gridDim.x, c + 2 gridDim.x, ...  Ring slots, accumulator
@@ -459,7 +502,6 @@ k_tc_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CU
   const int item0 = blockIdx.x, item_step = kMulti ? (int)gridDim.x : (1 << 30);
   if (!kMulti) items = item0 + 1;
   const int nblk0 = item_blocks(item0, chunks, chunk_blocks, n);
-  constexpr bool single_item = !kMulti;
   constexpr int m = NH * 128;
   const int group = kMulti ? 0 : blockIdx.z;   // feature group: rows of W^T, and which of the group-major results
 
@@ -479,7 +521,7 @@ k_tc_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CU
       mbar_init(&bars->d1_free[b], 1);
     }
     mbar_init(&bars->acc_done, NH);
-    mbar_init(&bars->acc_free, 8);
+    mbar_init(&bars->acc_free, 4 * NH);
     mbar_init(&bars->w_full, 1);
     bars->abort_flag = 0;
     fence_mbar_init();
@@ -677,7 +719,11 @@ k_tc_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CU
       const int slab = it / chunks;
       const int units = item_blocks(it, chunks, chunk_blocks, n) * 2 * NH;
       float zacc = 0.f;
-      for (int u = g; u < units; u += 2) {
+      // The groups take the units in turn, except (NH = 1) while one of them still writes the summary of the item before.
+      const int alone = NH == 1 && ic > 0 ? min(units, kDrainUnits) : 0;   // units of the other group alone
+      const int writer = (ic - 1) & 1;
+      for (int u = 0; u < units; ++u) {
+        if (NH == 1 ? (u < alone ? g == writer : ((u - alone + writer) & 1) != g) : (u & 1) != g) continue;
         const int gu = gu0 + u;
         if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&bars->d1_full[gu % 6], (gu / 6) & 1, abort_flag, status, kErrRelu));
         if (ok) {
@@ -689,102 +735,50 @@ k_tc_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CU
       }
       gu0 += units;
       if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&bars->acc_done, ic & 1, abort_flag, status, kErrRelu));
-      if (ok) tc_fence_after_sync();
+      // Each warp takes 32 features and all columns.  With one half the groups write the items' summaries in turn.
+      const bool writes = NH == 2 || g == (ic & 1);
+      const int feat0 = (NH == 2 ? g * 128 : 0) + (int)lane_base;
+      if (NH == 1) {   // both warpgroups saw the same 128 features on alternating tiles
+        if (ic > 0) named_bar_sync(kBarZsum, 256);    // the sums of the item before have been read
+        if (!writes) zx[row] = zacc;
+        named_bar_sync(kBarZsum, 256);
+        if (writes) zacc = (g == 0 ? zacc : zx[row]) + (g == 0 ? zx[row] : zacc);
+      }
+      if (!writes) continue;
+      uint32_t s0[32], s1[32];
+      if (ok) {
+        tc_fence_after_sync();
+        const uint32_t acc_addr = tmem + (lane_base << 16) + kAccCol + (NH == 2 ? g * 64 : 0);
+        tmem_ld32(acc_addr, s0);
+        tmem_ld32(acc_addr + 32, s1);
+        tmem_ld_wait();
+        reg_fence32(s0);
+        reg_fence32(s1);
+        tc_fence_before_sync();
+        warp_arrive(&bars->acc_free);   // the next item may overwrite the accumulators
+      }
       // (group * slabs + slab) * chunks + chunk
       const size_t pidx = (size_t)it + (kMulti ? 0 : (size_t)group * gridDim.x);
       // S' and z' themselves have the features of all groups side by side
-      const size_t sidx = kMulti || sbf == nullptr ? pidx : (size_t)slab * gridDim.z + group;
-      if (NH == 1) {   // both warpgroups saw the same 128 features on alternating tiles
-        if (ic > 0) named_bar_sync(kBarZsum, 256);    // the sums of the item before have been read
-        if (g == 1) zx[row] = zacc;
-        named_bar_sync(kBarZsum, 256);
-        if (g == 0) zacc += zx[row];
-      }
-      if (ok && (NH == 2 || g == 0)) {
-        const int feat0 = (NH == 2 ? g * 128 : 0) + (int)lane_base;   // first feature of this warp
+      const size_t sidx = kMulti || simg_out == nullptr ? pidx : (size_t)slab * gridDim.z + group;
+      if (ok) {
         // the filter stage left K_F, and with it the features, scaled by r (see haar_block_inplace)
         const float inv_r = 1.f / haar_scale(f[(size_t)slab * (L + 1)]);
-        const uint32_t acc_addr = tmem + (lane_base << 16) + kAccCol + (NH == 2 ? g * 64 : 0);
-        if (single_item) {
-          // The accumulator row of a thread is one feature's 64 values; written straight from the registers
-          // a warp would touch 32 different 256-byte rows per store.  With one item per CTA the K ring is
-          // idle by now: each warp turns its 32 x 32 chunk around in it (rows padded to 33 floats) and
-          // writes whole 128-byte row segments.
-          float* stage = reinterpret_cast<float*>(smem + SL::x) + (warp - kReluWarp0) * (32 * 33);
-          float* dst = spart + (sidx * m + feat0) * kD;
-#pragma unroll 1
-          for (int c = 0; c < 2; ++c) {
-            uint32_t r[32];
-            tmem_ld32(acc_addr + 32 * c, r);
-            tmem_ld_wait();
-            reg_fence32(r);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) stage[lane * 33 + j] = __uint_as_float(r[j]) * inv_r;
-            if (sbf != nullptr) {   // ... and the operand image of the query side (features along a row)
-              uint8_t* img = simg_out + pidx * simg_bytes(m);
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                *reinterpret_cast<__nv_bfloat16*>(img + simg_offset(feat0 + lane, 32 * c + j)) =
-                    __float2bfloat16_rn(__uint_as_float(r[j]) * inv_r);
-            }
-            __syncwarp();
-#pragma unroll 8
-            for (int rr = 0; rr < 32; ++rr) dst[(size_t)rr * kD + 32 * c + lane] = stage[rr * 33 + lane];
-            if (sbf != nullptr) {   // one chunk per slab: this is S' itself, leave its bf16 image as well
-              __nv_bfloat16* bdst = sbf + (pidx * m + feat0) * kD + 32 * c;
-#pragma unroll 8
-              for (int rr = 0; rr < 32; rr += 2) {   // two rows per instruction, a pair of columns per lane
-                const int rw = rr + (lane >> 4), cc = 2 * (lane & 15);
-                *reinterpret_cast<uint32_t*>(bdst + (size_t)rw * kD + cc) =
-                    pack_bf16x2(stage[rw * 33 + cc], stage[rw * 33 + cc + 1]);
-              }
-            }
-            __syncwarp();
-          }
-        } else {
-          // More items follow and the rings already hold their tiles: every thread writes its own row
-          // (16-byte stores; half-used sectors, but the accumulators are free again sooner).
-          float* dst = spart + (sidx * m + feat0 + lane) * kD;
-#pragma unroll 1
-          for (int c = 0; c < 2; ++c) {
-            uint32_t r[32];
-            tmem_ld32(acc_addr + 32 * c, r);
-            tmem_ld_wait();
-            reg_fence32(r);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) * inv_r);
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-              *reinterpret_cast<uint4*>(dst + 32 * c + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
-            if (sbf != nullptr) {
-              uint8_t* img = simg_out + pidx * simg_bytes(m);
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                *reinterpret_cast<__nv_bfloat16*>(img + simg_offset(feat0 + lane, 32 * c + j)) =
-                    __float2bfloat16_rn(__uint_as_float(r[j]));
-              __nv_bfloat16* bdst = sbf + (pidx * m + feat0 + lane) * kD + 32 * c;
-#pragma unroll
-              for (int q = 0; q < 4; ++q)
-                *reinterpret_cast<uint4*>(bdst + 8 * q) =
-                    make_uint4(pack_bf16x2(__uint_as_float(r[8 * q]), __uint_as_float(r[8 * q + 1])),
-                               pack_bf16x2(__uint_as_float(r[8 * q + 2]), __uint_as_float(r[8 * q + 3])),
-                               pack_bf16x2(__uint_as_float(r[8 * q + 4]), __uint_as_float(r[8 * q + 5])),
-                               pack_bf16x2(__uint_as_float(r[8 * q + 6]), __uint_as_float(r[8 * q + 7])));
-            }
-          }
-        }
+        float* stage = reinterpret_cast<float*>(smem + SL::stage) + (warp - kReluWarp0) * (32 * 12);
+        float* dst = spart + (sidx * m + feat0) * kD;
+        // with one chunk per slab this is S' itself: its bf16 image and the query side's operand image as well
+        __nv_bfloat16* bdst = sbf != nullptr ? sbf + (pidx * m + feat0) * kD : nullptr;
+        uint8_t* img = simg_out != nullptr ? simg_out + pidx * simg_bytes(m) : nullptr;
+        drain_columns(s0, inv_r, stage, dst, bdst, img, feat0, 0, lane);
+        drain_columns(s1, inv_r, stage, dst, bdst, img, feat0, 32, lane);
         zpart[sidx * m + feat0 + lane] = zacc * inv_r;
-        if (sbf != nullptr) {   // z' is row 64 of the image, rows 65-79 are zero
-          uint8_t* img = simg_out + pidx * simg_bytes(m);
+        if (img != nullptr) {   // z' is row 64 of the image, rows 65-79 are zero: 15 rows x 4 chunks of eight features
           *reinterpret_cast<__nv_bfloat16*>(img + simg_offset(feat0 + lane, kD)) = __float2bfloat16_rn(zacc * inv_r);
 #pragma unroll
-          for (int row = kD + 1; row < kSimgRows; ++row)
-            *reinterpret_cast<uint16_t*>(img + simg_offset(feat0 + lane, row)) = 0;
+          for (int e = lane; e < 4 * (kSimgRows - kD - 1); e += 32)
+            *reinterpret_cast<uint4*>(img + simg_offset(feat0 + 8 * (e & 3), kD + 1 + (e >> 2))) = make_uint4(0u, 0u, 0u, 0u);
         }
       }
-      // the accumulators may be overwritten by the next item
-      tc_fence_before_sync();
-      if (ok) warp_arrive(&bars->acc_free);
     }
   } else {
     reg_inc<kRegsAux>();
@@ -1176,7 +1170,7 @@ cudaError_t launch_tc_kside(const Plan& p, const Ws& w, const void* K, const voi
   const bool single = p.tchunks == 1;
   float* sp = single ? w.S : w.spart;
   float* zp = single ? w.z : w.zpart;
-  __nv_bfloat16* sb = single ? w.Sbf : nullptr;
+  __nv_bfloat16* sb = single && p.with_backward ? w.Sbf : nullptr;   // (the backward alone reads it)
   uint8_t* si = single ? w.Simg : nullptr;
   // Some CTA walks more than one item?  Never with feature groups: their CTAs come in waves (see make_plan).  Without
   // groups walking is the faster way (64 x 12 x 1024, m = 128: 130 us, in waves 164 us; m = 256: 186 and 202 us).
