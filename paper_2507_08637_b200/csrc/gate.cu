@@ -302,8 +302,18 @@ __device__ __forceinline__ float gate_df(const float* __restrict__ df, int b, in
   for (int hh = 0; hh < H; ++hh) s += __ldcg(df + ((size_t)b * H + hh) * kBandVals + i);
   return s;
 }
-constexpr int kGateRound = 28;   // batch elements of a round: a multiple of four, 28 x 9 values for the 256 threads
-__global__ void __launch_bounds__(256) k_gate_backward(
+// kParts = 4 parts of 64 threads, 16 where the batch is more than one round of four: at B=341 H=3 13 rounds of two
+// latencies each, and 22 for domega, took 37 us of a training step of 291, with 16 parts 16 (the step 271).
+// Sum of the parts' values in pairs of pairs.
+template <int kParts, typename F>
+__device__ __forceinline__ float sum_parts(F value) {
+  float s = (value(0) + value(1)) + (value(2) + value(3));
+#pragma unroll
+  for (int a = 4; a < kParts; a += 4) s += (value(a) + value(a + 1)) + (value(a + 2) + value(a + 3));
+  return s;
+}
+template <int kParts>
+__global__ void __launch_bounds__(64 * kParts) k_gate_backward(
     const float* __restrict__ df, const float* __restrict__ sg, const float* __restrict__ qbar,
     const float* __restrict__ gate_w, const float* __restrict__ omega, const float* __restrict__ sumdD,
     int n_sumdD, const float* __restrict__ beta, float eps, float bw_floor, int m, int B, int H, int dcols, int L1,
@@ -313,8 +323,11 @@ __global__ void __launch_bounds__(256) k_gate_backward(
   // wait, and unless it is the first one of its pass the gate weights are fetched ahead of it)
   if (first) wait_for_stream_predecessor();
   let_stream_successor_start();
-  __shared__ float part[4][kMaxLevels + 1][kD];
-  __shared__ float gbs[4][kMaxLevels + 1];
+  constexpr int kThreads = 64 * kParts;
+  constexpr int kGateRound = 7 * kParts;   // batch elements of a round: seven a part, 7 x 9 values for its 64 threads
+  static_assert(kGateRound * (kMaxLevels + 1) <= kThreads, "a value of a round per thread");
+  __shared__ float part[kParts][kMaxLevels + 1][kD];
+  __shared__ float gbs[kParts][kMaxLevels + 1];
   __shared__ float dus[kGateRound][kMaxLevels + 1];
   float* flat = &part[0][0][0];
   const int tid = threadIdx.x;
@@ -329,10 +342,10 @@ __global__ void __launch_bounds__(256) k_gate_backward(
     wait_for_stream_predecessor();
     const int db = tid / (kMaxLevels + 1), di = tid - db * (kMaxLevels + 1);   // this thread's du of a round
     for (int b0 = 0; b0 < B; b0 += kGateRound) {
-      float qb[kGateRound / 4];
+      float qb[kGateRound / kParts];
 #pragma unroll
-      for (int r = 0; r < kGateRound / 4; ++r) {
-        const int b = b0 + q + 4 * r;
+      for (int r = 0; r < kGateRound / kParts; ++r) {
+        const int b = b0 + q + kParts * r;
         qb[r] = b < B ? qbar[((size_t)b * H + h) * kD + c] : 0.f;
       }
       if (b0 > 0) __syncthreads();   // the round before has been read
@@ -346,14 +359,14 @@ __global__ void __launch_bounds__(256) k_gate_backward(
       }
       __syncthreads();
 #pragma unroll
-      for (int r = 0; r < kGateRound / 4; ++r) {
-        const int b = b0 + q + 4 * r;
+      for (int r = 0; r < kGateRound / kParts; ++r) {
+        const int b = b0 + q + kParts * r;
         if (b >= B) break;
         float dq = 0.f;
 #pragma unroll
         for (int i = 0; i <= kMaxLevels; ++i)
           if (i < L1) {
-            const float du = dus[q + 4 * r][i];
+            const float du = dus[q + kParts * r][i];
             gw_acc[i] += qb[r] * du;
             gb_acc[i] += du;
             if (gate_w != nullptr) dq += gw[i] * du;   // (none without weights, whatever du is)
@@ -367,21 +380,21 @@ __global__ void __launch_bounds__(256) k_gate_backward(
       if (c == 0) gbs[q][i] = gb_acc[i];
     }
     __syncthreads();
-    for (int e = tid; e < dcols * L1; e += 256) {   // (columns past the head dimension are padding of qbar)
+    for (int e = tid; e < dcols * L1; e += kThreads) {   // (columns past the head dimension are padding of qbar)
       const int cc = e / L1, i = e - cc * L1;
       if (dgate_w != nullptr)
-        dgate_w[(size_t)h * dcols * L1 + e] = (part[0][i][cc] + part[1][i][cc]) + (part[2][i][cc] + part[3][i][cc]);
+        dgate_w[(size_t)h * dcols * L1 + e] = sum_parts<kParts>([&](int a) { return part[a][i][cc]; });
     }
     if (dgate_b != nullptr && tid < L1)
-      dgate_b[h * L1 + tid] = per_head || h == 0 ? (gbs[0][tid] + gbs[1][tid]) + (gbs[2][tid] + gbs[3][tid]) : 0.f;
+      dgate_b[h * L1 + tid] = per_head || h == 0 ? sum_parts<kParts>([&](int a) { return gbs[a][tid]; }) : 0.f;
   } else if ((int)blockIdx.x == H) {
-    // domega[i] = sum over slabs of df_i * sigmoid(u_i): thread (i = tid & 15, q = tid >> 4) takes every 16th batch
+    // domega[i] = sum over slabs of df_i * sigmoid(u_i): thread (i = tid & 15, q = tid >> 4) takes every (4 kParts)th batch
     // element, then the parts are added in order
     const int i = tid & 15, q = tid >> 4;
     float acc = 0.f;
     wait_for_stream_predecessor();
     if (domega != nullptr && i < L1) {
-      for (int b = q; b < B; b += 16) {
+      for (int b = q; b < B; b += 4 * kParts) {
         if (per_head) {
 #pragma unroll 4
           for (int h = 0; h < H; ++h) {
@@ -398,17 +411,17 @@ __global__ void __launch_bounds__(256) k_gate_backward(
     if (domega != nullptr && tid < L1) {
       float s = 0.f;
 #pragma unroll
-      for (int r = 0; r < 16; ++r) s += flat[16 * r + tid];
+      for (int r = 0; r < 4 * kParts; ++r) s += flat[16 * r + tid];
       domega[tid] = s;
     }
   } else {
     wait_for_stream_predecessor();
     float tot = 0.f;
 #pragma unroll 4
-    for (int i = tid; i < n_sumdD; i += 256) tot += __ldcg(sumdD + i);
+    for (int i = tid; i < n_sumdD; i += kThreads) tot += __ldcg(sumdD + i);
     flat[tid] = tot;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
+    for (int o = kThreads / 2; o > 0; o >>= 1) {
       if (tid < o) flat[tid] += flat[tid + o];
       __syncthreads();
     }
@@ -523,6 +536,18 @@ size_t static_scratch_floats_needed(const Plan& p) {
 }
 size_t static_scratch_counters_needed(const Plan& p) { return (size_t)p.slabs + (size_t)p.cfg.batch; }
 
+static void gate_backward_kernel(const Plan& p, const Ws& w, const float* df, const float* beta, const float* gate_w,
+                                 const float* omega, const float* sumdD, int n_sumdD, float* dbeta, float* dgate_w,
+                                 float* dgate_b, float* domega, bool first, cudaStream_t st) {
+  auto go = [&](auto kernel, int threads) {
+    launch_after(kernel, dim3(p.cfg.heads + 2), dim3(threads), 0, st, df, w.sg, w.qbar, gate_w, omega, sumdD, n_sumdD, beta,
+                 p.cfg.eps, p.cfg.bw_floor, p.cfg.features, p.cfg.batch, p.cfg.heads, p.cfg.head_dim, p.L1, p.cfg.gate_per_head,
+                 dbeta, dgate_w, dgate_b, domega, w.dqbar, first);
+  };
+  if (p.cfg.batch <= 28) go(k_gate_backward<4>, 256);
+  else go(k_gate_backward<16>, 1024);
+}
+
 // The two halves of launch_gate_backward, for sequence shards: this shard's band inner products (df, slabs x 16)
 // and its sum of dD'; then, from the sums over all shards, the parameter gradients and d(qbar).
 cudaError_t launch_band_sums(const Plan& p, const Ws& w, int band_blocks, int n_sumdD, float* df, float* sumdD_total,
@@ -535,9 +560,7 @@ cudaError_t launch_band_sums(const Plan& p, const Ws& w, int band_blocks, int n_
 cudaError_t launch_gate_backward_from(const Plan& p, const Ws& w, const float* df, const float* sumdD_total,
                                       const float* beta, const float* gate_w, const float* omega, float* dbeta,
                                       float* dgate_w, float* dgate_b, float* domega, cudaStream_t st, int* launches) {
-  launch_after(k_gate_backward, dim3(p.cfg.heads + 2), dim3(256), 0, st, df, w.sg, w.qbar, gate_w, omega, sumdD_total, 1,
-               beta, p.cfg.eps, p.cfg.bw_floor, p.cfg.features, p.cfg.batch, p.cfg.heads, p.cfg.head_dim, p.L1, p.cfg.gate_per_head,
-               dbeta, dgate_w, dgate_b, domega, w.dqbar, true);
+  gate_backward_kernel(p, w, df, beta, gate_w, omega, sumdD_total, 1, dbeta, dgate_w, dgate_b, domega, true, st);
   *launches += 1;
   return cudaGetLastError();
 }
@@ -547,10 +570,7 @@ cudaError_t launch_gate_backward(const Plan& p, const Ws& w, int band_blocks, co
                                  float* domega, cudaStream_t st, int* launches) {
   float* df = w.dqbar + (size_t)p.slabs * kD;   // df lives behind dqbar in the same region
   launch_after(k_band_reduce, dim3(p.slabs), dim3(256), 0, st, w.bands, p.slabs, band_blocks, p.cfg.levels, df);
-  launch_after(k_gate_backward, dim3(p.cfg.heads + 2), dim3(256), 0, st, df, w.sg, w.qbar, gate_w, omega, w.sumdD, n_sumdD, beta,
-                                    p.cfg.eps, p.cfg.bw_floor, p.cfg.features, p.cfg.batch, p.cfg.heads,
-                                    p.cfg.head_dim, p.L1, p.cfg.gate_per_head, dbeta, dgate_w, dgate_b, domega, w.dqbar,
-                                    false);
+  gate_backward_kernel(p, w, df, beta, gate_w, omega, w.sumdD, n_sumdD, dbeta, dgate_w, dgate_b, domega, false, st);
   *launches += 2;
   return cudaGetLastError();
 }
