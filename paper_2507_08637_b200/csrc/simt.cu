@@ -712,16 +712,18 @@ __device__ __forceinline__ T sum_chunks4(const T* __restrict__ p, size_t stride,
   return a[0];
 }
 
-// grid (m / 8, slabs, feature groups), block 512 / V + 32: one CTA adds the partials of eight consecutive features (512 elements of
-// S', V = 1 or 4 per thread, and by the last warp their eight entries of z') in chunk order.  With Sbf it also leaves the bf16
+// grid (m / (8 J), slabs, feature groups), block 512 / V + 32: one CTA adds the partials of J times eight consecutive features (512
+// elements of S', V = 1 or 4 per thread, and by the last warp their eight entries of z') in chunk order.  With Sbf it also leaves the bf16
 // copy of S', with Simg the operand image of the query-side kernel (see simg_offset): eight consecutive features
 // are one 16-byte chunk of an image row, so the 80 rows of the CTA's part go out as one 16-byte store each.
 // ctas > 0: the partials are the segments of the tensor-core backward instead of `chunks` per slab.
 // What bounds it is the number of bytes in flight: with one element per thread most of a large grid's time went into
 // waves of threads that live for two or three loads, with four a small grid leaves the SMs with too few threads
 // (32 x 128 CTAs with 2 or 3 partials, as fp32 S' and bf16: 21 us with V = 1, 14 with 4; 24 x 192: 16 and 12 us;
-// 32 x 8 CTAs with 18 partials: a whole forward of 1 x 8 x 131072 201 us with V = 1, 203 with 4).
-template <int V>
+// 32 x 8 CTAs with 18 partials: a whole forward of 1 x 8 x 131072 201 us with V = 1, 203 with 4).  From 16 such CTAs per SM
+// on, four parts in one CTA (J = 4), whose loads go out together where there are up to three partials, as many slabs have:
+// 1023 slabs, m = 128 38 -> 26 us of a training step of 271, 192 slabs 16.5 -> 15.6.
+template <int V, int J>
 __global__ void __launch_bounds__(512 / V + 32) k_reduce_partials(const float* __restrict__ spart,
                                                          const float* __restrict__ zpart, int chunks, int tps, int ctas,
                                                          int m, float* __restrict__ S, float* __restrict__ z,
@@ -731,9 +733,9 @@ __global__ void __launch_bounds__(512 / V + 32) k_reduce_partials(const float* _
   // complete once the kernel before it has finished.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  __shared__ __align__(16) __nv_bfloat16 tile[kSimgRows][8];   // [image row][feature - f0]
+  __shared__ __align__(16) __nv_bfloat16 tile[J][kSimgRows][8];   // [part][image row][feature of the part]
   // slab counts through the slabs of one group after the other; S and z have a slab's features together
-  const int slab = blockIdx.z * gridDim.y + blockIdx.y, f0 = blockIdx.x * 8;
+  const int slab = blockIdx.z * gridDim.y + blockIdx.y, f0 = blockIdx.x * 8 * J;
   const size_t out = blockIdx.y * gridDim.z + blockIdx.z;
   const int ns = m * kD;
   size_t slot = (size_t)slab * chunks;          // first partial of this slab
@@ -743,36 +745,59 @@ __global__ void __launch_bounds__(512 / V + 32) k_reduce_partials(const float* _
     slot = (size_t)c0 + slab;
     chunks = c1 - c0 + 1;
   }
-  constexpr int kMain = 512 / V;
+  constexpr int kMain = 512 / V, kThreads = kMain + 32;
   using T = typename std::conditional<V == 4, float4, float>::type;
   if (threadIdx.x < kMain) {
-    const int e = V * threadIdx.x;                // first element of the thread in the CTA's 8 x 64 part
-    const int i = f0 * kD + e;                    // element of S' (feature i / 64, column i % 64)
-    const T s = sum_chunks4(reinterpret_cast<const T*>(spart + slot * ns + i), ns / V, chunks);
-    *reinterpret_cast<T*>(S + out * ns + i) = s;
-    union {
-      __nv_bfloat16 b[V];
-      typename std::conditional<V == 4, uint2, uint16_t>::type all;
-    } r;
+    const int e = V * threadIdx.x;                // first element of the thread in each 8 x 64 part
+    const int i = f0 * kD + e;                    // element of S' (feature i / 64, column i % 64) in the first part
+    const T* src = reinterpret_cast<const T*>(spart + slot * ns + i);
+    T s[J];
+    if (J > 1 && chunks <= 3) {   // (the sums of sum_chunks4)
 #pragma unroll
-    for (int q = 0; q < V; ++q) {
-      r.b[q] = __float2bfloat16_rn(reinterpret_cast<const float*>(&s)[q]);
-      tile[(e & (kD - 1)) + q][e >> 6] = r.b[q];
+      for (int j = 0; j < J; ++j) s[j] = src[j * kMain];
+      for (int k = 1; k < chunks; ++k) {
+        T v[J];
+#pragma unroll
+        for (int j = 0; j < J; ++j) v[j] = src[(size_t)k * (ns / V) + j * kMain];
+#pragma unroll
+        for (int j = 0; j < J; ++j) add_to(s[j], v[j]);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < J; ++j) s[j] = sum_chunks4(src + j * kMain, ns / V, chunks);
     }
-    if (Sbf != nullptr) *reinterpret_cast<decltype(r.all)*>(Sbf + (size_t)slab * ns + i) = r.all;
-  } else if (threadIdx.x < kMain + 8) {
-    const int q = threadIdx.x - kMain, r = f0 + q;
-    const float zr = sum_chunks4(zpart + slot * m + r, m, chunks);
-    z[out * m + r] = zr;
-    tile[kD][q] = __float2bfloat16_rn(zr);   // z' is row 64 of the image
-  } else if (threadIdx.x < kMain + 8 + kSimgRows - kD - 1) {   // rows 65-79 are zero
-    *reinterpret_cast<uint4*>(&tile[kD + 1 + threadIdx.x - kMain - 8][0]) = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      *reinterpret_cast<T*>(S + out * ns + i + 512 * j) = s[j];
+      union {
+        __nv_bfloat16 b[V];
+        typename std::conditional<V == 4, uint2, uint16_t>::type all;
+      } r;
+#pragma unroll
+      for (int q = 0; q < V; ++q) {
+        r.b[q] = __float2bfloat16_rn(reinterpret_cast<const float*>(&s[j])[q]);
+        tile[j][(e & (kD - 1)) + q][e >> 6] = r.b[q];
+      }
+      if (Sbf != nullptr) *reinterpret_cast<decltype(r.all)*>(Sbf + (size_t)slab * ns + i + 512 * j) = r.all;
+    }
+  } else {
+    const int q = threadIdx.x - kMain;
+    if (q < 8 * J) {
+      const int r = f0 + q;
+      const float zr = sum_chunks4(zpart + slot * m + r, m, chunks);
+      z[out * m + r] = zr;
+      tile[q >> 3][kD][q & 7] = __float2bfloat16_rn(zr);   // z' is row 64 of the image
+    }
+    for (int e = q; e < J * (kSimgRows - kD - 1); e += 32)   // rows 65-79 are zero
+      *reinterpret_cast<uint4*>(&tile[e / (kSimgRows - kD - 1)][kD + 1 + e % (kSimgRows - kD - 1)][0]) = make_uint4(0u, 0u, 0u, 0u);
   }
   if (Simg == nullptr) return;
   __syncthreads();
-  if (threadIdx.x < kSimgRows)
-    *reinterpret_cast<uint4*>(Simg + (size_t)slab * simg_bytes(m) + simg_offset(f0, threadIdx.x)) =
-        *reinterpret_cast<const uint4*>(&tile[threadIdx.x][0]);
+  for (int e = threadIdx.x; e < J * kSimgRows; e += kThreads) {
+    const int j = e / kSimgRows, row = e - j * kSimgRows;
+    *reinterpret_cast<uint4*>(Simg + (size_t)slab * simg_bytes(m) + simg_offset(f0 + 8 * j, row)) =
+        *reinterpret_cast<const uint4*>(&tile[j][row][0]);
+  }
 }
 
 template <typename K>
@@ -824,10 +849,13 @@ static cudaError_t launch_reduce(const Plan& p, int groups, const float* spart, 
   // (four CTAs per SM: see k_reduce_partials; a sequence shard's caller may hand in sums that lie at any float, such as a
   // view into the buffer of a larger all-reduce, and those are read one by one)
   const bool aligned = (reinterpret_cast<uintptr_t>(spart) & 15u) == 0;
-  const cudaError_t err =
-      aligned && grid.x * grid.y * grid.z > 4u * p.sms
-          ? launch_after(k_reduce_partials<4>, grid, dim3(160), 0, st, spart, zpart, chunks, tps, ctas, m, S, z, Sbf, Simg)
-          : launch_after(k_reduce_partials<1>, grid, dim3(544), 0, st, spart, zpart, chunks, tps, ctas, m, S, z, Sbf, Simg);
+  const unsigned ctas8 = grid.x * grid.y * grid.z;
+  auto go = [&](auto kernel, dim3 g, int threads) {
+    return launch_after(kernel, g, dim3(threads), 0, st, spart, zpart, chunks, tps, ctas, m, S, z, Sbf, Simg);
+  };
+  const cudaError_t err = !aligned || ctas8 <= 4u * p.sms ? go(k_reduce_partials<1, 1>, grid, 544)
+                          : ctas8 <= 16u * p.sms          ? go(k_reduce_partials<4, 1>, grid, 160)
+                                                          : go(k_reduce_partials<4, 4>, dim3(m / 32, grid.y, grid.z), 160);
   *launches += 1;
   return err != cudaSuccess ? err : cudaGetLastError();
 }
