@@ -769,8 +769,23 @@ k_tc_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CU
         // with one chunk per slab this is S' itself: its bf16 image and the query side's operand image as well
         __nv_bfloat16* bdst = sbf != nullptr ? sbf + (pidx * m + feat0) * kD : nullptr;
         uint8_t* img = simg_out != nullptr ? simg_out + pidx * simg_bytes(m) : nullptr;
-        drain_columns(s0, inv_r, stage, dst, bdst, img, feat0, 0, lane);
-        drain_columns(s1, inv_r, stage, dst, bdst, img, feat0, 32, lane);
+        if (!kMulti && img == nullptr) {
+          // The partial of a CTA's only item: the K ring is idle by now, and whole 32 x 32 pieces turn around in it (rows of
+          // 33 floats), so that a store is one row's 128 bytes (6 x 832, m = 256: a forward of 18.3 us, with drain_columns 19.3).
+          float* piece = reinterpret_cast<float*>(smem + SL::x) + (warp - kReluWarp0) * (32 * 33);
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) piece[lane * 33 + j] = __uint_as_float(c == 0 ? s0[j] : s1[j]) * inv_r;
+            __syncwarp();
+#pragma unroll 8
+            for (int rr = 0; rr < 32; ++rr) dst[(size_t)rr * kD + 32 * c + lane] = piece[rr * 33 + lane];
+            __syncwarp();
+          }
+        } else {
+          drain_columns(s0, inv_r, stage, dst, bdst, img, feat0, 0, lane);
+          drain_columns(s1, inv_r, stage, dst, bdst, img, feat0, 32, lane);
+        }
         zpart[sidx * m + feat0 + lane] = zacc * inv_r;
         if (img != nullptr) {   // z' is row 64 of the image, rows 65-79 are zero: 15 rows x 4 chunks of eight features
           *reinterpret_cast<__nv_bfloat16*>(img + simg_offset(feat0 + lane, kD)) = __float2bfloat16_rn(zacc * inv_r);
