@@ -227,6 +227,11 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 __device__ __forceinline__ float sum2(f32x2 v) {
   float lo, hi;
   upk2(v, lo, hi);
@@ -280,6 +285,13 @@ template <typename T> __device__ __forceinline__ T from_f32(float x);
 template <> __device__ __forceinline__ float from_f32<float>(float x) { return x; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float x) {
   return __float2bfloat16_rn(x);
+}
+
+// A finite value inside the range of bf16, whose largest is 2^128 - 2^120 (what is above it rounds to infinity); infinities and
+// NaN as they are.
+__device__ __forceinline__ float bf16_range(float x) {
+  const float most = __uint_as_float(0x7F7F0000u);
+  return fabsf(x) < INFINITY ? fminf(fmaxf(x, -most), most) : x;
 }
 
 // Loads 8 consecutive elements (16-byte aligned for bf16, 32-byte for float) as floats.

@@ -273,7 +273,10 @@ __global__ void __launch_bounds__(256, 3) k_f32_planes(const float* __restrict__
     if (kKeep && filtered) store4(keep + first + (size_t)j * d, x[j]);
 #pragma unroll
     for (int pl = 0; pl < 3; ++pl) {   // what a plane leaves is the next one's input
-      const __nv_bfloat162 a = __floats2bfloat162_rn(x[j][0], x[j][1]), b = __floats2bfloat162_rn(x[j][2], x[j][3]);
+      float v[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[c] = pl == 0 ? bf16_range(x[j][c]) : x[j][c];
+      const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
       const uint2 w = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
       *reinterpret_cast<uint2*>(dst + (size_t)pl * plane + (size_t)j * d) = w;
       x[j][0] -= __uint_as_float(w.x << 16);

@@ -83,9 +83,11 @@ static_assert(QxSmem::total <= 232448 && KxSmem::total <= 232448 && sizeof(XBars
 // to begin on an 8-byte boundary where n is odd).
 __host__ __device__ __forceinline__ int padded_tokens(int n) { return (n + kTile - 1) / kTile * kTile; }
 
-// Two floats -> one packed pair per plane.
+// Two floats -> one packed pair per plane.  kLarge: values above the largest bf16 keep a finite first plane (see
+// bf16_range); features go without, since what a feature of that size adds to is beyond 32 bits with anything above 1.
+template <bool kLarge = false>
 __device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-  hi = pack_bf16x2(a, b);
+  hi = kLarge ? pack_bf16x2(bf16_range(a), bf16_range(b)) : pack_bf16x2(a, b);
   a -= __uint_as_float(hi << 16);
   b -= __uint_as_float(hi & 0xFFFF0000u);
   mid = pack_bf16x2(a, b);
@@ -97,7 +99,7 @@ __device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t&
 __device__ __forceinline__ void put_planes8(uint8_t* tile, int row, int chunk, const float (&v)[8]) {
   uint32_t p[3][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) split3(v[2 * i], v[2 * i + 1], p[0][i], p[1][i], p[2][i]);
+  for (int i = 0; i < 4; ++i) split3<true>(v[2 * i], v[2 * i + 1], p[0][i], p[1][i], p[2][i]);
 #pragma unroll
   for (int s = 0; s < 3; ++s)
     *reinterpret_cast<uint4*>(tile + s * kTileBytes + swz128(row, chunk)) = make_uint4(p[s][0], p[s][1], p[s][2], p[s][3]);
@@ -130,20 +132,75 @@ __device__ __forceinline__ void load_s_planes(const float* S, const float* zg, s
   if (threadIdx.x < kXFeatures) zs[threadIdx.x] = __ldcg(zg + row0 + threadIdx.x);
 }
 
+// The planes of an infinite value are infinity, NaN and NaN: what the tensor cores make of a dot product that meets one is NaN,
+// and a ReLU would drop it.  In 32 bits it is infinite, or NaN where infinities cancel: such elements are formed again, from
+// the planes' sums and W.  (Only their class matters: a NaN came from an operand that is not finite.)
+struct Operands {
+  const __nv_bfloat16* x3;   // first plane of the slab: n rows of d values
+  size_t plane;              // values of a plane
+  const float* W;            // d x m
+  int n, d, m;
+};
+// Are there NaN among 32 columns of the warp?  (False alarms, such as opposite infinities, cost time only.)
+__device__ __forceinline__ bool warp_meets_nan(const uint32_t (&r)[32]) {
+  f32x2 t[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) t[j] = pk2u(r[2 * j], r[2 * j + 1]);
+#pragma unroll
+  for (int j = 4; j < 16; ++j) t[j & 3] = add2(t[j & 3], pk2u(r[2 * j], r[2 * j + 1]));
+  const float s = sum2(add2(add2(t[0], t[1]), add2(t[2], t[3])));
+  return __any_sync(0xffffffffu, s != s);
+}
+// The NaN among the 32 columns at taddr again.  Column j of a lane is token tok + j * dtok, feature feat + j * dfeat.
+__device__ __noinline__ void form_again(uint32_t taddr, const Operands op, int tok, int dtok, int feat, int dfeat) {
+  for (int j = 0; j < 32; ++j, tok += dtok, feat += dfeat) {
+    uint32_t r;
+    tmem_ld1(taddr + j, r);
+    tmem_ld_wait();
+    float a = __uint_as_float(r);
+    if (a != a && tok < op.n) {   // (rows past n are zeros: NaN against an infinite W, and no feature either way)
+      const __nv_bfloat16* x = op.x3 + (size_t)tok * op.d;
+      a = 0.f;
+      for (int c = 0; c < op.d && a == a; ++c) {
+        float v = __bfloat162float(__ldcg(x + c));
+        if (fabsf(v) < INFINITY) v = (v + __bfloat162float(__ldcg(x + op.plane + c))) + __bfloat162float(__ldcg(x + 2 * op.plane + c));
+        a = fmaf(v, op.W[(size_t)c * op.m + feat], a);
+      }
+      r = __float_as_uint(a);
+    }
+    __syncwarp();
+    tmem_st1(taddr + j, r);
+  }
+  tmem_st_wait();
+}
+// 32 columns of pre-activations.
+__device__ __forceinline__ void load_projected(uint32_t taddr, uint32_t (&r)[32], const Operands& op, int tok, int dtok, int feat,
+                                               int dfeat) {
+  tmem_ld32(taddr, r);
+  tmem_ld_wait();
+  reg_fence32(r);
+  if (warp_meets_nan(r)) {
+    form_again(taddr, op, tok, dtok, feat, dfeat);
+    tmem_ld32(taddr, r);
+    tmem_ld_wait();
+    reg_fence32(r);
+  }
+}
+
 // One D1 buffer: 128 fp32 columns -> ReLU -> planes.  32 columns hold 16 hi and 16 mid pairs of their features, the lo pairs
 // go to the columns behind them.  Returns the sum of the row's values, kWeighted: each times w[column], in chains of
 // eight, as few additions in a row as the FFMA kernels have (two chains of 64: D' 8e-8 off, more than all else together).
 // kScaled: the values are multiplied by s[column] first, and the sum is of those times w[column]; both arrays in global
 // memory, on an 8-byte boundary, and may hold anything where the value is zero.
-template <bool kWeighted, bool kScaled = false>
-__device__ __forceinline__ float relu_planes(uint32_t taddr, const float* w, const float* s = nullptr) {
+// kTokens: the columns are tokens from tok on and the lane is feature feat, else the other way round.
+template <bool kTokens, bool kWeighted, bool kScaled = false>
+__device__ __forceinline__ float relu_planes(uint32_t taddr, const Operands& op, int tok, int feat, const float* w,
+                                             const float* s = nullptr) {
   uint32_t r[32];
   float total = 0.f;
 #pragma unroll 1
   for (int c = 0; c < 4; ++c) {
-    tmem_ld32(taddr + 32 * c, r);
-    tmem_ld_wait();
-    reg_fence32(r);
+    load_projected(taddr + 32 * c, r, op, tok + (kTokens ? 32 * c : 0), kTokens, feat + (kTokens ? 0 : 32 * c), !kTokens);
     uint32_t hi[16], mid[16], lo[16];
     float e[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -153,10 +210,11 @@ __device__ __forceinline__ float relu_planes(uint32_t taddr, const float* w, con
       if constexpr (kScaled) {
         const float2 z = __ldg(reinterpret_cast<const float2*>(w + 32 * c + 2 * j));
         const float2 f = __ldg(reinterpret_cast<const float2*>(s + 32 * c + 2 * j));
-        a = a > 0.f ? a * f.x : 0.f;
-        b = b > 0.f ? b * f.y : 0.f;
-        e[k] += a > 0.f ? a * z.x : 0.f;
-        e[k + 1] += b > 0.f ? b * z.y : 0.f;
+        const bool on_a = a > 0.f, on_b = b > 0.f;
+        a = on_a ? a * f.x : 0.f;
+        b = on_b ? b * f.y : 0.f;
+        e[k] += on_a ? a * z.x : 0.f;
+        e[k + 1] += on_b ? b * z.y : 0.f;
       } else if constexpr (kWeighted) {
         const float2 z = *reinterpret_cast<const float2*>(w + 32 * c + 2 * j);
         e[k] = fmaf(a, z.x, e[k]);
@@ -282,7 +340,7 @@ template <bool kScaled>
 __global__ void __launch_bounds__(kXThreads, 1)
 k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const float* __restrict__ W,
             float* __restrict__ spart, float* __restrict__ zpart, int n, int d, int m, int chunk_tiles, int* __restrict__ status,
-            const float* __restrict__ scale, const float* __restrict__ weight) {
+            const __nv_bfloat16* x3, const float* __restrict__ scale, const float* __restrict__ weight) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
   using SL = KxSmem;
@@ -344,6 +402,7 @@ k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ C
     const uint32_t row = 32u * (warp & 3) + lane;   // feature of the group = TMEM lane
     const uint32_t taddr = tmem + ((32u * (warp & 3)) << 16) + g * kBufCols;
     float* zx = reinterpret_cast<float*>(smem + SL::zx);
+    const Operands op = {x3 + (size_t)slab * n * d, (size_t)slabs * n * d, W, n, d, m};
     float z = 0.f;
     bool ok = true;
     for (int t = g; t < nt && ok; t += 2) {
@@ -352,9 +411,9 @@ k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ C
       tc_fence_after_sync();
       if constexpr (kScaled) {
         const size_t tok = (size_t)slab * padded_tokens(n) + (size_t)(t0 + t) * kTile;
-        z += relu_planes<true, true>(taddr, weight + tok, scale + tok);
+        z += relu_planes<true, true, true>(taddr, op, (t0 + t) * kTile, f0 + row, weight + tok, scale + tok);
       } else {
-        z += relu_planes<false>(taddr, nullptr);
+        z += relu_planes<true, false>(taddr, op, (t0 + t) * kTile, f0 + row, nullptr);
       }
       tc_fence_before_sync();
       warp_arrive(&bars->phi_ready[g]);
@@ -401,7 +460,7 @@ __global__ void __launch_bounds__(kXThreads, 1)
 k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o, const float* __restrict__ W,
             const float* __restrict__ S, const float* __restrict__ zg, const float* __restrict__ beta, float eps, float bw_floor,
             float* __restrict__ den_out, const __grid_constant__ CUtensorMap map_keep, int keep, int n, int d, int m, int chunk_tiles,
-            int* __restrict__ status) {
+            int* __restrict__ status, const __nv_bfloat16* x3) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
   using SL = QxSmem;
@@ -453,12 +512,13 @@ k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     const int g = (warp - 4) >> 2;
     const uint32_t row = 32u * (warp & 3) + lane;   // token of the tile = TMEM lane
     const uint32_t taddr = tmem + ((32u * (warp & 3)) << 16) + g * kBufCols;
+    const Operands op = {x3 + (size_t)slab * n * d, (size_t)slabs * n * d, W, n, d, m};
     bool ok = true;
     for (int t = g; t < nt && ok; t += 2) {
       ok = __all_sync(0xffffffffu, mbar_wait(&bars->d1_full[g], (t >> 1) & 1, abort_flag, status, kErrXElem));
       if (!ok) break;
       tc_fence_after_sync();
-      const float sum = relu_planes<true>(taddr, zs);
+      const float sum = relu_planes<false, true>(taddr, op, (t0 + t) * kTile + row, f0, zs);
       if (t >= 2) {   // the drain has read the denominators of tile t - 2
         ok = __all_sync(0xffffffffu, mbar_wait(&bars->den_free[g], ((t >> 1) - 1) & 1, abort_flag, status, kErrXElem));
         if (!ok) break;
@@ -562,7 +622,7 @@ k_tcx_bwd_prep(const float* __restrict__ dO, const float* __restrict__ O, const 
 #pragma unroll
       for (int j = 0; j < 8; ++j) dot = fmaf(g[j], o[j], dot);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) split3(g[2 * j], g[2 * j + 1], pl[0][j], pl[1][j], pl[2][j]);
+      for (int j = 0; j < 4; ++j) split3<true>(g[2 * j], g[2 * j + 1], pl[0][j], pl[1][j], pl[2][j]);
 #pragma unroll
       for (int s = 0; s < 3; ++s)
         *reinterpret_cast<uint4*>(dO3 + s * plane + tok * d + c0) = make_uint4(pl[s][0], pl[s][1], pl[s][2], pl[s][3]);
@@ -630,7 +690,7 @@ __global__ void __launch_bounds__(kXThreads, 1)
 k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y, const float* __restrict__ W,
           const float* __restrict__ S, const float* __restrict__ zg, const float* __restrict__ tok_inv,
           const float* __restrict__ tok_c, const __grid_constant__ CUtensorMap map_dx, const __grid_constant__ CUtensorMap map_dv,
-          int add, int n, int d, int m, int f0, int chunk_tiles, int* __restrict__ status) {
+          int add, int n, int d, int m, int f0, int chunk_tiles, int* __restrict__ status, const __nv_bfloat16* x3) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
   using SL = YSmem;
@@ -723,6 +783,7 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
     const int g = (warp - 4) >> 2;                        // features 64 g .. 64 g + 63
     const uint32_t row = 32u * (warp & 3) + lane;         // token of the tile = TMEM lane
     const uint32_t lanes = tmem + ((32u * (warp & 3)) << 16);
+    const Operands op = {x3 + (size_t)slab * n * d, (size_t)slabs * n * d, W, n, d, m};
     bool ok = true;
     for (int t = 0; t < nt && ok; ++t) {
       float inv = 0.f, c = 0.f;
@@ -740,9 +801,7 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
       uint32_t r[32];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        tmem_ld32(lanes + 64 * g + 32 * h, r);
-        tmem_ld_wait();
-        reg_fence32(r);
+        load_projected(lanes + 64 * g + 32 * h, r, op, (t0 + t) * kTile + row, 0, f0 + 64 * g + 32 * h, 1);
         on[h] = 0;
         float v[32];
 #pragma unroll
@@ -832,8 +891,8 @@ cudaError_t launch_summary(const Plan& p, const Ws& w, const __nv_bfloat16* x3, 
   if ((err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, KxSmem::total)) != cudaSuccess) return err;
   *launches += 1;
   return launch_after(kernel, dim3(p.xchunks, p.slabs, p.cfg.features / kXFeatures), dim3(kXThreads), KxSmem::total, st, map_x, map_y,
-                      (const float*)W, w.spart, w.zpart, p.cfg.seq_len, p.cfg.head_dim, p.cfg.features, p.xchunk_tiles, w.status, scale,
-                      weight);
+                      (const float*)W, w.spart, w.zpart, p.cfg.seq_len, p.cfg.head_dim, p.cfg.features, p.xchunk_tiles, w.status,
+                      x3, scale, weight);
 }
 
 template <bool kKeys>
@@ -852,7 +911,7 @@ cudaError_t launch_bwd(const Plan& p, const Ws& w, const __nv_bfloat16* x3, cons
     *launches += 1;
     err = launch_after(kernel, dim3(p.xbchunks, p.slabs), dim3(kXThreads), YSmem::total, st, map_x, map_y, (const float*)W, S, z,
                        (const float*)w.xinv, (const float*)w.xc, map_dx, map_dv, f0 > 0 ? 1 : 0, n, d, p.cfg.features, f0,
-                       p.xbchunk_tiles, w.status);
+                       p.xbchunk_tiles, w.status, x3);
     if (err != cudaSuccess) return err;
   }
   return cudaSuccess;
@@ -881,7 +940,8 @@ cudaError_t launch_tcx_qside(const Plan& p, const Ws& w, const void* W, const fl
   *launches += 1;
   err = launch_after(k_tcx_qside, dim3(p.xchunks, p.slabs, groups), dim3(kXThreads), QxSmem::total, st, map_q, map_o, (const float*)W,
                      (const float*)w.S, (const float*)w.z, beta, p.cfg.eps, p.cfg.bw_floor, den, map_keep,
-                     keep != nullptr && groups == 1 ? 1 : 0, n, d, p.cfg.features, p.xchunk_tiles, w.status);
+                     keep != nullptr && groups == 1 ? 1 : 0, n, d, p.cfg.features, p.xchunk_tiles, w.status,
+                     (const __nv_bfloat16*)w.QF3);
   if (err != cudaSuccess || groups == 1) return err;
   *launches += 1;
   return launch_after(k_tcx_combine, dim3((unsigned)((tokens * (d >> 2) + 255) / 256)), dim3(256), 0, st, (const float*)share,
