@@ -577,7 +577,7 @@ wersa_status wersa_shard_keys(wersa_ctx* ctx, const void* K, const void* V, void
   DeviceGuard guard(p.cfg.device);
   if (guard.err != cudaSuccess) return WERSA_ERR_CUDA;
   int launches = 0;
-  WERSA_CUDA(launch_tc_kside(p, w, K, V, st, &launches));
+  WERSA_CUDA(launch_tc_kside(p, w, K, V, st, &launches, true));
   if (p.tchunks > 1)
     WERSA_CUDA(launch_reduce_partials(p, w.spart, w.zpart, p.tchunks, w.S, w.z, p.with_backward ? w.Sbf : nullptr, w.Simg, st, &launches));
   ctx->launches_fwd += launches;
@@ -598,7 +598,7 @@ wersa_status wersa_shard_output(wersa_ctx* ctx, const void* Q, const float* S_to
   if (guard.err != cudaSuccess) return WERSA_ERR_CUDA;
   int launches = 0;
   // the totals take the place of a single partial: the reduction copies them and writes the operand images
-  WERSA_CUDA(launch_reduce_partials(p, S_total, z_total, 1, w.S, w.z, p.with_backward ? w.Sbf : nullptr, w.Simg, st, &launches));
+  WERSA_CUDA(launch_reduce_partials(p, S_total, z_total, 1, w.S, w.z, p.with_backward ? w.Sbf : nullptr, w.Simg, st, &launches, true));
   WERSA_CUDA(launch_tc_qside(p, w, Q, beta, O, nullptr, st, &launches));
   ctx->launches_fwd += launches;
   return WERSA_OK;

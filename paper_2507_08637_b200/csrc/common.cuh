@@ -129,10 +129,11 @@ cudaError_t launch_haar_backward(const Plan& p, const Ws& w, int which, const vo
 // ---- simt.cu -------------------------------------------------------------------------------
 cudaError_t launch_simt_kside(const Plan& p, const Ws& w, const void* V, const void* W,
                               cudaStream_t st, int* launches);
-// S = sum_chunks spart, z = sum_chunks zpart in chunk order (also used for dS, dz).
+// S = sum_chunks spart, z = sum_chunks zpart in chunk order (also used for dS, dz).  first: the first kernel of its pass, and
+// the next one fetches arguments ahead of its wait (see launch_behind).
 cudaError_t launch_reduce_partials(const Plan& p, const float* spart, const float* zpart, int chunks,
                                    float* S, float* z, __nv_bfloat16* Sbf, uint8_t* Simg, cudaStream_t st,
-                                   int* launches);
+                                   int* launches, bool first = false);
 // The same for the segments the tensor-core backward leaves (slot CTA + slab for every CTA that has tiles of the
 // slab): dS, dz and the bf16 image of dS.
 cudaError_t launch_reduce_segments(const Plan& p, const Ws& w, cudaStream_t st, int* launches);
@@ -155,9 +156,10 @@ cudaError_t launch_tcx_bwd_qside(const Plan& p, const Ws& w, const void* W, cuda
 cudaError_t launch_tcx_bwd_kside(const Plan& p, const Ws& w, const void* W, void* dV, cudaStream_t st, int* launches);
 
 // ---- tc_fwd.cu -----------------------------------------------------------------------------
-// Both read the raw bf16 tensors and apply the Haar filter (coefficients from w.f) on chip.
-cudaError_t launch_tc_kside(const Plan& p, const Ws& w, const void* K, const void* V, cudaStream_t st,
-                            int* launches);
+// Both read the raw bf16 tensors and apply the Haar filter (coefficients from w.f) on chip.  first: the first kernel of its
+// pass (see launch_behind).
+cudaError_t launch_tc_kside(const Plan& p, const Ws& w, const void* K, const void* V, cudaStream_t st, int* launches,
+                            bool first = false);
 // den != nullptr (features == 256 only): also leaves every token's denominator in den[slab * n + token].
 cudaError_t launch_tc_qside(const Plan& p, const Ws& w, const void* Q, const float* beta, void* O, float* den,
                             cudaStream_t st, int* launches);
@@ -240,15 +242,21 @@ __device__ __forceinline__ float sum2(f32x2 v) {
 
 // Launch as a programmatic dependent of the work before it in the stream.  Ordering and visibility are those of a plain
 // launch, since the kernel writes nothing and reads nothing of that work before wait_for_stream_predecessor(); only the
-// placement of its CTAs, and what they set up or fetch ahead of the wait, overlaps the end of that work.  What may be
-// fetched ahead: what was complete before the kernel in front of this one in its pass passed its own wait (the arguments
-// of the call and the results of earlier kernels), hence nothing in the first kernel of a pass.  Where work stands ahead of
-// the wait, results of the kernel in front are read with load_after_wait (or __ldcg where the L1 has no use for them), not
-// through a const __restrict__ pointer: such a load counts as free of order with anything, and the compiler did move the row
-// vector of dQ above the wait.
+// placement of its CTAs, and what they set up or fetch ahead of the wait, overlaps the end of that work.
+// What may be fetched ahead of the wait: what a kernel wrote behind which, and in front of this one, there is a kernel of the
+// same pass that lets its successor start only after its own wait, or at its end (call it closed).  Not every kernel is:
+// k_reduce_partials, k_band_reduce and k_gate_backward (unless first) let the next one start at once, and that one then runs
+// beside the kernel in front of THEM.  So the arguments of a call may be fetched ahead behind the first closed kernel of the
+// pass (k_qmean_gate in the forward, whatever comes first in a backward; dQ_F by the last pass of a backward: k_haar_backward is
+// closed), and the first kernel of a pass fetches nothing: what stands in front of it may be the end of another pass, such
+// as a gate backward beside a k_haar_backward that still writes dQ.  Kernels that fetch arguments ahead and may be the first
+// of a pass, or stand behind a first one that is not closed, are told: overlap = false is a plain launch.
+// Where work stands ahead of the wait, results of the kernel in front are read with load_after_wait (or __ldcg where the L1
+// has no use for them), not through a const __restrict__ pointer: such a load counts as free of order with anything, and the
+// compiler did move the row vector of dQ above the wait.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                                Args&&... args) {
+inline cudaError_t launch_behind(bool overlap, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                 Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -256,10 +264,14 @@ inline cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block,
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  return launch_behind(true, kernel, grid, block, smem, st, args...);
 }
 __device__ __forceinline__ void wait_for_stream_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ float load_after_wait(const float* p) {

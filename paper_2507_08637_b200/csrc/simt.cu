@@ -843,7 +843,8 @@ cudaError_t launch_simt_kside(const Plan& p, const Ws& w, const void* V, const v
 }
 
 static cudaError_t launch_reduce(const Plan& p, int groups, const float* spart, const float* zpart, int chunks, int tps, int ctas,
-                                 float* S, float* z, __nv_bfloat16* Sbf, uint8_t* Simg, cudaStream_t st, int* launches) {
+                                 float* S, float* z, __nv_bfloat16* Sbf, uint8_t* Simg, cudaStream_t st, int* launches,
+                                 bool first = false) {
   const int m = p.cfg.features;
   const dim3 grid(m / 8, p.slabs, groups);
   // (four CTAs per SM: see k_reduce_partials; a sequence shard's caller may hand in sums that lie at any float, such as a
@@ -851,7 +852,7 @@ static cudaError_t launch_reduce(const Plan& p, int groups, const float* spart, 
   const bool aligned = (reinterpret_cast<uintptr_t>(spart) & 15u) == 0;
   const unsigned ctas8 = grid.x * grid.y * grid.z;
   auto go = [&](auto kernel, dim3 g, int threads) {
-    return launch_after(kernel, g, dim3(threads), 0, st, spart, zpart, chunks, tps, ctas, m, S, z, Sbf, Simg);
+    return launch_behind(!first, kernel, g, dim3(threads), 0, st, spart, zpart, chunks, tps, ctas, m, S, z, Sbf, Simg);
   };
   const cudaError_t err = !aligned || ctas8 <= 4u * p.sms ? go(k_reduce_partials<1, 1>, grid, 544)
                           : ctas8 <= 16u * p.sms          ? go(k_reduce_partials<4, 1>, grid, 160)
@@ -860,8 +861,8 @@ static cudaError_t launch_reduce(const Plan& p, int groups, const float* spart, 
   return err != cudaSuccess ? err : cudaGetLastError();
 }
 cudaError_t launch_reduce_partials(const Plan& p, const float* spart, const float* zpart, int chunks, float* S,
-                                   float* z, __nv_bfloat16* Sbf, uint8_t* Simg, cudaStream_t st, int* launches) {
-  return launch_reduce(p, p.groups, spart, zpart, chunks, 0, 0, S, z, Sbf, Simg, st, launches);
+                                   float* z, __nv_bfloat16* Sbf, uint8_t* Simg, cudaStream_t st, int* launches, bool first) {
+  return launch_reduce(p, p.groups, spart, zpart, chunks, 0, 0, S, z, Sbf, Simg, st, launches, first);
 }
 cudaError_t launch_reduce_segments(const Plan& p, const Ws& w, cudaStream_t st, int* launches) {
   return launch_reduce(p, 1, w.spart, w.zpart, 0, (p.cfg.seq_len + 127) / 128, p.bctas, w.dS, w.dz, w.dSbf, nullptr, st, launches);

@@ -526,7 +526,7 @@ k_tc_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CU
     bars->abort_flag = 0;
     fence_mbar_init();
     // K and V are inputs: the first copies of both rings (tiles of the first item) go out before the
-    // dependency wait below.  K, V and the output are touched once per forward: their copies carry the
+    // dependency wait below (behind another pass the launch is a plain one: see launch_behind).  K, V and the output are touched once per forward: their copies carry the
     // evict-first L2 policy (measured: 1-5 us per forward over the default policy; the same hint on the
     // query side's Q tiles cost 4 us and is not used).
     const int slab = item0 / chunks, row0 = (item0 % chunks) * chunk_blocks * kBlk;
@@ -1152,26 +1152,15 @@ bool tc_supported(const wersa_config& cfg) {
   else if (p.cfg.head_dim > 16) { constexpr int CW = 4; __VA_ARGS__ }          \
   else { constexpr int CW = 2; __VA_ARGS__ }
 
-// Both tensor-core kernels are launched as programmatic dependents of the kernel before them.
+// Both kernels are launched as programmatic dependents of the kernel before them, unless that would be another pass's.
 template <typename... Args>
-static cudaError_t launch_pdl(void (*k)(Args...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
-  cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, args...);
+static cudaError_t launch_pdl(bool overlap, void (*k)(Args...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+  const cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return err != cudaSuccess ? err : launch_behind(overlap, k, grid, dim3(threads), smem, st, args...);
 }
 
-cudaError_t launch_tc_kside(const Plan& p, const Ws& w, const void* K, const void* V, cudaStream_t st,
-                            int* launches) {
+cudaError_t launch_tc_kside(const Plan& p, const Ws& w, const void* K, const void* V, cudaStream_t st, int* launches,
+                            bool first) {
   CUtensorMap map_k, map_v;
   cudaError_t err;
   if ((err = make_tile_map(K, p.slabs, p.cfg.seq_len, &map_k, p.cfg.head_dim)) != cudaSuccess) return err;
@@ -1192,7 +1181,7 @@ cudaError_t launch_tc_kside(const Plan& p, const Ws& w, const void* K, const voi
   const bool multi = p.groups == 1 && items > (int)grid.x;
   if (!multi) grid = dim3(items, 1, p.groups);
   auto launch = [&](auto kernel, size_t smem_bytes) {
-    return launch_pdl(kernel, grid, kThreads, smem_bytes, st, map_k, map_v, map_w, (const float*)w.f, sp, zp, sb, si,
+    return launch_pdl(!first, kernel, grid, kThreads, smem_bytes, st, map_k, map_v, map_w, (const float*)w.f, sp, zp, sb, si,
                       p.cfg.seq_len, p.cfg.head_dim, p.cfg.levels, p.tchunk_blocks, p.tchunks, items, w.status);
   };
   WERSA_HEAD_CHUNKS({
@@ -1221,7 +1210,7 @@ cudaError_t launch_tc_qside(const Plan& p, const Ws& w, const void* Q, const flo
   const bool multi = p.groups == 1 && items > (int)grid.x;
   if (!multi) grid = dim3(items, 1, p.groups);   // see launch_tc_kside
   auto launch = [&](auto kernel, size_t smem_bytes) {
-    return launch_pdl(kernel, grid, kThreadsQ, smem_bytes, st, map_q, map_o, map_w, (const uint8_t*)w.Simg,
+    return launch_pdl(true, kernel, grid, kThreadsQ, smem_bytes, st, map_q, map_o, map_w, (const uint8_t*)w.Simg,
                       (const float*)w.f, beta, p.cfg.eps, p.cfg.bw_floor, p.cfg.seq_len, p.cfg.head_dim, p.cfg.levels,
                       p.tqchunk_blocks, p.tqchunks, items, w.status, den);
   };
