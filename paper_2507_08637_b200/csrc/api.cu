@@ -298,6 +298,7 @@ Ws resolve(const Plan& p, void* workspace) {
   char* b = static_cast<char*>(workspace);
   Ws w;
   w.status = reinterpret_cast<int*>(b + p.off_status);
+  w.seen = w.status + 16;   // (the status word has 256 bytes to itself)
   w.counters = reinterpret_cast<int*>(b + p.off_counters);
   w.qpart = reinterpret_cast<float*>(b + p.off_qpart);
   w.qbar = reinterpret_cast<float*>(b + p.off_qbar);

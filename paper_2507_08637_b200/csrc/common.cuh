@@ -54,6 +54,7 @@ wersa_status make_plan(const wersa_config& cfg, Plan* p);
 
 struct Ws {   // resolved workspace pointers
   int* status;
+  int* seen;       // fp32 on the tensor cores: not 0 where T_f(Q) [0], T_f(K) [1] hold a value that is not finite
   int* counters;   // arrival counters (slabs + batch + slabs ints), zero between launches
   float *qpart, *qbar, *sg, *f, *spart, *zpart, *S, *z, *dS, *dz, *sumdD, *bands, *dqbar;
   float *xO, *xden, *xinv, *xc, *xshare;   // fp32 on the tensor cores: O and D'_g for the backward, 1 / D and -dO.O per token, shares of N'

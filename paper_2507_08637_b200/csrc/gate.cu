@@ -118,13 +118,14 @@ __global__ void __launch_bounds__(256) k_qmean_gate(const T* __restrict__ Q, flo
                                                     float* __restrict__ sg, float* __restrict__ f,
                                                     int* __restrict__ slab_count, int* __restrict__ batch_count,
                                                     const __nv_bfloat16* __restrict__ W, __nv_bfloat16* __restrict__ Wt,
-                                                    int m, int dcols_arg) {
+                                                    int m, int dcols_arg, int* __restrict__ seen) {
   const int dcols = kFull ? kD : dcols_arg;
   // This grid may have been placed while the work before it in the stream was still running: nothing is
   // read or written before that work has completed.  After that the key-side kernel may be staged
   // (programmatic dependent launch; it waits for this grid before it reads W^T or the gate).
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (seen != nullptr && blockIdx.x + blockIdx.y == 0 && threadIdx.x < 2) seen[threadIdx.x] = 0;   // (see k_f32_planes)
   if ((int)blockIdx.y == slabs) {
     // A thread takes eight columns of W^T's row r: neighbouring threads read neighbouring features and store 16 bytes.  (An
     // element a thread reads 2 bytes out of 32 different sectors a warp, and the grid's other CTAs wait for nothing else:
@@ -439,7 +440,7 @@ __global__ void __launch_bounds__(64 * kParts) k_gate_backward(
 static cudaError_t launch_qmean_gate_impl(const Plan& p, const void* Q, float* qpart, const float* gate_w,
                                           const float* gate_b, const float* omega, float* qbar, float* sg, float* f,
                                           int* counters, const void* W, __nv_bfloat16* Wt, int cols,
-                                          cudaStream_t st) {
+                                          int* seen, cudaStream_t st) {
   dim3 grid(p.qchunks, p.slabs + (W != nullptr ? 1 : 0));
   int* slab_count = counters;
   int* batch_count = counters + p.slabs;
@@ -459,7 +460,7 @@ static cudaError_t launch_qmean_gate_impl(const Plan& p, const void* Q, float* q
     lc.numAttrs = 1;
     launch_err = cudaLaunchKernelEx(&lc, kernel, q, qpart, p.cfg.seq_len, p.qchunk_rows, p.slabs, p.cfg.heads, p.L1,
                                     p.cfg.gate_per_head, gate_w, gate_b, omega, qbar, sg, f, slab_count, batch_count,
-                                    (const __nv_bfloat16*)W, Wt, p.cfg.features, cols);
+                                    (const __nv_bfloat16*)W, Wt, p.cfg.features, cols, seen);
   };
   if (p.bf16) {
     if (cols == kD) launch(k_qmean_gate<__nv_bfloat16, true>, (const __nv_bfloat16*)Q);
@@ -475,7 +476,8 @@ cudaError_t launch_qmean_gate(const Plan& p, const Ws& w, const void* Q, const f
                               const float* gate_b, const float* omega, const void* W, int cols, cudaStream_t st,
                               int* launches) {
   *launches += 1;
-  return launch_qmean_gate_impl(p, Q, w.qpart, gate_w, gate_b, omega, w.qbar, w.sg, w.f, w.counters, W, w.Wt, cols, st);
+  return launch_qmean_gate_impl(p, Q, w.qpart, gate_w, gate_b, omega, w.qbar, w.sg, w.f, w.counters, W, w.Wt, cols,
+                                p.use_x ? w.seen : nullptr, st);
 }
 
 cudaError_t launch_shard_qsum(const Plan& p, const Ws& w, float* qsum, cudaStream_t st, int* launches) {
@@ -528,7 +530,7 @@ cudaError_t launch_qmean_gate_static(const Plan& p, float* scratch, const void* 
   int* counters = reinterpret_cast<int*>(scratch + (kStaticScratchFloats - kStaticCounterInts));
   cudaError_t err = cudaMemsetAsync(counters, 0, sizeof(int) * ((size_t)p.slabs + (size_t)p.cfg.batch), st);
   if (err != cudaSuccess) return err;
-  return launch_qmean_gate_impl(p, Q, qpart, gate_w, gate_b, omega, qbar, sg, f, counters, nullptr, nullptr, kD, st);
+  return launch_qmean_gate_impl(p, Q, qpart, gate_w, gate_b, omega, qbar, sg, f, counters, nullptr, nullptr, kD, nullptr, st);
 }
 
 size_t static_scratch_floats_needed(const Plan& p) {

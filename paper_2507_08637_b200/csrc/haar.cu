@@ -214,7 +214,8 @@ __global__ void __launch_bounds__(256, 3) k_f32_planes(const float* __restrict__
                                                        const float* __restrict__ V, const float* __restrict__ f,
                                                        __nv_bfloat16* __restrict__ Q3, __nv_bfloat16* __restrict__ K3,
                                                        __nv_bfloat16* __restrict__ V3, float* __restrict__ QF,
-                                                       float* __restrict__ KF, size_t plane, int n, int d_arg, int L) {
+                                                       float* __restrict__ KF, size_t plane, int n, int d_arg, int L,
+                                                       int* __restrict__ seen) {
   const int d = kFull ? kD : d_arg;
   __shared__ __align__(16) float ex[8][kHalfD];   // 32-row sums of the warps
   const int slab = blockIdx.y, warp = threadIdx.x >> 5, cg = threadIdx.x & 7, rg = threadIdx.x >> 3;
@@ -267,6 +268,7 @@ __global__ void __launch_bounds__(256, 3) k_f32_planes(const float* __restrict__
   }
   __nv_bfloat16* dst = (blockIdx.z == 0 ? Q3 : blockIdx.z == 1 ? K3 : V3) + first;
   float* keep = blockIdx.z == 0 ? QF : KF;
+  uint32_t top = 0;   // bits 15 and 31: an exponent of all ones in a first plane
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     if (j >= rows) break;
@@ -279,12 +281,14 @@ __global__ void __launch_bounds__(256, 3) k_f32_planes(const float* __restrict__
       const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
       const uint2 w = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
       *reinterpret_cast<uint2*>(dst + (size_t)pl * plane + (size_t)j * d) = w;
+      if (pl == 0) top |= ((w.x & 0x7F807F80u) + 0x00800080u) | ((w.y & 0x7F807F80u) + 0x00800080u);
       x[j][0] -= __uint_as_float(w.x << 16);
       x[j][1] -= __uint_as_float(w.x & 0xFFFF0000u);
       x[j][2] -= __uint_as_float(w.y << 16);
       x[j][3] -= __uint_as_float(w.y & 0xFFFF0000u);
     }
   }
+  if (filtered && (top & 0x80008000u) != 0) seen[blockIdx.z] = 1;   // (who multiplies by W wants to know: see Operands)
 }
 
 // The same pass for bf16 input: a thread keeps its 8 rows x 8 columns as the 32 packed words it loaded
@@ -688,7 +692,7 @@ cudaError_t launch_f32_planes(const Plan& p, const Ws& w, const float* Q, const 
   const size_t plane = (size_t)p.slabs * n * d;
   cudaError_t err;
   auto go = [&](auto kernel) {
-    return launch_after(kernel, grid, dim3(256), 0, st, Q, K, V, (const float*)w.f, w.QF3, w.KF3, w.V3, w.QF, w.KF, plane, n, d, L);
+    return launch_after(kernel, grid, dim3(256), 0, st, Q, K, V, (const float*)w.f, w.QF3, w.KF3, w.V3, w.QF, w.KF, plane, n, d, L, w.seen);
   };
   WERSA_FULL({ err = keep ? go(k_f32_planes<kFull, true>) : go(k_f32_planes<kFull, false>); })
   *launches += 1;

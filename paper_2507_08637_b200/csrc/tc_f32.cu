@@ -104,9 +104,11 @@ __device__ __forceinline__ void put_planes8(uint8_t* tile, int row, int chunk, c
   for (int s = 0; s < 3; ++s)
     *reinterpret_cast<uint4*>(tile + s * kTileBytes + swz128(row, chunk)) = make_uint4(p[s][0], p[s][1], p[s][2], p[s][3]);
 }
-// W (d x m, row-major) -> planes of rows f0 .. f0 + 127 of W^T, zero past column d.  512 threads.
-__device__ __forceinline__ void load_w_planes(const float* __restrict__ W, int d, int m, int f0, uint8_t* wt) {
+// W (d x m, row-major) -> planes of rows f0 .. f0 + 127 of W^T, zero past column d.  512 threads.  Is one of this thread's
+// values not finite?
+__device__ __forceinline__ bool load_w_planes(const float* __restrict__ W, int d, int m, int f0, uint8_t* wt) {
   const int f = threadIdx.x & 127, part = threadIdx.x >> 7;   // 16 columns
+  bool bad = false;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     float v[8];
@@ -114,9 +116,11 @@ __device__ __forceinline__ void load_w_planes(const float* __restrict__ W, int d
     for (int j = 0; j < 8; ++j) {
       const int c = 16 * part + 8 * h + j;
       v[j] = c < d ? W[(size_t)c * m + f0 + f] : 0.f;
+      bad |= !(fabsf(v[j]) < INFINITY);
     }
     put_planes8(wt, f, 2 * part + h, v);
   }
+  return bad;
 }
 // S' or dS' of a slab's features f0 .. f0 + 127 (64 columns) -> planes, and the group's z' or dz' -> zs: results of the kernel
 // in front (see launch_after).  512 threads.
@@ -134,12 +138,14 @@ __device__ __forceinline__ void load_s_planes(const float* S, const float* zg, s
 
 // The planes of an infinite value are infinity, NaN and NaN: what the tensor cores make of a dot product that meets one is NaN,
 // and a ReLU would drop it.  In 32 bits it is infinite, or NaN where infinities cancel: such elements are formed again, from
-// the planes' sums and W.  (Only their class matters: a NaN came from an operand that is not finite.)
+// the planes' sums and W.  (Only their class matters: a NaN came from an operand that is not finite.)  The kernels look for
+// them where W holds one (which they see as they read it) or the projected tensor does (k_f32_planes leaves word); looking
+// every time cost 1 us in each of the kernels of 2 x 4 x 4096, d = 32, m = 128 (a training step 107 -> 110).
 struct Operands {
-  const __nv_bfloat16* x3;   // first plane of the slab: n rows of d values
-  size_t plane;              // values of a plane
+  const __nv_bfloat16* x3;   // first plane: slabs x n rows of d values
   const float* W;            // d x m
-  int n, d, m;
+  int slab, slabs, n, d, m;
+  bool look;                 // is there anything that is not finite?
 };
 // Are there NaN among 32 columns of the warp?  (False alarms, such as opposite infinities, cost time only.)
 __device__ __forceinline__ bool warp_meets_nan(const uint32_t (&r)[32]) {
@@ -153,17 +159,18 @@ __device__ __forceinline__ bool warp_meets_nan(const uint32_t (&r)[32]) {
 }
 // The NaN among the 32 columns at taddr again.  Column j of a lane is token tok + j * dtok, feature feat + j * dfeat.
 __device__ __noinline__ void form_again(uint32_t taddr, const Operands op, int tok, int dtok, int feat, int dfeat) {
+  const size_t plane = (size_t)op.slabs * op.n * op.d;
   for (int j = 0; j < 32; ++j, tok += dtok, feat += dfeat) {
     uint32_t r;
     tmem_ld1(taddr + j, r);
     tmem_ld_wait();
     float a = __uint_as_float(r);
     if (a != a && tok < op.n) {   // (rows past n are zeros: NaN against an infinite W, and no feature either way)
-      const __nv_bfloat16* x = op.x3 + (size_t)tok * op.d;
+      const __nv_bfloat16* x = op.x3 + ((size_t)op.slab * op.n + tok) * op.d;
       a = 0.f;
       for (int c = 0; c < op.d && a == a; ++c) {
         float v = __bfloat162float(__ldcg(x + c));
-        if (fabsf(v) < INFINITY) v = (v + __bfloat162float(__ldcg(x + op.plane + c))) + __bfloat162float(__ldcg(x + 2 * op.plane + c));
+        if (fabsf(v) < INFINITY) v = (v + __bfloat162float(__ldcg(x + plane + c))) + __bfloat162float(__ldcg(x + 2 * plane + c));
         a = fmaf(v, op.W[(size_t)c * op.m + feat], a);
       }
       r = __float_as_uint(a);
@@ -179,7 +186,7 @@ __device__ __forceinline__ void load_projected(uint32_t taddr, uint32_t (&r)[32]
   tmem_ld32(taddr, r);
   tmem_ld_wait();
   reg_fence32(r);
-  if (warp_meets_nan(r)) {
+  if (op.look && warp_meets_nan(r)) {
     form_again(taddr, op, tok, dtok, feat, dfeat);
     tmem_ld32(taddr, r);
     tmem_ld_wait();
@@ -340,7 +347,7 @@ template <bool kScaled>
 __global__ void __launch_bounds__(kXThreads, 1)
 k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const float* __restrict__ W,
             float* __restrict__ spart, float* __restrict__ zpart, int n, int d, int m, int chunk_tiles, int* __restrict__ status,
-            const __nv_bfloat16* x3, const float* __restrict__ scale, const float* __restrict__ weight) {
+            const __nv_bfloat16* x3, const int* seen, const float* __restrict__ scale, const float* __restrict__ weight) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
   using SL = KxSmem;
@@ -353,10 +360,10 @@ k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ C
     tmem_alloc(&bars->tmem_base, 512);
     tmem_relinquish();
   }
-  load_w_planes(W, d, m, f0, smem + SL::wt);
+  const bool bad_w = load_w_planes(W, d, m, f0, smem + SL::wt);
   fence_proxy_async_smem();
   tc_fence_before_sync();
-  __syncthreads();
+  const bool look_w = __syncthreads_or(bad_w);
   tc_fence_after_sync();
   wait_for_stream_predecessor();   // (launched as a programmatic dependent: the planes come from the kernel before)
   let_stream_successor_start();
@@ -402,7 +409,7 @@ k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ C
     const uint32_t row = 32u * (warp & 3) + lane;   // feature of the group = TMEM lane
     const uint32_t taddr = tmem + ((32u * (warp & 3)) << 16) + g * kBufCols;
     float* zx = reinterpret_cast<float*>(smem + SL::zx);
-    const Operands op = {x3 + (size_t)slab * n * d, (size_t)slabs * n * d, W, n, d, m};
+    const Operands op = {x3, W, slab, slabs, n, d, m, look_w || __ldcg(seen) != 0};
     float z = 0.f;
     bool ok = true;
     for (int t = g; t < nt && ok; t += 2) {
@@ -460,7 +467,8 @@ __global__ void __launch_bounds__(kXThreads, 1)
 k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o, const float* __restrict__ W,
             const float* __restrict__ S, const float* __restrict__ zg, const float* __restrict__ beta, float eps, float bw_floor,
             float* __restrict__ den_out, const __grid_constant__ CUtensorMap map_keep, int keep, int n, int d, int m, int chunk_tiles,
-            int* __restrict__ status, const __nv_bfloat16* x3) {
+            int* __restrict__ status, const __nv_bfloat16* x3,
+            const int* seen) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
   using SL = QxSmem;
@@ -480,12 +488,12 @@ k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     tmem_alloc(&bars->tmem_base, 512);
     tmem_relinquish();
   }
-  load_w_planes(W, d, m, f0, smem + SL::wt);
+  const bool bad_w = load_w_planes(W, d, m, f0, smem + SL::wt);
   wait_for_stream_predecessor();
   load_s_planes(S, zg, (size_t)slab * m + f0, smem + SL::s, zs);
   fence_proxy_async_smem();
   tc_fence_before_sync();
-  __syncthreads();
+  const bool look_w = __syncthreads_or(bad_w);
   tc_fence_after_sync();
   const uint32_t tmem = bars->tmem_base;
   volatile int* abort_flag = &bars->abort_flag;
@@ -512,7 +520,7 @@ k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     const int g = (warp - 4) >> 2;
     const uint32_t row = 32u * (warp & 3) + lane;   // token of the tile = TMEM lane
     const uint32_t taddr = tmem + ((32u * (warp & 3)) << 16) + g * kBufCols;
-    const Operands op = {x3 + (size_t)slab * n * d, (size_t)slabs * n * d, W, n, d, m};
+    const Operands op = {x3, W, slab, slabs, n, d, m, look_w || __ldcg(seen) != 0};
     bool ok = true;
     for (int t = g; t < nt && ok; t += 2) {
       ok = __all_sync(0xffffffffu, mbar_wait(&bars->d1_full[g], (t >> 1) & 1, abort_flag, status, kErrXElem));
@@ -690,7 +698,8 @@ __global__ void __launch_bounds__(kXThreads, 1)
 k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y, const float* __restrict__ W,
           const float* __restrict__ S, const float* __restrict__ zg, const float* __restrict__ tok_inv,
           const float* __restrict__ tok_c, const __grid_constant__ CUtensorMap map_dx, const __grid_constant__ CUtensorMap map_dv,
-          int add, int n, int d, int m, int f0, int chunk_tiles, int* __restrict__ status, const __nv_bfloat16* x3) {
+          int add, int n, int d, int m, int f0, int chunk_tiles, int* __restrict__ status, const __nv_bfloat16* x3,
+            const int* seen) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
   using SL = YSmem;
@@ -723,14 +732,14 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
     tmem_alloc(&bars->tmem_base, 512);
     tmem_relinquish();
   }
-  load_w_planes(W, d, m, f0, smem + SL::wt);
+  const bool bad_w = load_w_planes(W, d, m, f0, smem + SL::wt);
   wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   // (behind the key side come kernels that start with reads of what it writes and that lost time placed early)
   if constexpr (!kKeys) let_stream_successor_start();
   load_s_planes(S, zg, (size_t)slab * m + f0, smem + SL::s, zs);
   fence_proxy_async_smem();
   tc_fence_before_sync();
-  __syncthreads();
+  const bool look_w = __syncthreads_or(bad_w);
   tc_fence_after_sync();
   const uint32_t tmem = bars->tmem_base;
   volatile int* abort_flag = &bars->abort_flag;
@@ -783,7 +792,7 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
     const int g = (warp - 4) >> 2;                        // features 64 g .. 64 g + 63
     const uint32_t row = 32u * (warp & 3) + lane;         // token of the tile = TMEM lane
     const uint32_t lanes = tmem + ((32u * (warp & 3)) << 16);
-    const Operands op = {x3 + (size_t)slab * n * d, (size_t)slabs * n * d, W, n, d, m};
+    const Operands op = {x3, W, slab, slabs, n, d, m, look_w || __ldcg(seen) != 0};
     bool ok = true;
     for (int t = 0; t < nt && ok; ++t) {
       float inv = 0.f, c = 0.f;
@@ -892,7 +901,7 @@ cudaError_t launch_summary(const Plan& p, const Ws& w, const __nv_bfloat16* x3, 
   *launches += 1;
   return launch_after(kernel, dim3(p.xchunks, p.slabs, p.cfg.features / kXFeatures), dim3(kXThreads), KxSmem::total, st, map_x, map_y,
                       (const float*)W, w.spart, w.zpart, p.cfg.seq_len, p.cfg.head_dim, p.cfg.features, p.xchunk_tiles, w.status,
-                      x3, scale, weight);
+                      x3, (const int*)(x3 == w.KF3 ? w.seen + 1 : w.seen), scale, weight);
 }
 
 template <bool kKeys>
@@ -911,7 +920,7 @@ cudaError_t launch_bwd(const Plan& p, const Ws& w, const __nv_bfloat16* x3, cons
     *launches += 1;
     err = launch_after(kernel, dim3(p.xbchunks, p.slabs), dim3(kXThreads), YSmem::total, st, map_x, map_y, (const float*)W, S, z,
                        (const float*)w.xinv, (const float*)w.xc, map_dx, map_dv, f0 > 0 ? 1 : 0, n, d, p.cfg.features, f0,
-                       p.xbchunk_tiles, w.status, x3);
+                       p.xbchunk_tiles, w.status, x3, (const int*)(kKeys ? w.seen + 1 : w.seen));
     if (err != cudaSuccess) return err;
   }
   return cudaSuccess;
@@ -941,7 +950,7 @@ cudaError_t launch_tcx_qside(const Plan& p, const Ws& w, const void* W, const fl
   err = launch_after(k_tcx_qside, dim3(p.xchunks, p.slabs, groups), dim3(kXThreads), QxSmem::total, st, map_q, map_o, (const float*)W,
                      (const float*)w.S, (const float*)w.z, beta, p.cfg.eps, p.cfg.bw_floor, den, map_keep,
                      keep != nullptr && groups == 1 ? 1 : 0, n, d, p.cfg.features, p.xchunk_tiles, w.status,
-                     (const __nv_bfloat16*)w.QF3);
+                     (const __nv_bfloat16*)w.QF3, (const int*)w.seen);
   if (err != cudaSuccess || groups == 1) return err;
   *launches += 1;
   return launch_after(k_tcx_combine, dim3((unsigned)((tokens * (d >> 2) + 255) / 256)), dim3(256), 0, st, (const float*)share,
