@@ -127,12 +127,14 @@ __device__ __forceinline__ void add_coarse4(const float (*ex)[W], const LevelCoe
 // inputs_ready: X and X2 were complete before the kernel in front of this one passed its wait (see launch_after), and are
 // fetched ahead of this one's.  That holds for dQ_F too, and the rows of the pass that writes dQ are on their way while the
 // gate backward is still at work.
+// place_next: the kernel behind this one may be placed early (see launch_haar_filter).
 // grid (col_blocks<32>, slabs, 1 or 2 tensors: X -> XF, X2 -> XF2); block 256.
 template <bool kFull, typename Tin, typename Tout, bool kAddVec>
 __global__ void __launch_bounds__(256, 4) k_haar_filter(const Tin* __restrict__ X, const float* __restrict__ f,
                                                      Tout* __restrict__ XF, const Tin* __restrict__ X2,
                                                      Tout* __restrict__ XF2, int n, int d_arg, int L,
-                                                     const float* __restrict__ vec, float vec_scale, bool inputs_ready) {
+                                                     const float* __restrict__ vec, float vec_scale, bool inputs_ready,
+                                                     bool place_next) {
   // (launched as a programmatic dependent: see launch_after)
   if (!kAddVec && !inputs_ready) wait_for_stream_predecessor();
   const int d = kFull ? kD : d_arg;
@@ -158,7 +160,7 @@ __global__ void __launch_bounds__(256, 4) k_haar_filter(const Tin* __restrict__ 
   }
   if constexpr (!kAddVec) {   // (with the row vector it is the last kernel of its pass, and f is the forward's)
     wait_for_stream_predecessor();
-    let_stream_successor_start();
+    if (place_next) let_stream_successor_start();
   }
   const LevelCoef k = level_coef<!kAddVec>(f + (size_t)slab * (L + 1), L);
   float hi[4], s5[4];
@@ -332,7 +334,7 @@ __global__ void __launch_bounds__(256, 3) k_haar_filter_bf16(const __nv_bfloat16
                                                              const float* __restrict__ f, Tout* __restrict__ XF,
                                                              const __nv_bfloat16* __restrict__ X2,
                                                              Tout* __restrict__ XF2, int n, int d_arg, int L,
-                                                             bool inputs_ready) {
+                                                             bool inputs_ready, bool place_next) {
   if (!inputs_ready) wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   const int d = kFull ? kD : d_arg;
   __shared__ __align__(16) float ex[8][kD];   // 32-row sums of the warps
@@ -352,7 +354,7 @@ __global__ void __launch_bounds__(256, 3) k_haar_filter_bf16(const __nv_bfloat16
     }
   }
   wait_for_stream_predecessor();   // f may be the gate kernel's result
-  let_stream_successor_start();
+  if (place_next) let_stream_successor_start();
   const LevelCoef k = level_coef<true>(f + (size_t)slab * (L + 1), L);
   float hi[8];
   packed_coarse(u, k, L, ex, hi);
@@ -669,17 +671,26 @@ cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const 
   const dim3 grid(col_blocks<32>(p.htiles, d), p.slabs, z), grid_bf(col_blocks<64>(p.htiles, d), p.slabs, z);
   const int n = p.cfg.seq_len, L = p.cfg.levels;
   using bf = __nv_bfloat16;
+  // In a pass the FFMA key side follows.  Not placed early where several of its small tiles' CTAs come to share an SM and this
+  // grid covers more than a third of the SMs: they gather on the others.  Forwards, placed early and not: 80 x 130, d = 32, m = 64
+  // 38.3 and 31.0 us; 40 x 200 30.0 and 27.2; 4 x 1024, d = 64 28.9 and 25.2; 10 x 1344 49.6 and 41.9; 16 x 500, m = 128 47.7 and
+  // 42.7; 30 x 130, d = 16 24.6 and 22.0.  One CTA an SM, full tiles or a small grid of this kernel: 1 x 1024, m = 64 21.1 and
+  // 22.5; 64 x 1024 87.8 and 89.7; 4 x 700, m = 256 38.4 and 39.6; 12 x 256, d = 32, m = 128 (24 CTAs here) 23.5 and 24.6; 20 x
+  // 200, m = 64 (40) 21.6 and 21.7.
+  const unsigned ctas = in_kind == 1 ? grid_bf.x * grid_bf.y * z : grid.x * grid.y * z;
+  const bool gathers = p.simt_small && p.cfg.features < 256 && (long long)p.schunks * p.slabs > p.sms && 3 * ctas > (unsigned)p.sms;
+  const bool place_next = inputs_ready && !gathers;   // (else it is the end of its pass)
   cudaError_t err;
   WERSA_FULL({
     if (in_kind == 1 && out_kind == 1)
       err = launch_after(k_haar_filter_bf16<kFull, bf>, grid_bf, dim3(256), 0, st, (const bf*)X, f, (bf*)XF, (const bf*)X2, (bf*)XF2, n, d, L,
-                         inputs_ready);
+                         inputs_ready, place_next);
     else if (in_kind == 1 && out_kind == 0)
       err = launch_after(k_haar_filter_bf16<kFull, float>, grid_bf, dim3(256), 0, st, (const bf*)X, f, (float*)XF, (const bf*)X2,
-                         (float*)XF2, n, d, L, inputs_ready);
+                         (float*)XF2, n, d, L, inputs_ready, place_next);
     else
       err = launch_after(k_haar_filter<kFull, float, float, false>, grid, dim3(256), 0, st, (const float*)X, f, (float*)XF,
-                         (const float*)X2, (float*)XF2, n, d, L, nullptr, 0.f, inputs_ready);
+                         (const float*)X2, (float*)XF2, n, d, L, nullptr, 0.f, inputs_ready, place_next);
   })
   *launches += 1;
   return err != cudaSuccess ? err : cudaGetLastError();
@@ -707,9 +718,9 @@ cudaError_t launch_haar_filter_addvec(const Plan& p, const float* G, const float
   cudaError_t err;
   WERSA_FULL({
     if (out_kind == 0)
-      err = launch_after(k_haar_filter<kFull, float, float, true>, grid, dim3(256), 0, st, G, f, (float*)dX, nullptr, nullptr, n, d, L, vec, vec_scale, true);
+      err = launch_after(k_haar_filter<kFull, float, float, true>, grid, dim3(256), 0, st, G, f, (float*)dX, nullptr, nullptr, n, d, L, vec, vec_scale, true, false);
     else
-      err = launch_after(k_haar_filter<kFull, float, bf, true>, grid, dim3(256), 0, st, G, f, (bf*)dX, nullptr, nullptr, n, d, L, vec, vec_scale, true);
+      err = launch_after(k_haar_filter<kFull, float, bf, true>, grid, dim3(256), 0, st, G, f, (bf*)dX, nullptr, nullptr, n, d, L, vec, vec_scale, true, false);
   })
   *launches += 1;
   return err != cudaSuccess ? err : cudaGetLastError();
