@@ -125,7 +125,9 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
 
   // fp32 forward on the tensor cores, from kXUnits tiles x groups of 128 features on: 2 x 4 x 1024, m = 128 (64 units) 49 -> 26
   // us, in d = 32 37 -> 23; 1 x 4 x 1024, m = 256 (64) 40 -> 26.  One CTA per SM and group, in chunks that minimise
-  // waves x (tiles + 3), 3 tiles being about what a CTA spends before its first and after its last one.
+  // waves x (tiles + 3), 3 tiles being about what a CTA spends before its first and after its last one, and a 64th of a tile
+  // for a chunk's partial in the reduction.  Up to a chunk per SM: one slab of 131072, m = 128 in 64 chunks against 147, forward
+  // d = 16 121 -> 83 us (FFMA 101), d = 64 165 -> 124; training step d = 16 368 -> 239 (294), d = 64 500 -> 348.
   // The backward from one tile per SM on: 2 x 3 x 4097, m = 128 150 -> 72 us, 5 x 4223, m = 256 203 -> 115, 8 x 4 x 1024,
   // d = 32 92 -> 65, narrower heads about as fast as before (40 x 4 x 130, d = 24 106 -> 107).  It is ahead below that line
   // too (64 tiles, m = 128 66 -> 48; 32 tiles 46 -> 46), but a feature within rounding of zero, which planes may decide
@@ -138,8 +140,8 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     const int tiles = ceil_div(n, 128), groups = m / 128;
     p->use_x = (long long)p->slabs * tiles * groups >= kXUnits;
     long long best = 0;
-    for (int ch = 1; ch <= tiles && ch <= 64; ++ch) {
-      const long long cost = (long long)ceil_div(p->slabs * groups * ch, p->sms) * (ceil_div(tiles, ch) + 3);
+    for (int ch = 1; ch <= tiles && ch <= p->sms; ++ch) {
+      const long long cost = (long long)ceil_div(p->slabs * groups * ch, p->sms) * (ceil_div(tiles, ch) + 3) * 64 + ch;
       if (ch == 1 || cost < best) {
         best = cost;
         p->xchunks = ch;
@@ -148,7 +150,7 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     p->xchunk_tiles = ceil_div(tiles, p->xchunks);
     p->xchunks = ceil_div(tiles, p->xchunk_tiles);
     p->use_xb = p->use_x && p->with_backward && !p->grad_bf16 && (long long)p->slabs * tiles >= p->sms;
-    for (int ch = 1; ch <= tiles && ch <= 64; ++ch) {
+    for (int ch = 1; ch <= tiles && ch <= p->sms; ++ch) {
       const long long cost = (long long)ceil_div(p->slabs * ch, p->sms) * (ceil_div(tiles, ch) + 1);
       if (ch == 1 || cost < best) {
         best = cost;
