@@ -12,6 +12,7 @@ namespace {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 constexpr long long kXUnits = 64;   // (see make_plan)
+constexpr double kXBytes = 64. * (1 << 30);
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 int next_pow2(int n) {
   int p = 1;
@@ -132,13 +133,16 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   // d = 32 92 -> 65, narrower heads about as fast as before (40 x 4 x 130, d = 24 106 -> 107).  It is ahead below that line
   // too (64 tiles, m = 128 66 -> 48; 32 tiles 46 -> 46), but a feature within rounding of zero, which planes may decide
   // otherwise than 32-bit sums, shows in a whole block of the coarsest level: in slabs of few tokens that is much of dQ.
+  // Their operands as planes take more memory than the FFMA kernels' fp32 ones (see the layout below): a problem that asks
+  // for more than kXBytes of it stays with those, so that what fitted the device beside its tensors before still does.
   p->use_x = p->use_xb = false;
   p->xchunks = p->xbchunks = 1;
   p->xchunk_tiles = p->xbchunk_tiles = 1;
   p->xprep = 0;
   if (!p->bf16 && !(c.flags & WERSA_FLAG_SIMT_ONLY) && m >= 128) {
     const int tiles = ceil_div(n, 128), groups = m / 128;
-    p->use_x = (long long)p->slabs * tiles * groups >= kXUnits;
+    const double plane_bytes = (p->with_backward ? 32. : 18.) * p->slabs * n * c.head_dim;
+    p->use_x = (long long)p->slabs * tiles * groups >= kXUnits && plane_bytes <= kXBytes;
     long long best = 0;
     for (int ch = 1; ch <= tiles && ch <= p->sms; ++ch) {
       const long long cost = (long long)ceil_div(p->slabs * groups * ch, p->sms) * (ceil_div(tiles, ch) + 3) * 64 + ch;
@@ -232,7 +236,8 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   // rows of partial sums: chunks of the forward or of the fp32 kernels, or the segments of the tensor-core
   // backward (slot = CTA + slab) of one feature group; of all feature groups in the forward
   size_t part_rows = slabs * p->groups * (p->use_tc ? p->tchunks : p->schunks) * (m < kGroupFeatures ? m : kGroupFeatures);
-  if (p->use_x && p->xchunks > p->schunks) part_rows = slabs * p->xchunks * m;
+  const bool ffma_bwd = p->use_x && p->with_backward && !p->use_xb;
+  if (p->use_x) part_rows = slabs * m * (ffma_bwd ? std::max(p->xchunks, p->schunks) : p->xchunks);
   if (p->use_tc && p->with_backward) {
     const size_t seg_rows = ((size_t)p->bctas + slabs) * (m < kGroupFeatures ? m : kGroupFeatures);
     if (seg_rows > part_rows) part_rows = seg_rows;
@@ -252,16 +257,27 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   take(p->dpad ? 256 : 0);
   p->off_Og = take(grouped ? io_bytes * slab_elems * p->groups : 0);
   p->off_den = take(grouped ? sizeof(float) * slabs * n * p->groups : 0);
+  // fp32 on the tensor cores: bytes per element of a tensor (slabs x n x head_dim: narrow heads pay for their own columns).
+  // Planes of T_f(Q), T_f(K) and V, 18 in all, over whose last two lie first the query side's shares of a forward without a
+  // backward (see launch_tcx_qside), then dQ_F and dK_F of an FFMA backward, which keeps T_f(Q) and T_f(K) as well: 26.  A
+  // backward on the planes: O (4), dQ_F (4) and planes of dO (6), 32 in all; the forward's shares lie over the last two,
+  // dK_F over the planes of dO, which its kernels no longer read.  FFMA alone: 8 and 16, 64 columns each.
+  const size_t tensor = slabs * (size_t)n * c.head_dim, plane3 = 3 * sizeof(__nv_bfloat16) * tensor;
   p->off_dO3 = p->off_xO = p->off_xden = p->off_xinv = p->off_xc = p->off_xshare = 0;
-  const bool need_xf = !p->use_tc && (!p->use_x || (p->with_backward && !p->use_xb));   // the tensor-core kernels filter on chip (forward) or read bf16 planes (backward)
-  p->off_QF = take(need_xf ? sizeof(float) * slab_elems : 0);
-  p->off_KF = take(need_xf ? sizeof(float) * slab_elems : 0);
-  if (p->use_x) {   // (the query side's shares follow on from KF3 into V3: see launch_tcx_qside)
-    p->off_QF3 = take(3 * sizeof(__nv_bfloat16) * slab_elems);
-    p->off_KF3 = take(3 * sizeof(__nv_bfloat16) * slab_elems);
-    p->off_V3 = take(3 * sizeof(__nv_bfloat16) * slab_elems);
-  } else {
-    p->off_QF3 = p->off_KF3 = p->off_V3 = 0;
+  p->off_QF = p->off_KF = p->off_QF3 = p->off_KF3 = p->off_V3 = p->off_dQF = p->off_dKF = 0;
+  if (p->use_x) {
+    p->off_QF3 = take(plane3);
+    p->off_KF3 = take(plane3);
+    p->off_V3 = take(plane3);
+    if (ffma_bwd) {
+      p->off_QF = take(sizeof(float) * tensor);
+      p->off_KF = take(sizeof(float) * tensor);
+      p->off_dQF = p->off_KF3;
+      p->off_dKF = p->off_KF3 + align_up(sizeof(float) * tensor, 256);
+    }
+  } else if (!p->use_tc) {   // (the bf16 kernels of the tensor cores filter on chip, or read planes in the backward)
+    p->off_QF = take(sizeof(float) * slab_elems);
+    p->off_KF = take(sizeof(float) * slab_elems);
   }
   if (p->with_backward) {
     p->off_dS = take(sizeof(float) * slabs * m * kD);
@@ -269,17 +285,19 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     p->off_sumdD = take(sizeof(float) * (p->use_tc ? (size_t)p->bctas : p->use_xb ? (size_t)p->xprep : slabs * p->schunks));
     if (p->use_xb) {
       const size_t groups = c.features / 128, padded = (size_t)ceil_div(c.seq_len, 128) * 128;
-      p->off_dO3 = take(3 * sizeof(__nv_bfloat16) * slab_elems);
-      p->off_xO = take(sizeof(float) * slab_elems);
+      p->off_xO = take(sizeof(float) * tensor);
       p->off_xden = take(sizeof(float) * groups * slabs * c.seq_len);
       p->off_xinv = take(sizeof(float) * slabs * padded);
       p->off_xc = take(sizeof(float) * slabs * padded);
-      p->off_xshare = take(groups > 1 ? sizeof(float) * groups * slab_elems : 0);
+      p->off_dQF = p->off_xshare = take(sizeof(float) * tensor);
+      p->off_dO3 = p->off_dKF = take(plane3);
     }
     p->off_bands = take(sizeof(float) * 2 * slabs * 2 * p->htiles * kBandVals);   // Q and K; two column halves per tile
     p->off_dqbar = take(sizeof(float) * slabs * (kD + kBandVals));
-    p->off_dQF = take(sizeof(float) * slab_elems);
-    p->off_dKF = take(sizeof(float) * slab_elems);
+    if (!p->use_x) {
+      p->off_dQF = take(sizeof(float) * slab_elems);
+      p->off_dKF = take(sizeof(float) * slab_elems);
+    }
     p->off_dSbf = take(sizeof(__nv_bfloat16) * slabs * m * kD);
     if (p->use_tc) {
       p->off_KF3 = take(3 * sizeof(__nv_bfloat16) * slab_elems);
@@ -290,7 +308,7 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     p->off_shardtot = take(256);
   } else {
     p->off_Dtot = p->off_shardtot = 0;
-    p->off_dS = p->off_dz = p->off_sumdD = p->off_bands = p->off_dqbar = p->off_dQF = p->off_dKF = p->off_dSbf = p->off_Slo = 0;
+    p->off_dS = p->off_dz = p->off_sumdD = p->off_bands = p->off_dqbar = p->off_dSbf = p->off_Slo = 0;
   }
   p->total = off;
   return WERSA_OK;

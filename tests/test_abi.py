@@ -61,6 +61,29 @@ def test_workspace_bytes_and_validation():
     assert w.wersa_workspace_bytes(_cfg(seq_len=200, levels=8)) > 0
 
 
+def test_workspace_of_fp32_on_the_tensor_cores():
+    """Operands as planes against the FFMA kernels' workspace: 18 bytes an element of a tensor against 8 for a forward, 32
+    against 16 with a backward, by the head's own width where the FFMA kernels' is 64 columns always, and a 20th for the
+    per-token and per-slab arrays; the FFMA kernels' own where the planes would take more than 64 GiB."""
+    import paper_2507_08637_b200 as w
+
+    def nbytes(flags, **shape):
+        return w.wersa_workspace_bytes(_cfg(dtype="f32", grad_dtype="f32", flags=flags, levels=4, **shape))
+
+    for shape in (dict(batch=2, heads=8, seq_len=4096), dict(batch=1, heads=8, seq_len=30000)):
+        for features in (128, 256):
+            for d in (8, 16, 32, 64):
+                kw = dict(shape, features=features, head_dim=d)
+                fwd, ffma_fwd = (nbytes(f | w.WERSA_FLAG_FORWARD_ONLY, **kw) for f in (0, w.WERSA_FLAG_SIMT_ONLY))
+                train, ffma_train = nbytes(0, **kw), nbytes(w.WERSA_FLAG_SIMT_ONLY, **kw)
+                tensor = shape["batch"] * shape["heads"] * shape["seq_len"] * 64
+                assert fwd <= ffma_fwd + (18 * d / 64 - 8 + 0.9) * tensor, (kw, fwd, ffma_fwd)
+                assert train <= ffma_train + (32 * d / 64 - 16 + 1.6) * tensor, (kw, train, ffma_train)
+    for flags in (0, w.WERSA_FLAG_FORWARD_ONLY):
+        kw = dict(batch=64, heads=64, seq_len=32768, features=256)
+        assert nbytes(flags, **kw) == nbytes(flags | w.WERSA_FLAG_SIMT_ONLY, **kw)
+
+
 def test_create_rejects_bad_arguments_without_a_device(lib):
     import paper_2507_08637_b200 as w
     lib.wersa_create.restype = ctypes.c_int
