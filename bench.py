@@ -355,17 +355,18 @@ def main():
     # algorithmic work of each step per launch
     m_launch = min(m, 256)                           # feature maps wider than 256 run one launch per 256 features
     unit_flops = TH * (4 * d * m_launch + 2 * m_launch)   # one projection + one (m x d) contraction per token-head
-    flops = {"tc_kside": unit_flops, "tc_qside": unit_flops, "simt_kside": unit_flops, "simt_qside": unit_flops}
+    flops = {side + "side": unit_flops for side in ("tc_k", "tc_q", "simt_k", "simt_q", "tcx_k", "tcx_q")}
     bytes_ = {"qmean_gate": TH * d * s_bytes, "haar_filter_q": TH * d * (s_bytes + 4),
               "haar_filter_k": TH * d * (s_bytes + 4),
               "tc_kside": 2 * TH * d * s_bytes,      # K and V read once
               "tc_qside": 2 * TH * d * s_bytes,      # Q read once, O written once
+              "f32_planes": 3 * TH * d * (4 + 6),    # Q, K, V -> three bf16 planes each
               # feature groups: G outputs of 64 columns and G denominators in, O out
               "combine_groups": TH * ((m // 256) * (64 * s_bytes + 4) + d * s_bytes)}
     ncu_bytes_per_th, traffic_source = load_traffic()
     if dom in flops:
-        if dom.startswith("tc_"):
-            bound, peak, unit = "tensor", tensor_peak, "TFLOP/s"
+        if dom.startswith("tc"):   # (fp32 as bf16 planes: six products for one)
+            bound, peak, unit = "tensor", tensor_peak / (6 if dom.startswith("tcx") else 1), "TFLOP/s"
         else:
             bound, peak, unit = "alu", fp32_alu_tflops(sms, sm_max_mhz), "TFLOP/s"
         achieved = flops[dom] / (avg[dom] * 1e-3) / 1e12
@@ -400,7 +401,9 @@ def main():
         "data": "synthetic",
         "config": {"workload": workload_string(cfg), "per_gpu": True,
                    "l2": "inputs+output 4 x %.0f MB per step exceed the 126 MB L2" % (TH * d * s_bytes / 1e6),
-                   "kernels": "tcgen05 bf16, fp32 accumulate" if tensor_cores else "fp32 FFMA", "storage": dtype},
+                   "kernels": ("tcgen05 bf16, fp32 accumulate" if tensor_cores else
+                               "tcgen05, fp32 as three bf16 planes" if "tcx_kside" in per_kernel else "fp32 FFMA"),
+                   "storage": dtype},
         "clocks": clocks,
         "e2e": {"value": e2e_value, "unit": "tokens/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "steps": args.e2e_steps, "serial_value": e2e_serial,

@@ -56,8 +56,9 @@ typedef enum { WERSA_F32 = 0, WERSA_BF16 = 1 } wersa_dtype;
 
 /* Flags for wersa_config.flags. */
 enum {
-  WERSA_FLAG_SIMT_ONLY = 1,    /* bf16 storage but fp32 FFMA arithmetic everywhere (no tensor
-                                  cores); the fp32 dtype always computes this way        */
+  WERSA_FLAG_SIMT_ONLY = 1,    /* fp32 FFMA arithmetic everywhere, no tensor cores: with bf16
+                                  storage, and with fp32 where a context would otherwise run
+                                  on them (see wersa_uses_tensor_cores)                  */
   WERSA_FLAG_FORWARD_ONLY = 2  /* the context will never run wersa_backward: its workspace
                                   omits the gradient scratch buffers                     */
 };
@@ -86,7 +87,11 @@ typedef struct wersa_config {
 } wersa_config;
 
 /* Bytes of device workspace a context of this configuration needs (a multiple of 256);
- * 0 if the configuration is invalid or unsupported.  Pure host arithmetic. */
+ * 0 if the configuration is invalid or unsupported.  Pure host arithmetic.
+ * What grows with the tensors, per element of one of them (batch*heads*seq_len*head_dim): with dtype fp32 on the
+ * tensor cores (see wersa_uses_tensor_cores) 18 bytes for a forward alone and 32 with a backward (26 where that runs
+ * on the FFMA kernels); on the FFMA kernels 8 and 16, but for 64 columns whatever head_dim is.  Problems whose planes
+ * would take more than 64 GiB stay on the FFMA kernels. */
 size_t wersa_workspace_bytes(const wersa_config* cfg);
 
 /* Validates cfg, records the plan (tiling, split-sequence chunking) and adopts `workspace`
@@ -127,7 +132,8 @@ wersa_status wersa_forward_host(wersa_ctx* ctx, const void* hQ, const void* hK, 
  * when gate_per_head = 0) and omega (levels+1).  The paper does not write the backward pass;
  * it is the chain rule through Eqs. 1-7 with dReLU(a)/da = 1[a > 0].  W is a fixed random
  * matrix (Sec. 3.1 step 7) and gets no gradient.  Must follow a wersa_forward on the same
- * context with the same inputs (it reuses f, qbar, S, z).  Any of the five parameter-gradient
+ * context with the same inputs (it reuses f, qbar, S, z, and with dtype fp32 what the forward read
+ * of Q, K, V and left in O).  Any of the five parameter-gradient
  * pointers may be NULL. */
 wersa_status wersa_backward(wersa_ctx* ctx, const void* Q, const void* K, const void* V,
                             const void* W, const float* beta, const float* gate_w,
@@ -251,9 +257,14 @@ const char* wersa_status_string(wersa_status status);
  * launched; 0 before the first call. */
 int32_t wersa_launch_count(const wersa_ctx* ctx, int which);
 
-/* 1 if this context's forward runs the bf16 tcgen05 tensor-core kernels, 0 if it runs the fp32
- * FFMA kernels (fp32 storage, WERSA_FLAG_SIMT_ONLY, or a shape the tensor-core kernels do not
- * cover). */
+/* 1 if this context multiplies bf16 operands (the filtered tensors and the features rounded to bf16, sums in fp32):
+ * dtype bf16 without WERSA_FLAG_SIMT_ONLY, on the tensor cores.  0 if it computes in fp32.  That is on the FFMA kernels,
+ * or, with dtype fp32, 128 or 256 features and a problem for which it is the faster way, on the tensor cores as well,
+ * with every operand split into three bf16 planes whose sum is its fp32 value: O is as close to 64 bits as with the
+ * FFMA kernels, in the 2-norm, but not the same bits.  Such a context's steps are called f32_planes and tcx_... (see
+ * wersa_step_times), and WERSA_FLAG_SIMT_ONLY keeps a context off them.  What differs at the ends of the range: values
+ * below 2^-110 lose low-order bits (a bf16 plane ends at 2^-133), and a sum that meets an infinity comes out as NaN
+ * where an FFMA sum may be infinite. */
 int32_t wersa_uses_tensor_cores(const wersa_ctx* ctx);
 
 /* Step timing (a measurement aid; the paper has no counterpart).  When enabled, forward and

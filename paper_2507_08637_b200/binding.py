@@ -369,6 +369,7 @@ class WersaContext:
         return [(names[i].decode(), float(ms[i])) for i in range(min(count.value, cap))]
 
     def uses_tensor_cores(self):
+        """True where bf16 operands are multiplied; fp32 contexts compute in fp32, be it on the tensor cores or not."""
         return bool(_lib().wersa_uses_tensor_cores(self._h))
 
     def launch_count(self, which=0):
