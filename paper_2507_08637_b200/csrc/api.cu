@@ -94,6 +94,7 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   p->simt_small = false;
   p->schunks = 1;
   p->schunk_rows = n;
+  double ffma_cost = 0;
   if (!p->use_tc) {
     const int mt = m < 256 ? m : 256;
     const int big = 64 * (256 / mt), share = 256 / mt;
@@ -122,17 +123,23 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     }
     p->schunk_rows = rows_best;
     p->schunks = ceil_div(n, rows_best);
+    ffma_cost = best;
   }
 
-  // fp32 forward on the tensor cores, from kXUnits tiles x groups of 128 features on: 2 x 4 x 1024, m = 128 (64 units) 49 -> 26
-  // us, in d = 32 37 -> 23; 1 x 4 x 1024, m = 256 (64) 40 -> 26.  One CTA per SM and group, in chunks that minimise
-  // waves x (tiles + 3), 3 tiles being about what a CTA spends before its first and after its last one, and a 64th of a tile
-  // for a chunk's partial in the reduction.  Up to a chunk per SM: one slab of 131072, m = 128 in 64 chunks against 147, forward
-  // d = 16 121 -> 83 us (FFMA 101), d = 64 165 -> 124; training step d = 16 368 -> 239 (294), d = 64 500 -> 348.
-  // The backward from one tile per SM on: 2 x 3 x 4097, m = 128 150 -> 72 us, 5 x 4223, m = 256 203 -> 115, 8 x 4 x 1024,
-  // d = 32 92 -> 65, narrower heads about as fast as before (40 x 4 x 130, d = 24 106 -> 107).  It is ahead below that line
-  // too (64 tiles, m = 128 66 -> 48; 32 tiles 46 -> 46), but a feature within rounding of zero, which planes may decide
-  // otherwise than 32-bit sums, shows in a whole block of the coarsest level: in slabs of few tokens that is much of dQ.
+  // fp32 on the tensor cores: one CTA per SM and group, in chunks that minimise waves x (tiles + 3), 3 tiles being about what
+  // a CTA spends before its first and after its last one, and a 64th of a tile for a chunk's partial in the reduction.  Up to
+  // a chunk per SM: one slab of 131072, m = 128 in 64 chunks against 147, forward d = 16 121 -> 83 us (FFMA 101), d = 64 165 ->
+  // 124; training step d = 16 368 -> 239 (294), d = 64 500 -> 348.
+  // Planes multiply tiles of 128 tokens and 64 columns whatever is in them, the FFMA kernels 16 tokens and 16, 32 or 64 columns:
+  // short slabs and narrow heads are theirs.  The line lies where two estimates in us meet, fitted to 435 shapes of 1 to
+  // 1023 slabs, 16 to 131072 tokens, d = 8 to 64, m = 128 and 256 (rms 4 % off for planes, 10 % for FFMA; 10 of the 435 choices
+  // cost more than 5 %).  Per unit of the FFMA plan's cost, with full and small tiles.  FFMA and planes, us:
+  //   forward  1 x 8192, d = 16, m = 128 37 27;  1 x 16384 29 34;   300 x 128 56 64;    148 x 256 38 37;    1023 x 16 60 153
+  //            512 x 64, d = 32, m = 128 77 89;  256 x 64 54 49;    300 x 128 77 65;    100 x 200 62 34
+  //            512 x 32, d = 64, m = 256 164 156; 148 x 40 50 52;   1023 x 16 192 314;  200 x 50, m = 128 76 50
+  //   backward 300 x 128, d = 16, m = 128 109 123; 8 x 8192 111 97; 512 x 64, d = 32 146 178; 300 x 128 155 136
+  // From kXUnits tiles x groups of 128 features on, the backward from one tile per SM on (below these lines planes have not
+  // been chosen, whatever the estimates say).
   // Their operands as planes take more memory than the FFMA kernels' fp32 ones (see the layout below): a problem that asks
   // for more than kXBytes of it stays with those, so that what fitted the device beside its tensors before still does.
   p->use_x = p->use_xb = false;
@@ -142,7 +149,6 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   if (!p->bf16 && !(c.flags & WERSA_FLAG_SIMT_ONLY) && m >= 128) {
     const int tiles = ceil_div(n, 128), groups = m / 128;
     const double plane_bytes = (p->with_backward ? 32. : 18.) * p->slabs * n * c.head_dim;
-    p->use_x = (long long)p->slabs * tiles * groups >= kXUnits && plane_bytes <= kXBytes;
     long long best = 0;
     for (int ch = 1; ch <= tiles && ch <= p->sms; ++ch) {
       const long long cost = (long long)ceil_div(p->slabs * groups * ch, p->sms) * (ceil_div(tiles, ch) + 3) * 64 + ch;
@@ -153,7 +159,6 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     }
     p->xchunk_tiles = ceil_div(tiles, p->xchunks);
     p->xchunks = ceil_div(tiles, p->xchunk_tiles);
-    p->use_xb = p->use_x && p->with_backward && !p->grad_bf16 && (long long)p->slabs * tiles >= p->sms;
     for (int ch = 1; ch <= tiles && ch <= p->sms; ++ch) {
       const long long cost = (long long)ceil_div(p->slabs * ch, p->sms) * (ceil_div(tiles, ch) + 1);
       if (ch == 1 || cost < best) {
@@ -163,6 +168,14 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     }
     p->xbchunk_tiles = ceil_div(tiles, p->xbchunks);
     p->xbchunks = ceil_div(tiles, p->xbchunk_tiles);
+    const int width = c.head_dim <= 16 ? 0 : c.head_dim <= 32 ? 1 : 2;
+    constexpr double kFwd[2][3] = {{0.13, 0.205, 0.345}, {0.17, 0.25, 0.46}}, kBwd[2][3] = {{0.275, 0.445, 0.745}, {0.33, 0.53, 0.8}};
+    const double f_fwd = 14 + kFwd[p->simt_small][width] * ffma_cost, f_bwd = 15 + kBwd[p->simt_small][width] * ffma_cost;
+    const int waves = ceil_div(p->slabs * groups * p->xchunks, p->sms), bwaves = ceil_div(p->slabs * p->xbchunks, p->sms) * groups;
+    const double x_fwd = 9 + (12.5 + 6 * p->xchunk_tiles) * waves + 0.02 * p->xchunks;
+    const double x_bwd = 14.5 + (15 + 3 * p->xchunk_tiles) * waves + 9. * bwaves * (p->xbchunk_tiles + 1);
+    p->use_x = (long long)p->slabs * tiles * groups >= kXUnits && x_fwd <= f_fwd && plane_bytes <= kXBytes;
+    p->use_xb = p->use_x && p->with_backward && !p->grad_bf16 && (long long)p->slabs * tiles >= p->sms && x_bwd <= f_bwd;
     p->xprep = (int)std::min<long long>(((long long)p->slabs * n * 8 + 255) / 256, 8LL * p->sms);
   }
 
