@@ -306,6 +306,8 @@ __device__ __forceinline__ float bf16_range(float x) {
   const float most = __uint_as_float(0x7F7F0000u);
   return fabsf(x) < INFINITY ? fminf(fmaxf(x, -most), most) : x;
 }
+// Not 0 where one of two packed bf16 has an exponent of all ones: infinity, NaN, or what rounded to infinity.
+__device__ __forceinline__ uint32_t full_exponents(uint32_t w) { return ((w & 0x7F807F80u) + 0x00800080u) & 0x80008000u; }
 
 // Loads 8 consecutive elements (16-byte aligned for bf16, 32-byte for float) as floats.
 __device__ __forceinline__ void load8(const float* p, float (&v)[8]) {

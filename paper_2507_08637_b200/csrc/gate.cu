@@ -125,7 +125,9 @@ __global__ void __launch_bounds__(256) k_qmean_gate(const T* __restrict__ Q, flo
   // (programmatic dependent launch; it waits for this grid before it reads W^T or the gate).
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (seen != nullptr && blockIdx.x + blockIdx.y == 0 && threadIdx.x < 2) seen[threadIdx.x] = 0;   // (see k_f32_planes)
+  if constexpr (sizeof(T) == 4) {   // (in the bf16 kernels, which have no use for it, four registers and a CTA per SM)
+    if (seen != nullptr && blockIdx.x + blockIdx.y == 0 && threadIdx.x < 2) seen[threadIdx.x] = 0;   // see k_f32_planes
+  }
   if ((int)blockIdx.y == slabs) {
     // A thread takes eight columns of W^T's row r: neighbouring threads read neighbouring features and store 16 bytes.  (An
     // element a thread reads 2 bytes out of 32 different sectors a warp, and the grid's other CTAs wait for nothing else:

@@ -270,27 +270,31 @@ __global__ void __launch_bounds__(256, 3) k_f32_planes(const float* __restrict__
   }
   __nv_bfloat16* dst = (blockIdx.z == 0 ? Q3 : blockIdx.z == 1 ? K3 : V3) + first;
   float* keep = blockIdx.z == 0 ? QF : KF;
-  uint32_t top = 0;   // bits 15 and 31: an exponent of all ones in a first plane
+  uint32_t top = 0;   // not 0: a value that is not finite, or above the largest bf16
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     if (j >= rows) break;
     if (kKeep && filtered) store4(keep + first + (size_t)j * d, x[j]);
 #pragma unroll
     for (int pl = 0; pl < 3; ++pl) {   // what a plane leaves is the next one's input
-      float v[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) v[c] = pl == 0 ? bf16_range(x[j][c]) : x[j][c];
-      const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
-      const uint2 w = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+      auto plane_of = [](float x0, float x1, float x2, float x3) {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(x0, x1), b = __floats2bfloat162_rn(x2, x3);
+        return make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+      };
+      uint2 w = plane_of(x[j][0], x[j][1], x[j][2], x[j][3]);
+      if (pl == 0) {
+        const uint32_t t = full_exponents(w.x) | full_exponents(w.y);
+        if (t != 0) w = plane_of(bf16_range(x[j][0]), bf16_range(x[j][1]), bf16_range(x[j][2]), bf16_range(x[j][3]));
+        top |= t;
+      }
       *reinterpret_cast<uint2*>(dst + (size_t)pl * plane + (size_t)j * d) = w;
-      if (pl == 0) top |= ((w.x & 0x7F807F80u) + 0x00800080u) | ((w.y & 0x7F807F80u) + 0x00800080u);
       x[j][0] -= __uint_as_float(w.x << 16);
       x[j][1] -= __uint_as_float(w.x & 0xFFFF0000u);
       x[j][2] -= __uint_as_float(w.y << 16);
       x[j][3] -= __uint_as_float(w.y & 0xFFFF0000u);
     }
   }
-  if (filtered && (top & 0x80008000u) != 0) seen[blockIdx.z] = 1;   // (who multiplies by W wants to know: see Operands)
+  if (filtered && top != 0) seen[blockIdx.z] = 1;   // (who multiplies by W wants to know: see Operands)
 }
 
 // The same pass for bf16 input: a thread keeps its 8 rows x 8 columns as the 32 packed words it loaded

@@ -22,9 +22,9 @@
 // the contractions (MMA2), warps 4-11 two groups that take the tiles in turn: accumulator -> ReLU -> planes back into
 // TMEM; warps 12-15 drain.  TMEM: two buffers of 192 columns (128 of D1, replaced in place by the hi and mid planes, 64 of
 // the lo plane), two accumulators of 64 (k_tcx_bwd has its own).  Every wait is bounded, as in tc_fwd.cu.
-// 2 x 8 x 4096, d = 64, m = 256: planes 19 us, key side 28, query side 29, combining 7; the forward 235 -> 95 us.  A tile and
-// group takes some 5 k cycles of tensor pipe (MMA1 reads both operands of its 24 instructions from shared memory, 105-115
-// cycles each instead of 64; the 48 of MMA2 45 each), 60 % of the time.
+// 2 x 8 x 4096, d = 64, m = 256: planes 19 us, key side 28, query side 29, combining 7; the forward 235 -> 96 us.  Alone and on a
+// cold L2 the key side takes 49 k cycles for the eight tiles of a CTA, the query side 47 k, with the tensor pipe active 43
+// and 46 % of them.
 #include "common.cuh"
 #include "tc_common.cuh"
 #include "tc_maps.cuh"
@@ -95,17 +95,30 @@ __device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t&
   b -= __uint_as_float(mid & 0xFFFF0000u);
   lo = pack_bf16x2(a, b);
 }
-// Eight floats -> 16-byte chunk `chunk` of row `row` of the three plane tiles at `tile`.
-__device__ __forceinline__ void put_planes8(uint8_t* tile, int row, int chunk, const float (&v)[8]) {
-  uint32_t p[3][4];
+// Eight floats -> planes.  Is one of them not finite (or above the largest bf16)?
+__device__ __forceinline__ bool split8(const float (&v)[8], uint32_t (&p)[3][4]) {
+  uint32_t top = 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) split3<true>(v[2 * i], v[2 * i + 1], p[0][i], p[1][i], p[2][i]);
+  for (int i = 0; i < 4; ++i) {
+    split3(v[2 * i], v[2 * i + 1], p[0][i], p[1][i], p[2][i]);
+    top |= full_exponents(p[0][i]);
+  }
+  if (top != 0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) split3<true>(v[2 * i], v[2 * i + 1], p[0][i], p[1][i], p[2][i]);
+  }
+  return top != 0;
+}
+// The same -> 16-byte chunk `chunk` of row `row` of the three plane tiles at `tile`.
+__device__ __forceinline__ bool put_planes8(uint8_t* tile, int row, int chunk, const float (&v)[8]) {
+  uint32_t p[3][4];
+  const bool bad = split8(v, p);
 #pragma unroll
   for (int s = 0; s < 3; ++s)
     *reinterpret_cast<uint4*>(tile + s * kTileBytes + swz128(row, chunk)) = make_uint4(p[s][0], p[s][1], p[s][2], p[s][3]);
+  return bad;
 }
-// W (d x m, row-major) -> planes of rows f0 .. f0 + 127 of W^T, zero past column d.  512 threads.  Is one of this thread's
-// values not finite?
+// W (d x m, row-major) -> planes of rows f0 .. f0 + 127 of W^T, zero past column d.  512 threads.  The answer is split8's.
 __device__ __forceinline__ bool load_w_planes(const float* __restrict__ W, int d, int m, int f0, uint8_t* wt) {
   const int f = threadIdx.x & 127, part = threadIdx.x >> 7;   // 16 columns
   bool bad = false;
@@ -116,9 +129,8 @@ __device__ __forceinline__ bool load_w_planes(const float* __restrict__ W, int d
     for (int j = 0; j < 8; ++j) {
       const int c = 16 * part + 8 * h + j;
       v[j] = c < d ? W[(size_t)c * m + f0 + f] : 0.f;
-      bad |= !(fabsf(v[j]) < INFINITY);
     }
-    put_planes8(wt, f, 2 * part + h, v);
+    bad |= put_planes8(wt, f, 2 * part + h, v);
   }
   return bad;
 }
@@ -606,7 +618,7 @@ __global__ void __launch_bounds__(256) k_tcx_combine(const float* __restrict__ N
 // ---- backward ------------------------------------------------------------------------------------
 // Per token: planes of dO, 1 / D (D = sum_g D'_g + eps'), c = -dO.O; sum of dD = c / D per CTA.  tpt threads (a power of
 // two >= d / 8) on a token, eight columns each.  Bound by memory (2 x 8 x 4096, d = 64: 59 MB).
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 6)
 k_tcx_bwd_prep(const float* __restrict__ dO, const float* __restrict__ O, const float* __restrict__ den, int groups,
                const float* __restrict__ beta, float eps, float bw_floor, int m, int d, int tpt, size_t tokens, int n,
                __nv_bfloat16* __restrict__ dO3, float* __restrict__ inv, float* __restrict__ c, float* __restrict__ sumdD) {
@@ -629,8 +641,7 @@ k_tcx_bwd_prep(const float* __restrict__ dO, const float* __restrict__ O, const 
       uint32_t pl[3][4];
 #pragma unroll
       for (int j = 0; j < 8; ++j) dot = fmaf(g[j], o[j], dot);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) split3<true>(g[2 * j], g[2 * j + 1], pl[0][j], pl[1][j], pl[2][j]);
+      split8(g, pl);
 #pragma unroll
       for (int s = 0; s < 3; ++s)
         *reinterpret_cast<uint4*>(dO3 + s * plane + tok * d + c0) = make_uint4(pl[s][0], pl[s][1], pl[s][2], pl[s][3]);
