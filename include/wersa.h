@@ -59,8 +59,10 @@ enum {
   WERSA_FLAG_SIMT_ONLY = 1,    /* fp32 FFMA arithmetic everywhere, no tensor cores: with bf16
                                   storage, and with fp32 where a context would otherwise run
                                   on them (see wersa_uses_tensor_cores)                  */
-  WERSA_FLAG_FORWARD_ONLY = 2  /* the context will never run wersa_backward: its workspace
+  WERSA_FLAG_FORWARD_ONLY = 2, /* the context will never run wersa_backward: its workspace
                                   omits the gradient scratch buffers                     */
+  WERSA_FLAG_STEPWISE = 4      /* bf16: a launch per step of the forward for short sequences
+                                  too, where it would otherwise be one launch            */
 };
 
 typedef struct wersa_config {

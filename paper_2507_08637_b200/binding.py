@@ -16,6 +16,7 @@ WERSA_OK = 0
 WERSA_F32, WERSA_BF16 = 0, 1
 WERSA_FLAG_SIMT_ONLY = 1
 WERSA_FLAG_FORWARD_ONLY = 2
+WERSA_FLAG_STEPWISE = 4
 
 STATUS_NAMES = ["WERSA_OK", "WERSA_ERR_INVALID_ARG", "WERSA_ERR_UNSUPPORTED", "WERSA_ERR_WORKSPACE",
                 "WERSA_ERR_CUDA", "WERSA_ERR_TIMEOUT", "WERSA_ERR_STATE", "WERSA_ERR_TOO_LARGE"]

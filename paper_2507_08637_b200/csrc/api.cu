@@ -224,6 +224,7 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     p->tqchunk_blocks = ceil_div(blocks, p->tqchunks);
     p->tqchunks = ceil_div(blocks, p->tqchunk_blocks);
   }
+  p->small_tokens = p->small_blocks = 0;
   {
     // tensor-core backward: one wave of CTAs that share the list of all 128-token tiles evenly
     const long long tiles = (long long)ceil_div(n, 128) * p->slabs;
@@ -489,6 +490,10 @@ wersa_status wersa_create(const wersa_config* cfg, void* workspace, size_t works
   if (s != WERSA_OK) return s;
   if (workspace == nullptr || (reinterpret_cast<uintptr_t>(workspace) & 255u) != 0 || workspace_bytes < p.total)
     return WERSA_ERR_WORKSPACE;
+  {
+    DeviceGuard guard(p.cfg.device);
+    if (guard.err == cudaSuccess) choose_small_forward(&p);
+  }
   wersa_ctx* ctx = new (std::nothrow) wersa_ctx;
   if (ctx == nullptr) return WERSA_ERR_INVALID_ARG;
   ctx->plan = p;
@@ -521,6 +526,14 @@ wersa_status wersa_forward(wersa_ctx* ctx, const void* Q, const void* K, const v
   if ((s = begin_pass(ctx, 0, st)) != WERSA_OK) return s;
   const size_t rows = (size_t)p.slabs * p.cfg.seq_len;
   const int d = p.cfg.head_dim;   // (narrow heads: every forward kernel reads and writes the narrow tensors themselves)
+  if (p.small_blocks > 0) {
+    WERSA_STEP(0, "small_forward", launch_small_forward(p, w, Q, K, V, W, beta, gate_w, gate_b, omega, O, st, &launches));
+    if (p.groups > 1)
+      WERSA_STEP(0, "combine_groups", launch_combine_groups(w.Og, w.den, O, rows, p.groups, d, st, &launches));
+    ctx->launches_fwd = launches;
+    ctx->forward_done = true;
+    return WERSA_OK;
+  }
   WERSA_STEP(0, "qmean_gate",
              launch_qmean_gate(p, w, Q, gate_w, gate_b, omega, p.use_tc ? W : nullptr, d, st, &launches));
   if (p.groups > 1) {

@@ -42,6 +42,7 @@ struct Plan {
   int xchunks, xchunk_tiles;   // its chunks per slab, 128-token tiles per chunk
   bool use_xb;        // fp32 backward on them too: chunks and tiles of its gradient kernels, CTAs of its first pass
   int xbchunks, xbchunk_tiles, xprep;
+  int small_tokens, small_blocks;   // bf16 forward in one launch (small.cu): tokens of a thread block, blocks of a slab; 0: not
   int bctas;          // tcgen05 backward: CTAs that share the list of all 128-token tiles
   // workspace offsets (bytes)
   size_t off_status, off_counters, status_bytes, off_qpart, off_qbar, off_sg, off_f, off_spart, off_zpart, off_S, off_z,
@@ -164,6 +165,16 @@ cudaError_t launch_tc_kside(const Plan& p, const Ws& w, const void* K, const voi
 // den != nullptr (features == 256 only): also leaves every token's denominator in den[slab * n + token].
 cudaError_t launch_tc_qside(const Plan& p, const Ws& w, const void* Q, const float* beta, void* O, float* den,
                             cudaStream_t st, int* launches);
+
+// ---- small.cu ------------------------------------------------------------------------------
+// The whole forward of slabs of p.small_blocks * p.small_tokens tokens in one launch: O (with several feature groups w.Og and
+// w.den), f, q-bar, S', z', and what a backward reads beside them.
+cudaError_t launch_small_forward(const Plan& p, const Ws& w, const void* Q, const void* K, const void* V, const void* W,
+                                 const float* beta, const float* gate_w, const float* gate_b, const float* omega, void* O,
+                                 cudaStream_t st, int* launches);
+
+// Decides p->small_tokens and p->small_blocks (asks the device, which is current).
+void choose_small_forward(Plan* p);
 
 // ---- tc_bwd.cu -----------------------------------------------------------------------------
 // Key-side backward on the tensor cores: dV and dK_F from K_F as three bf16 planes, V, the bf16 dS' image
