@@ -92,7 +92,8 @@ typedef struct wersa_config {
  * 0 if the configuration is invalid or unsupported.  Pure host arithmetic.
  * What grows with the tensors, per element of one of them (batch*heads*seq_len*head_dim): with dtype fp32 on the
  * tensor cores (see wersa_uses_tensor_cores) 18 bytes for a forward alone and 32 with a backward (26 where that runs
- * on the FFMA kernels); on the FFMA kernels 8 and 16, but for 64 columns whatever head_dim is.  Problems whose planes
+ * on the FFMA kernels), bf16 with 64 features there 12 and 24; on the FFMA kernels 8 and 16, but for 64 columns whatever
+ * head_dim is.  Problems whose planes
  * would take more than 64 GiB stay on the FFMA kernels. */
 size_t wersa_workspace_bytes(const wersa_config* cfg);
 

@@ -126,7 +126,7 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     ffma_cost = best;
   }
 
-  // fp32 on the tensor cores: one CTA per SM and group, in chunks that minimise waves x (tiles + 3), 3 tiles being about what
+  // fp32 arithmetic on the tensor cores, of fp32 tensors and of bf16 ones with m = 64: one CTA per SM and group, in chunks that minimise waves x (tiles + 3), 3 tiles being about what
   // a CTA spends before its first and after its last one, and a 64th of a tile for a chunk's partial in the reduction.  Up to
   // a chunk per SM: one slab of 131072, m = 128 in 64 chunks against 147, forward d = 16 121 -> 83 us (FFMA 101), d = 64 165 ->
   // 124; training step d = 16 368 -> 239 (294), d = 64 500 -> 348.
@@ -138,17 +138,17 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   //            512 x 64, d = 32, m = 128 77 89;  256 x 64 54 49;    300 x 128 77 65;    100 x 200 62 34
   //            512 x 32, d = 64, m = 256 164 156; 148 x 40 50 52;   1023 x 16 192 314;  200 x 50, m = 128 76 50
   //   backward 300 x 128, d = 16, m = 128 109 123; 8 x 8192 111 97; 512 x 64, d = 32 146 178; 300 x 128 155 136
-  // From kXUnits tiles x groups of 128 features on, the backward from one tile per SM on (below these lines planes have not
-  // been chosen, whatever the estimates say).
+  // With m = 128, 256 from kXUnits tiles x groups of 128 features on, the backward from one tile per SM on (below these lines
+  // planes have not been chosen, whatever the estimates say).
   // Their operands as planes take more memory than the FFMA kernels' fp32 ones (see the layout below): a problem that asks
   // for more than kXBytes of it stays with those, so that what fitted the device beside its tensors before still does.
   p->use_x = p->use_xb = false;
   p->xchunks = p->xbchunks = 1;
   p->xchunk_tiles = p->xbchunk_tiles = 1;
   p->xprep = 0;
-  if (!p->bf16 && !(c.flags & WERSA_FLAG_SIMT_ONLY) && m >= 128) {
-    const int tiles = ceil_div(n, 128), groups = m / 128;
-    const double plane_bytes = (p->with_backward ? 32. : 18.) * p->slabs * n * c.head_dim;
+  if (!p->use_tc && !(c.flags & WERSA_FLAG_SIMT_ONLY)) {
+    const int tiles = ceil_div(n, 128), groups = m <= 128 ? 1 : m / 128;
+    const double plane_bytes = (p->bf16 ? p->with_backward ? 24. : 12. : p->with_backward ? 32. : 18.) * p->slabs * n * c.head_dim;
     long long best = 0;
     for (int ch = 1; ch <= tiles && ch <= p->sms; ++ch) {
       const long long cost = (long long)ceil_div(p->slabs * groups * ch, p->sms) * (ceil_div(tiles, ch) + 3) * 64 + ch;
@@ -169,13 +169,32 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     p->xbchunk_tiles = ceil_div(tiles, p->xbchunks);
     p->xbchunks = ceil_div(tiles, p->xbchunk_tiles);
     const int width = c.head_dim <= 16 ? 0 : c.head_dim <= 32 ? 1 : 2;
-    constexpr double kFwd[2][3] = {{0.13, 0.205, 0.345}, {0.17, 0.25, 0.46}}, kBwd[2][3] = {{0.275, 0.445, 0.745}, {0.33, 0.53, 0.8}};
-    const double f_fwd = 14 + kFwd[p->simt_small][width] * ffma_cost, f_bwd = 15 + kBwd[p->simt_small][width] * ffma_cost;
     const int waves = ceil_div(p->slabs * groups * p->xchunks, p->sms), bwaves = ceil_div(p->slabs * p->xbchunks, p->sms) * groups;
-    const double x_fwd = 9 + (12.5 + 6 * p->xchunk_tiles) * waves + 0.02 * p->xchunks;
-    const double x_bwd = 14.5 + (15 + 3 * p->xchunk_tiles) * waves + 9. * bwaves * (p->xbchunk_tiles + 1);
-    p->use_x = (long long)p->slabs * tiles * groups >= kXUnits && x_fwd <= f_fwd && plane_bytes <= kXBytes;
-    p->use_xb = p->use_x && p->with_backward && !p->grad_bf16 && (long long)p->slabs * tiles >= p->sms && x_bwd <= f_bwd;
+    double f_fwd, f_bwd, x_fwd, x_bwd;
+    bool enough = true, enough_b = true;
+    if (m >= 128) {
+      constexpr double kFwd[2][3] = {{0.13, 0.205, 0.345}, {0.17, 0.25, 0.46}}, kBwd[2][3] = {{0.275, 0.445, 0.745}, {0.33, 0.53, 0.8}};
+      f_fwd = 14 + kFwd[p->simt_small][width] * ffma_cost;
+      f_bwd = 15 + kBwd[p->simt_small][width] * ffma_cost;
+      x_fwd = 9 + (12.5 + 6 * p->xchunk_tiles) * waves + 0.02 * p->xchunks;
+      x_bwd = 14.5 + (15 + 3 * p->xchunk_tiles) * waves + 9. * bwaves * (p->xbchunk_tiles + 1);
+      enough = (long long)p->slabs * tiles * groups >= kXUnits;
+      enough_b = (long long)p->slabs * tiles >= p->sms;
+    } else {
+      // m = 64, fitted to 220 shapes (1 to 1023 slabs, 16 to 131072 tokens, d = 16 to 64, fp32 and bf16; rms 5 % off for planes, 8
+      // and 13 % for FFMA; 14 of 440 choices cost more than 5 %, the worst 13 %).  FFMA and planes, us: forward bf16 1 x 7861, d = 16
+      // 26 24; 237 x 20 24 40; 1 x 7258, d = 64 32 24; 14 x 21903 405 160; fp32 1 x 1024 20.9 21.4; 2 x 36480 94 69; training step
+      // bf16 212 x 355 444 204.  From 24 tiles on, the fewest of the fit.
+      constexpr double kFwd[2][3] = {{0.144, 0.216, 0.371}, {0.184, 0.291, 0.426}}, kBwd[2][3] = {{0.291, 0.428, 0.754}, {0.404, 0.59, 0.805}};
+      const double elems = 1e-6 * p->slabs * n * c.head_dim, wt = (double)waves * p->xchunk_tiles, bt = (double)bwaves * (p->xbchunk_tiles + 1);
+      f_fwd = 11.2 + kFwd[p->simt_small][width] * ffma_cost;
+      f_bwd = 10.3 + kBwd[p->simt_small][width] * ffma_cost;
+      x_fwd = p->bf16 ? 6.8 + 12.7 * waves + 3.06 * wt + 4.34 * elems : 7.2 + 12.2 * waves + 4.23 * wt + 6.07 * elems;
+      enough = (long long)p->slabs * tiles >= 24;
+      x_bwd = p->bf16 ? 5.3 + 23.5 * waves + 3.47 * wt + 3.08 * bt + 8.23 * elems : 6.6 + 24 * waves + 5.64 * wt + 2.29 * bt + 10.2 * elems;
+    }
+    p->use_x = enough && x_fwd <= f_fwd && plane_bytes <= kXBytes && p->slabs < 65535;
+    p->use_xb = p->use_x && p->with_backward && (p->bf16 || !p->grad_bf16) && enough_b && x_bwd <= f_bwd;
     p->xprep = (int)std::min<long long>(((long long)p->slabs * n * 8 + 255) / 256, 8LL * p->sms);
   }
 
@@ -271,18 +290,19 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
   take(p->dpad ? 256 : 0);
   p->off_Og = take(grouped ? io_bytes * slab_elems * p->groups : 0);
   p->off_den = take(grouped ? sizeof(float) * slabs * n * p->groups : 0);
-  // fp32 on the tensor cores: bytes per element of a tensor (slabs x n x head_dim: narrow heads pay for their own columns).
+  // fp32 arithmetic on the tensor cores: bytes per element of a tensor (slabs x n x head_dim: narrow heads pay for their own columns).
   // Planes of T_f(Q), T_f(K) and V, 18 in all, over whose last two lie first the query side's shares of a forward without a
   // backward (see launch_tcx_qside), then dQ_F and dK_F of an FFMA backward, which keeps T_f(Q) and T_f(K) as well: 26.  A
   // backward on the planes: O (4), dQ_F (4) and planes of dO (6), 32 in all; the forward's shares lie over the last two,
-  // dK_F over the planes of dO, which its kernels no longer read.  FFMA alone: 8 and 16, 64 columns each.
+  // dK_F over the planes of dO, which its kernels no longer read.  bf16 tensors have planes of T_f(Q) and T_f(K) alone, 12 and 24
+  // (24 with an FFMA backward).  FFMA alone: 8 and 16, 64 columns each.
   const size_t tensor = slabs * (size_t)n * c.head_dim, plane3 = 3 * sizeof(__nv_bfloat16) * tensor;
   p->off_dO3 = p->off_xO = p->off_xden = p->off_xinv = p->off_xc = p->off_xshare = 0;
   p->off_QF = p->off_KF = p->off_QF3 = p->off_KF3 = p->off_V3 = p->off_dQF = p->off_dKF = 0;
   if (p->use_x) {
     p->off_QF3 = take(plane3);
     p->off_KF3 = take(plane3);
-    p->off_V3 = take(plane3);
+    p->off_V3 = take(!p->bf16 ? plane3 : ffma_bwd ? sizeof(float) * tensor : 0);   // (bf16: of use to dK_F below alone)
     if (ffma_bwd) {
       p->off_QF = take(sizeof(float) * tensor);
       p->off_KF = take(sizeof(float) * tensor);
@@ -298,13 +318,13 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     p->off_dz = take(sizeof(float) * slabs * m);
     p->off_sumdD = take(sizeof(float) * (p->use_tc ? (size_t)p->bctas : p->use_xb ? (size_t)p->xprep : slabs * p->schunks));
     if (p->use_xb) {
-      const size_t groups = c.features / 128, padded = (size_t)ceil_div(c.seq_len, 128) * 128;
+      const size_t groups = c.features <= 128 ? 1 : c.features / 128, padded = (size_t)ceil_div(c.seq_len, 128) * 128;
       p->off_xO = take(sizeof(float) * tensor);
       p->off_xden = take(sizeof(float) * groups * slabs * c.seq_len);
       p->off_xinv = take(sizeof(float) * slabs * padded);
       p->off_xc = take(sizeof(float) * slabs * padded);
       p->off_dQF = p->off_xshare = take(sizeof(float) * tensor);
-      p->off_dO3 = p->off_dKF = take(plane3);
+      p->off_dO3 = p->off_dKF = take(p->bf16 ? sizeof(float) * tensor : plane3);
     }
     p->off_bands = take(sizeof(float) * 2 * slabs * 2 * p->htiles * kBandVals);   // Q and K; two column halves per tile
     p->off_dqbar = take(sizeof(float) * slabs * (kD + kBandVals));
@@ -555,9 +575,8 @@ wersa_status wersa_forward(wersa_ctx* ctx, const void* Q, const void* K, const v
                  launch_reduce_partials(p, w.spart, w.zpart, p.tchunks, w.S, w.z, p.with_backward ? w.Sbf : nullptr, w.Simg, st, &launches));
     WERSA_STEP(0, "tc_qside", launch_tc_qside(p, w, Q, beta, O, nullptr, st, &launches));
   } else if (p.use_x) {
-    WERSA_STEP(0, "f32_planes", launch_f32_planes(p, w, static_cast<const float*>(Q), static_cast<const float*>(K),
-                                                  static_cast<const float*>(V), p.with_backward && !p.use_xb, st, &launches));
-    WERSA_STEP(0, "tcx_kside", launch_tcx_kside(p, w, W, st, &launches));
+    WERSA_STEP(0, "f32_planes", launch_f32_planes(p, w, Q, K, V, p.with_backward && !p.use_xb, st, &launches));
+    WERSA_STEP(0, "tcx_kside", launch_tcx_kside(p, w, V, W, st, &launches));
     WERSA_STEP(0, "reduce_partials",
                launch_reduce_partials(p, w.spart, w.zpart, p.xchunks, w.S, w.z, nullptr, nullptr, st, &launches));
     WERSA_STEP(0, "tcx_qside", launch_tcx_qside(p, w, W, beta, O, st, &launches));
@@ -793,7 +812,7 @@ wersa_status wersa_backward(wersa_ctx* ctx, const void* Q, const void* K, const 
     WERSA_STEP(1, "tc_bwd_qside", launch_tc_bwd_qside(p, w, w.QF3, beta, dO, nullptr, nullptr, false, st, &launches));
   } else if (p.use_xb) {
     WERSA_STEP(1, "tcx_bwd_prep", launch_tcx_bwd_prep(p, w, dO, beta, st, &launches));
-    WERSA_STEP(1, "tcx_bwd_qside", launch_tcx_bwd_qside(p, w, W, st, &launches));
+    WERSA_STEP(1, "tcx_bwd_qside", launch_tcx_bwd_qside(p, w, W, dO, st, &launches));
   } else {
     WERSA_STEP(1, "simt_bwd_qside", launch_simt_bwd_qside(p, w, W, beta, dO, st, &launches));
   }
@@ -807,7 +826,7 @@ wersa_status wersa_backward(wersa_ctx* ctx, const void* Q, const void* K, const 
   } else if (p.use_tc) {
     WERSA_STEP(1, "tc_bwd_kside", launch_tc_bwd_kside(p, w, w.KF3, V, dV, false, st, &launches));
   } else if (p.use_xb) {
-    WERSA_STEP(1, "tcx_bwd_kside", launch_tcx_bwd_kside(p, w, W, dV, st, &launches));
+    WERSA_STEP(1, "tcx_bwd_kside", launch_tcx_bwd_kside(p, w, V, W, dV, st, &launches));
   } else {
     WERSA_STEP(1, "simt_bwd_kside", launch_simt_bwd_kside(p, w, V, W, dV, st, &launches));
   }

@@ -114,8 +114,8 @@ cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const 
 // with X2 also XF3_2 from X2 in the same launch, with split_S also w.Slo = bf16(w.S - w.Sbf).
 cudaError_t launch_haar_filter_split3(const Plan& p, const Ws& w, const void* X, __nv_bfloat16* XF3, const void* X2,
                                       __nv_bfloat16* XF3_2, bool split_S, cudaStream_t st, int* launches);
-// fp32 tensors: w.QF3 = T_f(Q), w.KF3 = T_f(K) and w.V3 = V as planes; with keep also w.QF and w.KF.
-cudaError_t launch_f32_planes(const Plan& p, const Ws& w, const float* Q, const float* K, const float* V, bool keep,
+// w.QF3 = T_f(Q), w.KF3 = T_f(K) and, of fp32 tensors, w.V3 = V as planes; with keep also w.QF and w.KF.
+cudaError_t launch_f32_planes(const Plan& p, const Ws& w, const void* Q, const void* K, const void* V, bool keep,
                               cudaStream_t st, int* launches);
 // dX = T_f(G) + vec[slab] * vec_scale on every row (G fp32, vec = slabs x 64 floats).
 cudaError_t launch_haar_filter_addvec(const Plan& p, const float* G, const float* f, const float* vec,
@@ -150,12 +150,12 @@ cudaError_t launch_simt_bwd_kside(const Plan& p, const Ws& w, const void* V, con
 // fp32 on the tensor cores.  Forward: partial S', z' (p.xchunks per slab) from w.KF3 and w.V3; O from w.QF3, w.S and w.z,
 // with a backward also w.xO and w.xden.  Backward: dO as planes and what the division leaves per token; dQ_F, partial dS',
 // dz'; dK_F and dV.
-cudaError_t launch_tcx_kside(const Plan& p, const Ws& w, const void* W, cudaStream_t st, int* launches);
+cudaError_t launch_tcx_kside(const Plan& p, const Ws& w, const void* V, const void* W, cudaStream_t st, int* launches);
 cudaError_t launch_tcx_qside(const Plan& p, const Ws& w, const void* W, const float* beta, void* O, cudaStream_t st, int* launches);
 
 cudaError_t launch_tcx_bwd_prep(const Plan& p, const Ws& w, const void* dO, const float* beta, cudaStream_t st, int* launches);
-cudaError_t launch_tcx_bwd_qside(const Plan& p, const Ws& w, const void* W, cudaStream_t st, int* launches);
-cudaError_t launch_tcx_bwd_kside(const Plan& p, const Ws& w, const void* W, void* dV, cudaStream_t st, int* launches);
+cudaError_t launch_tcx_bwd_qside(const Plan& p, const Ws& w, const void* W, const void* dO, cudaStream_t st, int* launches);
+cudaError_t launch_tcx_bwd_kside(const Plan& p, const Ws& w, const void* V, const void* W, void* dV, cudaStream_t st, int* launches);
 
 // ---- tc_fwd.cu -----------------------------------------------------------------------------
 // Both read the raw bf16 tensors and apply the Haar filter (coefficients from w.f) on chip.  first: the first kernel of its

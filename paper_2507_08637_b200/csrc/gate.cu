@@ -104,8 +104,8 @@ __device__ __forceinline__ void batch_gate(int b, int H, int L1, const float* __
 // (a counter per slab) then runs slab_gate, and for the batch-wide gate the last slab of a batch
 // element (a counter per batch element) runs batch_gate; sums are taken in a fixed order, so the
 // result does not depend on which CTA comes last.  The counters start at zero and are left at zero.
-// Row y == slabs (only with W != nullptr): bf16 transpose Wt (m x 64) of W (64 x m) for the
-// tensor-core kernels.
+// Row y == slabs (only of bf16 tensors, with W or seen): bf16 transpose Wt (m x 64) of W (64 x m) for the tensor-core kernels;
+// seen is cleared there.
 // kFull = false: Q has dcols < 64 columns (a multiple of 8), gate_w dcols rows per head and W dcols rows;
 // dcols / 8 threads share a row, 256 / (dcols / 8) rows are in flight per pass, and the partial sums, q-bar
 // and W^T come out 64 wide with zeros in the columns past dcols.  fp32 tensors keep the 64-wide assignment
@@ -129,6 +129,8 @@ __global__ void __launch_bounds__(256) k_qmean_gate(const T* __restrict__ Q, flo
     if (seen != nullptr && blockIdx.x + blockIdx.y == 0 && threadIdx.x < 2) seen[threadIdx.x] = 0;   // see k_f32_planes
   }
   if ((int)blockIdx.y == slabs) {
+    if (sizeof(T) == 2 && seen != nullptr && blockIdx.x == 0 && threadIdx.x < 2) seen[threadIdx.x] = 0;   // see k_f32_planes
+    if (W == nullptr) return;
     // A thread takes eight columns of W^T's row r: neighbouring threads read neighbouring features and store 16 bytes.  (An
     // element a thread reads 2 bytes out of 32 different sectors a warp, and the grid's other CTAs wait for nothing else:
     // with two chunks a slab and m = 1024 this row took as long as all of the mean pool, 24.9 us; now 12.4.)
@@ -443,7 +445,7 @@ static cudaError_t launch_qmean_gate_impl(const Plan& p, const void* Q, float* q
                                           const float* gate_b, const float* omega, float* qbar, float* sg, float* f,
                                           int* counters, const void* W, __nv_bfloat16* Wt, int cols,
                                           int* seen, cudaStream_t st) {
-  dim3 grid(p.qchunks, p.slabs + (W != nullptr ? 1 : 0));
+  dim3 grid(p.qchunks, p.slabs + (W != nullptr || (p.bf16 && seen != nullptr) ? 1 : 0));
   int* slab_count = counters;
   int* batch_count = counters + p.slabs;
   cudaError_t launch_err = cudaSuccess;

@@ -210,10 +210,10 @@ __global__ void __launch_bounds__(256, 4) k_haar_filter(const Tin* __restrict__ 
 // carries the fp32 value; see k_haar_filter_split3), and for a backward that will want them T_f(Q) and T_f(K) themselves.
 // Tiles and arithmetic are those of k_haar_filter; all three tensors are arguments and fetched ahead of the wait.  Bound by
 // memory: 640 bytes a row of 64 columns and tensor, 2 x 8 x 4096 19 us, 6.6 TB/s.
-// grid (col_blocks<32>, slabs, 3), block 256.
-template <bool kFull, bool kKeep>
-__global__ void __launch_bounds__(256, 3) k_f32_planes(const float* __restrict__ Q, const float* __restrict__ K,
-                                                       const float* __restrict__ V, const float* __restrict__ f,
+// grid (col_blocks<32>, slabs, 3; of bf16 tensors 2: V is its own plane), block 256.
+template <bool kFull, bool kKeep, typename Tin>
+__global__ void __launch_bounds__(256, 3) k_f32_planes(const Tin* __restrict__ Q, const Tin* __restrict__ K,
+                                                       const Tin* __restrict__ V, const float* __restrict__ f,
                                                        __nv_bfloat16* __restrict__ Q3, __nv_bfloat16* __restrict__ K3,
                                                        __nv_bfloat16* __restrict__ V3, float* __restrict__ QF,
                                                        float* __restrict__ KF, size_t plane, int n, int d_arg, int L,
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(256, 3) k_f32_planes(const float* __restrict__
   const int rows = at.on ? n - row0 : 0;   // rows of this thread inside the sequence
   const size_t first = ((size_t)slab * n + row0) * d + at.col;
   const bool filtered = blockIdx.z < 2;
-  const float* __restrict__ X = blockIdx.z == 0 ? Q : blockIdx.z == 1 ? K : V;
+  const Tin* __restrict__ X = blockIdx.z == 0 ? Q : blockIdx.z == 1 ? K : V;
   float x[8][4];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -702,16 +702,21 @@ cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const 
   return err != cudaSuccess ? err : cudaGetLastError();
 }
 
-cudaError_t launch_f32_planes(const Plan& p, const Ws& w, const float* Q, const float* K, const float* V, bool keep,
+cudaError_t launch_f32_planes(const Plan& p, const Ws& w, const void* Q, const void* K, const void* V, bool keep,
                               cudaStream_t st, int* launches) {
   const int n = p.cfg.seq_len, L = p.cfg.levels, d = p.cfg.head_dim;
-  const dim3 grid(col_blocks<32>(p.htiles, d), p.slabs, 3);
+  const dim3 grid(col_blocks<32>(p.htiles, d), p.slabs, p.bf16 ? 2 : 3);
   const size_t plane = (size_t)p.slabs * n * d;
   cudaError_t err;
-  auto go = [&](auto kernel) {
-    return launch_after(kernel, grid, dim3(256), 0, st, Q, K, V, (const float*)w.f, w.QF3, w.KF3, w.V3, w.QF, w.KF, plane, n, d, L, w.seen);
+  auto go = [&](auto kernel, auto* q) {
+    using P = decltype(q);
+    return launch_after(kernel, grid, dim3(256), 0, st, q, (P)K, (P)V, (const float*)w.f, w.QF3, w.KF3, w.V3, w.QF, w.KF, plane, n, d, L, w.seen);
   };
-  WERSA_FULL({ err = keep ? go(k_f32_planes<kFull, true>) : go(k_f32_planes<kFull, false>); })
+  using bf = __nv_bfloat16;
+  WERSA_FULL({
+    if (p.bf16) err = keep ? go(k_f32_planes<kFull, true, bf>, (const bf*)Q) : go(k_f32_planes<kFull, false, bf>, (const bf*)Q);
+    else err = keep ? go(k_f32_planes<kFull, true, float>, (const float*)Q) : go(k_f32_planes<kFull, false, float>, (const float*)Q);
+  })
   *launches += 1;
   return err != cudaSuccess ? err : cudaGetLastError();
 }

@@ -37,10 +37,15 @@ namespace {
 constexpr int kTile = 128;
 constexpr uint32_t kTileBytes = kTile * kD * 2;   // one plane of a tile: 128 x 64 bf16
 constexpr uint32_t kTileStep = kTileBytes >> 4;   // in descriptor units
-constexpr int kXFeatures = 128;                   // features of a CTA
+constexpr int kXFeatures = 128;                   // features of a CTA at most
+// Features of a CTA in kernels of NF; planes of an argument of type T (a bf16 value is its own first plane, and the products
+// with the other two are left out).
+template <typename T> constexpr bool kExact = sizeof(T) == 2;
+template <typename T> constexpr uint32_t kPlanes = kExact<T> ? 1 : 3;
+__device__ __forceinline__ float arg(float x) { return x; }
+__device__ __forceinline__ float arg(__nv_bfloat16 x) { return __bfloat162float(x); }
 constexpr int kXThreads = 512;
 constexpr uint32_t kBufCols = 192, kLoCol = 128, kAccCol = 384;   // TMEM columns
-constexpr uint32_t kIdesc1 = make_idesc_bf16(128, 128, false, false);   // both operands K-major
 constexpr uint32_t kIdesc2 = make_idesc_bf16(128, 64, false, true);     // B = V or S', N-major
 enum { kErrXCopy = 31, kErrXMma = 32, kErrXElem = 33, kErrXDrain = 34 };
 enum { kBarZ = 1, kBarDrain = 2 };
@@ -52,32 +57,36 @@ __device__ __forceinline__ float put_back(float x) { return fmaf(x, kCut, x); }
 
 // Plane products in the order they are added.
 __device__ constexpr int kPa[6] = {2, 0, 1, 1, 0, 0}, kPb[6] = {0, 2, 1, 0, 1, 0};
+// (with kExactA / kExactB only those of the operand's first plane)
+template <bool kExactA, bool kExactB> __device__ constexpr bool product_on(int q) { return (!kExactA || kPa[q] == 0) && (!kExactB || kPb[q] == 0); }
+template <bool kExactA, bool kExactB> __device__ constexpr int first_product() { return product_on<kExactA, kExactB>(0) ? 0 : 1; }
 
 struct alignas(8) XBars {
   uint64_t x_full[2], x_empty[2], v_full, v_empty, d1_full[2], phi_ready[2], d1_free[2], acc_full[2], acc_free[2], den_free[2];
   uint32_t tmem_base;
   int abort_flag;
 };
-struct KxSmem {
+template <typename T> struct KxSmem {
   static constexpr uint32_t wt = 0;                          // planes of W^T (128 features x 64)
-  static constexpr uint32_t x = wt + 3 * kTileBytes;         // two stages of K_F planes
+  static constexpr uint32_t x = wt + kPlanes<T> * kTileBytes;   // two stages of K_F planes
   static constexpr uint32_t v = x + 6 * kTileBytes;          // planes of V
-  static constexpr uint32_t sum = v + 3 * kTileBytes;        // S' of the chunk so far: 64 x 128 floats, features side by side
+  static constexpr uint32_t sum = v + kPlanes<T> * kTileBytes;        // S' of the chunk so far: 64 x 128 floats, features side by side
   static constexpr uint32_t zx = sum + 2 * kTileBytes;       // 128 floats
   static constexpr uint32_t bars = zx + 512;
   static constexpr uint32_t total = bars + 256 + 1024;       // + alignment slack
 };
-struct QxSmem {
+template <typename T> struct QxSmem {
   static constexpr uint32_t wt = 0;
-  static constexpr uint32_t s = wt + 3 * kTileBytes;         // planes of S' (128 features x 64)
+  static constexpr uint32_t s = wt + kPlanes<T> * kTileBytes;   // planes of S' (128 features x 64)
   static constexpr uint32_t x = s + 3 * kTileBytes;          // two stages of Q_F planes
   static constexpr uint32_t out = x + 6 * kTileBytes;        // result tile: two boxes of 128 rows x 32 floats
-  static constexpr uint32_t zs = out + 2 * kTileBytes;       // z' of the group
+  static constexpr uint32_t out16 = out + 2 * kTileBytes;    // the same as bf16
+  static constexpr uint32_t zs = out16 + (kExact<T> ? kTileBytes : 0);       // z' of the group
   static constexpr uint32_t den = zs + 512;                  // denominators of two tiles
   static constexpr uint32_t bars = den + 2 * 512;
   static constexpr uint32_t total = bars + 256 + 1024;
 };
-static_assert(QxSmem::total <= 232448 && KxSmem::total <= 232448 && sizeof(XBars) <= 256, "shared memory of an SM");
+static_assert(QxSmem<float>::total <= 232448 && KxSmem<float>::total <= 232448 && sizeof(XBars) <= 256, "shared memory of an SM");
 
 // Tokens of a slab in the per-token arrays of the backward: whole tiles, since they are read past n and in pairs (a slab has
 // to begin on an 8-byte boundary where n is odd).
@@ -118,8 +127,9 @@ __device__ __forceinline__ bool put_planes8(uint8_t* tile, int row, int chunk, c
     *reinterpret_cast<uint4*>(tile + s * kTileBytes + swz128(row, chunk)) = make_uint4(p[s][0], p[s][1], p[s][2], p[s][3]);
   return bad;
 }
-// W (d x m, row-major) -> planes of rows f0 .. f0 + 127 of W^T, zero past column d.  512 threads.  The answer is split8's.
-__device__ __forceinline__ bool load_w_planes(const float* __restrict__ W, int d, int m, int f0, uint8_t* wt) {
+// W (d x m, row-major) -> planes of rows f0 .. f0 + 127 of W^T, zero past column d and row m.  512 threads.  The answer is split8's.
+template <typename T>
+__device__ __forceinline__ bool load_w_planes(const T* __restrict__ W, int d, int m, int f0, uint8_t* wt) {
   const int f = threadIdx.x & 127, part = threadIdx.x >> 7;   // 16 columns
   bool bad = false;
 #pragma unroll
@@ -128,24 +138,38 @@ __device__ __forceinline__ bool load_w_planes(const float* __restrict__ W, int d
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int c = 16 * part + 8 * h + j;
-      v[j] = c < d ? W[(size_t)c * m + f0 + f] : 0.f;
+      v[j] = c < d && f0 + f < m ? arg(W[(size_t)c * m + f0 + f]) : 0.f;
     }
-    bad |= put_planes8(wt, f, 2 * part + h, v);
+    if constexpr (kExact<T>) {
+      uint32_t u[4], top = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        u[i] = pack_bf16x2(v[2 * i], v[2 * i + 1]);
+        top |= full_exponents(u[i]);
+      }
+      bad |= top != 0;
+      *reinterpret_cast<uint4*>(wt + swz128(f, 2 * part + h)) = make_uint4(u[0], u[1], u[2], u[3]);
+    } else {
+      bad |= put_planes8(wt, f, 2 * part + h, v);
+    }
   }
   return bad;
 }
 // S' or dS' of a slab's features f0 .. f0 + 127 (64 columns) -> planes, and the group's z' or dz' -> zs: results of the kernel
 // in front (see launch_after).  512 threads.
+template <int NF>
 __device__ __forceinline__ void load_s_planes(const float* S, const float* zg, size_t row0, uint8_t* tile, float* zs) {
   const int f = threadIdx.x >> 2, part = threadIdx.x & 3;   // 16 columns of a feature's row
   const float* src = S + (row0 + f) * kD + 16 * part;
+  if (NF == kXFeatures || f < NF) {
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const float4 a = __ldcg(reinterpret_cast<const float4*>(src + 8 * h)), b = __ldcg(reinterpret_cast<const float4*>(src + 8 * h + 4));
-    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    put_planes8(tile, f, 2 * part + h, v);
+    for (int h = 0; h < 2; ++h) {
+      const float4 a = __ldcg(reinterpret_cast<const float4*>(src + 8 * h)), b = __ldcg(reinterpret_cast<const float4*>(src + 8 * h + 4));
+      const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+      put_planes8(tile, f, 2 * part + h, v);
+    }
   }
-  if (threadIdx.x < kXFeatures) zs[threadIdx.x] = __ldcg(zg + row0 + threadIdx.x);
+  if (threadIdx.x < NF) zs[threadIdx.x] = __ldcg(zg + row0 + threadIdx.x);
 }
 
 // The planes of an infinite value are infinity, NaN and NaN: what the tensor cores make of a dot product that meets one is NaN,
@@ -153,9 +177,9 @@ __device__ __forceinline__ void load_s_planes(const float* S, const float* zg, s
 // the planes' sums and W.  (Only their class matters: a NaN came from an operand that is not finite.)  The kernels look for
 // them where W holds one (which they see as they read it) or the projected tensor does (k_f32_planes leaves word); looking
 // every time cost 1 us in each of the kernels of 2 x 4 x 4096, d = 32, m = 128 (a training step 107 -> 110).
-struct Operands {
+template <typename T> struct Operands {
   const __nv_bfloat16* x3;   // first plane: slabs x n rows of d values
-  const float* W;            // d x m
+  const T* W;                // d x m
   int slab, slabs, n, d, m;
   bool look;                 // is there anything that is not finite?
 };
@@ -170,7 +194,8 @@ __device__ __forceinline__ bool warp_meets_nan(const uint32_t (&r)[32]) {
   return __any_sync(0xffffffffu, s != s);
 }
 // The NaN among the 32 columns at taddr again.  Column j of a lane is token tok + j * dtok, feature feat + j * dfeat.
-__device__ __noinline__ void form_again(uint32_t taddr, const Operands op, int tok, int dtok, int feat, int dfeat) {
+template <typename T>
+__device__ __noinline__ void form_again(uint32_t taddr, const Operands<T> op, int tok, int dtok, int feat, int dfeat) {
   const size_t plane = (size_t)op.slabs * op.n * op.d;
   for (int j = 0; j < 32; ++j, tok += dtok, feat += dfeat) {
     uint32_t r;
@@ -183,7 +208,7 @@ __device__ __noinline__ void form_again(uint32_t taddr, const Operands op, int t
       for (int c = 0; c < op.d && a == a; ++c) {
         float v = __bfloat162float(__ldcg(x + c));
         if (fabsf(v) < INFINITY) v = (v + __bfloat162float(__ldcg(x + plane + c))) + __bfloat162float(__ldcg(x + 2 * plane + c));
-        a = fmaf(v, op.W[(size_t)c * op.m + feat], a);
+        a = fmaf(v, arg(op.W[(size_t)c * op.m + feat]), a);
       }
       r = __float_as_uint(a);
     }
@@ -193,7 +218,8 @@ __device__ __noinline__ void form_again(uint32_t taddr, const Operands op, int t
   tmem_st_wait();
 }
 // 32 columns of pre-activations.
-__device__ __forceinline__ void load_projected(uint32_t taddr, uint32_t (&r)[32], const Operands& op, int tok, int dtok, int feat,
+template <typename T>
+__device__ __forceinline__ void load_projected(uint32_t taddr, uint32_t (&r)[32], const Operands<T>& op, int tok, int dtok, int feat,
                                                int dfeat) {
   tmem_ld32(taddr, r);
   tmem_ld_wait();
@@ -212,13 +238,14 @@ __device__ __forceinline__ void load_projected(uint32_t taddr, uint32_t (&r)[32]
 // kScaled: the values are multiplied by s[column] first, and the sum is of those times w[column]; both arrays in global
 // memory, on an 8-byte boundary, and may hold anything where the value is zero.
 // kTokens: the columns are tokens from tok on and the lane is feature feat, else the other way round.
-template <bool kTokens, bool kWeighted, bool kScaled = false>
-__device__ __forceinline__ float relu_planes(uint32_t taddr, const Operands& op, int tok, int feat, const float* w,
+// NC: columns / 32.
+template <int NC, bool kTokens, bool kWeighted, bool kScaled = false, typename T>
+__device__ __forceinline__ float relu_planes(uint32_t taddr, const Operands<T>& op, int tok, int feat, const float* w,
                                              const float* s = nullptr) {
   uint32_t r[32];
   float total = 0.f;
 #pragma unroll 1
-  for (int c = 0; c < 4; ++c) {
+  for (int c = 0; c < NC; ++c) {
     load_projected(taddr + 32 * c, r, op, tok + (kTokens ? 32 * c : 0), kTokens, feat + (kTokens ? 0 : 32 * c), !kTokens);
     uint32_t hi[16], mid[16], lo[16];
     float e[4] = {0.f, 0.f, 0.f, 0.f};
@@ -274,25 +301,29 @@ __device__ __forceinline__ void init_bars(XBars* b) {
   fence_mbar_init();
 }
 
-// Three planes of one tile.
+// The planes of one tile.
+template <uint32_t kN = 3>
 __device__ __forceinline__ void load_planes(uint8_t* dst, const CUtensorMap* map, int row0, int slab, int slabs, uint64_t* bar) {
-  mbar_arrive_expect_tx(bar, 3 * kTileBytes);
+  mbar_arrive_expect_tx(bar, kN * kTileBytes);
 #pragma unroll
-  for (int pl = 0; pl < 3; ++pl) tma_load_3d(dst + pl * kTileBytes, map, 0, row0, pl * slabs + slab, bar);
+  for (uint32_t pl = 0; pl < kN; ++pl) tma_load_3d(dst + pl * kTileBytes, map, 0, row0, pl * slabs + slab, bar);
 }
 
-// D[128 x 128] = A B^T over the head dimension in steps of 16 columns, both operands as planes of 128 rows x 64 columns.
+// D[128 x N] = A B^T over the head dimension in steps of 16 columns, both operands as planes of up to 128 rows x 64 columns.
+template <int N, bool kExactA, bool kExactB>
 __device__ __forceinline__ void issue_planes(uint32_t dst, uint32_t a_lo, uint32_t b_lo, int ksteps, uint32_t hi) {
+  constexpr uint32_t kIdesc1 = make_idesc_bf16(128, N, false, false);   // both operands K-major
 #pragma unroll
   for (int q = 0; q < 6; ++q)
+    if (product_on<kExactA, kExactB>(q))
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (k < ksteps)
-        mma_ss(dst, smem_desc_join(a_lo + kPa[q] * kTileStep + 2 * k, hi), smem_desc_join(b_lo + kPb[q] * kTileStep + 2 * k, hi),
-               kIdesc1, (q > 0 || k > 0) ? 1u : 0u);
+      for (int k = 0; k < 4; ++k)
+        if (k < ksteps)
+          mma_ss(dst, smem_desc_join(a_lo + kPa[q] * kTileStep + 2 * k, hi), smem_desc_join(b_lo + kPb[q] * kTileStep + 2 * k, hi),
+                 kIdesc1, (q > first_product<kExactA, kExactB>() || k > 0) ? 1u : 0u);
 }
-// MMA1 of every tile.  kXIsA: the tile is A (query side: tokens x features), else W^T is (key side: features x tokens).
-template <bool kXIsA>
+// MMA1 of every tile.  kXIsA: the tile is A (query side: tokens x NF features), else W^T is (key side: features x tokens).
+template <bool kXIsA, int NF, bool kExactW>
 __device__ __forceinline__ void issue_mma1(XBars* bars, uint8_t* x, uint8_t* wt, uint32_t tmem, int nt, int d,
                                            volatile int* abort_flag, int* status) {
   const uint32_t hi = smem_desc_hi(1024);
@@ -304,36 +335,38 @@ __device__ __forceinline__ void issue_mma1(XBars* bars, uint8_t* x, uint8_t* wt,
     if (t >= 2 && !mbar_wait(&bars->d1_free[b], ((t >> 1) - 1) & 1, abort_flag, status, kErrXMma)) break;
     tc_fence_after_sync();
     const uint32_t x_lo = x_lo0 + b * 3 * kTileStep;
-    issue_planes(tmem + b * kBufCols, kXIsA ? x_lo : wt_lo, kXIsA ? wt_lo : x_lo, ksteps, hi);
+    issue_planes<kXIsA ? NF : 128, !kXIsA && kExactW, kXIsA && kExactW>(tmem + b * kBufCols, kXIsA ? x_lo : wt_lo,
+                                                                        kXIsA ? wt_lo : x_lo, ksteps, hi);
     mma_commit(&bars->d1_full[b]);
     mma_commit(&bars->x_empty[b]);
   }
 }
-// The t-th contraction of a CTA, a quarter (32 of the 128 values of K) at a time: accumulator u % 2 (64 columns each, from
-// `acc` on) = Phi (planes in the buffer at `buf`) * B (planes of 128 rows x 64 columns at b_lo), u = 4 t + quarter.
-template <typename Bars>
+// The t-th contraction of a CTA, a part (32 of the 32 NC values of K) at a time: accumulator u % 2 (64 columns each, from
+// `acc` on) = Phi (planes in the buffer at `buf`) * B (planes of 64 columns at b_lo), u = NC t + part.
+template <int NC, bool kExactB, typename Bars>
 __device__ __forceinline__ bool issue_mma2(Bars* bars, uint32_t acc, uint32_t buf, int t, uint32_t b_lo, uint32_t hi,
                                            volatile int* abort_flag, int* status) {
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const int u = 4 * t + c, r = c & 1;
+  for (int c = 0; c < NC; ++c) {
+    const int u = NC * t + c, r = c & 1;
     if (u >= 2 && !mbar_wait(&bars->acc_free[r], ((u >> 1) - 1) & 1, abort_flag, status, kErrXMma)) return false;
     tc_fence_after_sync();
 #pragma unroll
     for (int q = 0; q < 6; ++q)
+      if (product_on<false, kExactB>(q))
 #pragma unroll
-      for (int k = 2 * c; k < 2 * c + 2; ++k)
-        mma_ts(acc + 64 * r, buf + phi_col(kPa[q], k), smem_desc_join(b_lo + kPb[q] * kTileStep + 128 * k, hi), kIdesc2,
-               (q > 0 || k > 2 * c) ? 1u : 0u);
+        for (int k = 2 * c; k < 2 * c + 2; ++k)
+          mma_ts(acc + 64 * r, buf + phi_col(kPa[q], k), smem_desc_join(b_lo + kPb[q] * kTileStep + 128 * k, hi), kIdesc2,
+                 (q > 0 || k > 2 * c) ? 1u : 0u);
     mma_commit(&bars->acc_full[r]);
   }
   return true;
 }
-// s[0 .. 63] += the four quarters of the t-th contraction.  One warp's share (32 lanes); taddr: its lanes, first accumulator.
-template <typename Bars>
+// s[0 .. 63] += the parts of the t-th contraction.  One warp's share (32 lanes); taddr: its lanes, first accumulator.
+template <int NC, typename Bars>
 __device__ __forceinline__ bool drain_tile(Bars* bars, uint32_t taddr, int t, float (&s)[64], volatile int* abort_flag, int* status) {
 #pragma unroll 1
-  for (int u = 4 * t; u < 4 * t + 4; ++u) {
+  for (int u = NC * t; u < NC * t + NC; ++u) {
     const int r = u & 1;
     if (!__all_sync(0xffffffffu, mbar_wait(&bars->acc_full[r], (u >> 1) & 1, abort_flag, status, kErrXDrain))) return false;
     tc_fence_after_sync();
@@ -355,17 +388,18 @@ __device__ __forceinline__ bool drain_tile(Bars* bars, uint32_t taddr, int t, fl
 // ---- key side.  grid (chunks, slabs, feature groups) ---------------------------------------------
 // kScaled: the query side of the backward, with Q_F and dO in the place of K_F and V.  Feature values are divided by their
 // token's D (scale, slabs of padded_tokens(n)), the sums weighted by c = -dO.O on top: dS' and dz'.
-template <bool kScaled>
+// NF = 64: the rows of the tile past them hold nothing (their warps keep step, and D1's zeros there are nobody's operand).
+template <bool kScaled, typename T, int NF>
 __global__ void __launch_bounds__(kXThreads, 1)
-k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const float* __restrict__ W,
+k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const T* __restrict__ W,
             float* __restrict__ spart, float* __restrict__ zpart, int n, int d, int m, int chunk_tiles, int* __restrict__ status,
             const __nv_bfloat16* x3, const int* seen, const float* __restrict__ scale, const float* __restrict__ weight) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
-  using SL = KxSmem;
+  using SL = KxSmem<T>;
   XBars* bars = reinterpret_cast<XBars*>(smem + SL::bars);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int chunk = blockIdx.x, slab = blockIdx.y, slabs = gridDim.y, f0 = blockIdx.z * kXFeatures;
+  const int chunk = blockIdx.x, slab = blockIdx.y, slabs = gridDim.y, f0 = blockIdx.z * NF;
   const int t0 = chunk * chunk_tiles, nt = min(chunk_tiles, (n + kTile - 1) / kTile - t0);
   if (threadIdx.x == 0) init_bars(bars);
   if (warp == 1) {
@@ -397,7 +431,7 @@ k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ C
     for (int t = 0; t < nt && ok; ++t) {
       if (t > 0) ok = mbar_wait(&bars->v_empty, (t - 1) & 1, abort_flag, status, kErrXCopy);
       if (!ok) break;
-      load_planes(smem + SL::v, &map_v, (t0 + t) * kTile, slab, slabs, &bars->v_full);
+      load_planes<kPlanes<T>>(smem + SL::v, &map_v, (t0 + t) * kTile, slab, slabs, &bars->v_full);
       ++vs;
       if (t + 2 < nt) load_x(t + 2);
     }
@@ -406,13 +440,13 @@ k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ C
       if (vs > 0) mbar_wait_drain(&bars->v_full, (vs - 1) & 1);
     }
   } else if (warp == 1 && lane == 0) {
-    issue_mma1<false>(bars, smem + SL::x, smem + SL::wt, tmem, nt, d, abort_flag, status);
+    issue_mma1<false, NF, kExact<T>>(bars, smem + SL::x, smem + SL::wt, tmem, nt, d, abort_flag, status);
   } else if (warp == 2 && lane == 0) {
     const uint32_t hi = smem_desc_hi(1024), v_lo = smem_desc_lo(smem_u32(smem + SL::v), 1024);
     for (int t = 0; t < nt; ++t) {
       if (!mbar_wait(&bars->v_full, t & 1, abort_flag, status, kErrXMma)) break;
       if (!mbar_wait(&bars->phi_ready[t & 1], (t >> 1) & 1, abort_flag, status, kErrXMma)) break;
-      if (!issue_mma2(bars, tmem + kAccCol, tmem + (t & 1) * kBufCols, t, v_lo, hi, abort_flag, status)) break;
+      if (!issue_mma2<4, kExact<T>>(bars, tmem + kAccCol, tmem + (t & 1) * kBufCols, t, v_lo, hi, abort_flag, status)) break;
       mma_commit(&bars->d1_free[t & 1]);
       mma_commit(&bars->v_empty);
     }
@@ -421,25 +455,26 @@ k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ C
     const uint32_t row = 32u * (warp & 3) + lane;   // feature of the group = TMEM lane
     const uint32_t taddr = tmem + ((32u * (warp & 3)) << 16) + g * kBufCols;
     float* zx = reinterpret_cast<float*>(smem + SL::zx);
-    const Operands op = {x3, W, slab, slabs, n, d, m, look_w || __ldcg(seen) != 0};
+    const Operands<T> op = {x3, W, slab, slabs, n, d, m, look_w || __ldcg(seen) != 0};
     float z = 0.f;
     bool ok = true;
     for (int t = g; t < nt && ok; t += 2) {
       ok = __all_sync(0xffffffffu, mbar_wait(&bars->d1_full[g], (t >> 1) & 1, abort_flag, status, kErrXElem));
       if (!ok) break;
       tc_fence_after_sync();
-      if constexpr (kScaled) {
+      if (row >= NF) {   // (whole warps)
+      } else if constexpr (kScaled) {
         const size_t tok = (size_t)slab * padded_tokens(n) + (size_t)(t0 + t) * kTile;
-        z += relu_planes<true, true, true>(taddr, op, (t0 + t) * kTile, f0 + row, weight + tok, scale + tok);
+        z += relu_planes<4, true, true, true>(taddr, op, (t0 + t) * kTile, f0 + row, weight + tok, scale + tok);
       } else {
-        z += relu_planes<true, false>(taddr, op, (t0 + t) * kTile, f0 + row, nullptr);
+        z += relu_planes<4, true, false>(taddr, op, (t0 + t) * kTile, f0 + row, nullptr);
       }
       tc_fence_before_sync();
       warp_arrive(&bars->phi_ready[g]);
     }
     if (g == 1) zx[row] = z;
     named_bar_sync(kBarZ, 256);
-    if (g == 0 && ok) zpart[((size_t)slab * gridDim.x + chunk) * m + f0 + row] = z + zx[row];
+    if (g == 0 && ok && row < NF) zpart[((size_t)slab * gridDim.x + chunk) * m + f0 + row] = z + zx[row];
   } else if (warp >= 12) {
     const uint32_t row = 32u * (warp & 3) + lane;
     const uint32_t taddr = tmem + ((32u * (warp & 3)) << 16) + kAccCol;
@@ -450,12 +485,12 @@ k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ C
       float s[64];
 #pragma unroll
       for (int j = 0; j < 64; ++j) s[j] = 0.f;
-      ok = drain_tile(bars, taddr, t, s, abort_flag, status);
+      ok = drain_tile<4>(bars, taddr, t, s, abort_flag, status);
       if (!ok) break;
 #pragma unroll
       for (int j = 0; j < 64; ++j) sum[j * kXFeatures] = t > 0 ? sum[j * kXFeatures] + s[j] : s[j];
     }
-    if (ok) {
+    if (ok && row < NF) {
       float* dst = spart + (((size_t)slab * gridDim.x + chunk) * m + f0 + row) * kD;
 #pragma unroll
       for (int j = 0; j < 64; j += 4)
@@ -475,18 +510,19 @@ k_tcx_kside(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ C
 // ---- query side.  grid (chunks, slabs, feature groups) -------------------------------------------
 // One group: O, divided, and with keep (for a backward) once more into map_keep.  Several: N'_g into map_o (group-major
 // slabs).  den_out, where given: D'_g at [(group * slabs + slab) * n + token].
+template <typename T, int NF>
 __global__ void __launch_bounds__(kXThreads, 1)
-k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o, const float* __restrict__ W,
+k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o, const T* __restrict__ W,
             const float* __restrict__ S, const float* __restrict__ zg, const float* __restrict__ beta, float eps, float bw_floor,
             float* __restrict__ den_out, const __grid_constant__ CUtensorMap map_keep, int keep, int n, int d, int m, int chunk_tiles,
             int* __restrict__ status, const __nv_bfloat16* x3,
             const int* seen) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
-  using SL = QxSmem;
+  using SL = QxSmem<T>;
   XBars* bars = reinterpret_cast<XBars*>(smem + SL::bars);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int chunk = blockIdx.x, slab = blockIdx.y, slabs = gridDim.y, f0 = blockIdx.z * kXFeatures;
+  const int chunk = blockIdx.x, slab = blockIdx.y, slabs = gridDim.y, f0 = blockIdx.z * NF;
   const int t0 = chunk * chunk_tiles, nt = min(chunk_tiles, (n + kTile - 1) / kTile - t0);
   float* zs = reinterpret_cast<float*>(smem + SL::zs);
   float* den = reinterpret_cast<float*>(smem + SL::den);
@@ -502,7 +538,7 @@ k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   }
   const bool bad_w = load_w_planes(W, d, m, f0, smem + SL::wt);
   wait_for_stream_predecessor();
-  load_s_planes(S, zg, (size_t)slab * m + f0, smem + SL::s, zs);
+  load_s_planes<NF>(S, zg, (size_t)slab * m + f0, smem + SL::s, zs);
   fence_proxy_async_smem();
   tc_fence_before_sync();
   const bool look_w = __syncthreads_or(bad_w);
@@ -520,25 +556,25 @@ k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     if (*abort_flag != 0)   // let copies in flight land before the CTA's shared memory goes away
       for (int t = max(0, xs - 2); t < xs; ++t) mbar_wait_drain(&bars->x_full[t & 1], (t >> 1) & 1);
   } else if (warp == 1 && lane == 0) {
-    issue_mma1<true>(bars, smem + SL::x, smem + SL::wt, tmem, nt, d, abort_flag, status);
+    issue_mma1<true, NF, kExact<T>>(bars, smem + SL::x, smem + SL::wt, tmem, nt, d, abort_flag, status);
   } else if (warp == 2 && lane == 0) {
     const uint32_t hi = smem_desc_hi(1024), s_lo = smem_desc_lo(smem_u32(smem + SL::s), 1024);
     for (int t = 0; t < nt; ++t) {
       if (!mbar_wait(&bars->phi_ready[t & 1], (t >> 1) & 1, abort_flag, status, kErrXMma)) break;
-      if (!issue_mma2(bars, tmem + kAccCol, tmem + (t & 1) * kBufCols, t, s_lo, hi, abort_flag, status)) break;
+      if (!issue_mma2<NF / 32, false>(bars, tmem + kAccCol, tmem + (t & 1) * kBufCols, t, s_lo, hi, abort_flag, status)) break;
       mma_commit(&bars->d1_free[t & 1]);
     }
   } else if (warp >= 4 && warp < 12) {
     const int g = (warp - 4) >> 2;
     const uint32_t row = 32u * (warp & 3) + lane;   // token of the tile = TMEM lane
     const uint32_t taddr = tmem + ((32u * (warp & 3)) << 16) + g * kBufCols;
-    const Operands op = {x3, W, slab, slabs, n, d, m, look_w || __ldcg(seen) != 0};
+    const Operands<T> op = {x3, W, slab, slabs, n, d, m, look_w || __ldcg(seen) != 0};
     bool ok = true;
     for (int t = g; t < nt && ok; t += 2) {
       ok = __all_sync(0xffffffffu, mbar_wait(&bars->d1_full[g], (t >> 1) & 1, abort_flag, status, kErrXElem));
       if (!ok) break;
       tc_fence_after_sync();
-      const float sum = relu_planes<false, true>(taddr, op, (t0 + t) * kTile + row, f0, zs);
+      const float sum = relu_planes<NF / 32, false, true>(taddr, op, (t0 + t) * kTile + row, f0, zs);
       if (t >= 2) {   // the drain has read the denominators of tile t - 2
         ok = __all_sync(0xffffffffu, mbar_wait(&bars->den_free[g], ((t >> 1) - 1) & 1, abort_flag, status, kErrXElem));
         if (!ok) break;
@@ -561,7 +597,7 @@ k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
       float s[64], scale = 1.f;
 #pragma unroll
       for (int j = 0; j < 64; ++j) s[j] = 0.f;
-      if (ok) ok = drain_tile(bars, taddr, t, s, abort_flag, status);
+      if (ok) ok = drain_tile<NF / 32>(bars, taddr, t, s, abort_flag, status);
       if (ok) {   // (the tile's denominators are older than its first accumulator)
         const float dn = den[b * kTile + et];
         if (divide) scale = put_back(1.f / (dn + epsp));
@@ -571,6 +607,14 @@ k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
       if (et == 0) bulk_wait_group_read0();   // the tile before has left the staging boxes
       named_bar_sync(kBarDrain, 128);
       if (ok) {
+        if constexpr (kExact<T>) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            *reinterpret_cast<uint4*>(smem + SL::out16 + swz128(et, j)) =
+                make_uint4(pack_bf16x2(s[8 * j] * scale, s[8 * j + 1] * scale), pack_bf16x2(s[8 * j + 2] * scale, s[8 * j + 3] * scale),
+                           pack_bf16x2(s[8 * j + 4] * scale, s[8 * j + 5] * scale), pack_bf16x2(s[8 * j + 6] * scale, s[8 * j + 7] * scale));
+        }
+        if (!kExact<T> || keep)
 #pragma unroll
         for (int j = 0; j < 16; ++j)
           *reinterpret_cast<float4*>(out + (j >> 3) * kTileBytes + swz128(et, j & 7)) =
@@ -579,8 +623,12 @@ k_tcx_qside(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
       }
       named_bar_sync(kBarDrain, 128);
       if (et == 0 && ok) {   // rows past n and columns past d are clipped
-        tma_store_3d(&map_o, out, 0, row0, out_slab);
-        if (d > 32) tma_store_3d(&map_o, out + kTileBytes, 32, row0, out_slab);
+        if constexpr (kExact<T>) {
+          tma_store_3d(&map_o, smem + SL::out16, 0, row0, out_slab);
+        } else {
+          tma_store_3d(&map_o, out, 0, row0, out_slab);
+          if (d > 32) tma_store_3d(&map_o, out + kTileBytes, 32, row0, out_slab);
+        }
         if (keep) {
           tma_store_3d(&map_keep, out, 0, row0, out_slab);
           if (d > 32) tma_store_3d(&map_keep, out + kTileBytes, 32, row0, out_slab);
@@ -618,8 +666,10 @@ __global__ void __launch_bounds__(256) k_tcx_combine(const float* __restrict__ N
 // ---- backward ------------------------------------------------------------------------------------
 // Per token: planes of dO, 1 / D (D = sum_g D'_g + eps'), c = -dO.O; sum of dD = c / D per CTA.  tpt threads (a power of
 // two >= d / 8) on a token, eight columns each.  Bound by memory (2 x 8 x 4096, d = 64: 59 MB).
+// (bf16 gradients are their own plane: dO3 stays unwritten)
+template <typename T>
 __global__ void __launch_bounds__(256, 6)
-k_tcx_bwd_prep(const float* __restrict__ dO, const float* __restrict__ O, const float* __restrict__ den, int groups,
+k_tcx_bwd_prep(const T* __restrict__ dO, const float* __restrict__ O, const float* __restrict__ den, int groups,
                const float* __restrict__ beta, float eps, float bw_floor, int m, int d, int tpt, size_t tokens, int n,
                __nv_bfloat16* __restrict__ dO3, float* __restrict__ inv, float* __restrict__ c, float* __restrict__ sumdD) {
   __shared__ float sums[8];
@@ -635,16 +685,19 @@ k_tcx_bwd_prep(const float* __restrict__ dO, const float* __restrict__ O, const 
     const int c0 = 8 * (int)(i % tpt);
     float dot = 0.f;
     if (tok < tokens && c0 < d) {
-      const float4 ga = *reinterpret_cast<const float4*>(dO + tok * d + c0), gb = *reinterpret_cast<const float4*>(dO + tok * d + c0 + 4);
+      float g[8];
+      load8(dO + tok * d + c0, g);
       const float4 oa = load4_after_wait(O + tok * d + c0), ob = load4_after_wait(O + tok * d + c0 + 4);
-      const float g[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w}, o[8] = {oa.x, oa.y, oa.z, oa.w, ob.x, ob.y, ob.z, ob.w};
-      uint32_t pl[3][4];
+      const float o[8] = {oa.x, oa.y, oa.z, oa.w, ob.x, ob.y, ob.z, ob.w};
 #pragma unroll
       for (int j = 0; j < 8; ++j) dot = fmaf(g[j], o[j], dot);
-      split8(g, pl);
+      if constexpr (!kExact<T>) {
+        uint32_t pl[3][4];
+        split8(g, pl);
 #pragma unroll
-      for (int s = 0; s < 3; ++s)
-        *reinterpret_cast<uint4*>(dO3 + s * plane + tok * d + c0) = make_uint4(pl[s][0], pl[s][1], pl[s][2], pl[s][3]);
+        for (int s = 0; s < 3; ++s)
+          *reinterpret_cast<uint4*>(dO3 + s * plane + tok * d + c0) = make_uint4(pl[s][0], pl[s][1], pl[s][2], pl[s][3]);
+      }
     }
     for (int o = tpt >> 1; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
     if (tok < tokens && c0 == 0) {
@@ -674,17 +727,17 @@ struct alignas(8) YBars {
   uint32_t tmem_base;
   int abort_flag;
 };
-struct YSmem {
+template <typename T> struct YSmem {
   static constexpr uint32_t wt = 0;                          // planes of W^T (128 features x 64)
-  static constexpr uint32_t s = wt + 3 * kTileBytes;         // planes of S' or dS'
+  static constexpr uint32_t s = wt + kPlanes<T> * kTileBytes;   // planes of S' or dS'
   static constexpr uint32_t x = s + 3 * kTileBytes;          // planes of Q_F or K_F
   static constexpr uint32_t y = x + 3 * kTileBytes;          // planes of dO or V
-  static constexpr uint32_t out = y + 3 * kTileBytes;        // result tile: two boxes of 128 rows x 32 floats
+  static constexpr uint32_t out = y + kPlanes<T> * kTileBytes;        // result tile: two boxes of 128 rows x 32 floats
   static constexpr uint32_t zs = out + 2 * kTileBytes;       // z' or dz' of the group
   static constexpr uint32_t bars = zs + 512;
   static constexpr uint32_t total = bars + 256 + 1024;
 };
-static_assert(YSmem::total <= 232448 && sizeof(YBars) <= 256, "shared memory of an SM");
+static_assert(YSmem<float>::total <= 232448 && sizeof(YBars) <= 256, "shared memory of an SM");
 
 // Chunk `chunk` (32 of 128 values) of a row -> planes, laid out as relu_planes leaves them.
 __device__ __forceinline__ void store_chunk_planes(uint32_t buf, int chunk, const float (&v)[32]) {
@@ -704,18 +757,20 @@ __device__ __forceinline__ void store_chunk_planes(uint32_t buf, int chunk, cons
 // Bound by latency: a tile is one chain copy -> MMA1 -> ReLU -> MMA2 -> drain with nothing of the next tile beside it but its
 // copies.  2 x 4 x 4096, d = 32, m = 128 (two tiles a CTA): queries 15 us, keys some 22; the backward of 8 x 4 x 1024 92 -> 65 us.
 // TMEM: keys: A and its planes 192, G and its planes 192; queries: A 128, G 192; then two accumulators of 64.
-template <bool kKeys>
+// TG: type of dV.
+template <bool kKeys, typename T, typename TG, int NF>
 __global__ void __launch_bounds__(kXThreads, 1)
-k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y, const float* __restrict__ W,
+k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y, const T* __restrict__ W,
           const float* __restrict__ S, const float* __restrict__ zg, const float* __restrict__ tok_inv,
           const float* __restrict__ tok_c, const __grid_constant__ CUtensorMap map_dx, const __grid_constant__ CUtensorMap map_dv,
           int add, int n, int d, int m, int f0, int chunk_tiles, int* __restrict__ status, const __nv_bfloat16* x3,
             const int* seen) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
-  using SL = YSmem;
+  using SL = YSmem<T>;
   constexpr uint32_t kG = kKeys ? kBufCols : 128, kAcc = kG + kBufCols;
   constexpr int kPer = kKeys ? 2 : 1;   // contractions of a tile
+  constexpr int kHalf = NF / 2, kH = NF / 64;   // features of a group of warps, and 32 at a time
   YBars* bars = reinterpret_cast<YBars*>(smem + SL::bars);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int chunk = blockIdx.x, slab = blockIdx.y, slabs = gridDim.y;
@@ -747,7 +802,7 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
   wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   // (behind the key side come kernels that start with reads of what it writes and that lost time placed early)
   if constexpr (!kKeys) let_stream_successor_start();
-  load_s_planes(S, zg, (size_t)slab * m + f0, smem + SL::s, zs);
+  load_s_planes<NF>(S, zg, (size_t)slab * m + f0, smem + SL::s, zs);
   fence_proxy_async_smem();
   tc_fence_before_sync();
   const bool look_w = __syncthreads_or(bad_w);
@@ -762,7 +817,7 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
       load_planes(smem + SL::x, &map_x, (t0 + t) * kTile, slab, slabs, &bars->x_full);
       ++xs;
       if (t > 0 && !mbar_wait(&bars->y_empty, (t - 1) & 1, abort_flag, status, kErrXCopy)) break;
-      load_planes(smem + SL::y, &map_y, (t0 + t) * kTile, slab, slabs, &bars->y_full);
+      load_planes<kPlanes<T>>(smem + SL::y, &map_y, (t0 + t) * kTile, slab, slabs, &bars->y_full);
       ++ys;
     }
     if (*abort_flag != 0) {   // let copies in flight land before the CTA's shared memory goes away
@@ -777,13 +832,13 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
       if (!mbar_wait(&bars->x_full, t & 1, abort_flag, status, kErrXMma)) break;
       if (t > 0 && !mbar_wait(&bars->a_done, (t - 1) & 1, abort_flag, status, kErrXMma)) break;
       tc_fence_after_sync();
-      issue_planes(tmem, x_lo, wt_lo, ksteps, hi);
+      issue_planes<NF, false, kExact<T>>(tmem, x_lo, wt_lo, ksteps, hi);
       mma_commit(&bars->a_full);
       mma_commit(&bars->x_empty);
       if (!mbar_wait(&bars->y_full, t & 1, abort_flag, status, kErrXMma)) break;
       if (t > 0 && !mbar_wait(&bars->g_done, (t - 1) & 1, abort_flag, status, kErrXMma)) break;
       tc_fence_after_sync();
-      issue_planes(tmem + kG, y_lo, s_lo, ksteps, hi);
+      issue_planes<NF, kExact<T>, false>(tmem + kG, y_lo, s_lo, ksteps, hi);
       mma_commit(&bars->g_full);
       mma_commit(&bars->y_empty);
     }
@@ -792,18 +847,18 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
     for (int t = 0; t < nt; ++t) {
       if constexpr (kKeys) {
         if (!mbar_wait(&bars->a_ready, t & 1, abort_flag, status, kErrXMma)) break;
-        if (!issue_mma2(bars, tmem + kAcc, tmem, 2 * t, s_lo, hi, abort_flag, status)) break;
+        if (!issue_mma2<NF / 32, false>(bars, tmem + kAcc, tmem, 2 * t, s_lo, hi, abort_flag, status)) break;
         mma_commit(&bars->a_done);
       }
       if (!mbar_wait(&bars->g_ready, t & 1, abort_flag, status, kErrXMma)) break;
-      if (!issue_mma2(bars, tmem + kAcc, tmem + kG, kPer * t + kPer - 1, wt_lo, hi, abort_flag, status)) break;
+      if (!issue_mma2<NF / 32, kExact<T>>(bars, tmem + kAcc, tmem + kG, kPer * t + kPer - 1, wt_lo, hi, abort_flag, status)) break;
       mma_commit(&bars->g_done);
     }
   } else if (warp >= 4 && warp < 12) {
-    const int g = (warp - 4) >> 2;                        // features 64 g .. 64 g + 63
+    const int g = (warp - 4) >> 2;                        // features kHalf g .. + kHalf - 1
     const uint32_t row = 32u * (warp & 3) + lane;         // token of the tile = TMEM lane
     const uint32_t lanes = tmem + ((32u * (warp & 3)) << 16);
-    const Operands op = {x3, W, slab, slabs, n, d, m, look_w || __ldcg(seen) != 0};
+    const Operands<T> op = {x3, W, slab, slabs, n, d, m, look_w || __ldcg(seen) != 0};
     bool ok = true;
     for (int t = 0; t < nt && ok; ++t) {
       float inv = 0.f, c = 0.f;
@@ -817,11 +872,11 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
       ok = __all_sync(0xffffffffu, mbar_wait(&bars->a_full, t & 1, abort_flag, status, kErrXElem));
       if (!ok) break;
       tc_fence_after_sync();
-      uint32_t on[2];
+      uint32_t on[kH];
       uint32_t r[32];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        load_projected(lanes + 64 * g + 32 * h, r, op, (t0 + t) * kTile + row, 0, f0 + 64 * g + 32 * h, 1);
+      for (int h = 0; h < kH; ++h) {
+        load_projected(lanes + kHalf * g + 32 * h, r, op, (t0 + t) * kTile + row, 0, f0 + kHalf * g + 32 * h, 1);
         on[h] = 0;
         float v[32];
 #pragma unroll
@@ -830,7 +885,7 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
           on[h] |= (x > 0.f ? 1u : 0u) << j;
           v[j] = fmaxf(put_back(x), 0.f);
         }
-        if constexpr (kKeys) store_chunk_planes(lanes, 2 * g + h, v);
+        if constexpr (kKeys) store_chunk_planes(lanes, kH * g + h, v);
       }
       if constexpr (kKeys) tmem_st_wait();
       tc_fence_before_sync();
@@ -839,19 +894,19 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
       if (!ok) break;
       tc_fence_after_sync();
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        tmem_ld32(lanes + kG + 64 * g + 32 * h, r);
+      for (int h = 0; h < kH; ++h) {
+        tmem_ld32(lanes + kG + kHalf * g + 32 * h, r);
         tmem_ld_wait();
         reg_fence32(r);
         float v[32];
-        const float* z = zs + 64 * g + 32 * h;
+        const float* z = zs + kHalf * g + 32 * h;
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
           const float x = put_back(__uint_as_float(r[j]));
           const float y = kKeys ? x + z[j] : fmaf(c, z[j], x) * inv;
           v[j] = ((on[h] >> j) & 1u) ? y : 0.f;
         }
-        store_chunk_planes(lanes + kG, 2 * g + h, v);
+        store_chunk_planes(lanes + kG, kH * g + h, v);
       }
       tmem_st_wait();
       tc_fence_before_sync();
@@ -867,10 +922,18 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
       float s[64];
 #pragma unroll
       for (int j = 0; j < 64; ++j) s[j] = 0.f;
-      if (ok) ok = drain_tile(bars, taddr, v, s, abort_flag, status);
+      if (ok) ok = drain_tile<NF / 32>(bars, taddr, v, s, abort_flag, status);
       if (et == 0) bulk_wait_group_read0();   // the tile before has left the staging boxes
       named_bar_sync(kBarDrain, 128);
-      if (ok) {
+      const bool values = kKeys && (v & 1) == 0;   // dV
+      if (ok && sizeof(TG) == 2 && values) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          *reinterpret_cast<uint4*>(out + swz128(et, j)) =
+              make_uint4(pack_bf16x2(put_back(s[8 * j]), put_back(s[8 * j + 1])), pack_bf16x2(put_back(s[8 * j + 2]), put_back(s[8 * j + 3])),
+                         pack_bf16x2(put_back(s[8 * j + 4]), put_back(s[8 * j + 5])), pack_bf16x2(put_back(s[8 * j + 6]), put_back(s[8 * j + 7])));
+        fence_proxy_async_smem();
+      } else if (ok) {
 #pragma unroll
         for (int j = 0; j < 16; ++j)
           *reinterpret_cast<float4*>(out + (j >> 3) * kTileBytes + swz128(et, j & 7)) =
@@ -879,8 +942,8 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
       }
       named_bar_sync(kBarDrain, 128);
       if (et == 0 && ok) {   // rows past n and columns past d are clipped
-        const CUtensorMap* map = kKeys && (v & 1) == 0 ? &map_dv : &map_dx;
-        for (int c = 0; c < (d > 32 ? 2 : 1); ++c) {
+        const CUtensorMap* map = values ? &map_dv : &map_dx;
+        for (int c = 0; c < (d > 32 && !(sizeof(TG) == 2 && values) ? 2 : 1); ++c) {
           if (add)
             tma_reduce_add_3d(map, out + c * kTileBytes, 32 * c, row0, slab);
           else
@@ -899,69 +962,94 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
   }
 }
 
-// S' and z' (or dS' and dz') per chunk from planes of X (the projected operand) and Y.
+// Runs body(T(), NF) with the type of the arguments and the features of a CTA as constants: fp32, or bf16 with 64 features
+// (wider bf16 maps: tc_fwd.cu, tc_bwd.cu).
+template <int V> struct Int { static constexpr int value = V; };
+template <typename F> cudaError_t with_args(const Plan& p, F&& body) {
+  if (p.bf16) return p.cfg.features == 64 ? body(__nv_bfloat16(), Int<64>()) : cudaErrorInvalidValue;
+  return p.cfg.features == 64 ? body(float(), Int<64>()) : body(float(), Int<128>());
+}
+int groups_of(const Plan& p) { return p.cfg.features <= kXFeatures ? 1 : p.cfg.features / kXFeatures; }
+
+// S' and z' (or dS' and dz') per chunk from planes of X (the projected operand) and Y (bf16: the tensor itself).
 template <bool kScaled>
-cudaError_t launch_summary(const Plan& p, const Ws& w, const __nv_bfloat16* x3, const __nv_bfloat16* y3, const void* W,
-                           const float* scale, const float* weight, cudaStream_t st, int* launches) {
-  auto kernel = k_tcx_kside<kScaled>;
-  CUtensorMap map_x, map_y;
-  cudaError_t err;
-  if ((err = make_tile_map(x3, 3 * p.slabs, p.cfg.seq_len, &map_x, p.cfg.head_dim)) != cudaSuccess) return err;
-  if ((err = make_tile_map(y3, 3 * p.slabs, p.cfg.seq_len, &map_y, p.cfg.head_dim)) != cudaSuccess) return err;
-  if ((err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, KxSmem::total)) != cudaSuccess) return err;
-  *launches += 1;
-  return launch_after(kernel, dim3(p.xchunks, p.slabs, p.cfg.features / kXFeatures), dim3(kXThreads), KxSmem::total, st, map_x, map_y,
-                      (const float*)W, w.spart, w.zpart, p.cfg.seq_len, p.cfg.head_dim, p.cfg.features, p.xchunk_tiles, w.status,
-                      x3, (const int*)(x3 == w.KF3 ? w.seen + 1 : w.seen), scale, weight);
+cudaError_t launch_summary(const Plan& p, const Ws& w, const __nv_bfloat16* x3, const void* y3, const void* W, const float* scale,
+                           const float* weight, cudaStream_t st, int* launches) {
+  return with_args(p, [&](auto tag, auto nf) {
+    using T = decltype(tag);
+    constexpr int NF = decltype(nf)::value;
+    auto kernel = k_tcx_kside<kScaled, T, NF>;
+    CUtensorMap map_x, map_y;
+    cudaError_t err;
+    if ((err = make_tile_map(x3, 3 * p.slabs, p.cfg.seq_len, &map_x, p.cfg.head_dim)) != cudaSuccess) return err;
+    if ((err = make_tile_map(y3, kPlanes<T> * p.slabs, p.cfg.seq_len, &map_y, p.cfg.head_dim)) != cudaSuccess) return err;
+    if ((err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, KxSmem<T>::total)) != cudaSuccess) return err;
+    *launches += 1;
+    return launch_after(kernel, dim3(p.xchunks, p.slabs, groups_of(p)), dim3(kXThreads), KxSmem<T>::total, st, map_x, map_y,
+                        (const T*)W, w.spart, w.zpart, p.cfg.seq_len, p.cfg.head_dim, p.cfg.features, p.xchunk_tiles, w.status,
+                        x3, (const int*)(x3 == w.KF3 ? w.seen + 1 : w.seen), scale, weight);
+  });
 }
 
 template <bool kKeys>
-cudaError_t launch_bwd(const Plan& p, const Ws& w, const __nv_bfloat16* x3, const __nv_bfloat16* y3, const void* W, const float* S,
-                       const float* z, float* dx, float* dv, cudaStream_t st, int* launches) {
-  auto kernel = k_tcx_bwd<kKeys>;
-  const int n = p.cfg.seq_len, d = p.cfg.head_dim;
-  CUtensorMap map_x, map_y, map_dx, map_dv;
-  cudaError_t err;
-  if ((err = make_tile_map(x3, 3 * p.slabs, n, &map_x, d)) != cudaSuccess) return err;
-  if ((err = make_tile_map(y3, 3 * p.slabs, n, &map_y, d)) != cudaSuccess) return err;
-  if ((err = make_out_map(dx, p.slabs, n, d, false, &map_dx)) != cudaSuccess) return err;
-  if ((err = make_out_map(dv, p.slabs, n, d, false, &map_dv)) != cudaSuccess) return err;
-  if ((err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, YSmem::total)) != cudaSuccess) return err;
-  for (int f0 = 0; f0 < p.cfg.features; f0 += kXFeatures) {
-    *launches += 1;
-    err = launch_after(kernel, dim3(p.xbchunks, p.slabs), dim3(kXThreads), YSmem::total, st, map_x, map_y, (const float*)W, S, z,
-                       (const float*)w.xinv, (const float*)w.xc, map_dx, map_dv, f0 > 0 ? 1 : 0, n, d, p.cfg.features, f0,
-                       p.xbchunk_tiles, w.status, x3, (const int*)(kKeys ? w.seen + 1 : w.seen));
-    if (err != cudaSuccess) return err;
-  }
-  return cudaSuccess;
+cudaError_t launch_bwd(const Plan& p, const Ws& w, const __nv_bfloat16* x3, const void* y3, const void* W, const float* S,
+                       const float* z, float* dx, void* dv, cudaStream_t st, int* launches) {
+  return with_args(p, [&](auto tag, auto nf) {
+    using T = decltype(tag);
+    constexpr int NF = decltype(nf)::value;
+    const int n = p.cfg.seq_len, d = p.cfg.head_dim;
+    const bool half = kKeys && p.grad_bf16;
+    auto kernel = kExact<T> && half ? k_tcx_bwd<kKeys, T, T, NF> : k_tcx_bwd<kKeys, T, float, NF>;   // (bf16 gradients: of bf16 tensors)
+    CUtensorMap map_x, map_y, map_dx, map_dv;
+    cudaError_t err;
+    if (half && !kExact<T>) return cudaErrorInvalidValue;
+    if ((err = make_tile_map(x3, 3 * p.slabs, n, &map_x, d)) != cudaSuccess) return err;
+    if ((err = make_tile_map(y3, kPlanes<T> * p.slabs, n, &map_y, d)) != cudaSuccess) return err;
+    if ((err = make_out_map(dx, p.slabs, n, d, false, &map_dx)) != cudaSuccess) return err;
+    if ((err = make_out_map(dv, p.slabs, n, d, half, &map_dv)) != cudaSuccess) return err;
+    if ((err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, YSmem<T>::total)) != cudaSuccess) return err;
+    for (int f0 = 0; f0 < p.cfg.features; f0 += NF) {
+      *launches += 1;
+      err = launch_after(kernel, dim3(p.xbchunks, p.slabs), dim3(kXThreads), YSmem<T>::total, st, map_x, map_y, (const T*)W, S, z,
+                         (const float*)w.xinv, (const float*)w.xc, map_dx, map_dv, f0 > 0 ? 1 : 0, n, d, p.cfg.features, f0,
+                         p.xbchunk_tiles, w.status, x3, (const int*)(kKeys ? w.seen + 1 : w.seen));
+      if (err != cudaSuccess) return err;
+    }
+    return cudaSuccess;
+  });
 }
 
 }  // namespace
 
-cudaError_t launch_tcx_kside(const Plan& p, const Ws& w, const void* W, cudaStream_t st, int* launches) {
-  return launch_summary<false>(p, w, w.KF3, w.V3, W, nullptr, nullptr, st, launches);
+cudaError_t launch_tcx_kside(const Plan& p, const Ws& w, const void* V, const void* W, cudaStream_t st, int* launches) {
+  return launch_summary<false>(p, w, w.KF3, p.bf16 ? V : w.V3, W, nullptr, nullptr, st, launches);
 }
 
 cudaError_t launch_tcx_qside(const Plan& p, const Ws& w, const void* W, const float* beta, void* O, cudaStream_t st, int* launches) {
-  const int groups = p.cfg.features / kXFeatures, n = p.cfg.seq_len, d = p.cfg.head_dim;
+  const int groups = groups_of(p), n = p.cfg.seq_len, d = p.cfg.head_dim;
   const size_t tokens = (size_t)p.slabs * n;
   // Several groups leave their shares where the planes of K_F and V were (which the key side has read), unless a backward
   // reads those again.
-  float* share = groups == 1 ? static_cast<float*>(O) : p.use_xb ? w.xshare : reinterpret_cast<float*>(w.KF3);
+  float* share = p.use_xb ? w.xshare : reinterpret_cast<float*>(w.KF3);
   float* den = p.use_xb ? w.xden : groups > 1 ? share + groups * tokens * d : nullptr;
   float* keep = p.use_xb ? w.xO : nullptr;
-  CUtensorMap map_q, map_o, map_keep;
-  cudaError_t err;
-  if ((err = make_tile_map(w.QF3, 3 * p.slabs, n, &map_q, d)) != cudaSuccess) return err;
-  if ((err = make_out_map(share, groups * p.slabs, n, d, false, &map_o)) != cudaSuccess) return err;
-  if ((err = make_out_map(keep != nullptr ? keep : share, p.slabs, n, d, false, &map_keep)) != cudaSuccess) return err;
-  if ((err = cudaFuncSetAttribute(k_tcx_qside, cudaFuncAttributeMaxDynamicSharedMemorySize, QxSmem::total)) != cudaSuccess) return err;
-  *launches += 1;
-  err = launch_after(k_tcx_qside, dim3(p.xchunks, p.slabs, groups), dim3(kXThreads), QxSmem::total, st, map_q, map_o, (const float*)W,
-                     (const float*)w.S, (const float*)w.z, beta, p.cfg.eps, p.cfg.bw_floor, den, map_keep,
-                     keep != nullptr && groups == 1 ? 1 : 0, n, d, p.cfg.features, p.xchunk_tiles, w.status,
-                     (const __nv_bfloat16*)w.QF3, (const int*)w.seen);
+  void* out = groups == 1 ? O : share;
+  const cudaError_t err = with_args(p, [&](auto tag, auto nf) {
+    using T = decltype(tag);
+    constexpr int NF = decltype(nf)::value;
+    auto kernel = k_tcx_qside<T, NF>;
+    CUtensorMap map_q, map_o, map_keep;
+    cudaError_t e;
+    if ((e = make_tile_map(w.QF3, 3 * p.slabs, n, &map_q, d)) != cudaSuccess) return e;
+    if ((e = make_out_map(out, groups * p.slabs, n, d, kExact<T>, &map_o)) != cudaSuccess) return e;
+    if ((e = make_out_map(keep != nullptr ? keep : out, p.slabs, n, d, keep == nullptr && kExact<T>, &map_keep)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, QxSmem<T>::total)) != cudaSuccess) return e;
+    *launches += 1;
+    return launch_after(kernel, dim3(p.xchunks, p.slabs, groups), dim3(kXThreads), QxSmem<T>::total, st, map_q, map_o, (const T*)W,
+                        (const float*)w.S, (const float*)w.z, beta, p.cfg.eps, p.cfg.bw_floor, den, map_keep,
+                        keep != nullptr && groups == 1 ? 1 : 0, n, d, p.cfg.features, p.xchunk_tiles, w.status,
+                        (const __nv_bfloat16*)w.QF3, (const int*)w.seen);
+  });
   if (err != cudaSuccess || groups == 1) return err;
   *launches += 1;
   return launch_after(k_tcx_combine, dim3((unsigned)((tokens * (d >> 2) + 255) / 256)), dim3(256), 0, st, (const float*)share,
@@ -972,19 +1060,23 @@ cudaError_t launch_tcx_bwd_prep(const Plan& p, const Ws& w, const void* dO, cons
   int tpt = 1;
   while (tpt * 8 < p.cfg.head_dim) tpt *= 2;
   *launches += 1;
-  return launch_after(k_tcx_bwd_prep, dim3(p.xprep), dim3(256), 0, st, (const float*)dO, (const float*)w.xO, (const float*)w.xden,
-                      p.cfg.features / kXFeatures, beta, p.cfg.eps, p.cfg.bw_floor, p.cfg.features, p.cfg.head_dim, tpt,
-                      (size_t)p.slabs * p.cfg.seq_len, p.cfg.seq_len, w.dO3, w.xinv, w.xc, w.sumdD);
+  auto go = [&](auto kernel, auto* g) {
+    return launch_after(kernel, dim3(p.xprep), dim3(256), 0, st, g, (const float*)w.xO, (const float*)w.xden, groups_of(p), beta,
+                        p.cfg.eps, p.cfg.bw_floor, p.cfg.features, p.cfg.head_dim, tpt, (size_t)p.slabs * p.cfg.seq_len,
+                        p.cfg.seq_len, w.dO3, w.xinv, w.xc, w.sumdD);
+  };
+  return p.bf16 ? go(k_tcx_bwd_prep<__nv_bfloat16>, (const __nv_bfloat16*)dO) : go(k_tcx_bwd_prep<float>, (const float*)dO);
 }
 
-cudaError_t launch_tcx_bwd_qside(const Plan& p, const Ws& w, const void* W, cudaStream_t st, int* launches) {
-  const cudaError_t err = launch_bwd<false>(p, w, w.QF3, w.dO3, W, w.S, w.z, w.dQF, w.dQF, st, launches);
+cudaError_t launch_tcx_bwd_qside(const Plan& p, const Ws& w, const void* W, const void* dO, cudaStream_t st, int* launches) {
+  const void* y = p.bf16 ? dO : w.dO3;
+  const cudaError_t err = launch_bwd<false>(p, w, w.QF3, y, W, w.S, w.z, w.dQF, w.dQF, st, launches);
   if (err != cudaSuccess) return err;
-  return launch_summary<true>(p, w, w.QF3, w.dO3, W, w.xinv, w.xc, st, launches);
+  return launch_summary<true>(p, w, w.QF3, y, W, w.xinv, w.xc, st, launches);
 }
 
-cudaError_t launch_tcx_bwd_kside(const Plan& p, const Ws& w, const void* W, void* dV, cudaStream_t st, int* launches) {
-  return launch_bwd<true>(p, w, w.KF3, w.V3, W, w.dS, w.dz, w.dKF, (float*)dV, st, launches);
+cudaError_t launch_tcx_bwd_kside(const Plan& p, const Ws& w, const void* V, const void* W, void* dV, cudaStream_t st, int* launches) {
+  return launch_bwd<true>(p, w, w.KF3, p.bf16 ? V : w.V3, W, w.dS, w.dz, w.dKF, dV, st, launches);
 }
 
 }  // namespace wersa
