@@ -836,13 +836,15 @@ wersa_status wersa_backward(wersa_ctx* ctx, const void* Q, const void* K, const 
   const bool pooled_term = gate_w != nullptr;
   WERSA_STEP(1, "haar_backward_kq",
              launch_haar_backward(p, w, 1, K, w.dKF, dK, Q, w.dQF, pooled_term ? nullptr : dQ, kind, gkind, d, st, &launches));
-  WERSA_STEP(1, "gate_backward",
-             launch_gate_backward(p, w, haar_band_blocks(p, d), beta, gate_w, omega,
-                                  p.use_tc ? p.bctas : p.use_xb ? p.xprep : p.slabs * p.schunks, dbeta, dgate_w, dgate_b, domega,
-                                  st, &launches));
+  const int n_sumdD = p.use_tc ? p.bctas : p.use_xb ? p.xprep : p.slabs * p.schunks;
   if (pooled_term)
-    WERSA_STEP(1, "haar_filter_dq",
-               launch_haar_filter_addvec(p, w.dQF, w.f, w.dqbar, 1.f / (float)p.cfg.seq_len, dQ, gkind, d, st, &launches));
+    WERSA_STEP(1, "gate_backward_dq",
+               launch_gate_backward_dq(p, w, haar_band_blocks(p, d), beta, gate_w, omega, n_sumdD, dbeta, dgate_w, dgate_b, domega, dQ,
+                                       gkind, st, &launches));
+  else
+    WERSA_STEP(1, "gate_backward",
+               launch_gate_backward(p, w, haar_band_blocks(p, d), beta, gate_w, omega, n_sumdD, dbeta, dgate_w, dgate_b, domega, st,
+                                    &launches));
   ctx->launches_bwd = launches;
   return WERSA_OK;
 }

@@ -95,6 +95,11 @@ cudaError_t launch_gate_backward(const Plan& p, const Ws& w, int band_blocks, co
                                  const float* omega, int n_sumdD, float* dbeta, float* dgate_w, float* dgate_b,
                                  float* domega, cudaStream_t st, int* launches);
 
+// Gate backward and dQ, in one launch or up to three (see launch_haar_dq).
+cudaError_t launch_gate_backward_dq(const Plan& p, const Ws& w, int band_blocks, const float* beta, const float* gate_w,
+                                    const float* omega, int n_sumdD, float* dbeta, float* dgate_w, float* dgate_b, float* domega,
+                                    void* dQ, int out_kind, cudaStream_t st, int* launches);
+
 // Mean pool + gate with their scratch in a file-scope device array (no caller workspace).
 cudaError_t static_scratch_address(int device, float** out);
 size_t static_scratch_capacity_floats();      // floats available to the partial sums and sigmoids
@@ -120,6 +125,12 @@ cudaError_t launch_f32_planes(const Plan& p, const Ws& w, const void* Q, const v
 // dX = T_f(G) + vec[slab] * vec_scale on every row (G fp32, vec = slabs x 64 floats).
 cudaError_t launch_haar_filter_addvec(const Plan& p, const float* G, const float* f, const float* vec,
                                       float vec_scale, void* dX, int out_kind, int d, cudaStream_t st, int* launches);
+// The same with the row vector d q-bar / n worked out in the pass, and with the gradients of the gate's parameters and of beta: where
+// haar_dq_takes_gate; from the partial band inner products themselves where haar_dq_sums_bands, else behind launch_band_reduce.
+struct GateBwdArgs;
+bool haar_dq_takes_gate(const Plan& p);
+bool haar_dq_sums_bands(const Plan& p);
+cudaError_t launch_haar_dq(const Plan& p, const Ws& w, const GateBwdArgs& args, void* dQ, int out_kind, cudaStream_t st, int* launches);
 // dX = T_f(G) (G fp32) and the band inner products of (G, X), one partial for each of haar_band_blocks(p, d)
 // CTAs per slab, into bands[which]; dX == nullptr: only the band inner products.  X2 / G2 / dX2: the other tensor
 // (bands[1 - which]) in the same launch, after the first, or null.

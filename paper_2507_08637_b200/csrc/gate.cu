@@ -2,6 +2,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "gate_backward.cuh"
 
 namespace wersa {
 namespace {
@@ -292,150 +293,13 @@ __global__ void __launch_bounds__(kD) k_sum_floats(const float* __restrict__ x, 
   if (c == 0) out[0] = part[0];
 }
 
-// Chain rule through f = sigmoid(u) * omega, u = gate(qbar): domega, dgate_b, dgate_w, dqbar; and the
-// bandwidth gradient dbeta = 2 eps m bw * sum_t dDh_t (ReLU is positively homogeneous, so beta only
-// acts through eps).  Grid H + 2, 256 threads: CTA h < H handles head h, CTA H sums domega, CTA H + 1 sums dbeta; every
-// sum has a fixed order.  In CTA h the 256 threads work out du of 28 batch elements x 9 levels at a time, one each, while
-// q-bar is on its way; then thread (c = column of q-bar, q) takes the batch elements q, q + 4, ... of the round.  All of
-// it is latency: with the reduction before it 36 us at B=32 H=4 with a barrier and a dependent load per batch element,
-// 20 us with every thread working out du itself (with the gate shared by the heads nine loads after one another:
-// 19 us at B=5 H=3), 11 now (9 at B=5 H=3).
-__device__ __forceinline__ float gate_df(const float* __restrict__ df, int b, int h, int H, int per_head, int i) {
-  if (per_head) return __ldcg(df + ((size_t)b * H + h) * kBandVals + i);
-  float s = 0.f;
-#pragma unroll 4
-  for (int hh = 0; hh < H; ++hh) s += __ldcg(df + ((size_t)b * H + hh) * kBandVals + i);
-  return s;
-}
-// kParts = 4 parts of 64 threads, 16 where the batch is more than one round of four: at B=341 H=3 13 rounds of two
-// latencies each, and 22 for domega, took 37 us of a training step of 291, with 16 parts 16 (the step 271).
-// Sum of the parts' values in pairs of pairs.
-template <int kParts, typename F>
-__device__ __forceinline__ float sum_parts(F value) {
-  float s = (value(0) + value(1)) + (value(2) + value(3));
-#pragma unroll
-  for (int a = 4; a < kParts; a += 4) s += (value(a) + value(a + 1)) + (value(a + 2) + value(a + 3));
-  return s;
-}
+// (launched as a programmatic dependent: see launch_after; the pass that writes dQ may be placed ahead of this kernel's wait, and
+// unless it is the first one of its pass the gate weights are fetched ahead of it)
 template <int kParts>
-__global__ void __launch_bounds__(64 * kParts) k_gate_backward(
-    const float* __restrict__ df, const float* __restrict__ sg, const float* __restrict__ qbar,
-    const float* __restrict__ gate_w, const float* __restrict__ omega, const float* __restrict__ sumdD,
-    int n_sumdD, const float* __restrict__ beta, float eps, float bw_floor, int m, int B, int H, int dcols, int L1,
-    int per_head, float* __restrict__ dbeta, float* __restrict__ dgate_w, float* __restrict__ dgate_b,
-    float* __restrict__ domega, float* __restrict__ dqbar, bool first) {
-  // (launched as a programmatic dependent: see launch_after; the pass that writes dQ may be placed ahead of this kernel's
-  // wait, and unless it is the first one of its pass the gate weights are fetched ahead of it)
+__global__ void __launch_bounds__(64 * kParts) k_gate_backward(const float* df, const GateBwdArgs args, bool first) {
   if (first) wait_for_stream_predecessor();
   let_stream_successor_start();
-  constexpr int kThreads = 64 * kParts;
-  constexpr int kGateRound = 7 * kParts;   // batch elements of a round: seven a part, 7 x 9 values for its 64 threads
-  static_assert(kGateRound * (kMaxLevels + 1) <= kThreads, "a value of a round per thread");
-  __shared__ float part[kParts][kMaxLevels + 1][kD];
-  __shared__ float gbs[kParts][kMaxLevels + 1];
-  __shared__ float dus[kGateRound][kMaxLevels + 1];
-  float* flat = &part[0][0][0];
-  const int tid = threadIdx.x;
-  if ((int)blockIdx.x < H) {
-    const int h = blockIdx.x, c = tid & (kD - 1), q = tid >> 6;
-    float gw[kMaxLevels + 1], gw_acc[kMaxLevels + 1], gb_acc[kMaxLevels + 1];
-#pragma unroll
-    for (int i = 0; i <= kMaxLevels; ++i) {
-      gw_acc[i] = gb_acc[i] = 0.f;
-      gw[i] = i < L1 && gate_w != nullptr && c < dcols ? gate_w[((size_t)h * dcols + c) * L1 + i] : 0.f;
-    }
-    wait_for_stream_predecessor();
-    const int db = tid / (kMaxLevels + 1), di = tid - db * (kMaxLevels + 1);   // this thread's du of a round
-    for (int b0 = 0; b0 < B; b0 += kGateRound) {
-      float qb[kGateRound / kParts];
-#pragma unroll
-      for (int r = 0; r < kGateRound / kParts; ++r) {
-        const int b = b0 + q + kParts * r;
-        qb[r] = b < B ? qbar[((size_t)b * H + h) * kD + c] : 0.f;
-      }
-      if (b0 > 0) __syncthreads();   // the round before has been read
-      if (db < kGateRound) {
-        float du = 0.f;
-        if (di < L1 && b0 + db < B) {
-          const float s = sg[((size_t)(b0 + db) * H + h) * L1 + di];
-          du = gate_df(df, b0 + db, h, H, per_head, di) * omega[di] * s * (1.f - s);
-        }
-        dus[db][di] = du;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int r = 0; r < kGateRound / kParts; ++r) {
-        const int b = b0 + q + kParts * r;
-        if (b >= B) break;
-        float dq = 0.f;
-#pragma unroll
-        for (int i = 0; i <= kMaxLevels; ++i)
-          if (i < L1) {
-            const float du = dus[q + kParts * r][i];
-            gw_acc[i] += qb[r] * du;
-            gb_acc[i] += du;
-            if (gate_w != nullptr) dq += gw[i] * du;   // (none without weights, whatever du is)
-          }
-        dqbar[((size_t)b * H + h) * kD + c] = dq;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i <= kMaxLevels; ++i) {
-      part[q][i][c] = gw_acc[i];
-      if (c == 0) gbs[q][i] = gb_acc[i];
-    }
-    __syncthreads();
-    for (int e = tid; e < dcols * L1; e += kThreads) {   // (columns past the head dimension are padding of qbar)
-      const int cc = e / L1, i = e - cc * L1;
-      if (dgate_w != nullptr)
-        dgate_w[(size_t)h * dcols * L1 + e] = sum_parts<kParts>([&](int a) { return part[a][i][cc]; });
-    }
-    if (dgate_b != nullptr && tid < L1)
-      dgate_b[h * L1 + tid] = per_head || h == 0 ? sum_parts<kParts>([&](int a) { return gbs[a][tid]; }) : 0.f;
-  } else if ((int)blockIdx.x == H) {
-    // domega[i] = sum over slabs of df_i * sigmoid(u_i): thread (i = tid & 15, q = tid >> 4) takes every (4 kParts)th batch
-    // element, then the parts are added in order
-    const int i = tid & 15, q = tid >> 4;
-    float acc = 0.f;
-    wait_for_stream_predecessor();
-    if (domega != nullptr && i < L1) {
-      for (int b = q; b < B; b += 4 * kParts) {
-        if (per_head) {
-#pragma unroll 4
-          for (int h = 0; h < H; ++h) {
-            const int slab = b * H + h;
-            acc += __ldcg(df + (size_t)slab * kBandVals + i) * sg[(size_t)slab * L1 + i];
-          }
-        } else {
-          acc += gate_df(df, b, 0, H, 0, i) * sg[((size_t)b * H) * L1 + i];
-        }
-      }
-    }
-    flat[tid] = acc;
-    __syncthreads();
-    if (domega != nullptr && tid < L1) {
-      float s = 0.f;
-#pragma unroll
-      for (int r = 0; r < 4 * kParts; ++r) s += flat[16 * r + tid];
-      domega[tid] = s;
-    }
-  } else {
-    wait_for_stream_predecessor();
-    float tot = 0.f;
-#pragma unroll 4
-    for (int i = tid; i < n_sumdD; i += kThreads) tot += __ldcg(sumdD + i);
-    flat[tid] = tot;
-    __syncthreads();
-    for (int o = kThreads / 2; o > 0; o >>= 1) {
-      if (tid < o) flat[tid] += flat[tid + o];
-      __syncthreads();
-    }
-    if (dbeta != nullptr && tid == 0) {
-      const float bt = beta[0];
-      const float bw = fmaxf(bt, bw_floor);
-      dbeta[0] = bt > bw_floor ? 2.f * eps * (float)m * bw * flat[0] : 0.f;
-    }
-  }
+  gate_backward_cta<kParts>(blockIdx.x, GivenDf{df}, args, []() { wait_for_stream_predecessor(); });
 }
 
 }  // namespace
@@ -542,14 +406,13 @@ size_t static_scratch_floats_needed(const Plan& p) {
 }
 size_t static_scratch_counters_needed(const Plan& p) { return (size_t)p.slabs + (size_t)p.cfg.batch; }
 
-static void gate_backward_kernel(const Plan& p, const Ws& w, const float* df, const float* beta, const float* gate_w,
-                                 const float* omega, const float* sumdD, int n_sumdD, float* dbeta, float* dgate_w,
-                                 float* dgate_b, float* domega, bool first, cudaStream_t st) {
-  auto go = [&](auto kernel, int threads) {
-    launch_after(kernel, dim3(p.cfg.heads + 2), dim3(threads), 0, st, df, w.sg, w.qbar, gate_w, omega, sumdD, n_sumdD, beta,
-                 p.cfg.eps, p.cfg.bw_floor, p.cfg.features, p.cfg.batch, p.cfg.heads, p.cfg.head_dim, p.L1, p.cfg.gate_per_head,
-                 dbeta, dgate_w, dgate_b, domega, w.dqbar, first);
-  };
+static GateBwdArgs gate_args(const Plan& p, const Ws& w, const float* beta, const float* gate_w, const float* omega, const float* sumdD,
+                             int n_sumdD, float* dbeta, float* dgate_w, float* dgate_b, float* domega, float* dqbar) {
+  return {w.sg, w.qbar, gate_w, omega, sumdD, beta, n_sumdD, p.cfg.eps, p.cfg.bw_floor, p.cfg.features, p.cfg.batch, p.cfg.heads,
+          p.cfg.head_dim, p.L1, p.cfg.gate_per_head, dbeta, dgate_w, dgate_b, domega, dqbar};
+}
+static void gate_backward_kernel(const Plan& p, const float* df, const GateBwdArgs& args, bool first, cudaStream_t st) {
+  auto go = [&](auto kernel, int threads) { launch_after(kernel, dim3(p.cfg.heads + 2), dim3(threads), 0, st, df, args, first); };
   if (p.cfg.batch <= 28) go(k_gate_backward<4>, 256);
   else go(k_gate_backward<16>, 1024);
 }
@@ -566,7 +429,7 @@ cudaError_t launch_band_sums(const Plan& p, const Ws& w, int band_blocks, int n_
 cudaError_t launch_gate_backward_from(const Plan& p, const Ws& w, const float* df, const float* sumdD_total,
                                       const float* beta, const float* gate_w, const float* omega, float* dbeta,
                                       float* dgate_w, float* dgate_b, float* domega, cudaStream_t st, int* launches) {
-  gate_backward_kernel(p, w, df, beta, gate_w, omega, sumdD_total, 1, dbeta, dgate_w, dgate_b, domega, true, st);
+  gate_backward_kernel(p, df, gate_args(p, w, beta, gate_w, omega, sumdD_total, 1, dbeta, dgate_w, dgate_b, domega, w.dqbar), true, st);
   *launches += 1;
   return cudaGetLastError();
 }
@@ -576,9 +439,26 @@ cudaError_t launch_gate_backward(const Plan& p, const Ws& w, int band_blocks, co
                                  float* domega, cudaStream_t st, int* launches) {
   float* df = w.dqbar + (size_t)p.slabs * kD;   // df lives behind dqbar in the same region
   launch_after(k_band_reduce, dim3(p.slabs), dim3(256), 0, st, w.bands, p.slabs, band_blocks, p.cfg.levels, df);
-  gate_backward_kernel(p, w, df, beta, gate_w, omega, w.sumdD, n_sumdD, dbeta, dgate_w, dgate_b, domega, false, st);
+  gate_backward_kernel(p, df, gate_args(p, w, beta, gate_w, omega, w.sumdD, n_sumdD, dbeta, dgate_w, dgate_b, domega, w.dqbar), false, st);
   *launches += 2;
   return cudaGetLastError();
+}
+
+cudaError_t launch_gate_backward_dq(const Plan& p, const Ws& w, int band_blocks, const float* beta, const float* gate_w,
+                                    const float* omega, int n_sumdD, float* dbeta, float* dgate_w, float* dgate_b, float* domega,
+                                    void* dQ, int out_kind, cudaStream_t st, int* launches) {
+  if (!haar_dq_takes_gate(p)) {
+    const cudaError_t err = launch_gate_backward(p, w, band_blocks, beta, gate_w, omega, n_sumdD, dbeta, dgate_w, dgate_b, domega, st, launches);
+    return err != cudaSuccess ? err
+                              : launch_haar_filter_addvec(p, w.dQF, w.f, w.dqbar, 1.f / (float)p.cfg.seq_len, dQ, out_kind,
+                                                          p.cfg.head_dim, st, launches);
+  }
+  if (!haar_dq_sums_bands(p)) {
+    launch_after(k_band_reduce, dim3(p.slabs), dim3(256), 0, st, w.bands, p.slabs, band_blocks, p.cfg.levels, w.dqbar + (size_t)p.slabs * kD);
+    *launches += 1;
+  }
+  return launch_haar_dq(p, w, gate_args(p, w, beta, gate_w, omega, w.sumdD, n_sumdD, dbeta, dgate_w, dgate_b, domega, nullptr), dQ, out_kind,
+                        st, launches);
 }
 
 }  // namespace wersa

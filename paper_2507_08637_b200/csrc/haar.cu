@@ -11,6 +11,7 @@
 // between a tile's loads and its stores; B=4 H=8 n=16384: inner products of Q 55 -> 47 us, dK with products 69 -> 61 us.)
 // Rows past the end of the sequence read as zero, which is the zero padding of Algorithm 2.
 #include "common.cuh"
+#include "gate_backward.cuh"
 
 namespace wersa {
 namespace {
@@ -187,6 +188,140 @@ __global__ void __launch_bounds__(256, 4) k_haar_filter(const Tin* __restrict__ 
     add_coarse4(ex, k, warp, cg * 4, hi);
   }
   Tout* dst = (blockIdx.z == 0 ? XF : XF2) + ((size_t)slab * n + row0) * d + col0;
+#pragma unroll
+  for (int j = 0; j < 8; j += 4) {   // four rows (one level-2 block) at a time
+    float y[4][4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float a0 = x[j][c] + x[j + 1][c], a1 = x[j + 2][c] + x[j + 3][c];
+      const float c2 = fmaf(k.k[2], a0 + a1, hi[c]);
+      const float c10 = fmaf(k.k[1], a0, c2), c11 = fmaf(k.k[1], a1, c2);
+      y[0][c] = fmaf(k.f0, x[j][c], c10);
+      y[1][c] = fmaf(k.f0, x[j + 1][c], c10);
+      y[2][c] = fmaf(k.f0, x[j + 2][c], c11);
+      y[3][c] = fmaf(k.f0, x[j + 3][c], c11);
+    }
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj)
+      if (j + jj < rows) store4(dst + (size_t)(j + jj) * d, y[jj]);
+  }
+}
+
+// The last pass of a backward with gate weights: dQ = T_f(dQ_F) + d q-bar / n on every row, as k_haar_filter with a row vector, which
+// is worked out here: every CTA of a slab takes df (16 numbers), du and the slab's d q-bar (64) for itself while its rows are on
+// their way, and the first H + 2 CTAs do what k_gate_backward does for the parameters.  All of that is latency, some 7 us of
+// it on 2 x 4 x 4096 whether in one launch or three; what one launch saves is their placement and the host's 2 us for each.  Training
+// steps: 2 x 2 x 256, d = 16, m = 256 bf16 56.1 -> 53 us (with the forward's one launch 46.6); 1 x 3 x 440, m = 256 fp32 70.4 -> 67.1; 5 x 3 x
+// 1777, m = 256 90.4 -> 89.3; 2 x 4 x 4096, d = 32, fp32 107.7 -> 106.7; from 16 x 12 x 1024 on the same.
+// kSum: df from the partials of `blocks` CTAs per slab and tensor, else from the reduction's result.
+// grid: H + 2 + slabs * blocks.
+template <bool kFull, typename Tout, bool kSum>
+__global__ void __launch_bounds__(256, 4) k_haar_dq(const float* __restrict__ G, const float* __restrict__ f, Tout* __restrict__ dQ,
+                                                    int n, int d_arg, int L, int slabs, int blocks, float inv_n, const float* df_in,
+                                                    const GateBwdArgs args) {
+  // (launched as a programmatic dependent: see launch_after)
+  const int H = args.H;
+  if ((int)blockIdx.x < H + 2) {
+    auto wait = []() { wait_for_stream_predecessor(); };
+    if constexpr (kSum) gate_backward_cta<4>(blockIdx.x, SummedDf{df_in, slabs, blocks, L}, args, wait);
+    else gate_backward_cta<4>(blockIdx.x, GivenDf{df_in}, args, wait);
+    return;
+  }
+  const int d = kFull ? kD : d_arg;
+  __shared__ __align__(16) float ex[8][kHalfD];   // 32-row sums of the warps
+  __shared__ float gws[kMaxLevels + 1][kD], red[16][kBandVals + 1], dus[kMaxLevels + 1];
+  __shared__ __align__(16) float vec[kD];
+  const int at_block = gridDim.x - 1 - blockIdx.x;   // (backwards: see k_haar_filter)
+  const int slab = at_block / blocks, bx = at_block - slab * blocks;
+  const int tid = threadIdx.x, warp = tid >> 5, cg = tid & 7, rg = tid >> 3;
+  const ColMap<32> at(bx, cg * 4, d);
+  const int row0 = at.row0 + rg * 8;
+  const int col0 = at.col;   // first of this thread's four columns
+  const int rows = at.on ? n - row0 : 0;   // rows of this thread inside the sequence
+  float x[8][4];
+  {
+    const float* xp = G + ((size_t)slab * n + row0) * d + col0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (j < rows) {
+        load4<true>(xp + (size_t)j * d, x[j]);
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) x[j][c] = 0.f;
+      }
+    }
+  }
+  // (gate weights are arguments, f and the sigmoids the forward's)
+  const int h = slab % H;
+  for (int e = tid; e < d * (L + 1); e += 256) {
+    const int c = e / (L + 1);
+    gws[e - c * (L + 1)][c] = args.gate_w[(size_t)h * d * (L + 1) + e];
+  }
+  float slope = 0.f;
+  if (tid <= L) {
+    const float sgm = args.sg[(size_t)slab * (L + 1) + tid];
+    slope = args.omega[tid] * sgm * (1.f - sgm) * inv_n;
+  }
+  const LevelCoef k = level_coef(f + (size_t)slab * (L + 1), L);
+  float hi[4], s5[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const float s3 = ((x[0][c] + x[1][c]) + (x[2][c] + x[3][c])) + ((x[4][c] + x[5][c]) + (x[6][c] + x[7][c]));
+    const float s4 = sum16(s3);
+    s5[c] = sum32(s4);
+    hi[c] = fmaf(k.k[3], s3, fmaf(k.k[4], s4, k.k[5] * s5[c]));
+  }
+  if (L > 5 && (tid & 24) == 0) *reinterpret_cast<float4*>(&ex[warp][cg * 4]) = make_float4(s5[0], s5[1], s5[2], s5[3]);
+  wait_for_stream_predecessor();
+  {
+    // df: slot j by sixteen threads; the gate of a batch element sums over its heads
+    const int j = tid & (kBandVals - 1), pt = tid >> 4;
+    const int first = args.per_head ? slab : slab - h, count = args.per_head ? 1 : H;
+    float s = 0.f;
+    if (j <= L) {
+      if constexpr (kSum) {
+        const float* src = df_in + (j < L ? j : 8 + L - 1);
+        const int all = count * blocks;   // of one tensor: the partials of neighbouring slabs lie side by side
+        for (int t = pt; t < all; t += 48) {   // (three at a time: see haar_dq_sums_bands)
+          float v[6];
+#pragma unroll
+          for (int e = 0; e < 3; ++e) {
+            const float* q = src + ((size_t)first * blocks + min(t + 16 * e, all - 1)) * kBandVals;
+            v[2 * e] = __ldcg(q);
+            v[2 * e + 1] = __ldcg(q + (size_t)slabs * blocks * kBandVals);
+          }
+#pragma unroll
+          for (int e = 0; e < 3; ++e) s += t + 16 * e < all ? v[2 * e] + v[2 * e + 1] : 0.f;
+        }
+      } else {
+        for (int t = pt; t < count; t += 16) s += __ldcg(df_in + (size_t)(first + t) * kBandVals + j);
+      }
+    }
+    red[pt][j] = s;
+    __syncthreads();
+    if (tid <= L) {
+      float df = 0.f;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) df += red[q][tid];
+      dus[tid] = df * slope;
+    }
+    __syncthreads();
+    if (tid < d) {
+      float v = 0.f;
+      for (int i = 0; i <= L; ++i) v = fmaf(gws[i][tid], dus[i], v);
+      vec[tid] = v;
+    }
+    __syncthreads();
+  }
+  if (at.on) {
+    const float4 v = *reinterpret_cast<const float4*>(&vec[col0]);
+    hi[0] += v.x;
+    hi[1] += v.y;
+    hi[2] += v.z;
+    hi[3] += v.w;
+  }
+  if (L > 5) add_coarse4(ex, k, warp, cg * 4, hi);
+  Tout* dst = dQ + ((size_t)slab * n + row0) * d + col0;
 #pragma unroll
   for (int j = 0; j < 8; j += 4) {   // four rows (one level-2 block) at a time
     float y[4][4];
@@ -732,6 +867,33 @@ cudaError_t launch_haar_filter_addvec(const Plan& p, const float* G, const float
       err = launch_after(k_haar_filter<kFull, float, float, true>, grid, dim3(256), 0, st, G, f, (float*)dX, nullptr, nullptr, n, d, L, vec, vec_scale, true, false);
     else
       err = launch_after(k_haar_filter<kFull, float, bf, true>, grid, dim3(256), 0, st, G, f, (bf*)dX, nullptr, nullptr, n, d, L, vec, vec_scale, true, false);
+  })
+  *launches += 1;
+  return err != cudaSuccess ? err : cudaGetLastError();
+}
+
+// The gate's CTAs take rounds of 28 batch elements after one another, and beyond four of them k_gate_backward with its 1024 threads
+// is the faster one; df is summed in place while a CTA reads at most some 40 partials a slot for its own slab (or batch element) and the
+// one of d omega 2048 for all of them.
+bool haar_dq_takes_gate(const Plan& p) { return p.cfg.batch <= 112; }
+bool haar_dq_sums_bands(const Plan& p) {
+  const long long blocks = haar_band_blocks(p, p.cfg.head_dim);
+  return blocks * (p.cfg.gate_per_head ? 1 : p.cfg.heads) <= 48 && blocks * p.slabs <= 2048;
+}
+cudaError_t launch_haar_dq(const Plan& p, const Ws& w, const GateBwdArgs& args, void* dQ, int out_kind, cudaStream_t st, int* launches) {
+  const int n = p.cfg.seq_len, L = p.cfg.levels, d = p.cfg.head_dim, blocks = col_blocks<32>(p.htiles, d);
+  const dim3 grid((unsigned)(p.cfg.heads + 2 + p.slabs * blocks));
+  const float* df = haar_dq_sums_bands(p) ? w.bands : w.dqbar + (size_t)p.slabs * kD;
+  using bf = __nv_bfloat16;
+  auto go = [&](auto kernel, auto* out) {
+    return launch_after(kernel, grid, dim3(256), 0, st, (const float*)w.dQF, (const float*)w.f, out, n, d, L, p.slabs, blocks,
+                        1.f / (float)n, df, args);
+  };
+  cudaError_t err;
+  const bool sum = haar_dq_sums_bands(p);
+  WERSA_FULL({
+    if (out_kind == 0) err = sum ? go(k_haar_dq<kFull, float, true>, (float*)dQ) : go(k_haar_dq<kFull, float, false>, (float*)dQ);
+    else err = sum ? go(k_haar_dq<kFull, bf, true>, (bf*)dQ) : go(k_haar_dq<kFull, bf, false>, (bf*)dQ);
   })
   *launches += 1;
   return err != cudaSuccess ? err : cudaGetLastError();
