@@ -452,7 +452,7 @@ static_assert(4 * kQRegsCtl + kQElemWarps * kQRegsElem <= (kQThreads / 32) * kQR
               "roles may not claim more registers than the CTA was launched with");
 
 struct alignas(8) BwdQBars {
-  uint64_t w_full, x_full, x_empty, do_full, do_empty, s_full, s_free, a_full, a_read, g_full, da_ready[4], dq_full, staged, p_free;
+  uint64_t w_full, x_full, x_empty, do_full[2], do_empty[2], s_full, s_free, a_full, a_read, g_full, da_ready[4], dq_full, staged, p_free;
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -463,8 +463,9 @@ template <int NH> struct BwdQSmem {
   static constexpr uint32_t p = slo + NH * kTileBytes;       // R / D, 2 NH blocks of 128 tokens x 64 features; result staging
   static constexpr uint32_t scratch = p + 2 * kTileBytes;    // (dz' sums at the end of a segment: R / D is dead then)
   static constexpr uint32_t x = p + 4 * kTileBytes;          // three Q_F planes
+  static constexpr int dos = NH == 1 ? 2 : 1;                // buffers of dO
   static constexpr uint32_t g = x + 3 * kTileBytes;          // dO
-  static constexpr uint32_t zs = g + kTileBytes;             // NH x 128 floats
+  static constexpr uint32_t zs = g + dos * kTileBytes;       // NH x 128 floats
   static constexpr uint32_t cs = zs + NH * 512;              // 128 floats
   static constexpr uint32_t bars = cs + 512;
   static constexpr uint32_t total = bars + 256 + 1024;       // + alignment slack
@@ -488,6 +489,8 @@ constexpr uint32_t kIdescT = make_idesc_bf16(128, 64, true, true);   // contract
 // pass (B=4 H=8 n=16384 m=256 202 us; 205 with R rounded first).  What bounds a tile (m = 256): 4.8 k cycles of tensor
 // pipe (1.5 A, 1.0 G, 0.8 dS', 1.4 dQ_F; 35 % of the time) plus num and the first half of dA, during which the pipe has
 // nothing to do (X is the only accumulator that fits).
+// With m = 128 X is double: A of the next tile is formed beside G and the last MMAs of this one, and taken before dz' and dQ_F
+// (16 x 12 x 1024 55.4 -> 53.5 us).
 // kGroup: the launch handles one group of 256 features of a wider feature map.  The denominator of Eq. 7 and
 // dD' then belong to the whole map and come from den_ext / dd_ext (one float per token), and with kAdd the
 // group's share of dQ_F is added to what the groups before it left.
@@ -512,10 +515,14 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
   const int g0 = (int)(tiles_all * blockIdx.x / gridDim.x), g1 = (int)(tiles_all * (blockIdx.x + 1) / gridDim.x);
 
   if (threadIdx.x == 0) {
-    uint64_t* one[] = {&bars->w_full, &bars->x_full, &bars->x_empty, &bars->do_full, &bars->do_empty, &bars->s_full,
-                       &bars->s_free, &bars->a_full, &bars->g_full, &bars->dq_full, &bars->p_free};
+    uint64_t* one[] = {&bars->w_full, &bars->x_full, &bars->x_empty, &bars->s_full, &bars->s_free, &bars->a_full, &bars->g_full,
+                       &bars->dq_full, &bars->p_free};
 #pragma unroll
-    for (int i = 0; i < 11; ++i) mbar_init(one[i], 1);
+    for (int i = 0; i < 9; ++i) mbar_init(one[i], 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&bars->do_full[i], 1);
+      mbar_init(&bars->do_empty[i], 1);
+    }
     mbar_init(&bars->a_read, kQElemWarps);
     for (int i = 0; i < 4; ++i) mbar_init(&bars->da_ready[i], kQElemWarps);
     mbar_init(&bars->staged, kQElemWarps);
@@ -535,8 +542,8 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kQRegsCtl));
     if (warp == 0 && lane == 0) {
-      // ---- copies.  Every buffer is single: the planes of the next tile are fetched as soon as A has been formed,
-      // dO as soon as dS' has taken it, both well before they are needed.
+      // ---- copies.  The planes of the next tile are fetched as soon as A has been formed, dO as soon as dS' has taken it (one
+      // buffer; two where the next tile's G is wanted before that), both before they are needed.
       mbar_arrive_expect_tx(&bars->w_full, NH * kTileBytes);
 #pragma unroll
       for (int h = 0; h < NH; ++h) tma_load_3d(smem + SL::wt + h * kTileBytes, &map_w, 0, h * kTile, 0, &bars->w_full);
@@ -552,10 +559,11 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
         for (int pl = 0; pl < 3; ++pl)
           tma_load_3d(smem + SL::x + pl * kTileBytes, &map_qf, 0, r0, pl * slabs + slab, &bars->x_full);
         ++x_sent;
-        if (it > 0) ok = mbar_wait(&bars->do_empty, (it - 1) & 1, abort_flag, status, kErrBwdCopy);
+        const int gb = it % SL::dos;
+        if (it >= SL::dos) ok = mbar_wait(&bars->do_empty[gb], (it / SL::dos - 1) & 1, abort_flag, status, kErrBwdCopy);
         if (!ok) break;
-        mbar_arrive_expect_tx(&bars->do_full, kTileBytes);
-        tma_load_3d(smem + SL::g, &map_do, 0, r0, slab, &bars->do_full);
+        mbar_arrive_expect_tx(&bars->do_full[gb], kTileBytes);
+        tma_load_3d(smem + SL::g + gb * kTileBytes, &map_do, 0, r0, slab, &bars->do_full[gb]);
         ++do_sent;
         if (slab != slab_now) {   // a segment begins: the images of S' of its slab
           slab_now = slab;
@@ -574,7 +582,7 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
       if (*abort_flag != 0) {   // let copies in flight land before the CTA's shared memory goes away
         mbar_wait_drain(&bars->w_full, 0);
         if (x_sent > 0) mbar_wait_drain(&bars->x_full, (x_sent - 1) & 1);
-        if (do_sent > 0) mbar_wait_drain(&bars->do_full, (do_sent - 1) & 1);
+        for (int t = max(0, do_sent - SL::dos); t < do_sent; ++t) mbar_wait_drain(&bars->do_full[t % SL::dos], (t / SL::dos) & 1);
         if (s_sent > 0) mbar_wait_drain(&bars->s_full, (s_sent - 1) & 1);
       }
     } else if (warp == 1 && lane == 0) {
@@ -588,16 +596,17 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
       uint32_t p_m = smem_desc_lo(smem_u32(smem + SL::p), kTileBytes);   // 64-feature blocks one tile apart
       constexpr uint32_t kTileStep = kTileBytes >> 4;
       // A and G take all features in one instruction: with N = 256 an instruction reads 12 KB of operands in its 128
-      // cycles, with N = 128 8 KB in 64, all the bandwidth shared memory has (measured: 105-115 cycles instead of 64)
+      // cycles, with N = 128 8 KB in 64, all the bandwidth shared memory has (measured: 105-115 cycles instead of 64; A in halves,
+      // the first of them as soon as dQ_F was done with that half of X, made 4 x 8 x 16384 2 % slower, m = 1024 3 %)
       constexpr uint32_t kIdescX = make_idesc_bf16(128, m, false, false);
-      auto issue_a = [&]() {
+      auto issue_a = [&](uint32_t dst) {
         asm volatile("" : "+r"(x_k), "+r"(wt_k));
 #pragma unroll
         for (int pl = 0; pl < 3; ++pl)
 #pragma unroll
           for (int k = 0; k < 4; ++k)
             if (k < ksteps)
-              mma_ss(tmem, smem_desc_join(x_k + pl * kTileStep + 2 * k, hi), smem_desc_join(wt_k + 2 * k, hi), kIdescX,
+              mma_ss(dst, smem_desc_join(x_k + pl * kTileStep + 2 * k, hi), smem_desc_join(wt_k + 2 * k, hi), kIdescX,
                      (pl > 0 || k > 0) ? 1u : 0u);
         mma_commit(&bars->a_full);
         mma_commit(&bars->x_empty);
@@ -608,19 +617,21 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
                 mbar_wait(&bars->x_full, 0, abort_flag, status, kErrBwdCopy);
       if (ok) {
         tc_fence_after_sync();
-        issue_a();
+        issue_a(tmem);
       }
       for (int it = 0; it < nt && ok; ++it) {
         const uint32_t par = it & 1;
+        const uint32_t x = tmem + (NH == 1 ? 128 * par : 0);   // this tile's X
+        const bool more = it + 1 < nt;
         // (the empty asm statements: the compiler would keep every descriptor of the unrolled loops in registers)
-        const int slab = (g0 + it) / tps;
+        const int slab = (g0 + it) / tps, gb = it % SL::dos;
         const bool fresh = slab != slab_now;   // first tile of a segment: dS' starts over
         if (fresh) {
           slab_now = slab;
           ok = mbar_wait(&bars->s_full, seg & 1, abort_flag, status, kErrBwdCopy);
           ++seg;
         }
-        ok = ok && mbar_wait(&bars->do_full, par, abort_flag, status, kErrBwdCopy) &&
+        ok = ok && mbar_wait(&bars->do_full[gb], (it / SL::dos) & 1, abort_flag, status, kErrBwdCopy) &&
              mbar_wait(&bars->a_read, par, abort_flag, status, kErrBwdMma);
         if (!ok) break;
         tc_fence_after_sync();
@@ -630,9 +641,16 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
 #pragma unroll
           for (int k = 0; k < 4; ++k)
             if (k < ksteps)
-              mma_ss(tmem, smem_desc_join(do_k + 2 * k, hi), smem_desc_join(s_k + part * NH * kTileStep + 2 * k, hi),
+              mma_ss(x, smem_desc_join(do_k + gb * kTileStep + 2 * k, hi), smem_desc_join(s_k + part * NH * kTileStep + 2 * k, hi),
                      kIdescX, (part > 0 || k > 0) ? 1u : 0u);
         mma_commit(&bars->g_full);
+        if (NH == 1 && more) {   // A of the next tile, in the other X, where the tile before had its dA
+          ok = (it == 0 || mbar_wait(&bars->dq_full, par ^ 1, abort_flag, status, kErrBwdMma)) &&
+               mbar_wait(&bars->x_full, par ^ 1, abort_flag, status, kErrBwdCopy);
+          if (!ok) break;
+          tc_fence_after_sync();
+          issue_a(tmem + 128 * (par ^ 1));
+        }
 #pragma unroll 1
         for (int h = 0; h < NH && ok; ++h) {
 #pragma unroll 1
@@ -645,27 +663,27 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
 #pragma unroll
               for (int k = 0; k < 8; ++k)
                 mma_ss(tmem + kAccS + h * 64, smem_desc_join(p_m + 2 * h * kTileStep + 128 * k, hi),
-                       smem_desc_join(do_n + 128 * k, hi), kIdescT, (!fresh || k > 0) ? 1u : 0u);
-              if (h == NH - 1) mma_commit(&bars->do_empty);
+                       smem_desc_join(do_n + gb * kTileStep + 128 * k, hi), kIdescT, (!fresh || k > 0) ? 1u : 0u);
+              if (h == NH - 1) mma_commit(&bars->do_empty[gb]);
             }
             asm volatile("" : "+r"(wt_n));
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
               for (int part = 0; part < 2; ++part)   // 16 columns per 16 features: 8 of hi pairs, 8 of lo pairs
-                mma_ts(tmem + kAccQ, tmem + h * 128 + 32 * i + 16 * q + 8 * part,
+                mma_ts(tmem + kAccQ, x + h * 128 + 32 * i + 16 * q + 8 * part,
                        smem_desc_join(wt_n + h * kTileStep + 128 * (2 * i + q), hi), kIdescC,
                        (h > 0 || q > 0 || i > 0 || part > 0) ? 1u : 0u);
           }
           if (ok && h == NH - 1) mma_commit(&bars->dq_full);   // (every MMA of the tile)
         }
-        if (ok && it + 1 < nt) {   // A of the next tile overwrites X once the MMAs that read dA there have completed
+        if (NH == 2 && ok && more) {   // A of the next tile overwrites X once the MMAs that read dA there have completed
           // (instructions with different shapes and accumulators are not ordered by being issued one after the other)
           ok = mbar_wait(&bars->dq_full, par, abort_flag, status, kErrBwdMma) &&
                mbar_wait(&bars->x_full, par ^ 1, abort_flag, status, kErrBwdCopy);
           if (!ok) break;
           tc_fence_after_sync();
-          issue_a();
+          issue_a(tmem);
         }
       }
     } else if (warp == 2 && lane == 0) {
@@ -704,207 +722,237 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
       ok = group_wait(bar, par, wq == 0, ok, 2 + (warp & 3), 128, abort_flag, status, kErrBwdMma);
       if (ok) tc_fence_after_sync();
     };
-    int it = 0;
-    for (int gt = g0; gt < g1 && ok;) {
-      const int slab = gt / tps, seg_end = min(g1, (slab + 1) * tps);
-      // (every thread is past its last use of z' and of the scratch)
-      if (et < m) zs[et] = zg[(size_t)slab * z_stride + et];
-      named_bar_sync(1, kQElem);
-      float dz[8];
+    const int nt = g1 - g0;
+    // The tile whose A is taken next.  (Stepped along: a division by the tiles of a slab in every thread and tile cost 1 k cycles a tile.)
+    int slab = g0 / tps, row0 = (g0 - slab * tps) * kTile;
+    uint32_t kept[NH][16];              // NH = 1: R / D of the tile whose A was read last
+    float inv = 0.f, c = 0.f;           // 1 / D of the tile whose A was read last (0 past the end: such rows contribute nothing); with kGroup c
+    // kGroup: D and dD' of the next tile's token, a tile ahead of their use (with the division above 183 -> 168 us a group of 32 x 4 x
+    // 4096, d = 32)
+    float ext_d = 1.f, ext_dd = 0.f;
+    const float* zr = zs + 32 * wq;
+    auto fetch_ext = [&]() {
+      const size_t tok = (size_t)slab * n + min(row0 + tl, n - 1);
+      ext_d = load_after_wait(den_ext + tok);   // (in this place, not where the values are used)
+      ext_dd = load_after_wait(dd_ext + tok);
+    };
+    if (kGroup && nt > 0) fetch_ext();
+    // row sums over the four threads of a token, through spare TMEM columns (four for D', four for num / D)
+    auto row_total = [&](int it, uint32_t col, float share) {
+      tmem_st1(trow + kStat + col + wq, __float_as_uint(share));
+      tmem_st_wait();
+      tc_fence_before_sync();
+      if (it > 0 && col > 0) wait_all(&bars->p_free, (it & 1) ^ 1);   // (long past, as a rule)
+      else named_bar_sync(2 + (warp & 3), 128);
+      tc_fence_after_sync();
+      uint32_t st[4];
+      tmem_ld4(trow + kStat + col, st);
+      tmem_ld_wait();
+      reg_fence4(st);
+      return (__uint_as_float(st[0]) + __uint_as_float(st[1])) + (__uint_as_float(st[2]) + __uint_as_float(st[3]));
+    };
+    // ---- D', and R / D, rounded to bf16 once from R in 32 bits
+    auto take_a = [&](int it, uint32_t (&pp)[NH][16]) {
+      const uint32_t xrow = trow + (NH == 1 ? 128u * (it & 1) : 0u);
+      const bool on = row0 + tl < n;
+      if (it == 0 || row0 == 0) {   // a segment begins (every thread is past its last use of z')
+        if (et < m) zs[et] = zg[(size_t)slab * z_stride + et];
+        named_bar_sync(1, kQElem);
+      }
+      row0 += kTile;
+      if (row0 >= n) {
+        row0 = 0;
+        ++slab;
+      }
+      inv = 0.f;
+      if constexpr (kGroup) {
+        inv = on ? 1.f / ext_d : 0.f;
+        c = on ? ext_dd * ext_d : 0.f;
+        if (it + 1 < nt) fetch_ext();
+      }
+      uint32_t r[NH][32];
+      wait_all(&bars->a_full, it & 1);
+      if (!ok) return;   // (every wait has one answer for the lane quarter: its barriers may stand inside)
 #pragma unroll
-      for (int i = 0; i < 8; ++i) dz[i] = 0.f;
-      for (; gt < seg_end; ++gt, ++it) {
-        const uint32_t par = it & 1;
-        const int row0 = (gt - slab * tps) * kTile, row = row0 + tl;
-        const float* zr = zs + 32 * wq;
-        // ---- D', and R / D, rounded to bf16 once from R in 32 bits
-        float inv = 0.f, c = 0.f;   // (rows past the end contribute nothing)
-        wait_all(&bars->a_full, par);
-        if (ok) {   // (every wait has one answer for the lane quarter: its barriers may stand inside)
-          // row sums over the four threads of a token, through spare TMEM columns (four for D', four for num / D)
-          auto row_total = [&](uint32_t col, float share) {
-            tmem_st1(trow + kStat + col + wq, __float_as_uint(share));
-            tmem_st_wait();
-            tc_fence_before_sync();
-            if (it > 0 && col > 0) wait_all(&bars->p_free, par ^ 1);   // (long past, as a rule)
-            else named_bar_sync(2 + (warp & 3), 128);
-            tc_fence_after_sync();
-            uint32_t st[4];
-            tmem_ld4(trow + kStat + col, st);
-            tmem_ld_wait();
-            reg_fence4(st);
-            return (__uint_as_float(st[0]) + __uint_as_float(st[1])) + (__uint_as_float(st[2]) + __uint_as_float(st[3]));
-          };
-          uint32_t pp[NH][16];
-          {
-            uint32_t r[NH][32];
+      for (int h = 0; h < NH; ++h) tmem_ld32(xrow + h * 128 + 32 * wq, r[h]);
+      tmem_ld_wait();
 #pragma unroll
-            for (int h = 0; h < NH; ++h) tmem_ld32(trow + h * 128 + 32 * wq, r[h]);
-            if constexpr (kGroup) {
-              if (row < n) {
-                const float D = __ldcg(den_ext + (size_t)slab * n + row);
-                inv = 1.f / D;
-                c = __ldcg(dd_ext + (size_t)slab * n + row) * D;
-              }
-            }
-            tmem_ld_wait();
+      for (int h = 0; h < NH; ++h) reg_fence32(r[h]);
+      tc_fence_before_sync();
+      warp_arrive(&bars->a_read);   // X may become G
+      if constexpr (!kGroup) {
+        float den = 0.f, den2 = 0.f;
 #pragma unroll
-            for (int h = 0; h < NH; ++h) reg_fence32(r[h]);
-            tc_fence_before_sync();
-            warp_arrive(&bars->a_read);   // X may become G
-            if constexpr (!kGroup) {
-              float den = 0.f, den2 = 0.f;
+        for (int h = 0; h < NH; ++h) {
 #pragma unroll
-              for (int h = 0; h < NH; ++h) {
-#pragma unroll
-                for (int j = 0; j < 32; j += 4) {
-                  if ((j & 7) == 0) asm volatile("" ::: "memory");   // (z' is read as it is used, not kept in registers)
-                  const float4 z = *reinterpret_cast<const float4*>(zr + h * 128 + j);
-                  den = fmaf(fmaxf(__uint_as_float(r[h][j]), 0.f), z.x, den);
-                  den2 = fmaf(fmaxf(__uint_as_float(r[h][j + 1]), 0.f), z.y, den2);
-                  den = fmaf(fmaxf(__uint_as_float(r[h][j + 2]), 0.f), z.z, den);
-                  den2 = fmaf(fmaxf(__uint_as_float(r[h][j + 3]), 0.f), z.w, den2);
-                }
-              }
-              const float total = row_total(0, den + den2);
-              if (row < n) inv = 1.f / (epsp + total);
-            }
-#pragma unroll
-            for (int h = 0; h < NH; ++h)
-#pragma unroll
-              for (int j = 0; j < 16; ++j)
-                pp[h][j] = relu_pack_bf16x2(__uint_as_float(r[h][2 * j]) * inv, __uint_as_float(r[h][2 * j + 1]) * inv);
+          for (int j = 0; j < 32; j += 4) {
+            if ((j & 7) == 0) asm volatile("" ::: "memory");   // (z' is read as it is used, not kept in registers)
+            const float4 z = *reinterpret_cast<const float4*>(zr + h * 128 + j);
+            den = fmaf(fmaxf(__uint_as_float(r[h][j]), 0.f), z.x, den);
+            den2 = fmaf(fmaxf(__uint_as_float(r[h][j + 1]), 0.f), z.y, den2);
+            den = fmaf(fmaxf(__uint_as_float(r[h][j + 2]), 0.f), z.z, den);
+            den2 = fmaf(fmaxf(__uint_as_float(r[h][j + 3]), 0.f), z.w, den2);
           }
-          // ---- num / D = (R / D) . G
-          wait_all(&bars->g_full, par);
-          if constexpr (!kGroup) {
-            if (ok) {
-              f32x2 num = pk2(0.f, 0.f);
-              uint32_t a[16], b[16];
-              tmem_ld16(trow + 32 * wq, a);
+        }
+        const float total = row_total(it, 0, den + den2);
+        if (on) inv = 1.f / (epsp + total);
+      }
 #pragma unroll
-              for (int h = 0; h < NH; ++h) {
-                reg_fence16(pp[h]);   // (R / D is unpacked again in every pass, not kept unpacked)
-                tmem_ld_wait();
-                reg_fence16(a);
-                tmem_ld16(trow + h * 128 + 32 * wq + 16, b);
+      for (int h = 0; h < NH; ++h)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(pp[h][j]), pk2u(a[2 * j], a[2 * j + 1]), num);
-                tmem_ld_wait();
-                reg_fence16(b);
-                if (h + 1 < NH) tmem_ld16(trow + (h + 1) * 128 + 32 * wq, a);
+        for (int j = 0; j < 16; ++j)
+          pp[h][j] = relu_pack_bf16x2(__uint_as_float(r[h][2 * j]) * inv, __uint_as_float(r[h][2 * j + 1]) * inv);
+    };
+    float dz[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(pp[h][8 + j]), pk2u(b[2 * j], b[2 * j + 1]), num);
-              }
-              c = -row_total(4, sum2(num));
-            }
-          } else if (it > 0) {
-            wait_all(&bars->p_free, par ^ 1);
-          }
+    for (int i = 0; i < 8; ++i) dz[i] = 0.f;
+    // With one half of features X is double, and a tile's A is taken while the MMAs of the tile before it still run.
+#pragma unroll 1
+    for (int it = NH == 1 ? -1 : 0; it < nt; ++it) {   // (left where a barrier of all threads has given them one answer)
+      const uint32_t par = it & 1;
+      const uint32_t xrow = trow + (NH == 1 ? 128u * par : 0u);
+      uint32_t own[NH][16];   // (of the iteration alone: what was kept would have to be, up to a wait that runs out)
+      uint32_t(&pp)[NH][16] = NH == 1 ? kept : own;
+      if constexpr (NH == 2) take_a(it, pp);
+      const bool last = row0 == 0 || it + 1 == nt;   // the tile ends its segment (its A has been taken, the next one's has not)
+      const int now = row0 == 0 ? slab - 1 : slab;   // its slab
+      float scale = 0.f;   // of this tile's dQ_F
+      if (it >= 0) {
+        // ---- num / D = (R / D) . G
+        wait_all(&bars->g_full, par);
+        if (ok && last && it + 1 < nt && et == 0) mbar_arrive(&bars->s_free);   // (G was the last to read the images of S')
+        if constexpr (!kGroup) {
           if (ok) {
-            if (wq == 0) {
-              cs[tl] = c;
-              sum_dd += c * inv;
-            }
-            // ---- dA D (hi + lo, in place) and R / D to shared memory, 16 features at a time
-            // (the mask 1[R > 0], taken from R / D, cuts the packed pairs: a factor would have to be 1 for the smallest R
-            // too, and would let an infinity or NaN of a feature that is off through)
-            const f32x2 c2 = pk2(c, c), minus1 = pk2(-1.f, -1.f);
-            uint32_t a[2][16];
-            tmem_ld16(trow + 32 * wq, a[0]);
+            f32x2 num = pk2(0.f, 0.f);
+            uint32_t a[16], b[16];
+            tmem_ld16(xrow + 32 * wq, a);
 #pragma unroll
-            for (int h = 0; h < NH; ++h) reg_fence16(pp[h]);
-#pragma unroll
-            for (int s = 0; s < 2 * NH; ++s) {
-              const int h = s >> 1, q = s & 1;
-              const uint32_t col = trow + h * 128 + 32 * wq + 16 * q;
-              uint32_t(&g)[16] = a[s & 1];
+            for (int h = 0; h < NH; ++h) {
+              reg_fence16(pp[h]);   // (R / D is unpacked again in every pass, not kept unpacked)
               tmem_ld_wait();
-              reg_fence16(g);
-              if (s + 1 < 2 * NH) tmem_ld16(trow + ((s + 1) >> 1) * 128 + 32 * wq + 16 * ((s + 1) & 1), a[(s + 1) & 1]);
-              const float* z = zr + h * 128 + 16 * q;
-              uint32_t ph[8], pl[8];
+              reg_fence16(a);
+              tmem_ld16(xrow + h * 128 + 32 * wq + 16, b);
 #pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                if ((j & 1) == 0) asm volatile("" ::: "memory");
-                const float2 zz = *reinterpret_cast<const float2*>(z + 2 * j);
-                const uint32_t mk = positive_mask_bf16x2(pp[h][8 * q + j]);
-                const f32x2 val = fma2(c2, pk2(zz.x, zz.y), pk2u(g[2 * j], g[2 * j + 1]));
-                const uint32_t hv = pack2_bf16(val);
-                ph[j] = hv & mk;
-                pl[j] = pack2_bf16(fma2(minus1, unpack2_bf16(hv), val)) & mk;
-              }
-              tmem_st8(col, ph);
-              tmem_st8(col + 8, pl);
-              uint8_t* blk = pt + (2 * h + (wq >> 1)) * kTileBytes;
-              const uint32_t ch = 4 * (wq & 1) + 2 * q;
-              const uint32_t* pq = pp[h] + 8 * q;
-              *reinterpret_cast<uint4*>(blk + swz128(tl, ch)) = make_uint4(pq[0], pq[1], pq[2], pq[3]);
-              *reinterpret_cast<uint4*>(blk + swz128(tl, ch + 1)) = make_uint4(pq[4], pq[5], pq[6], pq[7]);
-              tmem_st_wait();
-              if (q == 1) fence_proxy_async_smem();   // R / D of the half, for the MMA of dS'
-              else asm volatile("" ::: "memory");
-              tc_fence_before_sync();
-              warp_arrive(&bars->da_ready[s]);
+              for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(pp[h][j]), pk2u(a[2 * j], a[2 * j + 1]), num);
+              tmem_ld_wait();
+              reg_fence16(b);
+              if (h + 1 < NH) tmem_ld16(xrow + (h + 1) * 128 + 32 * wq, a);
+#pragma unroll
+              for (int j = 0; j < 8; ++j) num = fma2(unpack2_bf16(pp[h][8 + j]), pk2u(b[2 * j], b[2 * j + 1]), num);
             }
+            c = -row_total(it, 4, sum2(num));
+          }
+        } else if (it > 0) {
+          wait_all(&bars->p_free, par ^ 1);
+        }
+        if (ok) {
+          if (wq == 0) {
+            cs[tl] = c;
+            sum_dd += c * inv;
+          }
+          // (with eps = 0 a token without an active feature has D = 0; its dA is zero, and so is its dQ_F)
+          scale = inv <= 3.402823466e38f ? inv : 0.f;
+          // ---- dA D (hi + lo, in place) and R / D to shared memory, 16 features at a time
+          // (the mask 1[R > 0], taken from R / D, cuts the packed pairs: a factor would have to be 1 for the smallest R
+          // too, and would let an infinity or NaN of a feature that is off through)
+          const f32x2 c2 = pk2(c, c), minus1 = pk2(-1.f, -1.f);
+          uint32_t a[2][16];
+          tmem_ld16(xrow + 32 * wq, a[0]);
+#pragma unroll
+          for (int h = 0; h < NH; ++h) reg_fence16(pp[h]);
+#pragma unroll
+          for (int s = 0; s < 2 * NH; ++s) {
+            const int h = s >> 1, q = s & 1;
+            const uint32_t col = xrow + h * 128 + 32 * wq + 16 * q;
+            uint32_t(&g)[16] = a[s & 1];
+            tmem_ld_wait();
+            reg_fence16(g);
+            if (s + 1 < 2 * NH) tmem_ld16(xrow + ((s + 1) >> 1) * 128 + 32 * wq + 16 * ((s + 1) & 1), a[(s + 1) & 1]);
+            const float* z = zr + h * 128 + 16 * q;
+            uint32_t ph[8], pl[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              if ((j & 1) == 0) asm volatile("" ::: "memory");
+              const float2 zz = *reinterpret_cast<const float2*>(z + 2 * j);
+              const uint32_t mk = positive_mask_bf16x2(pp[h][8 * q + j]);
+              const f32x2 val = fma2(c2, pk2(zz.x, zz.y), pk2u(g[2 * j], g[2 * j + 1]));
+              const uint32_t hv = pack2_bf16(val);
+              ph[j] = hv & mk;
+              pl[j] = pack2_bf16(fma2(minus1, unpack2_bf16(hv), val)) & mk;
+            }
+            tmem_st8(col, ph);
+            tmem_st8(col + 8, pl);
+            uint8_t* blk = pt + (2 * h + (wq >> 1)) * kTileBytes;
+            const uint32_t ch = 4 * (wq & 1) + 2 * q;
+            const uint32_t* pq = pp[h] + 8 * q;
+            *reinterpret_cast<uint4*>(blk + swz128(tl, ch)) = make_uint4(pq[0], pq[1], pq[2], pq[3]);
+            *reinterpret_cast<uint4*>(blk + swz128(tl, ch + 1)) = make_uint4(pq[4], pq[5], pq[6], pq[7]);
+            tmem_st_wait();
+            if (q == 1) fence_proxy_async_smem();   // R / D of the half, for the MMA of dS'
+            else asm volatile("" ::: "memory");
+            tc_fence_before_sync();
+            warp_arrive(&bars->da_ready[s]);
           }
         }
         ok = named_bar_all(1, kQElem, ok);
         if (!ok) break;   // (all quarters together)
-        // ---- dz' += (R / D)^T c: thread = eight features (a 16-byte chunk) x kDzTok tokens.  (As warp-level MMAs the
-        // same sums waited for the tensor pipe, which is busy here: 2.9 k cycles.)
-        {
-          const uint8_t* blk = pt + (dz_ch >> 3) * kTileBytes;
+      }
+      if constexpr (NH == 1) {
+        if (it + 1 < nt) take_a(it + 1, pp);
+        if (it < 0) continue;
+      }
+      // ---- dz' += (R / D)^T c: thread = eight features (a 16-byte chunk) x kDzTok tokens.  (As warp-level MMAs the
+      // same sums waited for the tensor pipe, which is busy here: 2.9 k cycles.)
+      {
+        const uint8_t* blk = pt + (dz_ch >> 3) * kTileBytes;
 #pragma unroll
-          for (int t = 0; t < kDzTok; t += 4) {
-            const float4 cv = *reinterpret_cast<const float4*>(cs + dz_t0 + t);
-            const float cc[4] = {cv.x, cv.y, cv.z, cv.w};
+        for (int t = 0; t < kDzTok; t += 4) {
+          const float4 cv = *reinterpret_cast<const float4*>(cs + dz_t0 + t);
+          const float cc[4] = {cv.x, cv.y, cv.z, cv.w};
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const uint4 w = *reinterpret_cast<const uint4*>(blk + swz128(dz_t0 + t + i, dz_ch & 7));
-              const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+          for (int i = 0; i < 4; ++i) {
+            const uint4 w = *reinterpret_cast<const uint4*>(blk + swz128(dz_t0 + t + i, dz_ch & 7));
+            const uint32_t u[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                dz[2 * k] = fmaf(__uint_as_float(u[k] << 16), cc[i], dz[2 * k]);
-                dz[2 * k + 1] = fmaf(__uint_as_float(u[k] & 0xFFFF0000u), cc[i], dz[2 * k + 1]);
-              }
+            for (int k = 0; k < 4; ++k) {
+              dz[2 * k] = fmaf(__uint_as_float(u[k] << 16), cc[i], dz[2 * k]);
+              dz[2 * k + 1] = fmaf(__uint_as_float(u[k] & 0xFFFF0000u), cc[i], dz[2 * k + 1]);
             }
           }
         }
-        // ---- dQ_F: 16 columns per thread, times 1 / D, to the staging boxes and out
-        wait_all(&bars->dq_full, par);
-        uint32_t r[16];
-        if (ok) {
-          tmem_ld16(trow + kAccQ + 16 * wq, r);
-          tmem_ld_wait();
-          reg_fence16(r);
-          tc_fence_before_sync();
-        }
-        ok = named_bar_all(1, kQElem, ok);   // the dz' pass has read R / D (and dS' has: its MMAs precede dq_full)
-        if (!ok) break;
-        {
-          uint8_t* box = pt + (wq >> 1) * kTileBytes;
-          // (with eps = 0 a token without an active feature has D = 0; its dA is zero, and so is its dQ_F)
-          const float scale = inv <= 3.402823466e38f ? inv : 0.f;
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<float4*>(box + swz128(tl, 4 * (wq & 1) + q)) =
-                make_float4(__uint_as_float(r[4 * q]) * scale, __uint_as_float(r[4 * q + 1]) * scale,
-                            __uint_as_float(r[4 * q + 2]) * scale, __uint_as_float(r[4 * q + 3]) * scale);
-          fence_proxy_async_smem();
-        }
-        warp_arrive(&bars->staged);
       }
+      // ---- dQ_F: 16 columns per thread, times 1 / D, to the staging boxes and out
+      wait_all(&bars->dq_full, par);
+      uint32_t r[16];
+      if (ok) {
+        tmem_ld16(trow + kAccQ + 16 * wq, r);
+        tmem_ld_wait();
+        reg_fence16(r);
+        tc_fence_before_sync();
+      }
+      ok = named_bar_all(1, kQElem, ok);   // the dz' pass has read R / D (and dS' has: its MMAs precede dq_full)
       if (!ok) break;
+      {
+        uint8_t* box = pt + (wq >> 1) * kTileBytes;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          *reinterpret_cast<float4*>(box + swz128(tl, 4 * (wq & 1) + q)) =
+              make_float4(__uint_as_float(r[4 * q]) * scale, __uint_as_float(r[4 * q + 1]) * scale,
+                          __uint_as_float(r[4 * q + 2]) * scale, __uint_as_float(r[4 * q + 3]) * scale);
+        fence_proxy_async_smem();
+      }
+      warp_arrive(&bars->staged);
+      if (!last) continue;
       // ---- end of the segment: partial dS', dz' (every MMA of the segment has completed)
-      if (et == 0 && gt < g1) mbar_arrive(&bars->s_free);
       {
         float* dst = scratch + (et / kChunks) * m + 8 * dz_ch;
         *reinterpret_cast<float4*>(dst) = make_float4(dz[0], dz[1], dz[2], dz[3]);
         *reinterpret_cast<float4*>(dst + 4) = make_float4(dz[4], dz[5], dz[6], dz[7]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) dz[i] = 0.f;
       }
       named_bar_sync(1, kQElem);
-      const size_t pidx = (size_t)blockIdx.x + slab;
+      const size_t pidx = (size_t)blockIdx.x + now;
       tc_fence_after_sync();
       if (et < m) {
         float s = 0.f;
@@ -915,14 +963,14 @@ k_tc_bwd_qside(const __grid_constant__ CUtensorMap map_qf, const __grid_constant
 #pragma unroll
       for (int ii = 0; ii < NH; ++ii) {
         const int i = wq * NH + ii, h = i >> 2, cc = i & 3;   // 16 columns of one half
-        uint32_t r[16];
-        tmem_ld16(trow + kAccS + h * 64 + 16 * cc, r);
+        uint32_t r16[16];
+        tmem_ld16(trow + kAccS + h * 64 + 16 * cc, r16);
         tmem_ld_wait();
-        reg_fence16(r);
+        reg_fence16(r16);
         float* dst = dspart + (pidx * m + h * 128 + tl) * kD + 16 * cc;
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          *reinterpret_cast<uint4*>(dst + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+          *reinterpret_cast<uint4*>(dst + 4 * q) = make_uint4(r16[4 * q], r16[4 * q + 1], r16[4 * q + 2], r16[4 * q + 3]);
       }
       tc_fence_before_sync();
       named_bar_sync(1, kQElem);   // the scratch and z' may be written again
