@@ -70,6 +70,7 @@ static wersa_status make_pool_plan(const wersa_config& c, Plan* p) {
   p->qchunks = ceil_div(4 * p->sms, p->slabs);
   if (p->qchunks > ceil_div(n, 128)) p->qchunks = ceil_div(n, 128);
   if (p->qchunks < 1) p->qchunks = 1;
+  if (p->qchunks > 16 && 16 * p->slabs * 4 >= 3 * p->sms && n <= 16 * 1024) p->qchunks = 16;
   p->qchunk_rows = ceil_div(ceil_div(n, p->qchunks), 32) * 32;
   p->qchunks = ceil_div(n, p->qchunk_rows);
   return WERSA_OK;

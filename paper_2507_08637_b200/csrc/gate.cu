@@ -1,6 +1,7 @@
 // Mean-pooled query, content-adaptive gate (Eqs. 1-3 of the WERSA paper) and its backward pass.
 #include <mutex>
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "gate_backward.cuh"
 
@@ -17,11 +18,11 @@ constexpr int kMaxDevices = 64;
 float* g_static_scratch_addr[kMaxDevices] = {nullptr};
 std::mutex g_static_scratch_mutex;
 
-// Finish of one slab by the last CTA of that slab to arrive (256 threads): qbar = sum of the chunk
-// partials in chunk order / n (Eq. 1), the head's logits u = gate_w[h]^T qbar (Eq. 2) and, for the
+// Finish of one slab by one CTA (256 threads): qbar = sum of the chunk partials load(chunk, column) in chunk order / n (Eq. 1), the head's logits u = gate_w[h]^T qbar (Eq. 2) and, for the
 // per-head gate, sigmoid(u + gate_b[h]) and f = sigmoid * omega (Eq. 3).  For the batch-wide gate the
 // bias-free logits are parked in f for batch_gate.
-__device__ __forceinline__ void slab_gate(const float* __restrict__ qpart, int qchunks, int slab, int H, int n, int L1,
+template <typename Load>
+__device__ __forceinline__ void slab_gate(Load&& load, int qchunks, int slab, int H, int n, int L1,
                                           int per_head, const float* __restrict__ gate_w,
                                           const float* __restrict__ gate_b, const float* __restrict__ omega,
                                           float* __restrict__ qbar, float* __restrict__ sg, float* __restrict__ f,
@@ -41,17 +42,15 @@ __device__ __forceinline__ void slab_gate(const float* __restrict__ qpart, int q
     if (omega != nullptr) om = omega[i];
   }
   float s = 0.f;
-  const float* src = qpart + (size_t)slab * qchunks * kD + c;
   int k = part;
   for (; k + 12 < qchunks; k += 16) {
-    const float v0 = __ldcg(src + (size_t)k * kD), v1 = __ldcg(src + (size_t)(k + 4) * kD);
-    const float v2 = __ldcg(src + (size_t)(k + 8) * kD), v3 = __ldcg(src + (size_t)(k + 12) * kD);
+    const float v0 = load(k, c), v1 = load(k + 4, c), v2 = load(k + 8, c), v3 = load(k + 12, c);
     s += (v0 + v1) + (v2 + v3);
   }
   {
     float v[3];   // at most three left
 #pragma unroll
-    for (int j = 0; j < 3; ++j) v[j] = k + 4 * j < qchunks ? __ldcg(src + (size_t)(k + 4 * j) * kD) : 0.f;
+    for (int j = 0; j < 3; ++j) v[j] = k + 4 * j < qchunks ? load(k + 4 * j, c) : 0.f;
 #pragma unroll
     for (int j = 0; j < 3; ++j) s += v[j];
   }
@@ -101,9 +100,10 @@ __device__ __forceinline__ void batch_gate(int b, int H, int L1, const float* __
 // Mean pool and gate in one launch.  grid (qchunks, slabs [+ 1]), block 256.
 // Rows y < slabs: partial column sums of one row chunk of one slab of Q -- thread (cg = tid & 7,
 // rl = tid >> 3) owns 8 consecutive columns and every 32nd row, loads 16 bytes (bf16) / 32 bytes
-// (fp32) per row, four rows in flight, with the streaming cache hint (Q is read once here).  The CTA that finds it is the last of its slab to finish
-// (a counter per slab) then runs slab_gate, and for the batch-wide gate the last slab of a batch
-// element (a counter per batch element) runs batch_gate; sums are taken in a fixed order, so the
+// (fp32) per row, four rows in flight, with the streaming cache hint (Q is read once here).  kCluster: the chunks of a slab are a
+// cluster, whose first block gets the others' sums into its shared memory and runs slab_gate.  Otherwise the CTA that finds it is the
+// last of its slab to finish (a counter per slab) does, which takes two fences, an atomic and two more trips to the L2 (1 x 1024 fp32 4.3 us of a forward,
+// 3.2 as a cluster; 5 x 3 x 1777 9.5 and 8.2; 8 x 8 x 4096 12.2 and 10.6).  For the batch-wide gate the last slab of a batch element (a counter per batch element) runs batch_gate; sums are taken in a fixed order, so the
 // result does not depend on which CTA comes last.  The counters start at zero and are left at zero.
 // Row y == slabs (only of bf16 tensors, with W or seen): bf16 transpose Wt (m x 64) of W (64 x m) for the tensor-core kernels;
 // seen is cleared there.
@@ -111,7 +111,7 @@ __device__ __forceinline__ void batch_gate(int b, int H, int L1, const float* __
 // dcols / 8 threads share a row, 256 / (dcols / 8) rows are in flight per pass, and the partial sums, q-bar
 // and W^T come out 64 wide with zeros in the columns past dcols.  fp32 tensors keep the 64-wide assignment
 // (eight threads a row, those past dcols idle): their sums have the bits of the zero-padded problem.
-template <typename T, bool kFull>
+template <typename T, bool kFull, bool kCluster>
 __global__ void __launch_bounds__(256) k_qmean_gate(const T* __restrict__ Q, float* __restrict__ qpart, int n,
                                                     int chunk_rows, int slabs, int H, int L1, int per_head,
                                                     const float* __restrict__ gate_w, const float* __restrict__ gate_b,
@@ -150,6 +150,7 @@ __global__ void __launch_bounds__(256) k_qmean_gate(const T* __restrict__ Q, flo
     }
     return;
   }
+  if constexpr (kCluster) cluster_arrive();
   const int chunk = blockIdx.x, slab = blockIdx.y;
   const int cgs = kFull || sizeof(T) == 4 ? 8 : dcols >> 3;   // threads across a row
   const int rp = kFull ? 32 : 256 / cgs;       // rows per pass
@@ -187,22 +188,40 @@ __global__ void __launch_bounds__(256) k_qmean_gate(const T* __restrict__ Q, flo
     for (int j = 0; j < 8; ++j) red[rl * (dcols + 1) + cg * 8 + j] = acc[j];
   }
   __syncthreads();
+  float total = 0.f;   // kCluster
   if (threadIdx.x < kD) {
     float s = 0.f;
     if ((int)threadIdx.x < dcols) {
 #pragma unroll 8
       for (int i = 0; i < rp; ++i) s += red[i * (dcols + 1) + threadIdx.x];   // fixed order
     }
-    qpart[((size_t)slab * gridDim.x + chunk) * kD + threadIdx.x] = s;
-    __threadfence();
+    if constexpr (!kCluster) {
+      qpart[((size_t)slab * gridDim.x + chunk) * kD + threadIdx.x] = s;
+      __threadfence();
+    } else {
+      total = s;
+    }
   }
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&slab_count[slab], 1) == (int)gridDim.x - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  slab_gate(qpart, gridDim.x, slab, H, n, L1, per_head, gate_w, gate_b, omega, qbar, sg, f, red4, qs, dcols);
-  if (threadIdx.x == 0) slab_count[slab] = 0;
+  if constexpr (kCluster) {
+    __shared__ float shares[kMaxCluster][kD];
+    cluster_wait();   // (the first block has begun)
+    if (threadIdx.x < kD) peer_store(peer_addr(shared_addr(&shares[chunk][threadIdx.x]), 0), total);
+    cluster_release();
+    cluster_acquire();
+    if (chunk != 0) return;
+    slab_gate([&](int k, int c) { return shares[k][c]; }, gridDim.x, slab, H, n, L1, per_head, gate_w, gate_b, omega, qbar, sg, f, red4,
+              qs, dcols);
+  } else {
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&slab_count[slab], 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const float* src = qpart + (size_t)slab * gridDim.x * kD;
+    slab_gate([&](int k, int c) { return __ldcg(src + (size_t)k * kD + c); }, gridDim.x, slab, H, n, L1, per_head, gate_w, gate_b, omega,
+              qbar, sg, f, red4, qs, dcols);
+    if (threadIdx.x == 0) slab_count[slab] = 0;
+  }
   if (per_head) return;
   __threadfence();
   __syncthreads();
@@ -233,7 +252,8 @@ __global__ void __launch_bounds__(256) k_gate_from_sums(const float* __restrict_
   wait_for_stream_predecessor();   // (launched as a programmatic dependent: see launch_after)
   __shared__ float red4[4][kD];
   __shared__ float qs[kD];
-  slab_gate(qsum, 1, blockIdx.x, H, n_total, L1, per_head, gate_w, gate_b, omega, qbar, sg, f, red4, qs, dcols);
+  const float* src = qsum + (size_t)blockIdx.x * kD;
+  slab_gate([&](int, int c) { return __ldcg(src + c); }, 1, blockIdx.x, H, n_total, L1, per_head, gate_w, gate_b, omega, qbar, sg, f, red4, qs, dcols);
 }
 __global__ void __launch_bounds__(32) k_batch_gate(int H, int L1, const float* __restrict__ gate_b,
                                                    const float* __restrict__ omega, float* __restrict__ sg,
@@ -296,9 +316,15 @@ __global__ void __launch_bounds__(kD) k_sum_floats(const float* __restrict__ x, 
 // (launched as a programmatic dependent: see launch_after; the pass that writes dQ may be placed ahead of this kernel's wait, and
 // unless it is the first one of its pass the gate weights are fetched ahead of it)
 template <int kParts>
-__global__ void __launch_bounds__(64 * kParts) k_gate_backward(const float* df, const GateBwdArgs args, bool first) {
+__global__ void __launch_bounds__(64 * kParts) k_gate_backward(
+    const float* __restrict__ df, const float* __restrict__ sg, const float* __restrict__ qbar, const float* __restrict__ gate_w,
+    const float* __restrict__ omega, const float* __restrict__ sumdD, int n_sumdD, const float* __restrict__ beta, float eps,
+    float bw_floor, int m, int B, int H, int dcols, int L1, int per_head, float* __restrict__ dbeta, float* __restrict__ dgate_w,
+    float* __restrict__ dgate_b, float* __restrict__ domega, float* __restrict__ dqbar, bool first) {
   if (first) wait_for_stream_predecessor();
   let_stream_successor_start();
+  const GateBwdArgs args = {sg, qbar, gate_w, omega, sumdD, beta, n_sumdD, eps, bw_floor, m, B, H, dcols, L1, per_head,
+                            dbeta, dgate_w, dgate_b, domega, dqbar};
   gate_backward_cta<kParts>(blockIdx.x, GivenDf{df}, args, []() { wait_for_stream_predecessor(); });
 }
 
@@ -308,34 +334,33 @@ __global__ void __launch_bounds__(64 * kParts) k_gate_backward(const float* df, 
 static cudaError_t launch_qmean_gate_impl(const Plan& p, const void* Q, float* qpart, const float* gate_w,
                                           const float* gate_b, const float* omega, float* qbar, float* sg, float* f,
                                           int* counters, const void* W, __nv_bfloat16* Wt, int cols,
-                                          int* seen, cudaStream_t st) {
+                                          int* seen, bool cluster, cudaStream_t st) {
   dim3 grid(p.qchunks, p.slabs + (W != nullptr || (p.bf16 && seen != nullptr) ? 1 : 0));
   int* slab_count = counters;
   int* batch_count = counters + p.slabs;
   cudaError_t launch_err = cudaSuccess;
-  auto launch = [&](auto kernel, auto* q) {
-    // Launched as a programmatic dependent of whatever precedes it in the stream: the kernel's first
-    // instruction waits for that work to complete, so ordering and visibility are those of a plain launch,
-    // but its CTAs are already placed when the wait ends (2 us per forward in a sequence of steps).
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = grid;
-    lc.blockDim = dim3(256);
-    lc.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = attr;
-    lc.numAttrs = 1;
-    launch_err = cudaLaunchKernelEx(&lc, kernel, q, qpart, p.cfg.seq_len, p.qchunk_rows, p.slabs, p.cfg.heads, p.L1,
-                                    p.cfg.gate_per_head, gate_w, gate_b, omega, qbar, sg, f, slab_count, batch_count,
-                                    (const __nv_bfloat16*)W, Wt, p.cfg.features, cols, seen);
+  // Launched as a programmatic dependent of whatever precedes it in the stream: the kernel's first instruction waits for that
+  // work to complete, so ordering and visibility are those of a plain launch, but its CTAs are already placed when the wait
+  // ends (2 us per forward in a sequence of steps).
+  auto launch = [&](auto kernel, auto clustered, auto* q) {
+    auto go = [&](auto start) {
+      launch_err = start(q, qpart, p.cfg.seq_len, p.qchunk_rows, p.slabs, p.cfg.heads, p.L1, p.cfg.gate_per_head, gate_w, gate_b, omega,
+                         qbar, sg, f, slab_count, batch_count, (const __nv_bfloat16*)W, Wt, p.cfg.features, cols, seen);
+    };
+    if (cluster && prepare_cluster(clustered, 0, p.qchunks) == cudaSuccess) {
+      go([&](auto... args) { return launch_cluster(clustered, grid, dim3(256), 0, st, args...); });
+      if (launch_err == cudaSuccess) return;
+      cudaGetLastError();   // (a part of a GPU may have no room for a cluster of more than eight)
+    }
+    go([&](auto... args) { return launch_after(kernel, grid, dim3(256), 0, st, args...); });
   };
+  using bf = __nv_bfloat16;
   if (p.bf16) {
-    if (cols == kD) launch(k_qmean_gate<__nv_bfloat16, true>, (const __nv_bfloat16*)Q);
-    else launch(k_qmean_gate<__nv_bfloat16, false>, (const __nv_bfloat16*)Q);
+    if (cols == kD) launch(k_qmean_gate<bf, true, false>, k_qmean_gate<bf, true, true>, (const bf*)Q);
+    else launch(k_qmean_gate<bf, false, false>, k_qmean_gate<bf, false, true>, (const bf*)Q);
   } else {
-    if (cols == kD) launch(k_qmean_gate<float, true>, (const float*)Q);
-    else launch(k_qmean_gate<float, false>, (const float*)Q);
+    if (cols == kD) launch(k_qmean_gate<float, true, false>, k_qmean_gate<float, true, true>, (const float*)Q);
+    else launch(k_qmean_gate<float, false, false>, k_qmean_gate<float, false, true>, (const float*)Q);
   }
   return launch_err != cudaSuccess ? launch_err : cudaGetLastError();
 }
@@ -345,7 +370,7 @@ cudaError_t launch_qmean_gate(const Plan& p, const Ws& w, const void* Q, const f
                               int* launches) {
   *launches += 1;
   return launch_qmean_gate_impl(p, Q, w.qpart, gate_w, gate_b, omega, w.qbar, w.sg, w.f, w.counters, W, w.Wt, cols,
-                                p.use_x ? w.seen : nullptr, st);
+                                p.use_x ? w.seen : nullptr, p.qchunks <= kMaxCluster, st);
 }
 
 cudaError_t launch_shard_qsum(const Plan& p, const Ws& w, float* qsum, cudaStream_t st, int* launches) {
@@ -398,7 +423,7 @@ cudaError_t launch_qmean_gate_static(const Plan& p, float* scratch, const void* 
   int* counters = reinterpret_cast<int*>(scratch + (kStaticScratchFloats - kStaticCounterInts));
   cudaError_t err = cudaMemsetAsync(counters, 0, sizeof(int) * ((size_t)p.slabs + (size_t)p.cfg.batch), st);
   if (err != cudaSuccess) return err;
-  return launch_qmean_gate_impl(p, Q, qpart, gate_w, gate_b, omega, qbar, sg, f, counters, nullptr, nullptr, kD, nullptr, st);
+  return launch_qmean_gate_impl(p, Q, qpart, gate_w, gate_b, omega, qbar, sg, f, counters, nullptr, nullptr, kD, nullptr, false, st);
 }
 
 size_t static_scratch_floats_needed(const Plan& p) {
@@ -412,7 +437,11 @@ static GateBwdArgs gate_args(const Plan& p, const Ws& w, const float* beta, cons
           p.cfg.head_dim, p.L1, p.cfg.gate_per_head, dbeta, dgate_w, dgate_b, domega, dqbar};
 }
 static void gate_backward_kernel(const Plan& p, const float* df, const GateBwdArgs& args, bool first, cudaStream_t st) {
-  auto go = [&](auto kernel, int threads) { launch_after(kernel, dim3(p.cfg.heads + 2), dim3(threads), 0, st, df, args, first); };
+  auto go = [&](auto kernel, int threads) {
+    launch_after(kernel, dim3(p.cfg.heads + 2), dim3(threads), 0, st, df, args.sg, args.qbar, args.gate_w, args.omega, args.sumdD,
+                 args.n_sumdD, args.beta, args.eps, args.bw_floor, args.m, args.B, args.H, args.dcols, args.L1, args.per_head,
+                 args.dbeta, args.dgate_w, args.dgate_b, args.domega, args.dqbar, first);
+  };
   if (p.cfg.batch <= 28) go(k_gate_backward<4>, 256);
   else go(k_gate_backward<16>, 1024);
 }

@@ -209,20 +209,26 @@ __global__ void __launch_bounds__(256, 4) k_haar_filter(const Tin* __restrict__ 
 
 // The last pass of a backward with gate weights: dQ = T_f(dQ_F) + d q-bar / n on every row, as k_haar_filter with a row vector, which
 // is worked out here: every CTA of a slab takes df (16 numbers), du and the slab's d q-bar (64) for itself while its rows are on
-// their way, and the first H + 2 CTAs do what k_gate_backward does for the parameters.  All of that is latency, some 7 us of
-// it on 2 x 4 x 4096 whether in one launch or three; what one launch saves is their placement and the host's 2 us for each.  Training
-// steps: 2 x 2 x 256, d = 16, m = 256 bf16 56.1 -> 53 us (with the forward's one launch 46.6); 1 x 3 x 440, m = 256 fp32 70.4 -> 67.1; 5 x 3 x
-// 1777, m = 256 90.4 -> 89.3; 2 x 4 x 4096, d = 32, fp32 107.7 -> 106.7; from 16 x 12 x 1024 on the same.
+// their way, and the first H + 2 CTAs do what k_gate_backward does for the parameters.  The three launches before were latency from
+// end to end, as most of this one is: behind the pass over K and Q 8.4 us and now 5.7 on 5 x 3 x 1777, 7.2 and 5.9 on 2 x 4 x 4096, d = 32,
+// 16.5 and 11.9 on 16 x 12 x 1024 (25 MB of dQ_F in, half of it out); and the host has two launches less, 2 us each: training step of 2 x 2 x
+// 256, d = 16, m = 256 56.1 -> 53 us.
 // kSum: df from the partials of `blocks` CTAs per slab and tensor, else from the reduction's result.
 // grid: H + 2 + slabs * blocks.
 template <bool kFull, typename Tout, bool kSum>
 __global__ void __launch_bounds__(256, 4) k_haar_dq(const float* __restrict__ G, const float* __restrict__ f, Tout* __restrict__ dQ,
-                                                    int n, int d_arg, int L, int slabs, int blocks, float inv_n, const float* df_in,
-                                                    const GateBwdArgs args) {
+                                                    int n, int d_arg, int L, int slabs, int blocks, float inv_n,
+                                                    const float* __restrict__ df_in, const float* __restrict__ sg,
+                                                    const float* __restrict__ qbar, const float* __restrict__ gate_w,
+                                                    const float* __restrict__ omega, const float* __restrict__ sumdD, int n_sumdD,
+                                                    const float* __restrict__ beta, float eps, float bw_floor, int m, int B, int H,
+                                                    int per_head, float* __restrict__ dbeta, float* __restrict__ dgate_w,
+                                                    float* __restrict__ dgate_b, float* __restrict__ domega) {
   // (launched as a programmatic dependent: see launch_after)
-  const int H = args.H;
   if ((int)blockIdx.x < H + 2) {
     auto wait = []() { wait_for_stream_predecessor(); };
+    const GateBwdArgs args = {sg, qbar, gate_w, omega, sumdD, beta, n_sumdD, eps, bw_floor, m, B, H, kFull ? kD : d_arg, L + 1, per_head,
+                              dbeta, dgate_w, dgate_b, domega, nullptr};
     if constexpr (kSum) gate_backward_cta<4>(blockIdx.x, SummedDf{df_in, slabs, blocks, L}, args, wait);
     else gate_backward_cta<4>(blockIdx.x, GivenDf{df_in}, args, wait);
     return;
@@ -255,12 +261,12 @@ __global__ void __launch_bounds__(256, 4) k_haar_dq(const float* __restrict__ G,
   const int h = slab % H;
   for (int e = tid; e < d * (L + 1); e += 256) {
     const int c = e / (L + 1);
-    gws[e - c * (L + 1)][c] = args.gate_w[(size_t)h * d * (L + 1) + e];
+    gws[e - c * (L + 1)][c] = gate_w[(size_t)h * d * (L + 1) + e];
   }
   float slope = 0.f;
   if (tid <= L) {
-    const float sgm = args.sg[(size_t)slab * (L + 1) + tid];
-    slope = args.omega[tid] * sgm * (1.f - sgm) * inv_n;
+    const float sgm = sg[(size_t)slab * (L + 1) + tid];
+    slope = omega[tid] * sgm * (1.f - sgm) * inv_n;
   }
   const LevelCoef k = level_coef(f + (size_t)slab * (L + 1), L);
   float hi[4], s5[4];
@@ -276,7 +282,7 @@ __global__ void __launch_bounds__(256, 4) k_haar_dq(const float* __restrict__ G,
   {
     // df: slot j by sixteen threads; the gate of a batch element sums over its heads
     const int j = tid & (kBandVals - 1), pt = tid >> 4;
-    const int first = args.per_head ? slab : slab - h, count = args.per_head ? 1 : H;
+    const int first = per_head ? slab : slab - h, count = per_head ? 1 : H;
     float s = 0.f;
     if (j <= L) {
       if constexpr (kSum) {
@@ -872,10 +878,11 @@ cudaError_t launch_haar_filter_addvec(const Plan& p, const float* G, const float
   return err != cudaSuccess ? err : cudaGetLastError();
 }
 
-// The gate's CTAs take rounds of 28 batch elements after one another, and beyond four of them k_gate_backward with its 1024 threads
-// is the faster one; df is summed in place while a CTA reads at most some 40 partials a slot for its own slab (or batch element) and the
-// one of d omega 2048 for all of them.
-bool haar_dq_takes_gate(const Plan& p) { return p.cfg.batch <= 112; }
+// The gate's CTAs here have 256 threads: one round of 28 batch elements, and sixteen slabs a thread of d omega.  Beyond that
+// k_gate_backward with its 1024 threads is the faster one (88 x 372, m = 256 a training step 103.6 us, 107.4 with four rounds
+// here; 85 x 12 x 202, the gate of a batch element 432 and 458).  df is summed in place while a CTA reads at most some 40 partials a
+// slot for its own slab (or batch element) and the one of d omega 2048 for all of them.
+bool haar_dq_takes_gate(const Plan& p) { return p.cfg.batch <= 28 && p.slabs <= 256; }
 bool haar_dq_sums_bands(const Plan& p) {
   const long long blocks = haar_band_blocks(p, p.cfg.head_dim);
   return blocks * (p.cfg.gate_per_head ? 1 : p.cfg.heads) <= 48 && blocks * p.slabs <= 2048;
@@ -887,7 +894,8 @@ cudaError_t launch_haar_dq(const Plan& p, const Ws& w, const GateBwdArgs& args, 
   using bf = __nv_bfloat16;
   auto go = [&](auto kernel, auto* out) {
     return launch_after(kernel, grid, dim3(256), 0, st, (const float*)w.dQF, (const float*)w.f, out, n, d, L, p.slabs, blocks,
-                        1.f / (float)n, df, args);
+                        1.f / (float)n, df, args.sg, args.qbar, args.gate_w, args.omega, args.sumdD, args.n_sumdD, args.beta, args.eps,
+                        args.bw_floor, args.m, args.B, args.H, args.per_head, args.dbeta, args.dgate_w, args.dgate_b, args.domega);
   };
   cudaError_t err;
   const bool sum = haar_dq_sums_bands(p);

@@ -18,6 +18,7 @@
 // tokens and T features, likewise.
 #include <atomic>
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "tc_common.cuh"
 
@@ -25,38 +26,6 @@ namespace wersa {
 namespace {
 using tc::pack_bf16x2;
 using tc::relu_pack_bf16x2;
-
-constexpr int kMaxCluster = 16;   // blocks of a cluster (more than 8 are opt-in)
-
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// The two halves of a barrier of all threads of the cluster's blocks: what was written to shared memory before is visible behind.
-__device__ __forceinline__ void cluster_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// The same, nothing released: the blocks of the cluster have begun (their shared memory may be written to).
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t shared_addr(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-// The same place in the shared memory of block `rank`.  (Blocks only write to one another and read their own memory, and what is
-// more than a few hundred bytes goes as bulk copies.  The sums over S' of 3 x 130, m = 256 by reads of the peers' memory, 16 bytes a
-// lane, a row's side by side: 17 us a forward, row by row 26; by copies 13.  By 8-byte stores from the accumulators 14.)
-__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void peer_store2(uint32_t addr, float2 v) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
-}
-// `bytes` (a multiple of 16, not 0) of this block's shared memory to another block's, reported to a barrier over there.  What was
-// written here has to be fenced for the copy engine; the block may not end before the copy has (a barrier of the cluster).
-__device__ __forceinline__ void peer_copy(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src), "r"(bytes),
-               "r"(bar) : "memory");
-}
 
 // Two neighbouring columns of a row (packed as they were loaded until they are used).
 __device__ __forceinline__ float2 pair(uint32_t u) { return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u)); }
@@ -558,47 +527,6 @@ k_small_forward(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __rest
     if (c == 0) z[(size_t)slab * m + f0g + row] = sums[r * kSumPitch + 8 * kTiles];
   }
   if (blocks > 1) cluster_wait();   // (the others have what this block had for them)
-}
-
-template <typename K> cudaError_t prepare_cluster(K kernel, size_t smem, int blocks) {
-  const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  return err != cudaSuccess || blocks <= 8 ? err : cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-}
-// How many clusters of `blocks` the device holds at once (0: none, or no device).
-template <typename K> int clusters_at_once(K kernel, int threads, size_t smem, int blocks) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = blocks;
-  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int clusters = 0;
-  if (prepare_cluster(kernel, smem, blocks) == cudaSuccess && cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess)
-    return clusters;
-  cudaGetLastError();   // a failed query leaves no sticky error behind
-  return 0;
-}
-// A launch like launch_after's whose grid's first dimension is one cluster.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = grid.x;
-  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
 template <int V> struct Int { static constexpr int value = V; };
