@@ -61,8 +61,8 @@ enum {
                                   on them (see wersa_uses_tensor_cores)                  */
   WERSA_FLAG_FORWARD_ONLY = 2, /* the context will never run wersa_backward: its workspace
                                   omits the gradient scratch buffers                     */
-  WERSA_FLAG_STEPWISE = 4      /* bf16: a launch per step of the forward for short sequences
-                                  too, where it would otherwise be one launch            */
+  WERSA_FLAG_STEPWISE = 4      /* a launch per step of the forward for short sequences too,
+                                  where several would otherwise be one launch            */
 };
 
 typedef struct wersa_config {

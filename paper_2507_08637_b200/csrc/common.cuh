@@ -43,6 +43,7 @@ struct Plan {
   bool use_xb;        // fp32 backward on them too: chunks and tiles of its gradient kernels, CTAs of its first pass
   int xbchunks, xbchunk_tiles, xprep;
   int small_tokens, small_blocks;   // bf16 forward in one launch (small.cu): tokens of a thread block, blocks of a slab; 0: not
+  int filter_tokens;  // FFMA forward: mean pool, gate and filter in one launch (small.cu): tokens of a thread block; 0: in two
   int bctas;          // tcgen05 backward: CTAs that share the list of all 128-token tiles
   // workspace offsets (bytes)
   size_t off_status, off_counters, status_bytes, off_qpart, off_qbar, off_sg, off_f, off_spart, off_zpart, off_S, off_z,
@@ -112,6 +113,8 @@ cudaError_t launch_qmean_gate_static(const Plan& p, float* scratch, const void* 
 
 // ---- haar.cu -------------------------------------------------------------------------------
 // d: columns of the tensors as stored (a multiple of 8, at most 64).  in_kind/out_kind: 0 = float, 1 = bf16 (float input: float output).
+// Whether the FFMA key side may be placed early behind a filter of `ctas` CTAs.
+bool place_key_side_early(const Plan& p, unsigned ctas);
 // XF = T_f(X), and with X2 also XF2 = T_f(X2) in the same launch.
 cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const float* f, void* XF, const void* X2,
                                void* XF2, int out_kind, int d, bool inputs_ready, cudaStream_t st, int* launches);
@@ -184,7 +187,10 @@ cudaError_t launch_small_forward(const Plan& p, const Ws& w, const void* Q, cons
                                  const float* beta, const float* gate_w, const float* gate_b, const float* omega, void* O,
                                  cudaStream_t st, int* launches);
 
-// Decides p->small_tokens and p->small_blocks (asks the device, which is current).
+// Mean pool, gate, and w.QF = T_f(Q), w.KF = T_f(K), in one launch (p.filter_tokens).
+cudaError_t launch_small_filter(const Plan& p, const Ws& w, const void* Q, const void* K, const float* gate_w, const float* gate_b,
+                                const float* omega, cudaStream_t st, int* launches);
+// Decides p->small_tokens, p->small_blocks and p->filter_tokens (asks the device, which is current).
 void choose_small_forward(Plan* p);
 
 // ---- tc_bwd.cu -----------------------------------------------------------------------------

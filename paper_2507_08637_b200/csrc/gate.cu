@@ -101,10 +101,11 @@ __device__ __forceinline__ void batch_gate(int b, int H, int L1, const float* __
 // Rows y < slabs: partial column sums of one row chunk of one slab of Q -- thread (cg = tid & 7,
 // rl = tid >> 3) owns 8 consecutive columns and every 32nd row, loads 16 bytes (bf16) / 32 bytes
 // (fp32) per row, four rows in flight, with the streaming cache hint (Q is read once here).  kCluster: the chunks of a slab are a
-// cluster, whose first block gets the others' sums into its shared memory and runs slab_gate.  Otherwise the CTA that finds it is the
-// last of its slab to finish (a counter per slab) does, which takes two fences, an atomic and two more trips to the L2 (1 x 1024 fp32 4.3 us of a forward,
-// 3.2 as a cluster; 5 x 3 x 1777 9.5 and 8.2; 8 x 8 x 4096 12.2 and 10.6).  For the batch-wide gate the last slab of a batch element (a counter per batch element) runs batch_gate; sums are taken in a fixed order, so the
-// result does not depend on which CTA comes last.  The counters start at zero and are left at zero.
+// cluster, whose first block gets the others' sums into its shared memory and runs slab_gate.  Otherwise the CTA that finds it is
+// the last of its slab to finish (a counter per slab) does, which takes two fences, an atomic and two more trips to the L2 (1 x 1024
+// fp32 4.3 us of a forward, 3.2 as a cluster; 5 x 3 x 1777 9.5 and 8.2; 8 x 8 x 4096 12.2 and 10.6).  For the batch-wide gate the last
+// slab of a batch element (a counter per batch element) runs batch_gate; sums are taken in a fixed order, so the result does not
+// depend on which CTA comes last.  The counters start at zero and are left at zero.
 // Row y == slabs (only of bf16 tensors, with W or seen): bf16 transpose Wt (m x 64) of W (64 x m) for the tensor-core kernels;
 // seen is cleared there.
 // kFull = false: Q has dcols < 64 columns (a multiple of 8), gate_w dcols rows per head and W dcols rows;

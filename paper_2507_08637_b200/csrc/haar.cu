@@ -809,6 +809,16 @@ int haar_band_blocks(const Plan& p, int d) { return col_blocks<32>(p.htiles, d);
   if (d == kD) { constexpr bool kFull = true; __VA_ARGS__ } \
   else { constexpr bool kFull = false; __VA_ARGS__ }
 
+// The FFMA key side behind a filter: not placed early where several of its small tiles' CTAs come to share an SM and the
+// filter's grid covers more than a third of the SMs: they gather on the others.  Forwards, placed early and not: 80 x 130, d = 32, m = 64
+// 38.3 and 31.0 us; 40 x 200 30.0 and 27.2; 4 x 1024, d = 64 28.9 and 25.2; 10 x 1344 49.6 and 41.9; 16 x 500, m = 128 47.7 and
+// 42.7; 30 x 130, d = 16 24.6 and 22.0.  One CTA an SM, full tiles or a small grid of the filter: 1 x 1024, m = 64 21.1 and
+// 22.5; 64 x 1024 87.8 and 89.7; 4 x 700, m = 256 38.4 and 39.6; 12 x 256, d = 32, m = 128 (24 CTAs here) 23.5 and 24.6; 20 x
+// 200, m = 64 (40) 21.6 and 21.7.
+bool place_key_side_early(const Plan& p, unsigned ctas) {
+  return !(p.simt_small && p.cfg.features < 256 && (long long)p.schunks * p.slabs > p.sms && 3 * ctas > (unsigned)p.sms);
+}
+
 // X2 / XF2: a second tensor of the same shape in the same launch (or null).
 cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const float* f, void* XF, const void* X2,
                                void* XF2, int out_kind, int d, bool inputs_ready, cudaStream_t st, int* launches) {
@@ -816,17 +826,10 @@ cudaError_t launch_haar_filter(const Plan& p, const void* X, int in_kind, const 
   const dim3 grid(col_blocks<32>(p.htiles, d), p.slabs, z), grid_bf(col_blocks<64>(p.htiles, d), p.slabs, z);
   const int n = p.cfg.seq_len, L = p.cfg.levels;
   using bf = __nv_bfloat16;
-  // In a pass the FFMA key side follows.  Not placed early where several of its small tiles' CTAs come to share an SM and this
-  // grid covers more than a third of the SMs: they gather on the others.  Forwards, placed early and not: 80 x 130, d = 32, m = 64
-  // 38.3 and 31.0 us; 40 x 200 30.0 and 27.2; 4 x 1024, d = 64 28.9 and 25.2; 10 x 1344 49.6 and 41.9; 16 x 500, m = 128 47.7 and
-  // 42.7; 30 x 130, d = 16 24.6 and 22.0.  One CTA an SM, full tiles or a small grid of this kernel: 1 x 1024, m = 64 21.1 and
-  // 22.5; 64 x 1024 87.8 and 89.7; 4 x 700, m = 256 38.4 and 39.6; 12 x 256, d = 32, m = 128 (24 CTAs here) 23.5 and 24.6; 20 x
-  // 200, m = 64 (40) 21.6 and 21.7.
   const unsigned ctas = in_kind == 1 ? grid_bf.x * grid_bf.y * z : grid.x * grid.y * z;
-  const bool gathers = p.simt_small && p.cfg.features < 256 && (long long)p.schunks * p.slabs > p.sms && 3 * ctas > (unsigned)p.sms;
   // (without inputs_ready it is a pass of its own: 1 x 8 x 131072, bf16, call after call 51.1 us before it let the next one be
   // placed early, 48.2 to 48.8 since)
-  const bool place_next = !inputs_ready || !gathers;
+  const bool place_next = !inputs_ready || place_key_side_early(p, ctas);
   cudaError_t err;
   WERSA_FULL({
     if (in_kind == 1 && out_kind == 1)

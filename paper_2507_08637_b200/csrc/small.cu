@@ -27,7 +27,10 @@ namespace {
 using tc::pack_bf16x2;
 using tc::relu_pack_bf16x2;
 
-// Two neighbouring columns of a row (packed as they were loaded until they are used).
+// Two neighbouring columns of a row (bf16: packed as they were loaded until they are used).
+template <typename T> struct Pair { using type = float2; };
+template <> struct Pair<__nv_bfloat16> { using type = uint32_t; };
+__device__ __forceinline__ float2 pair(float2 v) { return v; }
 __device__ __forceinline__ float2 pair(uint32_t u) { return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u)); }
 
 struct GateArgs {
@@ -48,21 +51,22 @@ template <int T> struct alignas(16) FilterSmem {
 // from the segments of the block, those above from the blocks' totals, which are the partial sums of the mean pool too.
 // Every warp works out the gate for itself: no more barriers.  `late` runs while the other blocks' totals are
 // on their way.  Returns f_0.
-template <int T, int NW, typename Late, typename Put>
-__device__ __forceinline__ float pool_gate_filter(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __restrict__ K, const GateArgs& a, int row0,
+template <int T, int NW, typename Tin, typename Late, typename Put>
+__device__ __forceinline__ float pool_gate_filter(const Tin* __restrict__ Q, const Tin* __restrict__ K, const GateArgs& a, int row0,
                                                  uint32_t rank, uint32_t blocks, FilterSmem<T>& sm, Late&& late, Put&& put) {
   constexpr int kSegs = T / 8, kTasks = 2 * kSegs, kPer = (kTasks + NW - 1) / NW;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, c0 = 2 * lane;
   const int L1 = a.L + 1;
-  uint32_t raw[kPer][8];
+  using Raw = typename Pair<Tin>::type;
+  Raw raw[kPer][8];
 #pragma unroll
   for (int i = 0; i < kPer; ++i) {
     const int task = warp + i * NW, first = row0 + 8 * (task % kSegs);
-    const __nv_bfloat16* src = (task < kSegs ? Q : K) + (size_t)first * a.d + c0;
+    const Tin* src = (task < kSegs ? Q : K) + (size_t)first * a.d + c0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      raw[i][j] = 0u;
-      if (task < kTasks && c0 < a.d && first + j < a.n) raw[i][j] = *reinterpret_cast<const uint32_t*>(src + (size_t)j * a.d);
+      raw[i][j] = Raw();
+      if (task < kTasks && c0 < a.d && first + j < a.n) raw[i][j] = *reinterpret_cast<const Raw*>(src + (size_t)j * a.d);
     }
   }
   // (what the gate needs of its weights: the two columns of this lane, fetched ahead of the sums)
@@ -529,6 +533,34 @@ k_small_forward(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __rest
   if (blocks > 1) cluster_wait();   // (the others have what this block had for them)
 }
 
+// Mean pool, gate and filter alone, in front of the FFMA kernels (which follow as they are: with them in the same launch one head of
+// 1024 tokens, m = 64, fp32 went from 20.5 to 19.5 us, two thirds of it FFMA passes on 16 SMs).  One launch in the place of
+// k_qmean_gate and k_haar_filter, and Q is read once; bound by latency.  Forwards, us, before and now: fp32, d = 64, m = 64 1 x 1000
+// 20.7 -> 17.9, 4 x 200 18.7 -> 16.1; d = 16, m = 128 16 x 60 17.2 -> 15.2; bf16, m = 64 1 x 1000 22.5 -> 19.7.
+// grid (blocks, slabs), clusters of `blocks`.  place_next: see launch_haar_filter.
+constexpr int kFilterWarps = 8;
+template <int T, typename Tin>
+__global__ void __launch_bounds__(32 * kFilterWarps)
+k_small_filter(const Tin* __restrict__ Q, const Tin* __restrict__ K, const float* __restrict__ gate_w, const float* __restrict__ gate_b,
+               const float* __restrict__ omega, int n, int d, int L, int H, int per_head, float* __restrict__ qbar,
+               float* __restrict__ sg, float* __restrict__ f, float* __restrict__ QF, float* __restrict__ KF, bool place_next) {
+  __shared__ FilterSmem<T> sm;
+  const uint32_t rank = cluster_rank(), blocks = gridDim.x;
+  if (blocks > 1) cluster_arrive();
+  wait_for_stream_predecessor();   // (launched as a programmatic dependent; the first kernel of its pass: see launch_behind)
+  if (place_next) let_stream_successor_start();
+  const int slab = blockIdx.y, row0 = (int)rank * T;
+  const size_t slab_off = (size_t)slab * n * d;
+  const GateArgs gate = {gate_w, gate_b, omega, qbar + (size_t)slab * kD, sg + (size_t)slab * (L + 1), f + (size_t)slab * (L + 1),
+                         per_head ? slab % H : 0, slab % H, L, n, d};
+  pool_gate_filter<T, kFilterWarps>(Q + slab_off, K + slab_off, gate, row0, rank, blocks, sm, []() {},
+                                    [&](int tensor, int t, int at, float y0, float y1) {
+                                      if (row0 + t < n && 2 * at < d)
+                                        *reinterpret_cast<float2*>((tensor == 0 ? QF : KF) + slab_off + (size_t)(row0 + t) * d + 2 * at) =
+                                            make_float2(y0, y1);
+                                    });
+}
+
 template <int V> struct Int { static constexpr int value = V; };
 
 // Runs body(kernel, threads, shared memory) with the kernel of p's tile, if there is one.
@@ -570,6 +602,35 @@ cudaError_t launch_small_forward(const Plan& p, const Ws& w, const void* Q, cons
   return err;
 }
 
+// Runs body(kernel) with the kernel of p's tensors and tile.
+template <typename F> void with_filter(const Plan& p, F&& body) {
+  using bf = __nv_bfloat16;
+  if (p.bf16) {
+    if (p.filter_tokens == 32) body(k_small_filter<32, bf>, (const bf*)nullptr);
+    else body(k_small_filter<64, bf>, (const bf*)nullptr);
+  } else {
+    if (p.filter_tokens == 32) body(k_small_filter<32, float>, (const float*)nullptr);
+    else body(k_small_filter<64, float>, (const float*)nullptr);
+  }
+}
+static int filter_blocks(const Plan& p) { return (p.cfg.seq_len + p.filter_tokens - 1) / p.filter_tokens; }
+
+cudaError_t launch_small_filter(const Plan& p, const Ws& w, const void* Q, const void* K, const float* gate_w, const float* gate_b,
+                                const float* omega, cudaStream_t st, int* launches) {
+  const int blocks = filter_blocks(p);
+  const bool place_next = place_key_side_early(p, (unsigned)(p.slabs * blocks));
+  cudaError_t err = cudaErrorInvalidDeviceFunction;
+  with_filter(p, [&](auto kernel, auto* type) {
+    using P = decltype(type);
+    err = prepare_cluster(kernel, 0, blocks);
+    if (err != cudaSuccess) return;
+    err = launch_cluster(kernel, dim3(blocks, p.slabs), dim3(32 * kFilterWarps), 0, st, (P)Q, (P)K, gate_w, gate_b, omega, p.cfg.seq_len,
+                         p.cfg.head_dim, p.cfg.levels, p.cfg.heads, p.cfg.gate_per_head, w.qbar, w.sg, w.f, w.QF, w.KF, place_next);
+    *launches += 1;
+  });
+  return err;
+}
+
 // Clusters of p's tile that the device holds at once, asked for once per device, kernel and cluster size (the answer does not
 // change), and the shared memory of a block.
 static int small_clusters(const Plan& p, size_t* bytes) {
@@ -589,6 +650,33 @@ static int small_clusters(const Plan& p, size_t* bytes) {
   return clusters;
 }
 
+// Likewise of p's filter kernel.
+static int filter_clusters(const Plan& p) {
+  constexpr int kDevices = 16;
+  static std::atomic<int> known[kDevices][2][2][kMaxCluster + 1];
+  const int blocks = filter_blocks(p);
+  std::atomic<int>* at = p.cfg.device >= kDevices ? nullptr : &known[p.cfg.device][p.bf16][p.filter_tokens == 32][blocks];
+  int clusters = at != nullptr ? at->load(std::memory_order_relaxed) - 1 : -1;
+  if (clusters >= 0) return clusters;
+  with_filter(p, [&](auto kernel, auto*) { clusters = clusters_at_once(kernel, 32 * kFilterWarps, 0, blocks); });
+  if (at != nullptr) at->store(clusters + 1, std::memory_order_relaxed);
+  return clusters;
+}
+
+// Mean pool, gate and filter of the FFMA forward in one launch: slabs of up to 1024 tokens, in blocks of 32 tokens, 64 where 32
+// are too many for a cluster, and as long as the clusters are few.  Forwards, us, by two launches and by one: m = 64, d = 16 16 x 500 (256
+// blocks) 17.3 and 15.4, 40 x 200 (280) 18.7 and 18.1, 80 x 200 (560) 22.1 and 24.2; blocks of 64 4 x 1000 (64) 18.2 and
+// 16.7, m = 128 16 x 1000 (256) 24.1 and 24.7; of 128 (not built) 1 x 2000 17.7 and 20.1.  With 256 features and more the key side's
+// blocks are large and wait behind these: 4 x 200 (28) 17.5 and 15.9, 16 x 60 (32) 19.9 and 18.3, 4 x 500 (64) 19.9 and 21.9.
+// Contexts with a backward: see choose_small_forward.
+static void choose_small_filter(Plan* p) {
+  if (p->use_x || (p->cfg.flags & WERSA_FLAG_SIMT_ONLY) || p->cfg.seq_len > 64 * kMaxCluster) return;
+  p->filter_tokens = p->cfg.seq_len <= 32 * kMaxCluster ? 32 : 64;
+  const long long clusters = p->slabs, blocks = clusters * filter_blocks(*p);
+  const long long most = p->cfg.features >= 256 ? 32 : p->filter_tokens == 32 ? 2 * p->sms : 64;
+  if (blocks > most || filter_clusters(*p) <= 0) p->filter_tokens = 0;
+}
+
 // The one-launch forward where all slabs and groups fit the device at once, a block an SM: then it was faster than the general
 // path in each of 190 shapes (1 to 148 slabs of 64 to 2000 tokens, d = 16, 32, 64, m = 128, 256, 1024; by 1 to 15 us), and a second
 // wave of clusters loses (8 x 1000, m = 128: blocks of 64 tokens 20.5 us, of 128 14.1, general 16.6; 16 x 1000 27 and 18.8).  The
@@ -597,9 +685,13 @@ static int small_clusters(const Plan& p, size_t* bytes) {
 // heads is a sum over slabs, which the clusters do not exchange.  A context with a backward and one feature group may be that of
 // a sequence shard, whose steps (wersa_shard_*) give the bits of wersa_forward: there up to 512 tokens, which nobody cuts.
 void choose_small_forward(Plan* p) {
-  p->small_tokens = p->small_blocks = 0;
-  if (!p->use_tc || (p->cfg.flags & WERSA_FLAG_STEPWISE) || !(p->cfg.gate_per_head || p->cfg.heads == 1)) return;
+  p->small_tokens = p->small_blocks = p->filter_tokens = 0;
+  if ((p->cfg.flags & WERSA_FLAG_STEPWISE) || !(p->cfg.gate_per_head || p->cfg.heads == 1)) return;
   if (p->with_backward && p->groups == 1 && p->cfg.seq_len > 512) return;
+  if (!p->use_tc) {
+    choose_small_filter(p);
+    return;
+  }
   constexpr int kTokens[4] = {16, 32, 64, 128};
   constexpr double kCost[4] = {8.4, 9, 10.5, 14};
   Plan best = *p;
