@@ -521,7 +521,10 @@ wersa_status wersa_create(const wersa_config* cfg, void* workspace, size_t works
     return WERSA_ERR_WORKSPACE;
   {
     DeviceGuard guard(p.cfg.device);
-    if (guard.err == cudaSuccess) choose_small_forward(&p);
+    if (guard.err == cudaSuccess) {
+      choose_small_forward(&p);
+      prepare_qmean_gate(p);
+    }
   }
   wersa_ctx* ctx = new (std::nothrow) wersa_ctx;
   if (ctx == nullptr) return WERSA_ERR_INVALID_ARG;

@@ -40,6 +40,8 @@ __device__ __forceinline__ void peer_copy(uint32_t dst, uint32_t src, uint32_t b
                "r"(bar) : "memory");
 }
 
+// Once per device, ahead of the first launch (a context is created): 0.4 us a call, of which a forward that waits for the host has none
+// to spare (1 x 2531, m = 128 16.7 us with a plain launch, 17.4 with two of these at each launch of the mean pool).
 template <typename K> inline cudaError_t prepare_cluster(K kernel, size_t smem, int blocks) {
   const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   return err != cudaSuccess || blocks <= 8 ? err : cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);

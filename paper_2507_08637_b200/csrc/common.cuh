@@ -72,6 +72,8 @@ struct Ws {   // resolved workspace pointers
 Ws resolve(const Plan& p, void* workspace);
 
 // ---- gate.cu -------------------------------------------------------------------------------
+// What k_qmean_gate's launches as clusters need, once for a context (on its device).
+void prepare_qmean_gate(const Plan& p);
 // Partial column sums of Q over row chunks, then qbar, sigmoid(u) and f per slab (Eqs. 1-3).
 // With W != nullptr the second launch also leaves the bf16 transpose of W (m x 64) in w.Wt.
 // cols: columns of Q as stored (64, or the head dimension when Q comes unpadded; then gate_w has cols rows

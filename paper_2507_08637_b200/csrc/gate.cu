@@ -348,7 +348,7 @@ static cudaError_t launch_qmean_gate_impl(const Plan& p, const void* Q, float* q
       launch_err = start(q, qpart, p.cfg.seq_len, p.qchunk_rows, p.slabs, p.cfg.heads, p.L1, p.cfg.gate_per_head, gate_w, gate_b, omega,
                          qbar, sg, f, slab_count, batch_count, (const __nv_bfloat16*)W, Wt, p.cfg.features, cols, seen);
     };
-    if (cluster && prepare_cluster(clustered, 0, p.qchunks) == cudaSuccess) {
+    if (cluster) {
       go([&](auto... args) { return launch_cluster(clustered, grid, dim3(256), 0, st, args...); });
       if (launch_err == cudaSuccess) return;
       cudaGetLastError();   // (a part of a GPU may have no room for a cluster of more than eight)
@@ -372,6 +372,17 @@ cudaError_t launch_qmean_gate(const Plan& p, const Ws& w, const void* Q, const f
   *launches += 1;
   return launch_qmean_gate_impl(p, Q, w.qpart, gate_w, gate_b, omega, w.qbar, w.sg, w.f, w.counters, W, w.Wt, cols,
                                 p.use_x ? w.seen : nullptr, p.qchunks <= kMaxCluster, st);
+}
+
+void prepare_qmean_gate(const Plan& p) {
+  using bf = __nv_bfloat16;
+  const bool full = p.cfg.head_dim == kD;
+  if (p.qchunks > kMaxCluster) return;
+  auto go = [&](auto kernel) {
+    if (prepare_cluster(kernel, 0, p.qchunks) != cudaSuccess) cudaGetLastError();   // (the launch then falls back)
+  };
+  if (p.bf16) full ? go(k_qmean_gate<bf, true, true>) : go(k_qmean_gate<bf, false, true>);
+  else full ? go(k_qmean_gate<float, true, true>) : go(k_qmean_gate<float, false, true>);
 }
 
 cudaError_t launch_shard_qsum(const Plan& p, const Ws& w, float* qsum, cudaStream_t st, int* launches) {

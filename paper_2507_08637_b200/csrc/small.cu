@@ -592,7 +592,6 @@ cudaError_t launch_small_forward(const Plan& p, const Ws& w, const void* Q, cons
   *launches += 1;
   cudaError_t err = cudaErrorInvalidValue;
   with_small(p, [&](auto kernel, int threads, size_t bytes) {
-    if ((err = prepare_cluster(kernel, bytes, p.small_blocks)) != cudaSuccess) return;
     err = launch_cluster(kernel, dim3(p.small_blocks, p.slabs, p.groups), dim3(threads), bytes, st, (const bf*)Q, (const bf*)K,
                          (const bf*)V, (const bf*)W, beta, gate_w, gate_b, omega, p.cfg.eps, p.cfg.bw_floor, p.cfg.seq_len,
                          p.cfg.head_dim, p.cfg.levels, p.cfg.heads, p.cfg.gate_per_head, p.cfg.features,
@@ -622,8 +621,6 @@ cudaError_t launch_small_filter(const Plan& p, const Ws& w, const void* Q, const
   cudaError_t err = cudaErrorInvalidDeviceFunction;
   with_filter(p, [&](auto kernel, auto* type) {
     using P = decltype(type);
-    err = prepare_cluster(kernel, 0, blocks);
-    if (err != cudaSuccess) return;
     err = launch_cluster(kernel, dim3(blocks, p.slabs), dim3(32 * kFilterWarps), 0, st, (P)Q, (P)K, gate_w, gate_b, omega, p.cfg.seq_len,
                          p.cfg.head_dim, p.cfg.levels, p.cfg.heads, p.cfg.gate_per_head, w.qbar, w.sg, w.f, w.QF, w.KF, place_next);
     *launches += 1;
@@ -631,6 +628,7 @@ cudaError_t launch_small_filter(const Plan& p, const Ws& w, const void* Q, const
   return err;
 }
 
+// (The query also prepares the kernel for its launches: clusters_at_once.)
 // Clusters of p's tile that the device holds at once, asked for once per device, kernel and cluster size (the answer does not
 // change), and the shared memory of a block.
 static int small_clusters(const Plan& p, size_t* bytes) {
