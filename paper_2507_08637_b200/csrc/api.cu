@@ -55,6 +55,7 @@ static wersa_status make_pool_plan(const wersa_config& c, Plan* p) {
   }
   if ((long long)c.batch * c.heads > 65535) return WERSA_ERR_UNSUPPORTED;   // gridDim.y
 
+  *p = Plan();   // (what is not decided here or in make_plan, or not on this device, is 0)
   p->cfg = c;
   p->slabs = c.batch * c.heads;
   p->L1 = c.levels + 1;
@@ -252,7 +253,6 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
     p->tqchunk_blocks = ceil_div(blocks, p->tqchunks);
     p->tqchunks = ceil_div(blocks, p->tqchunk_blocks);
   }
-  p->small_tokens = p->small_blocks = 0;
   {
     // tensor-core backward: one wave of CTAs that share the list of all 128-token tiles evenly
     const long long tiles = (long long)ceil_div(n, 128) * p->slabs;

@@ -122,6 +122,21 @@ def test_status_strings(lib):
     assert len(seen) == 7 and all(s for s in seen)
 
 
+def test_plan_does_not_depend_on_what_its_memory_held(lib):
+    """Every part of a plan is decided when it is made, also what wersa_create decides again where there is a device: made over
+    memory of two fills, it differs nowhere but behind its end."""
+    make_plan = lib._ZN5wersa9make_planERK12wersa_configPNS_4PlanE   # wersa::make_plan(const wersa_config&, Plan*)
+    size = 4096
+    for kw in (dict(), dict(features=64), dict(features=1024), dict(dtype="f32"), dict(dtype="f32", features=64, seq_len=500)):
+        plans = []
+        for fill in (0x55, 0xAA):
+            plan = ctypes.create_string_buffer(bytes([fill]) * size, size)
+            assert make_plan(ctypes.byref(_cfg(**kw)), plan) == 0
+            plans.append(plan.raw)
+        first = next(i for i in range(size) if plans[0][i] != plans[1][i])
+        assert all(plans[0][i] != plans[1][i] for i in range(first, size)), kw
+
+
 def test_static_gate_makes_no_tile_plan():
     """wersa_gate_static needs none of the choices that fp32 contexts search for: refusing a problem that does not fit its
     array takes an fp32 call the time it takes a bf16 one (least of 20 batches of 200 calls)."""
