@@ -250,6 +250,15 @@ wersa_status wersa_query_status(wersa_ctx* ctx, void* cuda_stream);
 wersa_status wersa_selftest_wait_timeout(wersa_ctx* ctx, uint32_t limit_us, int32_t* observed,
                                          void* cuda_stream);
 
+/* The same for the one-launch forward of short sequences, whose thread blocks send one another partial sums and wait for them: the
+ * forward of wersa_forward with gate_w and gate_b NULL, in which the second block of every slab keeps to itself what it owes the
+ * others, its shares of S' and z' (loss = 1) or the rows that it has added up (loss = 2), and waits last a millisecond.  A
+ * block whose wait runs out writes no row of S', z' or O; with loss = 2 the second block has all it needs and writes its own.
+ * WERSA_ERR_UNSUPPORTED unless the context takes that launch with 128 features, head_dim <= 16 and at least two blocks of 16
+ * tokens. */
+wersa_status wersa_selftest_short_forward(wersa_ctx* ctx, int32_t loss, const void* Q, const void* K, const void* V, const void* W,
+                                          const float* beta, const float* omega, void* O, void* cuda_stream);
+
 /* Releases the host-side context.  Does not touch the workspace.  NULL is accepted. */
 wersa_status wersa_destroy(wersa_ctx* ctx);
 

@@ -89,6 +89,8 @@ def _lib():
     lib.wersa_shard_backward_gate.argtypes = [vp, fp, fp, ctypes.c_int64, fp, fp, fp, fp, fp, fp, fp, vp, vp]
     lib.wersa_selftest_wait_timeout.restype = ctypes.c_int
     lib.wersa_selftest_wait_timeout.argtypes = [vp, ctypes.c_uint32, vp, vp]
+    lib.wersa_selftest_short_forward.restype = ctypes.c_int
+    lib.wersa_selftest_short_forward.argtypes = [vp, ctypes.c_int32, vp, vp, vp, vp, fp, fp, vp, vp]
     lib.wersa_uses_tensor_cores.restype = ctypes.c_int32
     lib.wersa_uses_tensor_cores.argtypes = [vp]
     lib.wersa_set_step_timing.restype = ctypes.c_int
@@ -352,6 +354,15 @@ class WersaContext:
         if st != WERSA_OK:
             raise WersaError(st, "wersa_selftest_wait_timeout")
         return observed
+
+    def selftest_short_forward(self, loss, Q, K, V, W, beta, omega, out, stream=None):
+        """wersa_selftest_short_forward: a short forward, to `out`, in which one thread block keeps its data to itself."""
+        dt = self.io_dtype
+        st = _lib().wersa_selftest_short_forward(self._h, int(loss), _ptr(Q, dt, "Q"), _ptr(K, dt, "K"), _ptr(V, dt, "V"),
+                                                 _ptr(W, dt, "W"), _ptr(beta, torch.float32, "beta"),
+                                                 _ptr(omega, torch.float32, "omega"), _ptr(out, dt, "O"), _stream_ptr(stream))
+        if st != WERSA_OK:
+            raise WersaError(st, "wersa_selftest_short_forward")
 
     def set_step_timing(self, enable):
         st = _lib().wersa_set_step_timing(self._h, int(bool(enable)))

@@ -948,6 +948,23 @@ wersa_status wersa_selftest_wait_timeout(wersa_ctx* ctx, uint32_t limit_us, int3
   return WERSA_OK;
 }
 
+wersa_status wersa_selftest_short_forward(wersa_ctx* ctx, int32_t loss, const void* Q, const void* K, const void* V, const void* W,
+                                          const float* beta, const float* omega, void* O, void* cuda_stream) {
+  if (ctx == nullptr || loss < 1 || loss > 2 || Q == nullptr || K == nullptr || V == nullptr || W == nullptr || beta == nullptr ||
+      omega == nullptr || O == nullptr)
+    return WERSA_ERR_INVALID_ARG;
+  if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(W) || !aligned16(O)) return WERSA_ERR_INVALID_ARG;
+  const Plan& p = ctx->plan;
+  if (!selftest_small_supported(p)) return WERSA_ERR_UNSUPPORTED;
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  DeviceGuard guard(p.cfg.device);
+  if (guard.err != cudaSuccess) return WERSA_ERR_CUDA;
+  wersa_status s = clear_status_once(ctx, st);
+  if (s != WERSA_OK) return s;
+  WERSA_CUDA(launch_selftest_small(p, ctx->ws, loss, Q, K, V, W, beta, omega, O, st));
+  return WERSA_OK;
+}
+
 wersa_status wersa_set_step_timing(wersa_ctx* ctx, int enable) {
   if (ctx == nullptr) return WERSA_ERR_INVALID_ARG;
   StepTimer& t = ctx->timer;

@@ -188,7 +188,10 @@ cudaError_t launch_tc_qside(const Plan& p, const Ws& w, const void* Q, const flo
 cudaError_t launch_small_forward(const Plan& p, const Ws& w, const void* Q, const void* K, const void* V, const void* W,
                                  const float* beta, const float* gate_w, const float* gate_b, const float* omega, void* O,
                                  cudaStream_t st, int* launches);
-
+// Self-test of its waits that run out.
+bool selftest_small_supported(const Plan& p);
+cudaError_t launch_selftest_small(const Plan& p, const Ws& w, int loss, const void* Q, const void* K, const void* V, const void* W,
+                                  const float* beta, const float* omega, void* O, cudaStream_t st);
 // Mean pool, gate, and w.QF = T_f(Q), w.KF = T_f(K), in one launch (p.filter_tokens).
 cudaError_t launch_small_filter(const Plan& p, const Ws& w, const void* Q, const void* K, const float* gate_w, const float* gate_b,
                                 const float* omega, cudaStream_t st, int* launches);

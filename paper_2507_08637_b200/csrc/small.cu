@@ -275,7 +275,10 @@ __device__ __forceinline__ float bf_sum(uint32_t u) { return __uint_as_float(u <
 
 // grid (blocks, slabs, feature groups), clusters of `blocks`.  m: features of the whole map.  Sbf, Wt: for a backward, or null.
 // den: with several groups, every token's denominator times r = bf16(f_0) / f_0 as tc_fwd.cu leaves it, and O is the group's.
-template <int M, int T, int KS>
+// A block whose wait runs out sends and stores nothing from there on; it leaves through the barrier that every block of the cluster
+// passes, and not before the copies on their way to it have landed (or had their time).
+// kLoss: for the self-test of that, waits are short and block 1 keeps its shares of the sums (1) or its rows of the image (2) to itself.
+template <int M, int T, int KS, int kLoss = 0>
 __global__ void __launch_bounds__(SmallSmem<M, T, KS>::kThreads, 1)
 k_small_forward(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict__ V,
                 const __nv_bfloat16* __restrict__ W, const float* __restrict__ beta, const float* __restrict__ gate_w,
@@ -291,6 +294,7 @@ k_small_forward(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __rest
   const uint32_t rank = cluster_rank(), blocks = gridDim.x;
   const int slab = blockIdx.y, group = blockIdx.z, f0g = group * M, row0 = (int)rank * T;
   const int per = (M + (int)blocks - 1) / (int)blocks;   // rows of S' that a block adds up
+  constexpr unsigned long long kLimitNs = kLoss == 0 ? tc::kWaitLimitNs : 1000 * 1000;
   const uint32_t base = shared_addr(smem);
   const int count = max(0, min(per, M - (int)rank * per));   // (none for the last block or two where blocks are many)
   SmallBars* bars = reinterpret_cast<SmallBars*>(smem + SL::bars);
@@ -415,7 +419,7 @@ k_small_forward(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __rest
   }
   tc::fence_proxy_async_smem();
   __syncthreads();   // (the image may be written over W, by the other blocks too once they have this one's sums)
-  if (lane == 0) {   // their rows to the blocks that add them up, this one among them
+  if (lane == 0 && !(kLoss == 1 && rank == 1)) {   // their rows to the blocks that add them up, this one among them
     for (uint32_t r = warp; r < blocks; r += SL::kWarps) {
       const int rows = min(per, M - (int)r * per);
       if (rows > 0)
@@ -423,10 +427,12 @@ k_small_forward(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __rest
                   peer_addr(shared_addr(&bars->sums), r));
     }
   }
-  tc::mbar_wait(&bars->sums, 0, &bars->abort_flag, status, kErrSmall);
+  __syncwarp();
+  // (one answer per warp until the barriers that stand here anyway; to ask at all takes 0.1 of 10.4 us, 1 x 4 x 1000, m = 128)
+  bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->sums, 0, &bars->abort_flag, status, kErrSmall, kLimitNs));
   // ---- S', z' of this block's rows -> the place of the first block's share, and the image's rows
   float* sums = reinterpret_cast<float*>(smem + SL::recv);
-  for (int i = tid; i < count * (2 * kTiles + 1); i += NT) {
+  for (int i = ok ? tid : count * (2 * kTiles + 1); i < count * (2 * kTiles + 1); i += NT) {
     const int c = i / count, r = i - c * count;   // pieces of four columns, then z' and what lies behind it
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
@@ -453,18 +459,24 @@ k_small_forward(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __rest
     }
   }
   if (blocks > 1) tc::fence_proxy_async_smem();
-  __syncthreads();
-  if (blocks > 1) {
-    if (lane == 0 && count > 0)
+  ok = __syncthreads_and(ok);
+  if (blocks > 1 && ok) {
+    if (lane == 0 && count > 0 && !(kLoss == 2 && rank == 1))
       for (uint32_t r = warp; r < blocks; r += SL::kWarps) {
         const uint32_t at = base + SL::s + rank * per * kPitch * 2;
         if (r != rank) peer_copy(peer_addr(at, r), at, count * kPitch * 2, peer_addr(shared_addr(&bars->image), r));
       }
-    tc::mbar_wait(&bars->image, 0, &bars->abort_flag, status, kErrSmall);
-    cluster_arrive();   // (this block has what the others had for it)
+    __syncwarp();
+    ok = __all_sync(0xffffffffu, tc::mbar_wait(&bars->image, 0, &bars->abort_flag, status, kErrSmall, kLimitNs));
   }
+  if (!ok) {
+    tc::mbar_wait_drain(&bars->sums, 0, kLimitNs);
+    tc::mbar_wait_drain(&bars->image, 0, kLimitNs);
+    __syncwarp();
+  }
+  if (blocks > 1) cluster_arrive();   // (this block has what the others had for it)
   // ---- query side, the contraction
-  {
+  if (ok) {
     float acc[kTiles + 1][4];   // N', and D' from z' (hi, lo) behind it
 #pragma unroll
     for (int c = 0; c < kTiles + 1; ++c)
@@ -492,7 +504,10 @@ k_small_forward(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __rest
         *reinterpret_cast<float2*>(red + (tok + g + 8) * kSumPitch + 8 * c + 2 * q) = make_float2(acc[c][2], acc[c][3]);
       }
   }
-  __syncthreads();
+  if (!__syncthreads_and(ok)) {
+    if (blocks > 1) cluster_wait();
+    return;
+  }
   const float epsp = eps * (float)M * bw * bw;   // (of the group)
   const float* red = reinterpret_cast<const float*>(smem + SL::stage);
   for (int i = tid; i < T * kTiles; i += NT) {
@@ -585,20 +600,39 @@ template <typename F> bool with_small(const Plan& p, F&& body) {
 
 }  // namespace
 
+template <typename Kernel>
+static cudaError_t launch_small(Kernel kernel, int threads, size_t bytes, const Plan& p, const Ws& w, const void* Q, const void* K,
+                                const void* V, const void* W, const float* beta, const float* gate_w, const float* gate_b,
+                                const float* omega, void* O, cudaStream_t st) {
+  using bf = __nv_bfloat16;
+  return launch_cluster(kernel, dim3(p.small_blocks, p.slabs, p.groups), dim3(threads), bytes, st, (const bf*)Q, (const bf*)K,
+                        (const bf*)V, (const bf*)W, beta, gate_w, gate_b, omega, p.cfg.eps, p.cfg.bw_floor, p.cfg.seq_len,
+                        p.cfg.head_dim, p.cfg.levels, p.cfg.heads, p.cfg.gate_per_head, p.cfg.features,
+                        p.groups > 1 ? (bf*)w.Og : (bf*)O, p.groups > 1 ? w.den : nullptr, w.qbar, w.sg, w.f, w.S, w.z,
+                        p.with_backward ? w.Sbf : nullptr, p.with_backward ? w.Wt : nullptr, w.status);
+}
+
 cudaError_t launch_small_forward(const Plan& p, const Ws& w, const void* Q, const void* K, const void* V, const void* W,
                                  const float* beta, const float* gate_w, const float* gate_b, const float* omega, void* O,
                                  cudaStream_t st, int* launches) {
-  using bf = __nv_bfloat16;
   *launches += 1;
   cudaError_t err = cudaErrorInvalidValue;
   with_small(p, [&](auto kernel, int threads, size_t bytes) {
-    err = launch_cluster(kernel, dim3(p.small_blocks, p.slabs, p.groups), dim3(threads), bytes, st, (const bf*)Q, (const bf*)K,
-                         (const bf*)V, (const bf*)W, beta, gate_w, gate_b, omega, p.cfg.eps, p.cfg.bw_floor, p.cfg.seq_len,
-                         p.cfg.head_dim, p.cfg.levels, p.cfg.heads, p.cfg.gate_per_head, p.cfg.features,
-                         p.groups > 1 ? (bf*)w.Og : (bf*)O, p.groups > 1 ? w.den : nullptr, w.qbar, w.sg, w.f, w.S, w.z,
-                         p.with_backward ? w.Sbf : nullptr, p.with_backward ? w.Wt : nullptr, w.status);
+    err = launch_small(kernel, threads, bytes, p, w, Q, K, V, W, beta, gate_w, gate_b, omega, O, st);
   });
   return err;
+}
+
+// The same with block 1 of every cluster keeping its shares of the sums (loss = 1) or its rows of the image (2) to itself.
+bool selftest_small_supported(const Plan& p) {
+  return p.small_tokens == 16 && p.small_blocks > 1 && p.cfg.features == 128 && p.cfg.head_dim <= 16;
+}
+cudaError_t launch_selftest_small(const Plan& p, const Ws& w, int loss, const void* Q, const void* K, const void* V, const void* W,
+                                  const float* beta, const float* omega, void* O, cudaStream_t st) {
+  using SL = SmallSmem<128, 16, 1>;
+  auto kernel = loss == 1 ? k_small_forward<128, 16, 1, 1> : k_small_forward<128, 16, 1, 2>;
+  const cudaError_t err = prepare_cluster(kernel, SL::total, p.small_blocks);
+  return err != cudaSuccess ? err : launch_small(kernel, SL::kThreads, SL::total, p, w, Q, K, V, W, beta, nullptr, nullptr, omega, O, st);
 }
 
 // Runs body(kernel) with the kernel of p's tensors and tile.

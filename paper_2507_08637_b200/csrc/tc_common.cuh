@@ -76,11 +76,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 
 // Time-bounded wait that ignores the abort flag: used on the abort path to let copies that are
 // already in flight land before the CTA exits.
-__device__ __forceinline__ void mbar_wait_drain(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ void mbar_wait_drain(uint64_t* bar, uint32_t parity, unsigned long long limit_ns = kWaitLimitNs) {
   const unsigned long long t0 = global_timer_ns();
   uint32_t spins = 0;
   while (!mbar_try_wait(bar, parity)) {
-    if ((++spins & 255u) == 0 && global_timer_ns() - t0 > kWaitLimitNs) return;
+    if ((++spins & 255u) == 0 && global_timer_ns() - t0 > limit_ns) return;
   }
 }
 
