@@ -71,15 +71,20 @@ static wersa_status make_pool_plan(const wersa_config& c, Plan* p) {
   p->qchunks = ceil_div(4 * p->sms, p->slabs);
   if (p->qchunks > ceil_div(n, 128)) p->qchunks = ceil_div(n, 128);
   if (p->qchunks < 1) p->qchunks = 1;
-  // The chunks of a slab are one cluster (of at most 16) where that still covers most of the SMs and a chunk is not long: training
+  // In a context the chunks of a slab are one cluster (of at most 16) where that still covers most of the SMs and a chunk is not long: training
   // steps of 2 x 4 x 4096, d = 32, fp32 104.6 -> 103.3 us, of 4 x 8 x 16384 710.7 -> 703.9; forwards of 2 x 8 x 4096, fp32 96.6 -> 95.7.
   // With fewer slabs up to 1 MB of Q a slab (2 MB where the tensor-core key side has its first copies under way meanwhile): what
   // the counters take is then more than the longer chunks do.  Forwards, us, more chunks and 16: bf16 2 x 3994, d = 32, m = 512 22.1
   // and 20.3, 1 x 16000, d = 16, m = 128 21.9 and 19.0, d = 64, m = 256 22.8 and 21.8; m = 64 1 x 8000 25.1 and 24.0, 2 x 16000 (2 MB) 34.5
   // and 35.4; fp32 1 x 3994, m = 256 28.3 and 27.7, 1 x 11000 (2.8 MB) 37.5 and 38.6.
+  // (qchunks are those of launches that keep arrival counters: wersa_gate_static, and where a cluster finds no room.)
   const long long slab_bytes = (long long)n * c.head_dim * (p->bf16 ? 2 : 4);
   const bool few = slab_bytes <= (p->use_tc ? 2 << 20 : 1 << 20);
-  if (p->qchunks > 16 && (few || 16 * p->slabs * 4 >= 3 * p->sms) && n <= 16 * 1024) p->qchunks = 16;
+  int pool = p->qchunks;
+  if (pool > 16 && (few || 16 * p->slabs * 4 >= 3 * p->sms) && n <= 16 * 1024) pool = 16;
+  p->qcluster_rows = ceil_div(ceil_div(n, pool), 32) * 32;
+  p->qcluster = ceil_div(n, p->qcluster_rows);
+  if (p->qcluster > 16) p->qcluster = 0;
   p->qchunk_rows = ceil_div(ceil_div(n, p->qchunks), 32) * 32;
   p->qchunks = ceil_div(n, p->qchunk_rows);
   return WERSA_OK;

@@ -30,6 +30,7 @@ struct Plan {
   int groups;         // feature groups of kGroupFeatures (1 when cfg.features <= 256)
   // mean pool
   int qchunks, qchunk_rows;
+  int qcluster, qcluster_rows;   // the same where the chunks of a slab are one cluster; 0: they are not
   // haar tiles
   int htiles;
   // fp32 FFMA key-side / backward query-side split of the sequence

@@ -336,7 +336,7 @@ static cudaError_t launch_qmean_gate_impl(const Plan& p, const void* Q, float* q
                                           const float* gate_b, const float* omega, float* qbar, float* sg, float* f,
                                           int* counters, const void* W, __nv_bfloat16* Wt, int cols,
                                           int* seen, bool cluster, cudaStream_t st) {
-  dim3 grid(p.qchunks, p.slabs + (W != nullptr || (p.bf16 && seen != nullptr) ? 1 : 0));
+  const int rows = p.slabs + (W != nullptr || (p.bf16 && seen != nullptr) ? 1 : 0);
   int* slab_count = counters;
   int* batch_count = counters + p.slabs;
   cudaError_t launch_err = cudaSuccess;
@@ -344,16 +344,16 @@ static cudaError_t launch_qmean_gate_impl(const Plan& p, const void* Q, float* q
   // work to complete, so ordering and visibility are those of a plain launch, but its CTAs are already placed when the wait
   // ends (2 us per forward in a sequence of steps).
   auto launch = [&](auto kernel, auto clustered, auto* q) {
-    auto go = [&](auto start) {
-      launch_err = start(q, qpart, p.cfg.seq_len, p.qchunk_rows, p.slabs, p.cfg.heads, p.L1, p.cfg.gate_per_head, gate_w, gate_b, omega,
+    auto go = [&](int chunk_rows, auto start) {
+      launch_err = start(q, qpart, p.cfg.seq_len, chunk_rows, p.slabs, p.cfg.heads, p.L1, p.cfg.gate_per_head, gate_w, gate_b, omega,
                          qbar, sg, f, slab_count, batch_count, (const __nv_bfloat16*)W, Wt, p.cfg.features, cols, seen);
     };
     if (cluster) {
-      go([&](auto... args) { return launch_cluster(clustered, grid, dim3(256), 0, st, args...); });
+      go(p.qcluster_rows, [&](auto... args) { return launch_cluster(clustered, dim3(p.qcluster, rows), dim3(256), 0, st, args...); });
       if (launch_err == cudaSuccess) return;
       cudaGetLastError();   // (a part of a GPU may have no room for a cluster of more than eight)
     }
-    go([&](auto... args) { return launch_after(kernel, grid, dim3(256), 0, st, args...); });
+    go(p.qchunk_rows, [&](auto... args) { return launch_after(kernel, dim3(p.qchunks, rows), dim3(256), 0, st, args...); });
   };
   using bf = __nv_bfloat16;
   if (p.bf16) {
@@ -371,15 +371,15 @@ cudaError_t launch_qmean_gate(const Plan& p, const Ws& w, const void* Q, const f
                               int* launches) {
   *launches += 1;
   return launch_qmean_gate_impl(p, Q, w.qpart, gate_w, gate_b, omega, w.qbar, w.sg, w.f, w.counters, W, w.Wt, cols,
-                                p.use_x ? w.seen : nullptr, p.qchunks <= kMaxCluster, st);
+                                p.use_x ? w.seen : nullptr, p.qcluster > 0, st);
 }
 
 void prepare_qmean_gate(const Plan& p) {
   using bf = __nv_bfloat16;
   const bool full = p.cfg.head_dim == kD;
-  if (p.qchunks > kMaxCluster) return;
+  if (p.qcluster == 0) return;
   auto go = [&](auto kernel) {
-    if (prepare_cluster(kernel, 0, p.qchunks) != cudaSuccess) cudaGetLastError();   // (the launch then falls back)
+    if (prepare_cluster(kernel, 0, p.qcluster) != cudaSuccess) cudaGetLastError();   // (the launch then falls back)
   };
   if (p.bf16) full ? go(k_qmean_gate<bf, true, true>) : go(k_qmean_gate<bf, false, true>);
   else full ? go(k_qmean_gate<float, true, true>) : go(k_qmean_gate<float, false, true>);

@@ -137,6 +137,20 @@ def test_plan_does_not_depend_on_what_its_memory_held(lib):
         assert all(plans[0][i] != plans[1][i] for i in range(first, size)), kw
 
 
+@pytest.mark.parametrize("slabs,n,dtype", [(1, 16000, "bf16"), (1, 4000, "f32"), (8, 16384, "bf16"), (40, 2500, "bf16"), (8, 131072, "bf16")])
+def test_static_gate_cuts_a_slab_as_documented(lib, slabs, n, dtype):
+    """The mean pool of wersa_gate_static is no cluster, whatever contexts of the shape take: about four row chunks per
+    multiprocessor over all slabs, of 128 rows and more, in its scratch one after the other."""
+    make_plan = lib._ZN5wersa9make_planERK12wersa_configPNS_4PlanE   # wersa::make_plan(const wersa_config&, Plan*)
+    needed = lib._ZN5wersa28static_scratch_floats_neededERKNS_4PlanE   # wersa::static_scratch_floats_needed(const Plan&)
+    needed.restype = ctypes.c_size_t
+    plan = ctypes.create_string_buffer(4096)
+    assert make_plan(ctypes.byref(_cfg(batch=1, heads=slabs, seq_len=n, head_dim=64, levels=3, features=256, dtype=dtype)), plan) == 0
+    chunks = min(-(-592 // slabs), -(-n // 128))
+    rows = -(-(-(-n // chunks)) // 32) * 32
+    assert needed(plan) == slabs * (64 * -(-n // rows) + 4)
+
+
 def test_static_gate_makes_no_tile_plan():
     """wersa_gate_static needs none of the choices that fp32 contexts search for: refusing a problem that does not fit its
     array takes an fp32 call the time it takes a bf16 one (least of 20 batches of 200 calls)."""
