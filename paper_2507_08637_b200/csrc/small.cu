@@ -455,7 +455,8 @@ k_small_forward(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __rest
       *reinterpret_cast<uint2*>(img) = make_uint2(pack_bf16x2(s.x, s.y), pack_bf16x2(s.z, s.w));
     } else {
       const float top = __bfloat162float(__float2bfloat16_rn(s.x));
-      *reinterpret_cast<uint4*>(img) = make_uint4(pack_bf16x2(top, s.x - top), 0u, 0u, 0u);
+      const float low = fabsf(top) < INFINITY ? s.x - top : 0.f;   // (behind an infinite z' infinity again, or NaN: D' is infinite)
+      *reinterpret_cast<uint4*>(img) = make_uint4(pack_bf16x2(top, low), 0u, 0u, 0u);
     }
   }
   if (blocks > 1) tc::fence_proxy_async_smem();
