@@ -1,7 +1,10 @@
 // Clusters of thread blocks: barriers, and the shared memory of the other blocks.
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <atomic>
 
 namespace wersa {
 
@@ -40,7 +43,7 @@ __device__ __forceinline__ void peer_copy(uint32_t dst, uint32_t src, uint32_t b
                "r"(bar) : "memory");
 }
 
-// Once per device, ahead of the first launch (a context is created): 0.4 us a call, of which a forward that waits for the host has none
+// Once per CUDA context, ahead of the first launch (a wersa_ctx is created): 0.4 us a call, of which a forward that waits for the host has none
 // to spare (1 x 2531, m = 128 16.7 us with a plain launch, 17.4 with two of these at each launch of the mean pool).
 template <typename K> inline cudaError_t prepare_cluster(K kernel, size_t smem, int blocks) {
   const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -64,6 +67,35 @@ template <typename K> inline int clusters_at_once(K kernel, int threads, size_t 
   cudaGetLastError();   // a failed query leaves no sticky error behind
   return 0;
 }
+// The current CUDA context's number, which no other context of the process ever has; 0: none, or not to be had.
+inline unsigned long long current_context_id() {
+  using Fn = CUresult (*)(CUcontext, unsigned long long*);
+  static const Fn fn = []() -> Fn {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+      return reinterpret_cast<Fn>(p);
+    cudaGetLastError();
+    return nullptr;
+  }();
+  unsigned long long id = 0;
+  return fn != nullptr && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+// What clusters_at_once answered, for the CUDA context that it was asked in: the answer and the kernel's attributes belong to that,
+// not to the device, and another context (one more of the driver API's, the next one after a reset) asks again.  wersa_create
+// takes 30 to 140 us where it asks, 1.5 where it does not.  An answer of none is not kept: the query may have failed for a reason that
+// passes.
+struct KnownClusters {
+  std::atomic<unsigned long long> word{0};   // context number << 16 | answer
+  template <typename Ask> int get(Ask&& ask) {
+    const unsigned long long id = current_context_id(), w = word.load(std::memory_order_acquire);
+    if (id != 0 && w >> 16 == id) return (int)(w & 0xFFFF);
+    const int clusters = ask();
+    if (id != 0 && id >> 48 == 0 && clusters > 0 && clusters <= 0xFFFF)
+      word.store(id << 16 | (unsigned long long)clusters, std::memory_order_release);
+    return clusters;
+  }
+};
 // A launch like launch_after's whose grid's first dimension is one cluster.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {

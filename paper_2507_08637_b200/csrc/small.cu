@@ -16,8 +16,6 @@
 // one's operand in the registers, where tcgen05.mma would want its set-up and a way through TMEM for each.  A warp of the key side
 // owns 16 features, whose values (accumulators of the projection) are the A operand of S' += Phi^T V; one of the query side 16
 // tokens and T features, likewise.
-#include <atomic>
-
 #include "cluster.cuh"
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -663,22 +661,19 @@ cudaError_t launch_small_filter(const Plan& p, const Ws& w, const void* Q, const
   return err;
 }
 
-// (The query also prepares the kernel for its launches: clusters_at_once.)
-// Clusters of p's tile that the device holds at once, asked for once per device, kernel and cluster size (the answer does not
-// change), and the shared memory of a block.
+// Clusters of p's tile that the device holds at once, and the shared memory of a block.  (The query also prepares the kernel for its
+// launches: clusters_at_once.)
 static int small_clusters(const Plan& p, size_t* bytes) {
   constexpr int kDevices = 16;
-  static std::atomic<int> known[kDevices][4][2][3][kMaxCluster + 1];   // 1 + the answer; 0: not asked yet
+  static KnownClusters known[kDevices][4][2][3][kMaxCluster + 1];
   int clusters = 0;
   with_small(p, [&](auto kernel, int threads, size_t b) {
     *bytes = b;
     const int d = p.cfg.head_dim, t = p.small_tokens;
-    std::atomic<int>* at = p.cfg.device >= kDevices ? nullptr
-                                                    : &known[p.cfg.device][t == 16 ? 0 : t == 32 ? 1 : t == 64 ? 2 : 3]
-                                                            [p.cfg.features == 128 ? 0 : 1][d <= 16 ? 0 : d <= 32 ? 1 : 2][p.small_blocks];
-    if (at != nullptr && (clusters = at->load(std::memory_order_relaxed) - 1) >= 0) return;
-    clusters = clusters_at_once(kernel, threads, b, p.small_blocks);
-    if (at != nullptr) at->store(clusters + 1, std::memory_order_relaxed);
+    auto ask = [&]() { return clusters_at_once(kernel, threads, b, p.small_blocks); };
+    clusters = p.cfg.device >= kDevices ? ask()
+                                        : known[p.cfg.device][t == 16 ? 0 : t == 32 ? 1 : t == 64 ? 2 : 3]
+                                               [p.cfg.features == 128 ? 0 : 1][d <= 16 ? 0 : d <= 32 ? 1 : 2][p.small_blocks].get(ask);
   });
   return clusters;
 }
@@ -686,14 +681,14 @@ static int small_clusters(const Plan& p, size_t* bytes) {
 // Likewise of p's filter kernel.
 static int filter_clusters(const Plan& p) {
   constexpr int kDevices = 16;
-  static std::atomic<int> known[kDevices][2][2][kMaxCluster + 1];
+  static KnownClusters known[kDevices][2][2][kMaxCluster + 1];
   const int blocks = filter_blocks(p);
-  std::atomic<int>* at = p.cfg.device >= kDevices ? nullptr : &known[p.cfg.device][p.bf16][p.filter_tokens == 32][blocks];
-  int clusters = at != nullptr ? at->load(std::memory_order_relaxed) - 1 : -1;
-  if (clusters >= 0) return clusters;
-  with_filter(p, [&](auto kernel, auto*) { clusters = clusters_at_once(kernel, 32 * kFilterWarps, 0, blocks); });
-  if (at != nullptr) at->store(clusters + 1, std::memory_order_relaxed);
-  return clusters;
+  int clusters = 0;
+  auto ask = [&]() {
+    with_filter(p, [&](auto kernel, auto*) { clusters = clusters_at_once(kernel, 32 * kFilterWarps, 0, blocks); });
+    return clusters;
+  };
+  return p.cfg.device >= kDevices ? ask() : known[p.cfg.device][p.bf16][p.filter_tokens == 32][blocks].get(ask);
 }
 
 // Mean pool, gate and filter of the FFMA forward in one launch: slabs of up to 1024 tokens, in blocks of 32 tokens, 64 where 32
