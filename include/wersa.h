@@ -270,13 +270,14 @@ const char* wersa_status_string(wersa_status status);
 int32_t wersa_launch_count(const wersa_ctx* ctx, int which);
 
 /* 1 if this context multiplies bf16 operands (the filtered tensors and the features rounded to bf16, sums in fp32):
- * dtype bf16 without WERSA_FLAG_SIMT_ONLY, on the tensor cores.  0 if it computes in fp32.  That is on the FFMA kernels,
- * or, with dtype fp32, 128 or 256 features and a problem for which it is the faster way, on the tensor cores as well,
- * with every operand split into three bf16 planes whose sum is its fp32 value: O is as close to 64 bits as with the
- * FFMA kernels, in the 2-norm, but not the same bits.  Such a context's steps are called f32_planes and tcx_... (see
- * wersa_step_times), and WERSA_FLAG_SIMT_ONLY keeps a context off them.  What differs at the ends of the range: values
- * below 2^-110 lose low-order bits (a bf16 plane ends at 2^-133), and a sum that meets an infinity comes out as NaN
- * where an FFMA sum may be infinite. */
+ * dtype bf16 with 128 features or more and without WERSA_FLAG_SIMT_ONLY, on the tensor cores.  0 if it computes in
+ * fp32.  That is on the FFMA kernels, or, with dtype fp32 or 64 features and a problem for which it is the faster way, on
+ * the tensor cores as well, with every operand split into three bf16 planes whose sum is its fp32 value (V, W and dO of
+ * dtype bf16 are one plane as they are): O is as close to 64 bits as with the FFMA kernels, in the 2-norm, but not the
+ * same bits.  Such a context's steps are called f32_planes and tcx_... (see wersa_step_times), and WERSA_FLAG_SIMT_ONLY
+ * keeps a context off them.  What differs at the ends of the range, with dtype bf16 and 64 features too: values of split
+ * operands below 2^-110 lose low-order bits (a bf16 plane ends at 2^-133), and a sum that meets an infinity comes out as
+ * NaN where an FFMA sum may be infinite. */
 int32_t wersa_uses_tensor_cores(const wersa_ctx* ctx);
 
 /* Step timing (a measurement aid; the paper has no counterpart).  When enabled, forward and
