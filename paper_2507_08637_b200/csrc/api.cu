@@ -77,7 +77,12 @@ static wersa_status make_pool_plan(const wersa_config& c, Plan* p) {
   // the counters take is then more than the longer chunks do.  Forwards, us, more chunks and 16: bf16 2 x 3994, d = 32, m = 512 22.1
   // and 20.3, 1 x 16000, d = 16, m = 128 21.9 and 19.0, d = 64, m = 256 22.8 and 21.8; m = 64 1 x 8000 25.1 and 24.0, 2 x 16000 (2 MB) 34.5
   // and 35.4; fp32 1 x 3994, m = 256 28.3 and 27.7, 1 x 11000 (2.8 MB) 37.5 and 38.6.
-  // (qchunks are those of launches that keep arrival counters: wersa_gate_static, and where a cluster finds no room.)
+  // At the end of the range of lengths, forwards of 7, 8 and 12 slabs of d = 64, m = 256, bf16: 16384 tokens 40.5, 41.1, 52.2 and 39.7, 40.2,
+  // 50.9; beyond it 16 chunks would give 16500 41.4, 42.2, 52.2 and 40.9, 41.7, 51.5, 20000 42.1, 45.9, 57.5 and 42.7, 46.0, 57.1, 32768
+  // 56.8, 59.5, 77.8 and 59.5, 62.7, 79.6; fp32, m = 128 7 x 16384 103.3 and 103.7, 7 x 20000 119.5 and 121.1.  (Narrow heads would
+  // gain further on, 1 x 17000, d = 16 23.6 and 20.5, and are cut as before.)
+  // qchunks are those of launches that keep arrival counters: wersa_gate_static (8 slabs of 16384, fp32 14.5 us, with 16 chunks 16.6; but
+  // 32 slabs of 4096, bf16 12.2 and 10.4), and where a cluster finds no room.
   const long long slab_bytes = (long long)n * c.head_dim * (p->bf16 ? 2 : 4);
   const bool few = slab_bytes <= (p->use_tc ? 2 << 20 : 1 << 20);
   int pool = p->qchunks;

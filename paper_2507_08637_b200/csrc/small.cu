@@ -710,8 +710,12 @@ static void choose_small_filter(Plan* p) {
 // wave of clusters loses (8 x 1000, m = 128: blocks of 64 tokens 20.5 us, of 128 14.1, general 16.6; 16 x 1000 27 and 18.8).  The
 // tokens of a block: as few as fit, since a block's time grows with them (m = 128, d = 64 8.4, 9.0, 10.5 and 14.2 us for 16, 32, 64
 // and 128), unless that makes blocks share SMs (32 x 64, m = 128: 16 tokens 10.6, 32 9.3).  The gate of a batch element of several
-// heads is a sum over slabs, which the clusters do not exchange.  A context with a backward and one feature group may be that of
-// a sequence shard, whose steps (wersa_shard_*) give the bits of wersa_forward: there up to 512 tokens, which nobody cuts.
+// heads is a sum over slabs, which the clusters do not exchange.  A context with a backward and one feature group takes this launch
+// or k_small_filter up to 512 tokens.  They would pay beyond that too; such contexts have kept the bits of a launch per step, and
+// nothing else holds the line there.  Forwards of contexts with a backward, us, by steps and by one launch: 1 x 4 x 600, m = 128 20.1
+// and 10.3; 1 x 4 x 1000 15.7 and 11.0, m = 256 17.3 and 16.0; 3 x 700, d = 32, m = 256 17.7 and 10.8; 1 x 4 x 2000 16.2 and 14.5; fp32,
+// m = 64 1 x 1000 21.0 and 18.2.  (The steps of a sequence shard are launches of their own in every context, and give what
+// wersa_forward does up to rounding.)
 void choose_small_forward(Plan* p) {
   p->small_tokens = p->small_blocks = p->filter_tokens = 0;
   if ((p->cfg.flags & WERSA_FLAG_STEPWISE) || !(p->cfg.gate_per_head || p->cfg.heads == 1)) return;
