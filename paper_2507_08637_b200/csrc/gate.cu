@@ -97,7 +97,7 @@ __device__ __forceinline__ void batch_gate(int b, int H, int L1, const float* __
   }
 }
 
-// Mean pool and gate in one launch.  grid (qchunks, slabs [+ 1]), block 256.
+// Mean pool and gate in one launch.  grid (qcluster or qchunks, slabs [+ 1]), block 256.
 // Rows y < slabs: partial column sums of one row chunk of one slab of Q -- thread (cg = tid & 7,
 // rl = tid >> 3) owns 8 consecutive columns and every 32nd row, loads 16 bytes (bf16) / 32 bytes
 // (fp32) per row, four rows in flight, with the streaming cache hint (Q is read once here).  kCluster: the chunks of a slab are a
