@@ -204,7 +204,7 @@ wersa_status make_plan(const wersa_config& c, Plan* p) {
       // m = 64, fitted to 220 shapes (1 to 1023 slabs, 16 to 131072 tokens, d = 16 to 64, fp32 and bf16; rms 5 % off for planes, 8
       // and 13 % for FFMA; 14 of 440 choices cost more than 5 %, the worst 13 %).  FFMA and planes, us: forward bf16 1 x 7861, d = 16
       // 26 24; 237 x 20 24 40; 1 x 7258, d = 64 32 24; 14 x 21903 405 160; fp32 1 x 1024 20.9 21.4; 2 x 36480 94 69; training step
-      // bf16 212 x 355 444 204.  From 24 tiles on, the fewest of the fit.
+      // bf16 212 x 355 444 206.  From 24 tiles on, the fewest of the fit.
       constexpr double kFwd[2][3] = {{0.144, 0.216, 0.371}, {0.184, 0.291, 0.426}}, kBwd[2][3] = {{0.291, 0.428, 0.754}, {0.404, 0.59, 0.805}};
       const double elems = 1e-6 * p->slabs * n * c.head_dim, wt = (double)waves * p->xchunk_tiles, bt = (double)bwaves * (p->xbchunk_tiles + 1);
       f_fwd = 11.2 + kFwd[p->simt_small][width] * ffma_cost;

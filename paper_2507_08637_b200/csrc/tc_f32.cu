@@ -310,7 +310,9 @@ __device__ __forceinline__ void load_planes(uint8_t* dst, const CUtensorMap* map
 }
 
 // D[128 x N] = A B^T over the head dimension in steps of 16 columns, both operands as planes of up to 128 rows x 64 columns.
-template <int N, bool kExactA, bool kExactB>
+// kParts: the steps from the third on go to a second accumulator, kPartCol columns behind the first.
+constexpr uint32_t kPartCol = 64;
+template <int N, bool kExactA, bool kExactB, bool kParts = false>
 __device__ __forceinline__ void issue_planes(uint32_t dst, uint32_t a_lo, uint32_t b_lo, int ksteps, uint32_t hi) {
   constexpr uint32_t kIdesc1 = make_idesc_bf16(128, N, false, false);   // both operands K-major
 #pragma unroll
@@ -319,8 +321,9 @@ __device__ __forceinline__ void issue_planes(uint32_t dst, uint32_t a_lo, uint32
 #pragma unroll
       for (int k = 0; k < 4; ++k)
         if (k < ksteps)
-          mma_ss(dst, smem_desc_join(a_lo + kPa[q] * kTileStep + 2 * k, hi), smem_desc_join(b_lo + kPb[q] * kTileStep + 2 * k, hi),
-                 kIdesc1, (q > first_product<kExactA, kExactB>() || k > 0) ? 1u : 0u);
+          mma_ss(dst + (kParts && k >= 2 ? kPartCol : 0), smem_desc_join(a_lo + kPa[q] * kTileStep + 2 * k, hi),
+                 smem_desc_join(b_lo + kPb[q] * kTileStep + 2 * k, hi), kIdesc1,
+                 (q > first_product<kExactA, kExactB>() || (kParts ? k & 1 : k) > 0) ? 1u : 0u);
 }
 // MMA1 of every tile.  kXIsA: the tile is A (query side: tokens x NF features), else W^T is (key side: features x tokens).
 template <bool kXIsA, int NF, bool kExactW>
@@ -757,6 +760,13 @@ __device__ __forceinline__ void store_chunk_planes(uint32_t buf, int chunk, cons
 // Bound by latency: a tile is one chain copy -> MMA1 -> ReLU -> MMA2 -> drain with nothing of the next tile beside it but its
 // copies.  2 x 4 x 4096, d = 32, m = 128 (two tiles a CTA): queries 15 us, keys some 22; the backward of 8 x 4 x 1024 92 -> 65 us.
 // TMEM: keys: A and its planes 192, G and its planes 192; queries: A 128, G 192; then two accumulators of 64.
+// With 64 features G has room for two accumulators of its own, of 32 columns of Y each: chains of two steps, as long as those of
+// O and dS', lose the same in the mean.  phi . (G + c z') is zero for every token, the two terms being of opposite signs, and so is the
+// sum of phi (G + dz') over all keys and features: the gate's gradients, which are sums of such terms by bands, hold the
+// difference of the two losses many times over.  dgate_w, domega against 64 bits, medians of 20 seeds, with one chain of four, two of
+// two, FFMA, in 1e-6: bf16 60 x 2 x 900 2.6 5.1, 1.2 1.2, 0.6 0.9; 300 x 260 2.7 2.8, 1.1 1.2, 0.7 0.6; 1 x 2 x 20001 0.8 1.1, 0.7 0.7, 0.6
+// 0.6; fp32 300 x 260 3.3 3.5, 1.4 1.3, 0.6 0.7.  (Another constant than kCut for G: worse on either side.)  Training steps
+// 14 x 21903, bf16 447.3 -> 449.1 us, 53 x 4 x 355 204.0 -> 206.1.
 // TG: type of dV.
 template <bool kKeys, typename T, typename TG, int NF>
 __global__ void __launch_bounds__(kXThreads, 1)
@@ -771,6 +781,7 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
   constexpr uint32_t kG = kKeys ? kBufCols : 128, kAcc = kG + kBufCols;
   constexpr int kPer = kKeys ? 2 : 1;   // contractions of a tile
   constexpr int kHalf = NF / 2, kH = NF / 64;   // features of a group of warps, and 32 at a time
+  constexpr bool kParts = NF <= (int)kPartCol;
   YBars* bars = reinterpret_cast<YBars*>(smem + SL::bars);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int chunk = blockIdx.x, slab = blockIdx.y, slabs = gridDim.y;
@@ -838,7 +849,7 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
       if (!mbar_wait(&bars->y_full, t & 1, abort_flag, status, kErrXMma)) break;
       if (t > 0 && !mbar_wait(&bars->g_done, (t - 1) & 1, abort_flag, status, kErrXMma)) break;
       tc_fence_after_sync();
-      issue_planes<NF, kExact<T>, false>(tmem + kG, y_lo, s_lo, ksteps, hi);
+      issue_planes<NF, kExact<T>, false, kParts>(tmem + kG, y_lo, s_lo, ksteps, hi);
       mma_commit(&bars->g_full);
       mma_commit(&bars->y_empty);
     }
@@ -899,10 +910,19 @@ k_tcx_bwd(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUt
         tmem_ld_wait();
         reg_fence32(r);
         float v[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = put_back(__uint_as_float(r[j]));
+        if (kParts && d > 32) {
+          tmem_ld32(lanes + kG + kPartCol + kHalf * g + 32 * h, r);
+          tmem_ld_wait();
+          reg_fence32(r);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] += put_back(__uint_as_float(r[j]));
+        }
         const float* z = zs + kHalf * g + 32 * h;
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
-          const float x = put_back(__uint_as_float(r[j]));
+          const float x = v[j];
           const float y = kKeys ? x + z[j] : fmaf(c, z[j], x) * inv;
           v[j] = ((on[h] >> j) & 1u) ? y : 0.f;
         }
